@@ -7,15 +7,7 @@
 #include <mutex>
 
 #include "spechub.h"
-#include "spechub_common.cuh"
-#include "spechub_stream.cuh"
-#include "spechub_lean.cuh"
-#include "spechub_kary.cuh"
-#include "spechub_fused.cuh"
-#include "spechub_resident.cuh"
-#include "spechub_resident_kary.cuh"
-#include "spechub_shard.cuh"
-#include "spechub_shard_rrs.cuh"
+#include "spechub_launch.h"
 
 extern "C" size_t spechub_draft_stats_bytes(const spechub_desc *desc);
 
@@ -73,16 +65,6 @@ RowArgs base_args(const spechub_desc *d) {
     return a;
 }
 
-// The lean kernels take bf16 rows whose starts are 16-byte aligned and whose length is a
-// multiple of 8 and large enough to keep 512 threads busy.
-constexpr int kLeanDraftThreads = 128;
-constexpr int kLeanThreads = 256;  // 4 CTAs per SM measured best (256/512/1024: 1.54/1.65/1.87 ms)
-// Verification from draft statistics on shorter rows: 8 CTAs of 128 threads per SM overlap the fixed work of
-// a row (reductions, tests, draws) better (V = 32000, 3840 rows: SpecHub 0.180 -> 0.158 ms, RRS 0.230 ->
-// 0.205 ms; 64 threads: 0.171 ms; on V = 128256 the 256-thread CTA stays ahead, 1.02 against 1.06 ms).
-constexpr int kLeanSmallThreads = 128;
-constexpr int kLeanSmallVocab = 65536;
-
 // CTAs per row.  With 4 CTAs per SM and 148 SMs, 592/CS rows are between their first and second
 // read at any time; at CS = 4 on V = 128256 that fits L2 (DRAM reads drop from 2.0x to 1.0x the
 // algorithmic bytes) but the per-CTA fixed work grows 4x, and the two cancel (1.6 vs 1.8 ms).
@@ -95,214 +77,19 @@ int lean_split(const spechub_desc *d) {
     return 0;
 }
 
-constexpr int kMaxDevices = 64;
-std::mutex g_attr_mutex;
-
-template <class K, class... Args>
-int launch_group(K kern, int cs, unsigned rows, cudaStream_t s, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at; cfg.numAttrs = cs > 1 ? 1 : 0;
-    cfg.gridDim = dim3(rows * cs); cfg.blockDim = dim3(kLeanThreads); cfg.dynamicSmemBytes = 0; cfg.stream = s;
-    return cudaLaunchKernelEx(&cfg, kern, args...) == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH;
-}
-
-template <int CS>
-int launch_lean_verify_cs(int method, const RowArgs &a, unsigned rows, cudaStream_t s) {
-    if (method == kSpecHub) return launch_group(lean_verify_kernel<kSpecHub, kLeanThreads, CS>, CS, rows, s, a);
-    if (method == kRRS) return launch_group(lean_verify_kernel<kRRS, kLeanThreads, CS>, CS, rows, s, a);
-    return launch_group(lean_verify_kernel<kRRSw, kLeanThreads, CS>, CS, rows, s, a);
-}
-// The leaf rows of an unsplit call (same CTA shape as the draft step).
-int launch_lean_leaf(const RowArgs &a, const NodeOutPtrs *outs, int n_out, unsigned rows, cudaStream_t s) {
-    LeafArgs la = {};
-    la.r = a;
-    la.n_out = n_out;
-    for (int m = 0; m < n_out; ++m) la.out[m] = outs[m];
-    lean_leaf_kernel<kLeanDraftThreads><<<rows, kLeanDraftThreads, 0, s>>>(la);
-    return cudaGetLastError() == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH;
-}
-
-// One CTA per row, the passes fed by per-warp rings of bulk copies (spechub_ring.cuh).
-template <int METHOD>
-int launch_lean_verify_ring(const RowArgs &a, unsigned rows, cudaStream_t s) {
-    auto kern = lean_verify_kernel<METHOD, kLeanThreads, 1, true>;
-    constexpr int smem = kLeanThreads / 32 * kRingWarpBytes;
-    static bool configured[kMaxDevices] = {};
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return SPECHUB_ERR_LAUNCH;
-    {
-        std::lock_guard<std::mutex> lock(g_attr_mutex);
-        if (!configured[dev]) {
-            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
-                cudaGetLastError();
-                return SPECHUB_ERR_LAUNCH;
-            }
-            configured[dev] = true;
-        }
-    }
-    kern<<<rows, kLeanThreads, smem, s>>>(a);
-    return cudaGetLastError() == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH;
-}
-
-int launch_lean_verify(int method, int cs, const RowArgs &a, unsigned rows, cudaStream_t s) {
-    if (cs == 4) return launch_lean_verify_cs<4>(method, a, rows, s);
-    if (cs == 2) return launch_lean_verify_cs<2>(method, a, rows, s);
-    if (a.node_kind) {
-        const NodeOutPtrs o = {a.accept_idx, a.token, a.hub, a.beta, a.rate, a.status};
-        const int lrc = launch_lean_leaf(a, &o, 1, rows, s);
-        if (lrc != SPECHUB_OK) return lrc;
-    }
-    if (cs == 0 && a.draft_stats_in) {   // the draft row's statistics come from the draft step
-        if (a.vocab <= kLeanSmallVocab) {
-            if (method == kSpecHub) lean_verify_kernel<kSpecHub, kLeanSmallThreads, 1, false, true><<<rows, kLeanSmallThreads, 0, s>>>(a);
-            else if (method == kRRS) lean_verify_kernel<kRRS, kLeanSmallThreads, 1, false, true><<<rows, kLeanSmallThreads, 0, s>>>(a);
-            else lean_verify_kernel<kRRSw, kLeanSmallThreads, 1, false, true><<<rows, kLeanSmallThreads, 0, s>>>(a);
-        } else
-        if (method == kSpecHub) lean_verify_kernel<kSpecHub, kLeanThreads, 1, false, true><<<rows, kLeanThreads, 0, s>>>(a);
-        else if (method == kRRS) lean_verify_kernel<kRRS, kLeanThreads, 1, false, true><<<rows, kLeanThreads, 0, s>>>(a);
-        else lean_verify_kernel<kRRSw, kLeanThreads, 1, false, true><<<rows, kLeanThreads, 0, s>>>(a);
-        return cudaGetLastError() == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH;
-    }
-    if (cs == 1 || method == kSpecHub) return launch_lean_verify_cs<1>(method, a, rows, s);
-    if (method == kRRS) return launch_lean_verify_ring<kRRS>(a, rows, s);
-    return launch_lean_verify_ring<kRRSw>(a, rows, s);
-}
-int launch_lean_draft(int method, int cs, const RowArgs &a, unsigned rows, cudaStream_t s) {
-    if (cs == 4) return launch_group(lean_draft_kernel<kLeanThreads, 4>, 4, rows, s, a, method);
-    if (cs == 2) return launch_group(lean_draft_kernel<kLeanThreads, 2>, 2, rows, s, a, method);
-    // one CTA per row (cs 0 or 1): 128 threads, 8 CTAs per SM measured best for the single-pass draft step
-    // (64 / 128 / 256 / 512 threads: 0.41 / 0.36 / 0.38 / 0.52 ms on V = 128256; 0.078 / 0.081 / 0.102 /
-    // 0.165 ms on V = 32000)
-    lean_draft_ck_kernel<kLeanDraftThreads><<<rows, kLeanDraftThreads, 0, s>>>(a, method);
-    return cudaGetLastError() == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH;
-}
-
+// The lean kernels take bf16 rows whose starts are 16-byte aligned and whose length is a multiple of 8 and
+// large enough to keep a CTA's threads busy.
 bool lean_ok(const spechub_desc *d, bool aligned) {
     return d->dtype == SPECHUB_BF16 && aligned && d->vocab % 8 == 0 && d->vocab >= 8192;
 }
 
-// ---- verification with the exponentials resident on chip ------------------------------------------
-// A row is spread over `cs` CTAs of 8 warps; every lane keeps `nb` batches of four 16-byte vectors
-// of the row pair as fp32 exponentials (tensor memory, shared memory, registers).  The smallest
-// cluster that holds the row with at most four batches per lane is taken.
-struct ResShape { int cs, nb; };
-
-bool resident_fits(const spechub_desc *d, bool aligned, ResShape *out);
-
+bool resident_fits(const spechub_desc *d, bool aligned, ResShape *out) {
+    return lean_ok(d, aligned) && resident_fits(d->vocab, out);
+}
 // two drafts per node: on request (SPECHUB_FLAG_RESIDENT)
 bool resident_shape(const spechub_desc *d, bool aligned, ResShape *out) {
     return (d->flags & SPECHUB_FLAG_RESIDENT) && resident_fits(d, aligned, out);
 }
-
-bool resident_fits(const spechub_desc *d, bool aligned, ResShape *out) {
-    if (!lean_ok(d, aligned)) return false;
-    const int nvec = d->vocab / 8;
-    for (int cs = 1; cs <= 8; cs *= 2) {
-        const int parts = cs * kResWarps;
-        const int seg = (((nvec + parts - 1) / parts) + 7) & ~7;   // vectors per warp, as the kernel cuts them
-        const int nb = (seg + 127) / 128;
-        if (nb <= kResMaxBatches) { out->cs = cs; out->nb = nb; return true; }
-    }
-    return false;
-}
-
-template <int MASK, int CS>
-int launch_resident_one(int nb, const FusedArgs &f, unsigned rows, cudaStream_t s) {
-    auto kern = resident_verify_kernel<MASK, CS>;
-    // tensor-memory columns of a CTA: two warps share each lane quarter, 32 columns per batch each
-    const uint32_t cols = nb == 1 ? 64u : nb == 2 ? 128u : 256u;
-    // Shared memory: e_q of all batches but the last.  A CTA that takes 256 columns asks for at least a
-    // third of an SM's shared memory, so that no more than two such CTAs share the SM's 512 columns.
-    int smem = (nb - 1) * 4 * 2 * kResThreads * 16;
-    if (cols == 256u && smem < 76 * 1024) smem = 76 * 1024;
-    constexpr int smem_max = (kResMaxBatches - 1) * 4 * 2 * kResThreads * 16;
-    static bool configured[kMaxDevices] = {};
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return SPECHUB_ERR_LAUNCH;
-    {
-        std::lock_guard<std::mutex> lock(g_attr_mutex);
-        if (!configured[dev]) {
-            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max) != cudaSuccess) {
-                cudaGetLastError();
-                return SPECHUB_ERR_LAUNCH;
-            }
-            configured[dev] = true;
-        }
-    }
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at; cfg.numAttrs = CS > 1 ? 1 : 0;
-    cfg.gridDim = dim3(rows * CS); cfg.blockDim = dim3(kResThreads); cfg.dynamicSmemBytes = smem; cfg.stream = s;
-    return cudaLaunchKernelEx(&cfg, kern, f, nb, cols) == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH;
-}
-
-template <int MASK>
-int launch_resident_mask(ResShape sh, const FusedArgs &f, unsigned rows, cudaStream_t s) {
-    if (sh.cs == 1) return launch_resident_one<MASK, 1>(sh.nb, f, rows, s);
-    if (sh.cs == 2) return launch_resident_one<MASK, 2>(sh.nb, f, rows, s);
-    if (sh.cs == 4) return launch_resident_one<MASK, 4>(sh.nb, f, rows, s);
-    return launch_resident_one<MASK, 8>(sh.nb, f, rows, s);
-}
-
-// Algorithm 1 with k > 2 drafts: the stages run over the exponentials kept on chip
-template <int CS>
-int launch_resident_kary_one(int nb, const KaryArgs &ka, unsigned rows, cudaStream_t s) {
-    auto kern = resident_kary_kernel<CS>;
-    const uint32_t cols = nb == 1 ? 64u : nb == 2 ? 128u : 256u;
-    int smem = (nb - 1) * 4 * 2 * kResThreads * 16;
-    if (cols == 256u && smem < 76 * 1024) smem = 76 * 1024;   // at most two CTAs of 256 columns per SM
-    constexpr int smem_max = (kResMaxBatches - 1) * 4 * 2 * kResThreads * 16;
-    static bool configured[kMaxDevices] = {};
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return SPECHUB_ERR_LAUNCH;
-    {
-        std::lock_guard<std::mutex> lock(g_attr_mutex);
-        if (!configured[dev]) {
-            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max) != cudaSuccess) {
-                cudaGetLastError();
-                return SPECHUB_ERR_LAUNCH;
-            }
-            configured[dev] = true;
-        }
-    }
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at; cfg.numAttrs = CS > 1 ? 1 : 0;
-    cfg.gridDim = dim3(rows * CS); cfg.blockDim = dim3(kResThreads); cfg.dynamicSmemBytes = smem; cfg.stream = s;
-    return cudaLaunchKernelEx(&cfg, kern, ka, nb, cols) == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH;
-}
-
-int launch_resident_kary(ResShape sh, const KaryArgs &ka, unsigned rows, cudaStream_t s) {
-    if (sh.cs == 1) return launch_resident_kary_one<1>(sh.nb, ka, rows, s);
-    if (sh.cs == 2) return launch_resident_kary_one<2>(sh.nb, ka, rows, s);
-    if (sh.cs == 4) return launch_resident_kary_one<4>(sh.nb, ka, rows, s);
-    return launch_resident_kary_one<8>(sh.nb, ka, rows, s);
-}
-
-// mask: bit m set = method m (0 SpecHub, 1 RRS, 2 RRSw) is verified; leaf rows go to lean_leaf_kernel
-int launch_resident(int mask, ResShape sh, const FusedArgs &f, unsigned rows, cudaStream_t s) {
-    if (f.r.node_kind) {
-        NodeOutPtrs outs[3];
-        int n_out = 0;
-        for (int m = 0; m < 3; ++m)
-            if (mask & (1 << m)) outs[n_out++] = f.out[m];
-        const int lrc = launch_lean_leaf(f.r, outs, n_out, rows, s);
-        if (lrc != SPECHUB_OK) return lrc;
-    }
-    if (mask == kMaskSpecHub) return launch_resident_mask<kMaskSpecHub>(sh, f, rows, s);
-    if (mask == kMaskRRS) return launch_resident_mask<kMaskRRS>(sh, f, rows, s);
-    if (mask == kMaskRRSw) return launch_resident_mask<kMaskRRSw>(sh, f, rows, s);
-    return launch_resident_mask<7>(sh, f, rows, s);
-}
-
-int launch_status() { return cudaGetLastError() == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH; }
 
 int draft_common(const spechub_desc *d, const void *draft_logits, const float *uniforms, int method,
                  int32_t *draft_tokens, int32_t *hub, float *draft_prob, uint32_t *status,
@@ -331,36 +118,10 @@ int draft_common(const spechub_desc *d, const void *draft_logits, const float *u
         if (method == kSpecHub) return SPECHUB_ERR_SHAPE;
         KaryArgs ka;
         ka.r = a; ka.k = d->k; ka.without_replacement = (method == kRRSw);
-        if (d->dtype == SPECHUB_BF16) {
-            if (al) kary_draft_kernel<__nv_bfloat16, true><<<rows, th, 0, s>>>(ka);
-            else kary_draft_kernel<__nv_bfloat16, false><<<rows, th, 0, s>>>(ka);
-        } else {
-            if (al) kary_draft_kernel<float, true><<<rows, th, 0, s>>>(ka);
-            else kary_draft_kernel<float, false><<<rows, th, 0, s>>>(ka);
-        }
-    } else if (lean_ok(d, al)) {
-        const int lrc = launch_lean_draft(method, lean_split(d), a, rows, s);
-        if (lrc != SPECHUB_OK) return lrc;
-    } else if (d->dtype == SPECHUB_BF16) {
-        if (al) draft_rows_kernel<__nv_bfloat16, true><<<rows, th, 0, s>>>(a, method);
-        else draft_rows_kernel<__nv_bfloat16, false><<<rows, th, 0, s>>>(a, method);
-    } else {
-        if (al) draft_rows_kernel<float, true><<<rows, th, 0, s>>>(a, method);
-        else draft_rows_kernel<float, false><<<rows, th, 0, s>>>(a, method);
+        return launch_kary_draft(d->dtype, al, th, ka, rows, s);
     }
-    return launch_status();
-}
-
-template <int METHOD>
-void launch_verify(const spechub_desc *d, const RowArgs &a, bool al, unsigned rows, int th,
-                   cudaStream_t s) {
-    if (d->dtype == SPECHUB_BF16) {
-        if (al) verify_rows_kernel<__nv_bfloat16, true, METHOD><<<rows, th, 0, s>>>(a);
-        else verify_rows_kernel<__nv_bfloat16, false, METHOD><<<rows, th, 0, s>>>(a);
-    } else {
-        if (al) verify_rows_kernel<float, true, METHOD><<<rows, th, 0, s>>>(a);
-        else verify_rows_kernel<float, false, METHOD><<<rows, th, 0, s>>>(a);
-    }
+    if (lean_ok(d, al)) return launch_lean_draft(method, lean_split(d), a, rows, s);
+    return launch_rows_draft(d->dtype, al, th, a, method, rows, s);
 }
 
 int launch_walk(const spechub_desc *d, const spechub_node_out *no, const spechub_seq_out *so, cudaStream_t s) {
@@ -377,14 +138,9 @@ int launch_walk(const spechub_desc *d, const spechub_node_out *no, const spechub
     w.batch = d->batch;
     w.nodes = d->nodes;
     w.levels = d->levels;
-    if (d->k > 2) {
-        WalkKArgs wk;
-        wk.w = w; wk.k = d->k;
-        walk_k_kernel<<<(d->batch + 127) / 128, 128, 0, s>>>(wk);
-    } else {
-        walk_kernel<<<(d->batch + 127) / 128, 128, 0, s>>>(w);
-    }
-    return launch_status();
+    WalkKArgs wk;
+    wk.w = w; wk.k = d->k;
+    return launch_walk(wk, s);
 }
 
 int verify_common(const spechub_desc *d, const void *target_logits, const void *draft_logits,
@@ -416,35 +172,27 @@ int verify_common(const spechub_desc *d, const void *target_logits, const void *
     const int th = threads_for(d);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const bool al = rows_aligned(d, target_logits) && rows_aligned(d, draft_logits);
+    int lrc;
+    ResShape rs;
     if (d->k > 2) {
         if (method == kSpecHub) return SPECHUB_ERR_SHAPE;
         KaryArgs ka;
         ka.r = a; ka.k = d->k; ka.without_replacement = (method == kRRSw);
-        ResShape rs;
-        if (!(d->flags & 7u) && resident_fits(d, al, &rs)) {   // (a split flag asks for the streaming kernel)
-            const int lrc = launch_resident_kary(rs, ka, rows, s);
-            if (lrc != SPECHUB_OK) return lrc;
-        } else if (d->dtype == SPECHUB_BF16) {
-            if (al) kary_verify_kernel<__nv_bfloat16, true><<<rows, th, 0, s>>>(ka);
-            else kary_verify_kernel<__nv_bfloat16, false><<<rows, th, 0, s>>>(ka);
-        } else {
-            if (al) kary_verify_kernel<float, true><<<rows, th, 0, s>>>(ka);
-            else kary_verify_kernel<float, false><<<rows, th, 0, s>>>(ka);
-        }
-    } else if (ResShape rs; resident_shape(d, al, &rs)) {
+        if (!(d->flags & 7u) && resident_fits(d, al, &rs))   // (a split flag asks for the streaming kernel)
+            lrc = launch_resident_kary(rs, ka, rows, s);
+        else
+            lrc = launch_kary_verify(d->dtype, al, th, ka, rows, s);
+    } else if (resident_shape(d, al, &rs)) {
         FusedArgs f = {};
         f.r = a;
         f.tok[method] = draft_tokens;
         f.out[method] = NodeOutPtrs{a.accept_idx, a.token, a.hub, a.beta, a.rate, a.status};
-        const int lrc = launch_resident(1 << method, rs, f, rows, s);
-        if (lrc != SPECHUB_OK) return lrc;
+        lrc = launch_resident(1 << method, rs, f, rows, s);
     } else if (lean_ok(d, al)) {
-        const int lrc = launch_lean_verify(method, lean_split(d), a, rows, s);
-        if (lrc != SPECHUB_OK) return lrc;
-    } else if (method == kSpecHub) launch_verify<kSpecHub>(d, a, al, rows, th, s);
-    else if (method == kRRS) launch_verify<kRRS>(d, a, al, rows, th, s);
-    else launch_verify<kRRSw>(d, a, al, rows, th, s);
-    const int lrc = launch_status();
+        lrc = launch_lean_verify(method, lean_split(d), a, rows, s);
+    } else {
+        lrc = launch_rows_verify(d->dtype, al, th, a, method, rows, s);
+    }
     if (lrc != SPECHUB_OK) return lrc;
     return launch_walk(d, no, so, s);
 }
@@ -483,9 +231,7 @@ int compare_draft(const spechub_desc *d, const void *draft_logits, const float *
         f.dstatus[m] = status ? status[m] : nullptr;
     }
     const unsigned rows = (unsigned)(d->batch * (int64_t)d->nodes);
-    // same CTA shape as lean_draft_ck_kernel: the results are to be the same bit for bit
-    fused_draft_kernel<kLeanDraftThreads><<<rows, kLeanDraftThreads, 0, static_cast<cudaStream_t>(stream)>>>(f, hub, draft_prob);
-    return launch_status();
+    return launch_fused_draft(f, hub, draft_prob, rows, static_cast<cudaStream_t>(stream));
 }
 
 int compare_verify(const spechub_desc *d, const void *target_logits, const void *draft_logits,
@@ -529,15 +275,8 @@ int compare_verify(const spechub_desc *d, const void *target_logits, const void 
             const int llrc = launch_lean_leaf(f.r, f.out, 3, rows, s);
             if (llrc != SPECHUB_OK) return llrc;
         }
-        if (draft_stats && lean_split(d) == 0) {
-            f.r.draft_stats_in = draft_stats;
-            // (the CTA shape of the per-method kernels, whose results these are bit for bit)
-            if (d->vocab <= kLeanSmallVocab) fused_verify_kernel<kLeanSmallThreads, true><<<rows, kLeanSmallThreads, 0, s>>>(f);
-            else fused_verify_kernel<kLeanThreads, true><<<rows, kLeanThreads, 0, s>>>(f);
-        } else {
-            fused_verify_kernel<kLeanThreads><<<rows, kLeanThreads, 0, s>>>(f);
-        }
-        lrc = launch_status();
+        if (lean_split(d) == 0) f.r.draft_stats_in = draft_stats;
+        lrc = launch_fused_verify(f, rows, s);
     }
     for (int m = 0; m < 3 && lrc == SPECHUB_OK && so; ++m) lrc = launch_walk(d, &no[m], &so[m], s);
     return lrc;
@@ -563,35 +302,34 @@ ShardArgs shard_args(const spechub_desc *d, const spechub_shard *sh) {
     return a;
 }
 
-enum ShardPhase { kPhaseStats, kPhaseSums, kPhaseDecide, kPhaseDraft, kPhaseRrsSums, kPhaseRrsDecide, kPhaseRrsDraft };
-
-template <typename LT, bool AL>
-void launch_shard_phase(int phase, const ShardArgs &a, unsigned rows, int th, cudaStream_t s) {
-    if (phase == kPhaseStats) shard_stats_kernel<LT, AL><<<rows, th, 0, s>>>(a);
-    else if (phase == kPhaseSums) shard_sums_kernel<LT, AL><<<rows, th, 0, s>>>(a);
-    else if (phase == kPhaseDecide) shard_decide_kernel<LT, AL><<<rows, th, 0, s>>>(a);
-    else if (phase == kPhaseDraft) shard_draft_kernel<LT, AL><<<rows, th, 0, s>>>(a);
-    else if (phase == kPhaseRrsSums) rrs_shard_sums_kernel<LT, AL><<<rows, th, 0, s>>>(a);
-    else if (phase == kPhaseRrsDecide) rrs_shard_decide_kernel<LT, AL><<<rows, th, 0, s>>>(a);
-    else rrs_shard_draft_kernel<LT, AL><<<rows, th, 0, s>>>(a);
-}
-
 int run_shard_phase(int phase, const spechub_desc *d, const ShardArgs &a, void *stream) {
     const unsigned rows = (unsigned)a.rows;
     const int th = threads_for(d);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const bool al = (!a.r.target || rows_aligned(d, a.r.target)) && (!a.r.draft || rows_aligned(d, a.r.draft));
-    if (d->dtype == SPECHUB_BF16) {
-        if (al) launch_shard_phase<__nv_bfloat16, true>(phase, a, rows, th, s);
-        else launch_shard_phase<__nv_bfloat16, false>(phase, a, rows, th, s);
-    } else {
-        if (al) launch_shard_phase<float, true>(phase, a, rows, th, s);
-        else launch_shard_phase<float, false>(phase, a, rows, th, s);
-    }
-    return launch_status();
+    return launch_shard_phase(phase, d->dtype, al, th, a, rows, s);
 }
 
 }  // namespace
+
+namespace spechub {
+
+int allow_smem(const void *kern, int bytes, bool *configured) {
+    static std::mutex mutex;
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return SPECHUB_ERR_LAUNCH;
+    std::lock_guard<std::mutex> lock(mutex);
+    if (!configured[dev]) {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            return SPECHUB_ERR_LAUNCH;
+        }
+        configured[dev] = true;
+    }
+    return SPECHUB_OK;
+}
+
+}  // namespace spechub
 
 extern "C" {
 
@@ -773,8 +511,7 @@ int spechub_shard_draft_finish(const spechub_desc *desc, const spechub_shard *sh
     ShardArgs a = shard_args(desc, shard);
     a.gstats = gathered_stats; a.cand = cand_max;
     a.r.draft_tokens_out = draft_tokens; a.r.hub = hub; a.r.status = status;
-    shard_draft_finish_kernel<<<(unsigned)((a.rows + 127) / 128), 128, 0, static_cast<cudaStream_t>(stream)>>>(a);
-    return launch_status();
+    return launch_shard_draft_finish(false, a, static_cast<cudaStream_t>(stream));
 }
 
 int rrs_shard_sums(const spechub_desc *desc, const spechub_shard *shard, int without_replacement,
@@ -841,8 +578,7 @@ int rrs_shard_draft_finish(const spechub_desc *desc, const spechub_shard *shard,
     a.without_replacement = without_replacement;
     a.gstats = gathered_stats; a.cand = cand_max;
     a.r.draft_tokens_out = draft_tokens; a.r.status = status;
-    rrs_shard_draft_finish_kernel<<<(unsigned)((a.rows + 127) / 128), 128, 0, static_cast<cudaStream_t>(stream)>>>(a);
-    return launch_status();
+    return launch_shard_draft_finish(true, a, static_cast<cudaStream_t>(stream));
 }
 
 size_t spechub_workspace_bytes(const spechub_desc *desc) {

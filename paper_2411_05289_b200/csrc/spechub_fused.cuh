@@ -15,14 +15,6 @@
 
 namespace spechub {
 
-struct FusedArgs {
-    RowArgs r;                 // target, draft, uniforms, temperature, node_kind, shape
-    const int32_t *tok[3];     // draft tokens of SpecHub, RRS, RRSw (verify)
-    int32_t *tok_out[3];       // (draft)
-    NodeOutPtrs out[3];
-    uint32_t *dstatus[3];      // draft status
-};
-
 __device__ __forceinline__ void write_node3(const NodeOutPtrs &p, long long r, const NodeResult &o, bool tok_elsewhere) {
     p.accept_idx[r] = o.accept_idx;
     if (!tok_elsewhere) p.token[r] = o.token;

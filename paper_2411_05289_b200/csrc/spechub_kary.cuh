@@ -18,13 +18,7 @@
 
 namespace spechub {
 
-constexpr int kMaxK = SPECHUB_MAX_K;
 
-struct KaryArgs {
-    RowArgs r;
-    int k;
-    int without_replacement;
-};
 
 // Is token y one of x[0..n)?
 __device__ __forceinline__ bool in_set(const int *x, int n, int y) {
@@ -269,37 +263,6 @@ __global__ void __launch_bounds__(512) kary_verify_kernel(KaryArgs A) {
         token = tok;
     }
     write_out();
-}
-
-// ---- tree walk with k children per node -------------------------------------------------------------
-struct WalkKArgs {
-    WalkArgs w;
-    int k;
-};
-__global__ void walk_k_kernel(WalkKArgs A) {
-    const WalkArgs &a = A.w;
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= a.batch) return;
-    int n = 0, acc = 0, emitted = 0, step = 0;
-    for (; step < a.levels && n >= 0 && n < a.nodes; ++step) {
-        const long long r = static_cast<long long>(b) * a.nodes + n;
-        const int tok = a.token[r];
-        if (a.path_nodes) a.path_nodes[static_cast<long long>(b) * a.levels + step] = n;
-        if (a.path_tokens) a.path_tokens[static_cast<long long>(b) * a.levels + step] = tok;
-        if (tok < 0) { ++step; break; }
-        ++emitted;
-        if (a.node_kind && a.node_kind[n] == SPECHUB_NODE_LEAF) { ++step; break; }
-        const int idx = a.accept_idx[r];
-        if (idx < 0 || idx >= A.k) { ++step; break; }
-        ++acc;
-        n = a.child ? a.child[A.k * n + idx] : A.k * n + 1 + idx;
-    }
-    for (; step < a.levels; ++step) {
-        if (a.path_nodes) a.path_nodes[static_cast<long long>(b) * a.levels + step] = -1;
-        if (a.path_tokens) a.path_tokens[static_cast<long long>(b) * a.levels + step] = -1;
-    }
-    if (a.n_accepted) a.n_accepted[b] = acc;
-    if (a.n_emitted) a.n_emitted[b] = emitted;
 }
 
 }  // namespace spechub

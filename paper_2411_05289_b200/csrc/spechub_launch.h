@@ -1,0 +1,44 @@
+// Launch functions of the kernel families, one translation unit each (they compile in parallel).  Every
+// function enqueues on `s` and returns a SPECHUB_* code.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "spechub_args.cuh"
+
+namespace spechub {
+
+constexpr int kMaxDevices = 64;
+
+inline int launch_status() { return cudaGetLastError() == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH; }
+
+// Raise a kernel's dynamic shared memory limit once per device.  `configured`: one flag per device, kept by
+// the caller (one array per kernel).
+int allow_smem(const void *kern, int bytes, bool *configured);
+
+// general kernels (any shape); th = threads per row
+int launch_rows_draft(int dtype, bool aligned, int th, const RowArgs &a, int method, unsigned rows, cudaStream_t s);
+int launch_rows_verify(int dtype, bool aligned, int th, const RowArgs &a, int method, unsigned rows, cudaStream_t s);
+int launch_kary_draft(int dtype, bool aligned, int th, const KaryArgs &a, unsigned rows, cudaStream_t s);
+int launch_kary_verify(int dtype, bool aligned, int th, const KaryArgs &a, unsigned rows, cudaStream_t s);
+int launch_walk(const WalkKArgs &w, cudaStream_t s);
+
+// large-vocabulary kernels; cs = CTAs per row asked for (0: the library's choice)
+int launch_lean_draft(int method, int cs, const RowArgs &a, unsigned rows, cudaStream_t s);
+int launch_lean_leaf(const RowArgs &a, const NodeOutPtrs *outs, int n_out, unsigned rows, cudaStream_t s);
+int launch_lean_verify(int method, int cs, const RowArgs &a, unsigned rows, cudaStream_t s);
+int launch_fused_draft(const FusedArgs &f, int32_t *hub, float *draft_prob, unsigned rows, cudaStream_t s);
+int launch_fused_verify(const FusedArgs &f, unsigned rows, cudaStream_t s);
+
+// exponentials resident on chip.  A row is spread over `cs` CTAs; every lane keeps `nb` batches of vectors.
+struct ResShape { int cs, nb; };
+bool resident_fits(int vocab, ResShape *out);
+int launch_resident(int mask, ResShape sh, const FusedArgs &f, unsigned rows, cudaStream_t s);
+int launch_resident_kary(ResShape sh, const KaryArgs &ka, unsigned rows, cudaStream_t s);
+
+// vocabulary-sharded phases
+enum ShardPhase { kPhaseStats, kPhaseSums, kPhaseDecide, kPhaseDraft, kPhaseRrsSums, kPhaseRrsDecide, kPhaseRrsDraft };
+int launch_shard_phase(int phase, int dtype, bool aligned, int th, const ShardArgs &a, unsigned rows, cudaStream_t s);
+int launch_shard_draft_finish(bool rrs, const ShardArgs &a, cudaStream_t s);
+
+}  // namespace spechub

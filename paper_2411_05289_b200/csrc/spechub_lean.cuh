@@ -601,7 +601,7 @@ __device__ __forceinline__ float slice_mass(const LeanShared &sh, int r, const R
 // Draw inside this CTA's slice from softmax(row) without token `excl`, target t (row scale,
 // relative to the start of the slice).  sh.wmass[r] holds the per-warp sums of the slice on the
 // slice's own scale with the slice argmax left out.
-__device__ int lean_sample_slice(const Geo &g, const __nv_bfloat16 *row, float k, const RowStat &st,
+__device__ inline int lean_sample_slice(const Geo &g, const __nv_bfloat16 *row, float k, const RowStat &st,
                                  int excl, float t, int r, LeanShared &sh) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int locarg = sh.x_idx[r];
@@ -785,7 +785,7 @@ __device__ __forceinline__ void lean_pass_a_ck(const uint4 *rq, int lo, int hi, 
 // Inverse-CDF draw from softmax(row) without token `excl` (excl < 0: nothing left out) over the
 // checkpoint sub-blocks.  C = the row's exponent shift.  Returns to every thread the token, -1 if
 // nothing has mass.  Called by all threads of the CTA, after the checkpoints are visible.
-__device__ int lean_ck_sample(const Geo &g, const __nv_bfloat16 *row, float k, float C, int CK, int excl,
+__device__ inline int lean_ck_sample(const Geo &g, const __nv_bfloat16 *row, float k, float C, int CK, int excl,
                               float u, LeanCkShared &sh) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nslot = g.nwarps * kLeanCk;
@@ -876,17 +876,6 @@ __device__ int lean_ck_sample(const Geo &g, const __nv_bfloat16 *row, float k, f
 // pass A over p with checkpoints, then the sub-block sampler.  CTAs of verifying rows leave at
 // once; the verification kernels skip the leaf rows.  Up to three output sets receive the result
 // (the three-method call: the methods share u_res, hence the bonus token).
-struct NodeOutPtrs {
-    int32_t *accept_idx, *token, *hub;
-    float *beta, *rate;
-    uint32_t *status;
-};
-struct LeafArgs {
-    RowArgs r;
-    NodeOutPtrs out[3];
-    int n_out;
-};
-
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_leaf_kernel(LeafArgs A) {
     __shared__ LeanCkShared sh;

@@ -18,24 +18,6 @@
 
 namespace spechub {
 
-constexpr int kShardRecord = 8;  // floats per row in a phase output
-
-struct ShardArgs {
-    RowArgs r;             // r.target / r.draft: this rank's slices; r.vocab: their width
-    int rank, nranks, id_offset, vocab_total;
-    long long rows;
-    const float *gstats;   // [nranks][rows][8]: (ml, sx, idx) of p then of q, per rank
-    const float *gsums;    // [nranks][rows][8]
-    const float *gw2;      // [nranks][rows][8] (RRS / RRSw: second-stage residual masses)
-    int without_replacement;
-    const int32_t *x1_known;  // RRSw draft, second round: [rows][2] candidates after the maximum
-    const float *ex1_known;   // ... and the exponential of x1's logit, [rows]
-    float *ex1_out;           // first round: that exponential from x1's owner, -1 elsewhere
-    const int32_t *cand;   // [rows][2] after the element-wise maximum over ranks
-    float *out;            // [rows][8] phase output
-    int32_t *cand_out;     // [rows][2]
-};
-
 struct ShardStat {
     float ml, C, sx;
     float own;   // the row argmax's own term 2^(k ml - C)

@@ -7,47 +7,14 @@
 
 #include "spechub.h"
 #include "spechub_common.cuh"
+#include "spechub_args.cuh"
 
 namespace spechub {
 
-struct RowArgs {
-    const void *target;   // [B][N][V] (verify only)
-    const void *draft;    // [B][N][V]
-    const float *uniforms;  // [B][N][5]
-    const int32_t *draft_tokens_in;  // verify: [B][N][2]
-    int32_t *draft_tokens_out;       // draft: [B][N][2]
-    int32_t *hub;
-    float *draft_prob;
-    int32_t *accept_idx;
-    int32_t *token;
-    float *beta;
-    float *rate;
-    uint32_t *status;
-    const float *temperature_per_seq;
-    const uint8_t *node_kind;
-    float temperature;
-    int nodes, vocab;
-    long long stride_seq, stride_node;
-    // per-row statistics of the draft logits, handed from the draft step to verification: [B][N] DraftStat
-    void *draft_stats_out;       // draft step, may be NULL
-    const void *draft_stats_in;  // verification through a *_stats entry point
-};
-
-// What the draft step knows about a row of draft logits once it has read it, and what verification would
-// otherwise have to read the row for a second time to find out (Section 4: a = argmax q; q(a); 1 - q(a)).
-struct DraftStat {
-    float ml;       // the row's maximum logit
-    float sx;       // sum over ids != argmax of 2^(k l - k ml), k = log2(e) / T
-    int idx;        // argmax, lowest id on ties
-    unsigned tag;   // kDraftStatTag ^ bits of k: a record of another library version or temperature is refused
-};
-constexpr unsigned kDraftStatTag = 0x51a75u << 12;
 // a draft kernel that keeps no statistics leaves a record that no verification accepts
 __device__ __forceinline__ void void_draft_stat(const RowArgs &a, long long r) {
     if (a.draft_stats_out) static_cast<uint4 *>(a.draft_stats_out)[r] = make_uint4(0u, 0u, 0u, 0u);
 }
-
-enum Method { kSpecHub = 0, kRRS = 1, kRRSw = 2 };
 
 struct WarpPart {  // per-warp (max, argmax, sum without the argmax) of one row
     float ml[kMaxWarps], sx[kMaxWarps];
@@ -493,41 +460,6 @@ __global__ void __launch_bounds__(512) verify_rows_kernel(RowArgs a) {
         }
     }
     if (threadIdx.x == 0) write_node(a, r, o);
-}
-
-// ------------------------------------------------------------------------------------------------
-// Tree walk (Figure 2): one thread per sequence.
-// ------------------------------------------------------------------------------------------------
-struct WalkArgs {
-    const int32_t *accept_idx, *token, *child;
-    const uint8_t *node_kind;
-    int32_t *n_accepted, *n_emitted, *path_nodes, *path_tokens;
-    int batch, nodes, levels;
-};
-
-__global__ void walk_kernel(WalkArgs a) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= a.batch) return;
-    int n = 0, acc = 0, emitted = 0, step = 0;
-    for (; step < a.levels && n >= 0 && n < a.nodes; ++step) {
-        const long long r = static_cast<long long>(b) * a.nodes + n;
-        const int tok = a.token[r];
-        if (a.path_nodes) a.path_nodes[static_cast<long long>(b) * a.levels + step] = n;
-        if (a.path_tokens) a.path_tokens[static_cast<long long>(b) * a.levels + step] = tok;
-        if (tok < 0) { ++step; break; }
-        ++emitted;
-        if (a.node_kind && a.node_kind[n] == SPECHUB_NODE_LEAF) { ++step; break; }
-        const int idx = a.accept_idx[r];
-        if (idx < 0 || idx > 1) { ++step; break; }   // (a caller-supplied index outside {0, 1} ends the walk)
-        ++acc;
-        n = a.child ? a.child[2 * n + idx] : 2 * n + 1 + idx;
-    }
-    for (; step < a.levels; ++step) {
-        if (a.path_nodes) a.path_nodes[static_cast<long long>(b) * a.levels + step] = -1;
-        if (a.path_tokens) a.path_tokens[static_cast<long long>(b) * a.levels + step] = -1;
-    }
-    if (a.n_accepted) a.n_accepted[b] = acc;
-    if (a.n_emitted) a.n_emitted[b] = emitted;
 }
 
 }  // namespace spechub
