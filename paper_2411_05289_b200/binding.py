@@ -1,12 +1,15 @@
-"""ctypes binding of ``libspechub.so``: argument marshalling only.
+"""Binding of ``libspechub.so``: argument marshalling only.
 
 Function names and argument meaning follow ``include/spechub.h``.  Tensors are
-torch CUDA tensors; outputs are allocated here with torch (device memory is the
-only thing torch is used for) and returned in small dicts.
+torch CUDA tensors; outputs are allocated with torch (device memory is the only
+thing torch is used for) and returned in small dicts.  The calls of a decoding
+iteration are marshalled by a CPython module (``csrc/native_binding.cpp``);
+ctypes serves the rest of the C ABI.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from dataclasses import dataclass
 from typing import Optional
@@ -242,17 +245,6 @@ def _stream_ptr(stream):
     return ctypes.c_void_p(s.cuda_stream)
 
 
-def _hold(tensors, stream):
-    """Temporaries of a call (a converted temperature vector, a workspace) are freed when the Python
-    call returns, while the kernels may still be queued.  On the current stream torch's allocator
-    orders the reuse after them; on any other stream it has to be told."""
-    if stream is None:
-        return
-    for t in tensors:
-        if t is not None:
-            t.record_stream(stream)
-
-
 def _desc(logits: torch.Tensor, tree: Tree, temperature) -> tuple:
     if logits.dim() != 3 or logits.stride(2) != 1:
         raise ValueError("logits must be [batch][nodes][vocab] with a contiguous vocabulary axis")
@@ -312,80 +304,47 @@ def _need_k2(tree):
         raise ValueError("SpecHub takes exactly two drafts per node")
 
 
-def _alloc_stats(lib, d, dev):
-    """The caller-owned buffer of per-row draft statistics (16 bytes per row, opaque)."""
-    n = lib.spechub_draft_stats_bytes(ctypes.byref(d))
-    return torch.empty(max(n, 16) // 4, dtype=torch.int32, device=dev)
+def _load_native():
+    """The CPython module over ``libspechub.so`` (built when it is missing or stale)."""
+    global _native
+    load_library()
+    path = _build.build_binding()
+    spec = importlib.util.spec_from_file_location("_spechub_native", path)
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    mod.set_error(SpecHubError)
+    _native = mod
+    return mod
+
+
+_native = None
+_SPECHUB, _RRS, _RRSW = 0, 1, 2
 
 
 def spechub_draft_sample(draft_logits, uniforms, tree: Tree, temperature=1.0, stream=None):
     """Draw the k = 2 SpecHub drafts of every node.  Returns dict(tokens, hub, prob, status)."""
-    return _spechub_draft(draft_logits, uniforms, tree, temperature, stream, False)
+    return (_native or _load_native()).draft(_SPECHUB, draft_logits, uniforms, tree, temperature, stream, _split, False)
 
 
 def spechub_draft_sample_stats(draft_logits, uniforms, tree: Tree, temperature=1.0, stream=None):
-    """``spechub_draft_sample`` that also leaves the per-row draft statistics (key ``stats``) for
-    ``spechub_verify_tree_stats``."""
-    return _spechub_draft(draft_logits, uniforms, tree, temperature, stream, True)
-
-
-def _spechub_draft(draft_logits, uniforms, tree, temperature, stream, with_stats):
-    lib = load_library()
-    _need_k2(tree)
-    d, keep = _desc(draft_logits, tree, temperature)
-    B, N, _ = draft_logits.shape
-    dev = draft_logits.device
-    _check_uniforms(uniforms, B, N, dev)
-    tokens = torch.empty((B, N, 2), dtype=torch.int32, device=dev)
-    hub = torch.empty((B, N), dtype=torch.int32, device=dev)
-    prob = torch.empty((B, N, 2), dtype=torch.float32, device=dev)
-    status = torch.empty((B, N), dtype=torch.int32, device=dev)
-    out = dict(tokens=tokens, hub=hub, prob=prob, status=status)
-    if with_stats:
-        out["stats"] = _alloc_stats(lib, d, dev)
-        _check(lib.spechub_draft_sample_stats(ctypes.byref(d), _ptr(draft_logits), _ptr(uniforms), _ptr(tokens),
-                                              _ptr(hub), _ptr(prob), _ptr(status), _ptr(out["stats"]),
-                                              _stream_ptr(stream)))
-    else:
-        _check(lib.spechub_draft_sample(ctypes.byref(d), _ptr(draft_logits), _ptr(uniforms), _ptr(tokens),
-                                        _ptr(hub), _ptr(prob), _ptr(status), _stream_ptr(stream)))
-    _hold(keep + list(out.values()), stream)
-    return out
+    """``spechub_draft_sample`` that also leaves the per-row draft statistics (key ``stats``: 16 bytes per
+    row, opaque) for ``spechub_verify_tree_stats``."""
+    return (_native or _load_native()).draft(_SPECHUB, draft_logits, uniforms, tree, temperature, stream, _split, True)
 
 
 def rrs_draft_sample(draft_logits, uniforms, tree: Tree, without_replacement: bool, temperature=1.0,
                      stream=None):
     """Draw the k = tree.k RRS / RRSw drafts of every node.  Returns dict(tokens, status)."""
-    return _rrs_draft(draft_logits, uniforms, tree, without_replacement, temperature, stream, False)
+    return (_native or _load_native()).draft(_RRSW if without_replacement else _RRS, draft_logits, uniforms, tree,
+                                             temperature, stream, _split, False)
 
 
 def rrs_draft_sample_stats(draft_logits, uniforms, tree: Tree, without_replacement: bool, temperature=1.0,
                            stream=None):
     """``rrs_draft_sample`` that also leaves the per-row draft statistics (key ``stats``) for
     ``rrs_verify_tree_stats``."""
-    return _rrs_draft(draft_logits, uniforms, tree, without_replacement, temperature, stream, True)
-
-
-def _rrs_draft(draft_logits, uniforms, tree, without_replacement, temperature, stream, with_stats):
-    lib = load_library()
-    d, keep = _desc(draft_logits, tree, temperature)
-    B, N, _ = draft_logits.shape
-    dev = draft_logits.device
-    _check_uniforms(uniforms, B, N, dev, tree.k)
-    tokens = torch.empty((B, N, tree.k), dtype=torch.int32, device=dev)
-    status = torch.empty((B, N), dtype=torch.int32, device=dev)
-    out = dict(tokens=tokens, status=status)
-    if with_stats:
-        out["stats"] = _alloc_stats(lib, d, dev)
-        _check(lib.rrs_draft_sample_stats(ctypes.byref(d), _ptr(draft_logits), _ptr(uniforms),
-                                          int(bool(without_replacement)), _ptr(tokens), _ptr(status),
-                                          _ptr(out["stats"]), _stream_ptr(stream)))
-    else:
-        _check(lib.rrs_draft_sample(ctypes.byref(d), _ptr(draft_logits), _ptr(uniforms),
-                                    int(bool(without_replacement)), _ptr(tokens), _ptr(status),
-                                    _stream_ptr(stream)))
-    _hold(keep + list(out.values()), stream)
-    return out
+    return (_native or _load_native()).draft(_RRSW if without_replacement else _RRS, draft_logits, uniforms, tree,
+                                             temperature, stream, _split, True)
 
 
 def alloc_verify_outputs(B, N, levels, dev, k=2):
@@ -404,77 +363,39 @@ def alloc_verify_outputs(B, N, levels, dev, k=2):
     )
 
 
-def _verify(method, target_logits, draft_logits, draft_tokens, uniforms, tree, temperature, stream,
-            out, probabilities=True, stats=None, with_stats=False):
-    lib = load_library()
-    _same_layout(target_logits, draft_logits)
-    d, keep = _desc(target_logits, tree, temperature)
-    B, N, _ = target_logits.shape
-    dev = target_logits.device
-    if method == "spechub":
-        _need_k2(tree)
-    _check_uniforms(uniforms, B, N, dev, tree.k)
-    if (draft_tokens.dtype != torch.int32 or tuple(draft_tokens.shape) != (B, N, tree.k)
-            or not draft_tokens.is_contiguous() or draft_tokens.device != dev):
-        raise ValueError("draft_tokens must be a contiguous int32 [batch][nodes][k] tensor")
-    if out is None:
-        out = alloc_verify_outputs(B, N, tree.levels, dev, tree.k)
-    no = _NodeOut(*[out[k].data_ptr() if (probabilities or k not in ("beta", "rate")) else None
-                    for k in ("accept_idx", "token", "hub", "beta", "rate", "status")])
-    so = _SeqOut(*[out[k].data_ptr() for k in ("n_accepted", "n_emitted", "path_nodes", "path_tokens")])
-    ws_bytes = lib.spechub_workspace_bytes(ctypes.byref(d))
-    ws = torch.empty(ws_bytes, dtype=torch.uint8, device=dev) if ws_bytes else None
-    common = (ctypes.byref(d), _ptr(target_logits), _ptr(draft_logits), _ptr(draft_tokens), _ptr(uniforms))
-    tail = (ctypes.byref(no), ctypes.byref(so), _ptr(ws), ws_bytes, _stream_ptr(stream))
-    if with_stats:
-        need = lib.spechub_draft_stats_bytes(ctypes.byref(d))
-        if (stats is None or stats.dtype != torch.int32 or not stats.is_contiguous() or stats.device != dev
-                or stats.numel() * 4 < need):
-            raise ValueError("stats must be the tensor a *_draft_sample_stats call returned for this shape")
-        common = common[:3] + (_ptr(stats),) + common[3:]
-        if method == "spechub":
-            _check(lib.spechub_verify_tree_stats(*common, *tail))
-        else:
-            _check(lib.rrs_verify_tree_stats(*common, 1 if method == "rrsw" else 0, *tail))
-    elif method == "spechub":
-        _check(lib.spechub_verify_tree(*common, *tail))
-    else:
-        _check(lib.rrs_verify_tree(*common, 1 if method == "rrsw" else 0, *tail))
-    _hold(keep + [ws, stats] + list(out.values()), stream)
-    return out
-
-
 def spechub_verify_tree(target_logits, draft_logits, draft_tokens, uniforms, tree: Tree,
                         temperature=1.0, stream=None, out=None, probabilities=True):
     """SpecHub verification of every node and the tree walk.  Returns the dict of output
     tensors (see ``alloc_verify_outputs``); pass ``out`` to reuse buffers.  With
     ``probabilities=False`` the library is given no beta / rate buffers (their tensors are left
     untouched) and skips work that only they need."""
-    return _verify("spechub", target_logits, draft_logits, draft_tokens, uniforms, tree, temperature,
-                   stream, out, probabilities)
+    return (_native or _load_native()).verify(_SPECHUB, target_logits, draft_logits, None, draft_tokens, uniforms, tree,
+                                              temperature, stream, out, probabilities, _split, False)
 
 
 def rrs_verify_tree(target_logits, draft_logits, draft_tokens, uniforms, tree: Tree,
                     without_replacement: bool, temperature=1.0, stream=None, out=None, probabilities=True):
     """RRS / RRSw verification of every node and the tree walk."""
-    return _verify("rrsw" if without_replacement else "rrs", target_logits, draft_logits, draft_tokens,
-                   uniforms, tree, temperature, stream, out, probabilities)
+    return (_native or _load_native()).verify(_RRSW if without_replacement else _RRS, target_logits, draft_logits, None,
+                                              draft_tokens, uniforms, tree, temperature, stream, out, probabilities,
+                                              _split, False)
 
 
 def spechub_verify_tree_stats(target_logits, draft_logits, stats, draft_tokens, uniforms, tree: Tree,
                               temperature=1.0, stream=None, out=None, probabilities=True):
     """``spechub_verify_tree`` given the draft statistics ``spechub_draft_sample_stats`` left for the same
     draft logits, tree and temperature: the first pass reads the target rows only."""
-    return _verify("spechub", target_logits, draft_logits, draft_tokens, uniforms, tree, temperature,
-                   stream, out, probabilities, stats, True)
+    return (_native or _load_native()).verify(_SPECHUB, target_logits, draft_logits, stats, draft_tokens, uniforms, tree,
+                                              temperature, stream, out, probabilities, _split, True)
 
 
 def rrs_verify_tree_stats(target_logits, draft_logits, stats, draft_tokens, uniforms, tree: Tree,
                           without_replacement: bool, temperature=1.0, stream=None, out=None,
                           probabilities=True):
     """``rrs_verify_tree`` given the draft statistics ``rrs_draft_sample_stats`` left."""
-    return _verify("rrsw" if without_replacement else "rrs", target_logits, draft_logits, draft_tokens,
-                   uniforms, tree, temperature, stream, out, probabilities, stats, True)
+    return (_native or _load_native()).verify(_RRSW if without_replacement else _RRS, target_logits, draft_logits, stats,
+                                              draft_tokens, uniforms, tree, temperature, stream, out, probabilities,
+                                              _split, True)
 
 
 METHODS = ("spechub", "rrs", "rrsw")
@@ -483,43 +404,13 @@ METHODS = ("spechub", "rrs", "rrsw")
 def mdsd_compare_draft_sample(draft_logits, uniforms, tree: Tree, temperature=1.0, stream=None):
     """Draft step of SpecHub, RRS and RRSw on the same q and uniforms.  Returns a dict keyed by
     method name; each entry is what the method's own draft call returns."""
-    return _compare_draft(draft_logits, uniforms, tree, temperature, stream, False)
+    return (_native or _load_native()).compare_draft(draft_logits, uniforms, tree, temperature, stream, _split, False)
 
 
 def mdsd_compare_draft_sample_stats(draft_logits, uniforms, tree: Tree, temperature=1.0, stream=None):
     """``mdsd_compare_draft_sample`` that also leaves the per-row draft statistics (key ``stats`` of the
     returned dict, one buffer for the three methods) for ``mdsd_compare_verify_tree_stats``."""
-    return _compare_draft(draft_logits, uniforms, tree, temperature, stream, True)
-
-
-def _compare_draft(draft_logits, uniforms, tree, temperature, stream, with_stats):
-    lib = load_library()
-    _need_k2(tree)
-    d, keep = _desc(draft_logits, tree, temperature)
-    B, N, _ = draft_logits.shape
-    dev = draft_logits.device
-    _check_uniforms(uniforms, B, N, dev)
-    tokens = [torch.empty((B, N, 2), dtype=torch.int32, device=dev) for _ in METHODS]
-    status = [torch.empty((B, N), dtype=torch.int32, device=dev) for _ in METHODS]
-    hub = torch.empty((B, N), dtype=torch.int32, device=dev)
-    prob = torch.empty((B, N, 2), dtype=torch.float32, device=dev)
-    tp = (ctypes.c_void_p * 3)(*[t.data_ptr() for t in tokens])
-    sp = (ctypes.c_void_p * 3)(*[t.data_ptr() for t in status])
-    stats = None
-    if with_stats:
-        stats = _alloc_stats(lib, d, dev)
-        _check(lib.mdsd_compare_draft_sample_stats(ctypes.byref(d), _ptr(draft_logits), _ptr(uniforms), tp,
-                                                   _ptr(hub), _ptr(prob), sp, _ptr(stats), _stream_ptr(stream)))
-    else:
-        _check(lib.mdsd_compare_draft_sample(ctypes.byref(d), _ptr(draft_logits), _ptr(uniforms), tp, _ptr(hub),
-                                             _ptr(prob), sp, _stream_ptr(stream)))
-    _hold(keep + tokens + status + [hub, prob, stats], stream)
-    res = dict(spechub=dict(tokens=tokens[0], hub=hub, prob=prob, status=status[0]),
-               rrs=dict(tokens=tokens[1], status=status[1]),
-               rrsw=dict(tokens=tokens[2], status=status[2]))
-    if with_stats:
-        res["stats"] = stats
-    return res
+    return (_native or _load_native()).compare_draft(draft_logits, uniforms, tree, temperature, stream, _split, True)
 
 
 def mdsd_compare_verify_tree(target_logits, draft_logits, draft_tokens, uniforms, tree: Tree,
@@ -527,54 +418,15 @@ def mdsd_compare_verify_tree(target_logits, draft_logits, draft_tokens, uniforms
     """Verification and tree walk by SpecHub, RRS and RRSw from shared reads of p and q.
     ``draft_tokens`` and ``out`` are dicts keyed by method name (``out`` entries as made by
     ``alloc_verify_outputs``).  Returns ``out``."""
-    return _compare_verify(target_logits, draft_logits, draft_tokens, uniforms, tree, temperature, stream, out,
-                           probabilities, None, False)
+    return (_native or _load_native()).compare_verify(target_logits, draft_logits, None, draft_tokens, uniforms, tree,
+                                                      temperature, stream, out, probabilities, _split, False)
 
 
 def mdsd_compare_verify_tree_stats(target_logits, draft_logits, stats, draft_tokens, uniforms, tree: Tree,
                                    temperature=1.0, stream=None, out=None, probabilities=True):
     """``mdsd_compare_verify_tree`` given the draft statistics ``mdsd_compare_draft_sample_stats`` left."""
-    return _compare_verify(target_logits, draft_logits, draft_tokens, uniforms, tree, temperature, stream, out,
-                           probabilities, stats, True)
-
-
-def _compare_verify(target_logits, draft_logits, draft_tokens, uniforms, tree, temperature, stream, out,
-                    probabilities, stats, with_stats):
-    lib = load_library()
-    _need_k2(tree)
-    _same_layout(target_logits, draft_logits)
-    d, keep = _desc(target_logits, tree, temperature)
-    B, N, _ = target_logits.shape
-    dev = target_logits.device
-    _check_uniforms(uniforms, B, N, dev)
-    for m in METHODS:
-        t = draft_tokens[m]
-        if t.dtype != torch.int32 or tuple(t.shape) != (B, N, 2) or not t.is_contiguous() or t.device != dev:
-            raise ValueError("draft_tokens[%s] must be a contiguous int32 [batch][nodes][2] tensor" % m)
-    if out is None:
-        out = {m: alloc_verify_outputs(B, N, tree.levels, dev) for m in METHODS}
-    no = (_NodeOut * 3)(*[
-        _NodeOut(*[out[m][k].data_ptr() if (probabilities or k not in ("beta", "rate")) else None
-                   for k in ("accept_idx", "token", "hub", "beta", "rate", "status")]) for m in METHODS])
-    so = (_SeqOut * 3)(*[
-        _SeqOut(*[out[m][k].data_ptr() for k in ("n_accepted", "n_emitted", "path_nodes", "path_tokens")])
-        for m in METHODS])
-    tp = (ctypes.c_void_p * 3)(*[draft_tokens[m].data_ptr() for m in METHODS])
-    ws_bytes = lib.spechub_workspace_bytes(ctypes.byref(d))
-    ws = torch.empty(ws_bytes, dtype=torch.uint8, device=dev) if ws_bytes else None
-    if with_stats:
-        need = lib.spechub_draft_stats_bytes(ctypes.byref(d))
-        if (stats is None or stats.dtype != torch.int32 or not stats.is_contiguous() or stats.device != dev
-                or stats.numel() * 4 < need):
-            raise ValueError("stats must be the tensor a *_draft_sample_stats call returned for this shape")
-        _check(lib.mdsd_compare_verify_tree_stats(ctypes.byref(d), _ptr(target_logits), _ptr(draft_logits),
-                                                  _ptr(stats), tp, _ptr(uniforms), no, so, _ptr(ws), ws_bytes,
-                                                  _stream_ptr(stream)))
-    else:
-        _check(lib.mdsd_compare_verify_tree(ctypes.byref(d), _ptr(target_logits), _ptr(draft_logits), tp,
-                                            _ptr(uniforms), no, so, _ptr(ws), ws_bytes, _stream_ptr(stream)))
-    _hold(keep + [ws, stats] + [t for m in METHODS for t in out[m].values()], stream)
-    return out
+    return (_native or _load_native()).compare_verify(target_logits, draft_logits, stats, draft_tokens, uniforms, tree,
+                                                      temperature, stream, out, probabilities, _split, True)
 
 
 STATIC_MAX_ROWS = 16384
@@ -588,25 +440,8 @@ def spechub_verify_tree_static(target_logits, draft_logits, draft_tokens, unifor
     intermediate per-row records in a static array of its own, so at most ``STATIC_MAX_ROWS``
     (batch x nodes) rows per call, and calls on one device must not overlap.  Pass ``out`` (from
     ``alloc_verify_outputs``) to keep this wrapper from allocating the result tensors too."""
-    lib = load_library()
-    _need_k2(tree)
-    _same_layout(target_logits, draft_logits)
-    d, keep = _desc(target_logits, tree, temperature)
-    B, N, _ = target_logits.shape
-    dev = target_logits.device
-    _check_uniforms(uniforms, B, N, dev)
-    if (draft_tokens.dtype != torch.int32 or tuple(draft_tokens.shape) != (B, N, 2)
-            or not draft_tokens.is_contiguous() or draft_tokens.device != dev):
-        raise ValueError("draft_tokens must be a contiguous int32 [batch][nodes][2] tensor")
-    if out is None:
-        out = alloc_verify_outputs(B, N, tree.levels, dev)
-    no = _NodeOut(*[out[k].data_ptr() for k in ("accept_idx", "token", "hub", "beta", "rate", "status")])
-    so = _SeqOut(*[out[k].data_ptr() for k in ("n_accepted", "n_emitted", "path_nodes", "path_tokens")])
-    _check(lib.spechub_verify_tree_static(ctypes.byref(d), _ptr(target_logits), _ptr(draft_logits),
-                                          _ptr(draft_tokens), _ptr(uniforms), ctypes.byref(no),
-                                          ctypes.byref(so), _stream_ptr(stream)))
-    _hold(keep + list(out.values()), stream)
-    return out
+    return (_native or _load_native()).verify_static(target_logits, draft_logits, draft_tokens, uniforms, tree,
+                                                     temperature, stream, out, _split)
 
 
 def workspace_bytes(logits, tree: Tree, temperature=1.0) -> int:
