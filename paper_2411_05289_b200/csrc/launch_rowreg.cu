@@ -1,0 +1,85 @@
+// Rows held in registers: calls whose rows do not fill the GPU.
+#include "spechub_launch.h"
+#include "spechub_rowreg.cuh"
+
+namespace spechub {
+
+// Warps of the whole call from which the streaming kernels are faster, on rows of several warps: about 24 per SM, or
+// one and a half waves of these kernels (V = 32000: 224 rows, V = 128256: 56 rows; measured for each step, both types).
+constexpr long long kRegMaxWarps = 24 * 148;
+
+bool reg_plan(int dtype, int vocab, long long rows, RegPlan *out) {
+    const int nvec = (vocab + 7) / 8, max_nv = dtype == SPECHUB_BF16 ? 8 : 4;
+    RegPlan p = {};
+    // as many warps per row as one wave holds (16 per SM): the fewest vectors per lane that allow it
+    for (p.nv = 1;; p.nv *= 2) {
+        const int parts = (nvec + 32 * p.nv - 1) / (32 * p.nv);
+        if (parts > kRegMaxParts) {
+            if (p.nv == max_nv) return false;
+            continue;
+        }
+        p.cs = 1;
+        while (p.cs * 8 < parts && p.cs < 8) p.cs *= 2;   // CTAs of up to 8 warps measured as good as 4 and better than 16
+        p.w = (parts + p.cs - 1) / p.cs;
+        if (p.w == 3) p.w = 4;
+        if (p.nv == max_nv || rows * p.w * p.cs <= 16 * 148) break;
+    }
+    p.rows_per_cta = p.w <= 2 ? 4 / p.w : 1;
+    p.seg = (nvec + p.w * p.cs - 1) / (p.w * p.cs);
+    *out = p;
+    // rows of one warp (bf16: of two) are the faster ones here however many they are (7168 rows, fp32 V = 1000: draft
+    // step 27.7 -> 17.9 us, verification 50.4 -> 29.6 us; bf16 V = 4096: 45.6 -> 40.5, 92.6 -> 75.9 us)
+    return p.w * p.cs <= (dtype == SPECHUB_BF16 ? 2 : 1) || rows * p.w * p.cs <= kRegMaxWarps;
+}
+
+template <class K, class... Args>
+static int launch(const RegPlan &pl, K kern, unsigned rows, cudaStream_t s, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = pl.cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = pl.cs > 1 ? 1 : 0;
+    cfg.gridDim = dim3(pl.cs > 1 ? rows * pl.cs : (rows + pl.rows_per_cta - 1) / pl.rows_per_cta);
+    cfg.blockDim = dim3(pl.w * pl.rows_per_cta * 32);
+    cfg.stream = s;
+    const RegGeo geo = {pl.w, pl.cs, pl.rows_per_cta, pl.seg};
+    return cudaLaunchKernelEx(&cfg, kern, args..., rows, geo) == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH;
+}
+
+template <typename LT, int NV>
+static int draft(const RegPlan &pl, const KaryArgs &a, int method, unsigned rows, cudaStream_t s) {
+    if (a.k == 2) return launch(pl, reg_draft_kernel<LT, NV, 2>, rows, s, a, method);
+    return launch(pl, reg_draft_kernel<LT, NV, 0>, rows, s, a, method);
+}
+template <typename LT, int NV>
+static int verify(const RegPlan &pl, const KaryArgs &a, int method, unsigned rows, cudaStream_t s) {
+    if (method == kSpecHub) return launch(pl, reg_verify_spechub_kernel<LT, NV>, rows, s, a.r);
+    if (a.k == 2) return launch(pl, reg_verify_rrs_kernel<LT, NV, 2>, rows, s, a);
+    if (a.k == 3) return launch(pl, reg_verify_rrs_kernel<LT, NV, 3>, rows, s, a);
+    if (a.k == 4) return launch(pl, reg_verify_rrs_kernel<LT, NV, 4>, rows, s, a);
+    return launch(pl, reg_verify_rrs_kernel<LT, NV, 0>, rows, s, a);
+}
+
+template <typename LT>
+static int draft_nv(const RegPlan &pl, const KaryArgs &a, int method, unsigned rows, cudaStream_t s) {
+    if (pl.nv == 1) return draft<LT, 1>(pl, a, method, rows, s);
+    if (pl.nv == 2) return draft<LT, 2>(pl, a, method, rows, s);
+    if (pl.nv == 4) return draft<LT, 4>(pl, a, method, rows, s);
+    return draft<LT, sizeof(LT) == 2 ? 8 : 4>(pl, a, method, rows, s);
+}
+template <typename LT>
+static int verify_nv(const RegPlan &pl, const KaryArgs &a, int method, unsigned rows, cudaStream_t s) {
+    if (pl.nv == 1) return verify<LT, 1>(pl, a, method, rows, s);
+    if (pl.nv == 2) return verify<LT, 2>(pl, a, method, rows, s);
+    if (pl.nv == 4) return verify<LT, 4>(pl, a, method, rows, s);
+    return verify<LT, sizeof(LT) == 2 ? 8 : 4>(pl, a, method, rows, s);
+}
+
+int launch_reg_draft(const RegPlan &pl, int dtype, const KaryArgs &a, int method, unsigned rows, cudaStream_t s) {
+    return dtype == SPECHUB_BF16 ? draft_nv<__nv_bfloat16>(pl, a, method, rows, s) : draft_nv<float>(pl, a, method, rows, s);
+}
+int launch_reg_verify(const RegPlan &pl, int dtype, const KaryArgs &a, int method, unsigned rows, cudaStream_t s) {
+    return dtype == SPECHUB_BF16 ? verify_nv<__nv_bfloat16>(pl, a, method, rows, s) : verify_nv<float>(pl, a, method, rows, s);
+}
+
+}  // namespace spechub

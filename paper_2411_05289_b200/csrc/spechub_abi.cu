@@ -91,6 +91,14 @@ bool resident_shape(const spechub_desc *d, bool aligned, ResShape *out) {
     return (d->flags & SPECHUB_FLAG_RESIDENT) && resident_fits(d, aligned, out);
 }
 
+// Shapes whose draft step leaves records that verification reads (see spechub_draft_sample_stats).
+bool keeps_stats(const spechub_desc *d, bool aligned) { return d->k == 2 && d->flags == 0 && lean_ok(d, aligned); }
+
+// Rows held in registers: no flag asks for another kernel.
+bool use_reg(const spechub_desc *d, long long rows, RegPlan *pl) {
+    return d->flags == 0 && reg_plan(d->dtype, d->vocab, rows, pl);
+}
+
 int draft_common(const spechub_desc *d, const void *draft_logits, const float *uniforms, int method,
                  int32_t *draft_tokens, int32_t *hub, float *draft_prob, uint32_t *status,
                  void *stream, void *draft_stats = nullptr) {
@@ -114,10 +122,12 @@ int draft_common(const spechub_desc *d, const void *draft_logits, const float *u
     const int th = threads_for(d);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const bool al = rows_aligned(d, draft_logits);
+    if (d->k > 2 && method == kSpecHub) return SPECHUB_ERR_SHAPE;
+    KaryArgs ka;
+    ka.r = a; ka.k = d->k; ka.without_replacement = (method == kRRSw); ka.keep_stats = keeps_stats(d, al);
+    RegPlan pl;
+    if (use_reg(d, rows, &pl)) return launch_reg_draft(pl, d->dtype, ka, method, rows, s);
     if (d->k > 2) {
-        if (method == kSpecHub) return SPECHUB_ERR_SHAPE;
-        KaryArgs ka;
-        ka.r = a; ka.k = d->k; ka.without_replacement = (method == kRRSw);
         return launch_kary_draft(d->dtype, al, th, ka, rows, s);
     }
     if (lean_ok(d, al)) return launch_lean_draft(method, lean_split(d), a, rows, s);
@@ -174,10 +184,14 @@ int verify_common(const spechub_desc *d, const void *target_logits, const void *
     const bool al = rows_aligned(d, target_logits) && rows_aligned(d, draft_logits);
     int lrc;
     ResShape rs;
-    if (d->k > 2) {
-        if (method == kSpecHub) return SPECHUB_ERR_SHAPE;
-        KaryArgs ka;
-        ka.r = a; ka.k = d->k; ka.without_replacement = (method == kRRSw);
+    RegPlan pl;
+    if (d->k > 2 && method == kSpecHub) return SPECHUB_ERR_SHAPE;
+    KaryArgs ka;
+    ka.r = a; ka.k = d->k; ka.without_replacement = (method == kRRSw);
+    if (!keeps_stats(d, al)) ka.r.draft_stats_in = nullptr;
+    if (use_reg(d, rows, &pl)) {
+        lrc = launch_reg_verify(pl, d->dtype, ka, method, rows, s);
+    } else if (d->k > 2) {
         if (!(d->flags & 7u) && resident_fits(d, al, &rs))   // (a split flag asks for the streaming kernel)
             lrc = launch_resident_kary(rs, ka, rows, s);
         else
@@ -208,7 +222,9 @@ int compare_draft(const spechub_desc *d, const void *draft_logits, const float *
     if (!draft_logits || !uniforms || !draft_tokens || !draft_tokens[0] || !draft_tokens[1] || !draft_tokens[2])
         return SPECHUB_ERR_NULL;
     if (reinterpret_cast<uintptr_t>(draft_stats) % 16 != 0) return SPECHUB_ERR_STRIDE;
-    if (!lean_ok(d, rows_aligned(d, draft_logits))) {
+    const unsigned rows = (unsigned)(d->batch * (int64_t)d->nodes);
+    RegPlan pl;
+    if (!lean_ok(d, rows_aligned(d, draft_logits)) || use_reg(d, rows, &pl)) {
         for (int m = 0; m < 3; ++m) {
             const int mrc = draft_common(d, draft_logits, uniforms, m, draft_tokens[m], m == 0 ? hub : nullptr,
                                          m == 0 ? draft_prob : nullptr, status ? status[m] : nullptr, stream,
@@ -230,7 +246,6 @@ int compare_draft(const spechub_desc *d, const void *draft_logits, const float *
         f.tok_out[m] = draft_tokens[m];
         f.dstatus[m] = status ? status[m] : nullptr;
     }
-    const unsigned rows = (unsigned)(d->batch * (int64_t)d->nodes);
     return launch_fused_draft(f, hub, draft_prob, rows, static_cast<cudaStream_t>(stream));
 }
 
@@ -247,7 +262,9 @@ int compare_verify(const spechub_desc *d, const void *target_logits, const void 
         if (!draft_tokens[m] || !no[m].accept_idx || !no[m].token) return SPECHUB_ERR_NULL;
     if (workspace_bytes < spechub_workspace_bytes(d)) return SPECHUB_ERR_WORKSPACE;
     const bool al = rows_aligned(d, target_logits) && rows_aligned(d, draft_logits);
-    if (!lean_ok(d, al)) {
+    const unsigned rows = (unsigned)(d->batch * (int64_t)d->nodes);
+    RegPlan pl;
+    if (!lean_ok(d, al) || use_reg(d, rows, &pl)) {
         for (int m = 0; m < 3; ++m) {
             const int mrc = verify_common(d, target_logits, draft_logits, draft_tokens[m], uniforms, m, &no[m],
                                           so ? &so[m] : nullptr, workspace, workspace_bytes, stream, draft_stats);
@@ -265,7 +282,6 @@ int compare_verify(const spechub_desc *d, const void *target_logits, const void 
         f.out[m].accept_idx = no[m].accept_idx; f.out[m].token = no[m].token; f.out[m].hub = no[m].hub;
         f.out[m].beta = no[m].beta; f.out[m].rate = no[m].rate; f.out[m].status = no[m].status;
     }
-    const unsigned rows = (unsigned)(d->batch * (int64_t)d->nodes);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     int lrc;
     if (ResShape rs; resident_shape(d, al, &rs)) {

@@ -67,6 +67,7 @@ struct KaryArgs {
     RowArgs r;
     int k;
     int without_replacement;
+    bool keep_stats;   // draft step: leave records that verification accepts (else void ones)
 };
 
 constexpr int kShardRecord = 8;  // floats per row in a phase output

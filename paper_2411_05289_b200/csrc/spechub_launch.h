@@ -23,6 +23,13 @@ int launch_kary_draft(int dtype, bool aligned, int th, const KaryArgs &a, unsign
 int launch_kary_verify(int dtype, bool aligned, int th, const KaryArgs &a, unsigned rows, cudaStream_t s);
 int launch_walk(const WalkKArgs &w, cudaStream_t s);
 
+// Rows held in registers.  reg_plan: false if the row does not fit, or if the streaming kernels are the faster
+// ones for so many rows.
+struct RegPlan { int nv, w, cs, rows_per_cta, seg; };
+bool reg_plan(int dtype, int vocab, long long rows, RegPlan *out);
+int launch_reg_draft(const RegPlan &pl, int dtype, const KaryArgs &a, int method, unsigned rows, cudaStream_t s);
+int launch_reg_verify(const RegPlan &pl, int dtype, const KaryArgs &a, int method, unsigned rows, cudaStream_t s);
+
 // large-vocabulary kernels; cs = CTAs per row asked for (0: the library's choice)
 int launch_lean_draft(int method, int cs, const RowArgs &a, unsigned rows, cudaStream_t s);
 int launch_lean_leaf(const RowArgs &a, const NodeOutPtrs *outs, int n_out, unsigned rows, cudaStream_t s);

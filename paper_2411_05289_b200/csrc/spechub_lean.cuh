@@ -32,6 +32,7 @@
 #include "spechub_common.cuh"
 #include "spechub_stream.cuh"
 #include "spechub_ring.cuh"
+#include "spechub_vec.cuh"
 
 namespace spechub {
 namespace cg = cooperative_groups;
@@ -83,59 +84,6 @@ struct RowGroup {
     }
 };
 
-__device__ __forceinline__ unsigned bf2max(unsigned a, unsigned b) {
-    unsigned d;
-    asm("max.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-    return d;
-}
-__device__ __forceinline__ float bf2_hmax(unsigned m2) {
-    return fmaxf(__uint_as_float(m2 << 16), __uint_as_float(m2 & 0xffff0000u));
-}
-__device__ __forceinline__ void unpack_bf16x8(const uint4 &v, float (&o)[8]) {
-    o[0] = __uint_as_float(v.x << 16); o[1] = __uint_as_float(v.x & 0xffff0000u);
-    o[2] = __uint_as_float(v.y << 16); o[3] = __uint_as_float(v.y & 0xffff0000u);
-    o[4] = __uint_as_float(v.z << 16); o[5] = __uint_as_float(v.z & 0xffff0000u);
-    o[6] = __uint_as_float(v.w << 16); o[7] = __uint_as_float(v.w & 0xffff0000u);
-}
-
-// Two fp32 lanes per instruction (fma / add / sub .f32x2): half the issue slots of the scalar forms,
-// the same roundings (round to nearest, subnormals kept), so results do not depend on which form is used.
-struct F2 {
-    unsigned long long v;
-};
-__device__ __forceinline__ F2 f2_make(float lo, float hi) {
-    F2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void f2_get(F2 a, float &lo, float &hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.v));
-}
-__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
-    F2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-    return d;
-}
-__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
-    F2 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d.v) : "l"(a.v), "l"(b.v));
-    return d;
-}
-__device__ __forceinline__ F2 f2_sub(F2 a, F2 b) {
-    F2 d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d.v) : "l"(a.v), "l"(b.v));
-    return d;
-}
-__device__ __forceinline__ F2 f2_max0(F2 a) {
-    float lo, hi;
-    f2_get(a, lo, hi);
-    return f2_make(fmaxf(lo, 0.f), fmaxf(hi, 0.f));
-}
-__device__ __forceinline__ float f2_sum(F2 a) {
-    float lo, hi;
-    f2_get(a, lo, hi);
-    return lo + hi;
-}
 // the exponentials 2^(k l - c) of one 32-bit word (two bf16 logits), as a pair
 __device__ __forceinline__ F2 f2_exp_word(unsigned w, F2 k2, F2 nc2) {
     const F2 x = f2_fma(f2_make(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u)), k2, nc2);

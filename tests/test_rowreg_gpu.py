@@ -1,0 +1,38 @@
+"""Rows held in registers (calls whose rows do not fill the GPU, short vocabularies): the edges of a lane's vectors,
+of a warp's and a cluster's part, aligned and packed odd rows, both types, against the oracle."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+import workloads  # noqa: E402
+from test_parity_gpu import random_logits, random_uniforms, run_case, sh  # noqa: E402,F401
+
+
+# one warp of 1 / 2 / 4 / 8 vectors per lane, two warps, a CTA, clusters of 2 / 4 / 8 CTAs, each with its neighbours
+@pytest.mark.parametrize("pad", [0, 64])
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("V", [2, 255, 256, 257, 1025, 2048, 2049, 4097, 16385, 32769, 131071])
+def test_edges_of_parts(sh, V, dtype, pad):  # noqa: F811
+    rng = np.random.default_rng(V + 3)
+    B, N = 2, 3
+    lp, lq = random_logits(rng, B, N, V, dtype)
+    lq[0, 1] = lp[0, 1]                                      # p = q
+    lq[1, 2] = -np.inf; lq[1, 2, V - 1] = 0.0                # one-hot q at the last id
+    lp[1, 0, V // 2:] = -np.inf                              # whole parts without mass
+    lq[0, 2, V - 1] = lq[0, 2].max() + 6.0                   # the hub is the last id
+    lp, lq = workloads.round_to_storage(lp, dtype), workloads.round_to_storage(lq, dtype)
+    un = random_uniforms(rng, B, N)
+    for paper in (False, True):
+        run_case(sh, lp, lq, dtype, np.array([1.0, 0.6], np.float32), un, paper, pad_to=pad, label="rowreg V=%d" % V)
+
+
+@pytest.mark.parametrize("rows", [1, 3, 5, 1183, 2369])
+def test_rows_per_cta_and_vectors_per_lane(sh, rows):  # noqa: F811
+    """Row counts around a CTA's share of short rows and around one wave (fewer, wider warps from there on)."""
+    rng = np.random.default_rng(rows)
+    V = 384
+    lp, lq = random_logits(rng, rows, 1, V, "fp32", sd=3.0)
+    run_case(sh, lp, lq, "fp32", 1.0, random_uniforms(rng, rows, 1), False, label="rowreg rows=%d" % rows)
