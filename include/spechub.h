@@ -32,7 +32,8 @@
  *   - Layout: logits are [batch][nodes][vocab] with element strides
  *     `stride_seq`, `stride_node` (rows are contiguous in the vocabulary).
  *     Rows that start on a 16-byte boundary are read with 128-bit loads; other
- *     rows are still read correctly, element by element.
+ *     rows in the aligned words that cover them, shifted into place (results do
+ *     not depend on the alignment).
  *     uniforms are float [batch][nodes][5] = (u_d1, u_d2, r1, r2, u_res), each
  *     in [0, 1): u_d1, u_d2 drive the two draft draws; r1, r2 the first and
  *     second acceptance test performed at the node; u_res the residual (or
@@ -240,8 +241,9 @@ int spechub_verify_tree(const spechub_desc *desc, const void *target_logits,
  * or library), argmax out of range, or a draft logit at the argmax other than
  * the recorded maximum -- flags the row SPECHUB_ST_STATS with outputs -1; other
  * inconsistencies are the caller's responsibility.  Only the default path of
- * the large-vocabulary bf16 shapes (no SPECHUB_FLAG_*, k = 2, rows 16-byte
- * aligned, vocab % 8 == 0, vocab >= 8192) writes and reads records; on every
+ * the large-vocabulary shapes (no SPECHUB_FLAG_*, k = 2, rows on 16-byte (bf16)
+ * or 32-byte (fp32) boundaries, vocab % 8 == 0, vocab >= 8192) writes and reads
+ * records; on every
  * other path the draft call clears draft_stats and the verification call
  * ignores it, so the four calls may be used unconditionally.
  */

@@ -1,4 +1,4 @@
-// Draft step and leaf rows of the large-vocabulary shapes.
+// Streaming draft step and leaf rows.
 #include "spechub_launch.h"
 #include "spechub_lean.cuh"
 #include "spechub_shapes.h"
@@ -16,21 +16,45 @@ static int draft_group(const RowArgs &a, int method, unsigned rows, cudaStream_t
     return cudaLaunchKernelEx(&cfg, lean_draft_kernel<kLeanThreads, CS>, a, method) == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH;
 }
 
-int launch_lean_draft(int method, int cs, const RowArgs &a, unsigned rows, cudaStream_t s) {
+template <typename LT, bool SHIFT>
+static int draft_rows(const RowArgs &a, int method, bool keep_stats, unsigned rows, cudaStream_t s) {
+    const int th = draft_threads(a.vocab, rows);
+    if (th == 512) lean_draft_ck_kernel<LT, SHIFT, 512><<<rows, 512, 0, s>>>(a, method, keep_stats);
+    else if (th == 256) lean_draft_ck_kernel<LT, SHIFT, 256><<<rows, 256, 0, s>>>(a, method, keep_stats);
+    else if (th == 128) lean_draft_ck_kernel<LT, SHIFT, 128><<<rows, 128, 0, s>>>(a, method, keep_stats);
+    else lean_draft_ck_kernel<LT, SHIFT, 64><<<rows, 64, 0, s>>>(a, method, keep_stats);
+    return launch_status();
+}
+
+int launch_lean_draft(int format, int method, int cs, const RowArgs &a, bool keep_stats, unsigned rows, cudaStream_t s) {
     if (cs == 4) return draft_group<4>(a, method, rows, s);
     if (cs == 2) return draft_group<2>(a, method, rows, s);
-    lean_draft_ck_kernel<kLeanDraftThreads><<<rows, kLeanDraftThreads, 0, s>>>(a, method);
+    if (format == kBf16) return draft_rows<__nv_bfloat16, false>(a, method, keep_stats, rows, s);
+    if (format == kBf16Shift) return draft_rows<__nv_bfloat16, true>(a, method, keep_stats, rows, s);
+    if (format == kF32) return draft_rows<float, false>(a, method, keep_stats, rows, s);
+    return draft_rows<float, true>(a, method, keep_stats, rows, s);
+}
+
+template <typename LT, bool SHIFT>
+static int leaf_rows(const LeafArgs &la, unsigned rows, cudaStream_t s) {
+    const int th = draft_threads(la.r.vocab, rows);
+    if (th == 512) lean_leaf_kernel<LT, SHIFT, 512><<<rows, 512, 0, s>>>(la);
+    else if (th == 256) lean_leaf_kernel<LT, SHIFT, 256><<<rows, 256, 0, s>>>(la);
+    else if (th == 128) lean_leaf_kernel<LT, SHIFT, 128><<<rows, 128, 0, s>>>(la);
+    else lean_leaf_kernel<LT, SHIFT, 64><<<rows, 64, 0, s>>>(la);
     return launch_status();
 }
 
 // The leaf rows of an unsplit call (same CTA shape as the draft step).
-int launch_lean_leaf(const RowArgs &a, const NodeOutPtrs *outs, int n_out, unsigned rows, cudaStream_t s) {
+int launch_lean_leaf(int format, const RowArgs &a, const NodeOutPtrs *outs, int n_out, unsigned rows, cudaStream_t s) {
     LeafArgs la = {};
     la.r = a;
     la.n_out = n_out;
     for (int m = 0; m < n_out; ++m) la.out[m] = outs[m];
-    lean_leaf_kernel<kLeanDraftThreads><<<rows, kLeanDraftThreads, 0, s>>>(la);
-    return launch_status();
+    if (format == kBf16) return leaf_rows<__nv_bfloat16, false>(la, rows, s);
+    if (format == kBf16Shift) return leaf_rows<__nv_bfloat16, true>(la, rows, s);
+    if (format == kF32) return leaf_rows<float, false>(la, rows, s);
+    return leaf_rows<float, true>(la, rows, s);
 }
 
 }  // namespace spechub

@@ -1,0 +1,65 @@
+// Streaming verification of one method: its kernels and which of them a call takes.
+#pragma once
+
+#include "spechub_launch.h"
+#include "spechub_lean.cuh"
+#include "spechub_shapes.h"
+
+namespace spechub {
+
+template <int METHOD, int CS>
+int verify_split(const RowArgs &a, unsigned rows, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = CS > 1 ? 1 : 0;
+    cfg.gridDim = dim3(rows * CS); cfg.blockDim = dim3(kLeanThreads); cfg.stream = s;
+    return cudaLaunchKernelEx(&cfg, lean_verify_kernel<__nv_bfloat16, false, METHOD, kLeanThreads, CS>, a) == cudaSuccess
+               ? SPECHUB_OK : SPECHUB_ERR_LAUNCH;
+}
+
+// One CTA per row, the passes fed by per-warp rings of bulk copies (spechub_ring.cuh).
+template <int METHOD>
+int verify_ring(const RowArgs &a, unsigned rows, cudaStream_t s) {
+    auto kern = lean_verify_kernel<__nv_bfloat16, false, METHOD, kLeanThreads, 1, true>;
+    constexpr int smem = kLeanThreads / 32 * kRingWarpBytes;
+    static bool configured[kMaxDevices] = {};
+    const int rc = allow_smem(reinterpret_cast<const void *>(kern), smem, configured);
+    if (rc != SPECHUB_OK) return rc;
+    kern<<<rows, kLeanThreads, smem, s>>>(a);
+    return launch_status();
+}
+
+// One CTA per row.  STATS: the draft row's statistics come from the draft step.
+template <typename LT, bool SHIFT, int METHOD, bool STATS>
+int verify_rows(const RowArgs &a, unsigned rows, cudaStream_t s) {
+    const int th = verify_threads(a.vocab, rows);
+    if (th == 512) lean_verify_kernel<LT, SHIFT, METHOD, 512, 1, false, STATS><<<rows, 512, 0, s>>>(a);
+    else if (th == 256) lean_verify_kernel<LT, SHIFT, METHOD, 256, 1, false, STATS><<<rows, 256, 0, s>>>(a);
+    else lean_verify_kernel<LT, SHIFT, METHOD, 128, 1, false, STATS><<<rows, 128, 0, s>>>(a);
+    return launch_status();
+}
+
+template <int METHOD>
+int launch_lean_verify_method(int format, int cs, const RowArgs &a, unsigned rows, cudaStream_t s) {
+    if (cs == 4) return verify_split<METHOD, 4>(a, rows, s);
+    if (cs == 2) return verify_split<METHOD, 2>(a, rows, s);
+    if (a.node_kind) {
+        const NodeOutPtrs o = {a.accept_idx, a.token, a.hub, a.beta, a.rate, a.status};
+        const int lrc = launch_lean_leaf(format, a, &o, 1, rows, s);
+        if (lrc != SPECHUB_OK) return lrc;
+    }
+    const bool stats = cs == 0 && a.draft_stats_in;
+    if (format == kBf16Shift) return verify_rows<__nv_bfloat16, true, METHOD, false>(a, rows, s);
+    if (format == kF32Shift) return verify_rows<float, true, METHOD, false>(a, rows, s);
+    if (format == kF32)
+        return stats ? verify_rows<float, false, METHOD, true>(a, rows, s) : verify_rows<float, false, METHOD, false>(a, rows, s);
+    if (stats) return verify_rows<__nv_bfloat16, false, METHOD, true>(a, rows, s);
+    // (the plain calls and the three-method kernel: always 256 threads)
+    if constexpr (METHOD != kSpecHub)
+        if (cs == 0) return verify_ring<METHOD>(a, rows, s);
+    return verify_split<METHOD, 1>(a, rows, s);
+}
+
+}  // namespace spechub

@@ -77,8 +77,16 @@ int lean_split(const spechub_desc *d) {
     return 0;
 }
 
-// The lean kernels take bf16 rows whose starts are 16-byte aligned and whose length is a multiple of 8 and
-// large enough to keep a CTA's threads busy.
+// How the streaming kernels read the rows: in whole aligned words if every row starts on the boundary of a vector
+// of eight ids and has no remainder.  (`aligned`: on 16-byte boundaries.)
+int stream_format(const spechub_desc *d, bool aligned, const void *base0, const void *base1) {
+    if (d->dtype == SPECHUB_BF16) return aligned && d->vocab % 8 == 0 ? kBf16 : kBf16Shift;
+    const uintptr_t at = reinterpret_cast<uintptr_t>(base0) | reinterpret_cast<uintptr_t>(base1);
+    return at % 32 == 0 && d->stride_node % 8 == 0 && d->stride_seq % 8 == 0 && d->vocab % 8 == 0 ? kF32 : kF32Shift;
+}
+
+// Shapes of the kernels that take long bf16 rows in whole words only: split rows, the three-method kernels, rows
+// resident on chip.
 bool lean_ok(const spechub_desc *d, bool aligned) {
     return d->dtype == SPECHUB_BF16 && aligned && d->vocab % 8 == 0 && d->vocab >= 8192;
 }
@@ -92,11 +100,13 @@ bool resident_shape(const spechub_desc *d, bool aligned, ResShape *out) {
 }
 
 // Shapes whose draft step leaves records that verification reads (see spechub_draft_sample_stats).
-bool keeps_stats(const spechub_desc *d, bool aligned) { return d->k == 2 && d->flags == 0 && lean_ok(d, aligned); }
+bool keeps_stats(const spechub_desc *d, int format) {
+    return d->k == 2 && d->flags == 0 && (format == kBf16 || format == kF32) && d->vocab >= 8192;
+}
 
 // Rows held in registers: no flag asks for another kernel.
-bool use_reg(const spechub_desc *d, long long rows, RegPlan *pl) {
-    return d->flags == 0 && reg_plan(d->dtype, d->vocab, rows, pl);
+bool use_reg(const spechub_desc *d, bool aligned, long long rows, RegPlan *pl) {
+    return (d->flags == 0 || !lean_ok(d, aligned)) && reg_plan(d->dtype, d->vocab, rows, pl);
 }
 
 int draft_common(const spechub_desc *d, const void *draft_logits, const float *uniforms, int method,
@@ -119,19 +129,16 @@ int draft_common(const spechub_desc *d, const void *draft_logits, const float *u
     a.draft_prob = draft_prob;
     a.status = status;
     const unsigned rows = (unsigned)(d->batch * (int64_t)d->nodes);
-    const int th = threads_for(d);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const bool al = rows_aligned(d, draft_logits);
+    const int fmt = stream_format(d, al, draft_logits, nullptr);
     if (d->k > 2 && method == kSpecHub) return SPECHUB_ERR_SHAPE;
     KaryArgs ka;
-    ka.r = a; ka.k = d->k; ka.without_replacement = (method == kRRSw); ka.keep_stats = keeps_stats(d, al);
+    ka.r = a; ka.k = d->k; ka.without_replacement = (method == kRRSw); ka.keep_stats = keeps_stats(d, fmt);
     RegPlan pl;
-    if (use_reg(d, rows, &pl)) return launch_reg_draft(pl, d->dtype, ka, method, rows, s);
-    if (d->k > 2) {
-        return launch_kary_draft(d->dtype, al, th, ka, rows, s);
-    }
-    if (lean_ok(d, al)) return launch_lean_draft(method, lean_split(d), a, rows, s);
-    return launch_rows_draft(d->dtype, al, th, a, method, rows, s);
+    if (use_reg(d, al, rows, &pl)) return launch_reg_draft(pl, d->dtype, ka, method, rows, s);
+    if (d->k > 2) return launch_kary_draft(d->dtype, al, threads_for(d), ka, rows, s);
+    return launch_lean_draft(fmt, method, lean_ok(d, al) ? lean_split(d) : 0, a, ka.keep_stats, rows, s);
 }
 
 int launch_walk(const spechub_desc *d, const spechub_node_out *no, const spechub_seq_out *so, cudaStream_t s) {
@@ -179,33 +186,36 @@ int verify_common(const spechub_desc *d, const void *target_logits, const void *
     a.rate = no->rate;
     a.status = no->status;
     const unsigned rows = (unsigned)(d->batch * (int64_t)d->nodes);
-    const int th = threads_for(d);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const bool al = rows_aligned(d, target_logits) && rows_aligned(d, draft_logits);
+    const int fmt = stream_format(d, al, target_logits, draft_logits);
+    if (!keeps_stats(d, fmt)) a.draft_stats_in = nullptr;
     int lrc;
     ResShape rs;
     RegPlan pl;
     if (d->k > 2 && method == kSpecHub) return SPECHUB_ERR_SHAPE;
     KaryArgs ka;
     ka.r = a; ka.k = d->k; ka.without_replacement = (method == kRRSw);
-    if (!keeps_stats(d, al)) ka.r.draft_stats_in = nullptr;
-    if (use_reg(d, rows, &pl)) {
+    const int cs = lean_ok(d, al) ? lean_split(d) : 0;
+    if (use_reg(d, al, rows, &pl)) {
         lrc = launch_reg_verify(pl, d->dtype, ka, method, rows, s);
     } else if (d->k > 2) {
         if (!(d->flags & 7u) && resident_fits(d, al, &rs))   // (a split flag asks for the streaming kernel)
             lrc = launch_resident_kary(rs, ka, rows, s);
         else
-            lrc = launch_kary_verify(d->dtype, al, th, ka, rows, s);
+            lrc = launch_kary_verify(d->dtype, al, threads_for(d), ka, rows, s);
     } else if (resident_shape(d, al, &rs)) {
         FusedArgs f = {};
         f.r = a;
         f.tok[method] = draft_tokens;
         f.out[method] = NodeOutPtrs{a.accept_idx, a.token, a.hub, a.beta, a.rate, a.status};
         lrc = launch_resident(1 << method, rs, f, rows, s);
-    } else if (lean_ok(d, al)) {
-        lrc = launch_lean_verify(method, lean_split(d), a, rows, s);
+    } else if (method == kSpecHub) {
+        lrc = launch_lean_verify_spechub(fmt, cs, a, rows, s);
+    } else if (method == kRRS) {
+        lrc = launch_lean_verify_rrs(fmt, cs, a, rows, s);
     } else {
-        lrc = launch_rows_verify(d->dtype, al, th, a, method, rows, s);
+        lrc = launch_lean_verify_rrsw(fmt, cs, a, rows, s);
     }
     if (lrc != SPECHUB_OK) return lrc;
     return launch_walk(d, no, so, s);
@@ -224,7 +234,8 @@ int compare_draft(const spechub_desc *d, const void *draft_logits, const float *
     if (reinterpret_cast<uintptr_t>(draft_stats) % 16 != 0) return SPECHUB_ERR_STRIDE;
     const unsigned rows = (unsigned)(d->batch * (int64_t)d->nodes);
     RegPlan pl;
-    if (!lean_ok(d, rows_aligned(d, draft_logits)) || use_reg(d, rows, &pl)) {
+    const bool al = rows_aligned(d, draft_logits);
+    if (!lean_ok(d, al) || use_reg(d, al, rows, &pl)) {
         for (int m = 0; m < 3; ++m) {
             const int mrc = draft_common(d, draft_logits, uniforms, m, draft_tokens[m], m == 0 ? hub : nullptr,
                                          m == 0 ? draft_prob : nullptr, status ? status[m] : nullptr, stream,
@@ -264,7 +275,7 @@ int compare_verify(const spechub_desc *d, const void *target_logits, const void 
     const bool al = rows_aligned(d, target_logits) && rows_aligned(d, draft_logits);
     const unsigned rows = (unsigned)(d->batch * (int64_t)d->nodes);
     RegPlan pl;
-    if (!lean_ok(d, al) || use_reg(d, rows, &pl)) {
+    if (!lean_ok(d, al) || use_reg(d, al, rows, &pl)) {
         for (int m = 0; m < 3; ++m) {
             const int mrc = verify_common(d, target_logits, draft_logits, draft_tokens[m], uniforms, m, &no[m],
                                           so ? &so[m] : nullptr, workspace, workspace_bytes, stream, draft_stats);
@@ -288,7 +299,7 @@ int compare_verify(const spechub_desc *d, const void *target_logits, const void 
         lrc = launch_resident(7, rs, f, rows, s);
     } else {
         if (d->node_kind) {
-            const int llrc = launch_lean_leaf(f.r, f.out, 3, rows, s);
+            const int llrc = launch_lean_leaf(kBf16, f.r, f.out, 3, rows, s);
             if (llrc != SPECHUB_OK) return llrc;
         }
         if (lean_split(d) == 0) f.r.draft_stats_in = draft_stats;

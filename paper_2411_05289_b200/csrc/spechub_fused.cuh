@@ -35,7 +35,8 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
     const int b = static_cast<int>(r / a.nodes), n = static_cast<int>(r % a.nodes);
     const __nv_bfloat16 *rowp = static_cast<const __nv_bfloat16 *>(a.target) + b * a.stride_seq + n * a.stride_node;
     const __nv_bfloat16 *rowq = static_cast<const __nv_bfloat16 *>(a.draft) + b * a.stride_seq + n * a.stride_node;
-    const uint4 *vp = reinterpret_cast<const uint4 *>(rowp), *vq = reinterpret_cast<const uint4 *>(rowq);
+    using V = Vec8<__nv_bfloat16>;
+    const StreamRow<__nv_bfloat16, false> vp(rowp, a.vocab), vq(rowq, a.vocab);
     const Geo g = make_geo(a.vocab, 8);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int lo = g.seg_lo(warp), hi = g.seg_hi(warp);
@@ -60,9 +61,9 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
     };
 
     if (leaf) return;   // leaf rows belong to lean_leaf_kernel
-    LeanAcc tp, tq;
+    LeanAcc<__nv_bfloat16> tp, tq;
     if (STATS) lean_pass_a_deep(vp, lo, hi, lane, k, tp);
-    else lean_pass_a<true>(vp, vq, lo, hi, lane, k, tp, tq);
+    else lean_pass_a<true, false>(vp, vq, lo, hi, lane, k, tp, tq);
     {
         ArgMaxSum Ps, Qs;
         if (STATS) lean_reduce2<false>(tp, tq, vp, vq, lo, hi, k, sh, Ps, Qs);
@@ -97,7 +98,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
     }
     auto prob_p = [&](int y) { return prob_of(load_one<__nv_bfloat16>(rowp, y), k, cP, invZp); };
     auto prob_q = [&](int y) { return prob_of(load_one<__nv_bfloat16>(rowq, y), k, cQ, invZq); };
-    auto draw_from_p = [&]() { return lean_sample_row<1>(g, rowp, k, P, 0, -1, ures, 0, sh); };
+    auto draw_from_p = [&]() { return lean_sample_row<1>(g, vp, k, P, 0, -1, ures, 0, sh); };
 
     if (!(P.ml > neg_inf()) || !(P.ml < pinf) || !finite_pos(Zp)) {
         for (int m = 0; m < 3; ++m) o[m].status = SPECHUB_ST_NONFINITE;
@@ -145,14 +146,13 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
     const F2 nrho2 = f2_make(-rho, -rho), ncrho2 = f2_make(-crho, -crho);
 #pragma unroll 2
     for (int vi = last_vi; vi >= lo; vi -= 32) {
-        const uint4 rawp = vp[vi], rawq = vq[vi];
-        if (STATS) diff |= (rawp.x ^ rawq.x) | (rawp.y ^ rawq.y) | (rawp.z ^ rawq.z) | (rawp.w ^ rawq.w);
-        const unsigned wps[4] = {rawp.x, rawp.y, rawp.z, rawp.w}, wqs[4] = {rawq.x, rawq.y, rawq.z, rawq.w};
+        const V cp = vp[vi], cq = vq[vi];
+        if (STATS) diff |= cp.differs(cq);
         float qw[8];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const F2 ep = f2_exp_word(wps[i], k2, ncp2);
-            F2 eq = f2_exp_word(wqs[i], k2, ncq2);
+            const F2 ep = f2_exp(cp.pair(i), k2, ncp2);
+            F2 eq = f2_exp(cq.pair(i), k2, ncq2);
             if (!STATS) f2_get(eq, qw[2 * i], qw[2 * i + 1]);
             F2 d = f2_fma(nrho2, eq, ep);              // Z_p (p - q)
             F2 m = f2_max0(d);
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
     }
     float accB[5] = {s1a + s1b, s2a + s2b, ra + rb, a1a + a1b, dna + dnb};
     lean_block_sums<5, 0>(accB, sh);   // per-warp R stays in sh.acc[2]
-    if (STATS) accB[4] = wx1 >= 0 ? sum_without(Q, rowq, wx1, k) : 0.f;
+    if (STATS) accB[4] = wx1 >= 0 ? sum_without(Q, vq, wx1, k) : 0.f;
     const float Rraw = accB[2];
     const float S1 = accB[0] * invZp, S2 = degenerate ? qa : accB[1] * invZp, R = Rraw * invZp;
     const float A1 = accB[3] * invZp, den = accB[4] * invZq;
@@ -212,14 +212,13 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
         asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(polf));
 #pragma unroll 2
         for (int vi = lo + lane; vi < hi; vi += 32) {
-            const uint4 rawp = ld_l2_hint(vp + vi, polf), rawq = ld_l2_hint(vq + vi, polf);
-            const unsigned wps[4] = {rawp.x, rawp.y, rawp.z, rawp.w}, wqs[4] = {rawq.x, rawq.y, rawq.z, rawq.w};
+            const V cp = vp.fetch(vi, polf), cq = vq.fetch(vi, polf);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 F2 nsc = nsc1;
                 if (vi == wvec && i == (wel >> 1)) nsc = (wel & 1) ? f2_make(-A1grho[1], 0.f) : f2_make(0.f, -A1grho[1]);
-                const F2 eq = f2_exp_word(wqs[i], k2, ncq2);
-                const F2 m = f2_max0(f2_fma(nrho2, eq, f2_exp_word(wps[i], k2, ncp2)));
+                const F2 eq = f2_exp(cq.pair(i), k2, ncq2);
+                const F2 m = f2_max0(f2_fma(nrho2, eq, f2_exp(cp.pair(i), k2, ncp2)));
                 w0 = f2_add(w0, f2_max0(f2_fma(nsc0, eq, m)));
                 w1 = f2_add(w1, f2_max0(f2_fma(nsc, eq, m)));
             }
@@ -260,13 +259,11 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
                 if (threadIdx.x < g.nwarps) sh.mass[threadIdx.x] = sh.acc[2][threadIdx.x];
                 __syncthreads();
                 auto wf = [&](int vi, float(&w)[8]) {
-                    float fp[8], fq[8];
-                    unpack_bf16x8(vp[vi], fp);
-                    unpack_bf16x8(vq[vi], fq);
+                    const V fp = vp[vi], fq = vq[vi];
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         float d, t;
-                        lean_terms(lean_exp(fp[i], k, cP), lean_exp(fq[i], k, cQ), rho, crho, d, t);
+                        lean_terms(lean_exp(fp.get(i), k, cP), lean_exp(fq.get(i), k, cQ), rho, crho, d, t);
                         w[i] = (vi * 8 + i == hubtok) ? 0.f : fmaxf(t, 0.f);
                     }
                 };
@@ -307,14 +304,12 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
                 __syncthreads();
                 const float coef = A1grho[m];
                 auto wf = [&](int vi, float(&w)[8]) {
-                    float fp[8], fq[8];
-                    unpack_bf16x8(vp[vi], fp);
-                    unpack_bf16x8(vq[vi], fq);
+                    const V fp = vp[vi], fq = vq[vi];
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         float d, t;
                         const float sc = (wo && vi * 8 + i == x1) ? 0.f : coef;
-                        lean_terms(lean_exp(fp[i], k, cP), lean_exp(fq[i], k, cQ), rho, sc, d, t);
+                        lean_terms(lean_exp(fp.get(i), k, cP), lean_exp(fq.get(i), k, cQ), rho, sc, d, t);
                         w[i] = fmaxf(t, 0.f);
                     }
                 };
@@ -339,7 +334,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
     const long long r = blockIdx.x;
     const int b = static_cast<int>(r / a.nodes), n = static_cast<int>(r % a.nodes);
     const __nv_bfloat16 *rowq = static_cast<const __nv_bfloat16 *>(a.draft) + b * a.stride_seq + n * a.stride_node;
-    const uint4 *vq = reinterpret_cast<const uint4 *>(rowq);
+    const StreamRow<__nv_bfloat16, false> vq(rowq, a.vocab);
     const Geo g = make_geo(a.vocab, 8);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int lo = g.seg_lo(warp), hi = g.seg_hi(warp);
@@ -348,9 +343,9 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
     const bool t0 = threadIdx.x == 0;
     const int CK = lean_ck_interval(g);
 
-    LeanAcc tq, unused;
-    unused.m2 = 0xff80ff80u; unused.s = 0.f; unused.c = 0.f;
-    lean_pass_a_ck(vq, lo, hi, lane, k, CK, tq, sh.cks[warp], sh.ckc[warp]);
+    LeanAcc<__nv_bfloat16> tq, unused;
+    unused.init();
+    lean_pass_a_ck<false>(vq, lo, hi, lane, k, CK, tq, sh.cks[warp], sh.ckc[warp]);
     {
         ArgMaxSum q, unusedq;
         lean_reduce2<false>(tq, unused, vq, vq, lo, hi, k, sh, q, unusedq);
@@ -377,7 +372,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
         return;
     }
     const int hubtok = Q.idx;
-    const int x1 = lean_ck_sample(g, rowq, k, Q.C, CK, -1, u1, sh);
+    const int x1 = lean_ck_sample(g, vq, k, Q.C, CK, -1, u1, sh);
     uint32_t st[3] = {0, 0, 0};
     int x2[3];
     // SpecHub (Section 4)
@@ -390,13 +385,13 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
         x2[0] = (hubtok == 0) ? 1 : 0;
         st[0] |= SPECHUB_ST_DEGENERATE_Q;
     } else {
-        x2[0] = lean_ck_sample(g, rowq, k, Q.C, CK, hubtok, u2, sh);
+        x2[0] = lean_ck_sample(g, vq, k, Q.C, CK, hubtok, u2, sh);
         prob1 = prob0 * ex2(fmaf(load_one<__nv_bfloat16>(rowq, x2[0]), k, -Q.C)) / Q.sx;
     }
     // RRS: an independent second draw
-    x2[1] = lean_ck_sample(g, rowq, k, Q.C, CK, -1, u2, sh);
+    x2[1] = lean_ck_sample(g, vq, k, Q.C, CK, -1, u2, sh);
     // RRSw: q with q(x1) set to 0
-    x2[2] = lean_ck_sample(g, rowq, k, Q.C, CK, x1, u2, sh);
+    x2[2] = lean_ck_sample(g, vq, k, Q.C, CK, x1, u2, sh);
     if (x2[2] < 0) {
         x2[2] = (x1 == 0) ? 1 : 0;
         st[2] |= SPECHUB_ST_DEGENERATE_Q;

@@ -16,9 +16,7 @@ inline int launch_status() { return cudaGetLastError() == cudaSuccess ? SPECHUB_
 // the caller (one array per kernel).
 int allow_smem(const void *kern, int bytes, bool *configured);
 
-// general kernels (any shape); th = threads per row
-int launch_rows_draft(int dtype, bool aligned, int th, const RowArgs &a, int method, unsigned rows, cudaStream_t s);
-int launch_rows_verify(int dtype, bool aligned, int th, const RowArgs &a, int method, unsigned rows, cudaStream_t s);
+// more than two drafts per node, any shape; th = threads per row
 int launch_kary_draft(int dtype, bool aligned, int th, const KaryArgs &a, unsigned rows, cudaStream_t s);
 int launch_kary_verify(int dtype, bool aligned, int th, const KaryArgs &a, unsigned rows, cudaStream_t s);
 int launch_walk(const WalkKArgs &w, cudaStream_t s);
@@ -30,10 +28,15 @@ bool reg_plan(int dtype, int vocab, long long rows, RegPlan *out);
 int launch_reg_draft(const RegPlan &pl, int dtype, const KaryArgs &a, int method, unsigned rows, cudaStream_t s);
 int launch_reg_verify(const RegPlan &pl, int dtype, const KaryArgs &a, int method, unsigned rows, cudaStream_t s);
 
-// large-vocabulary kernels; cs = CTAs per row asked for (0: the library's choice)
-int launch_lean_draft(int method, int cs, const RowArgs &a, unsigned rows, cudaStream_t s);
-int launch_lean_leaf(const RowArgs &a, const NodeOutPtrs *outs, int n_out, unsigned rows, cudaStream_t s);
-int launch_lean_verify(int method, int cs, const RowArgs &a, unsigned rows, cudaStream_t s);
+// Streaming kernels.  How the rows are read: in whole aligned words (bf16: rows on 16-byte boundaries, fp32: on
+// 32-byte boundaries, vocab % 8 == 0), or shifted into place (any row).
+enum StreamFormat { kBf16, kBf16Shift, kF32, kF32Shift };
+int launch_lean_draft(int format, int method, int cs, const RowArgs &a, bool keep_stats, unsigned rows, cudaStream_t s);
+int launch_lean_leaf(int format, const RowArgs &a, const NodeOutPtrs *outs, int n_out, unsigned rows, cudaStream_t s);
+// cs = CTAs per row asked for (0: the library's choice; other than 0 and 1: kBf16 only)
+int launch_lean_verify_spechub(int format, int cs, const RowArgs &a, unsigned rows, cudaStream_t s);
+int launch_lean_verify_rrs(int format, int cs, const RowArgs &a, unsigned rows, cudaStream_t s);
+int launch_lean_verify_rrsw(int format, int cs, const RowArgs &a, unsigned rows, cudaStream_t s);
 int launch_fused_draft(const FusedArgs &f, int32_t *hub, float *draft_prob, unsigned rows, cudaStream_t s);
 int launch_fused_verify(const FusedArgs &f, unsigned rows, cudaStream_t s);
 

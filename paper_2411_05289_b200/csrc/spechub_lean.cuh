@@ -84,76 +84,69 @@ struct RowGroup {
     }
 };
 
-// the exponentials 2^(k l - c) of one 32-bit word (two bf16 logits), as a pair
-__device__ __forceinline__ F2 f2_exp_word(unsigned w, F2 k2, F2 nc2) {
-    const F2 x = f2_fma(f2_make(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u)), k2, nc2);
-    float x0, x1;
-    f2_get(x, x0, x1);
-    return f2_make(ex2(x0), ex2(x1));
-}
+// CTAs of THREADS threads per SM.  bf16 rows in whole words: 64 registers per thread (1024 threads per SM) measured
+// best; wider vectors, and the two words of a shifted one, take 80 (768 threads per SM).
+template <typename LT, bool SHIFT>
+constexpr int lean_ctas(int threads) { return (sizeof(LT) == 2 && !SHIFT ? 1024 : 768) / threads; }
 
-// a 16-byte load with an L2 eviction policy (createpolicy)
-__device__ __forceinline__ uint4 ld_l2_hint(const uint4 *p, uint64_t pol) {
-    uint4 v;
-    asm volatile("ld.global.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(pol));
-    return v;
-}
-
+template <typename LT>
 struct LeanAcc {  // one thread's pass-A state for one row
-    unsigned m2;  // packed running maximum
-    float c;      // exponent reference (k * some logit of this thread, or 0)
-    float s;      // sum of 2^(k l - c)
+    typename Vec8<LT>::Max m2;  // running maximum (packed)
+    float c;                    // exponent reference (k * some logit of this thread, or 0)
+    float s;                    // sum of 2^(k l - c)
+    __device__ __forceinline__ void init() { m2 = Vec8<LT>::max_none(); s = 0.f; c = 0.f; }
+    __device__ __forceinline__ float max() const { return Vec8<LT>::max_value(m2); }
 };
 
-__device__ __forceinline__ void lean_push(LeanAcc &st, const uint4 &raw, float k) {
-    const unsigned vm = bf2max(bf2max(raw.x, raw.y), bf2max(raw.z, raw.w));
-    st.m2 = bf2max(st.m2, vm);
+// a vector's sum of exponentials, two lanes at a time: (e0 + e2) + (e4 + e6) and (e1 + e3) + (e5 + e7)
+template <typename LT>
+__device__ __forceinline__ float vec_sum(const Vec8<LT> &v, F2 k2, F2 nc2) {
+    return f2_sum(f2_add(f2_add(f2_exp(v.pair(0), k2, nc2), f2_exp(v.pair(1), k2, nc2)),
+                         f2_add(f2_exp(v.pair(2), k2, nc2), f2_exp(v.pair(3), k2, nc2))));
+}
+
+template <typename LT>
+__device__ __forceinline__ void lean_push(LeanAcc<LT> &st, const Vec8<LT> &v, float k) {
+    const auto vm = v.packed_max();
+    st.m2 = Vec8<LT>::max_of(st.m2, vm);
     const F2 k2 = f2_make(k, k);
-    F2 nc2 = f2_make(-st.c, -st.c);
-    // the vector's sum, two lanes at a time: (e0 + e2) + (e4 + e6) and (e1 + e3) + (e5 + e7)
-    float a = f2_sum(f2_add(f2_add(f2_exp_word(raw.x, k2, nc2), f2_exp_word(raw.y, k2, nc2)),
-                            f2_add(f2_exp_word(raw.z, k2, nc2), f2_exp_word(raw.w, k2, nc2))));
+    float a = vec_sum(v, k2, f2_make(-st.c, -st.c));
     if (!(a < kHuge)) {  // out of range (or NaN / +inf input): move the reference to this vector's max
-        const float vmax = bf2_hmax(vm);
-        const float cn = shift_of(vmax, k);
+        const float cn = shift_of(Vec8<LT>::max_value(vm), k);
         st.s *= ex2(st.c - cn);
         st.c = cn;
-        nc2 = f2_make(-st.c, -st.c);
-        a = f2_sum(f2_add(f2_add(f2_exp_word(raw.x, k2, nc2), f2_exp_word(raw.y, k2, nc2)),
-                          f2_add(f2_exp_word(raw.z, k2, nc2), f2_exp_word(raw.w, k2, nc2))));
+        a = vec_sum(v, k2, f2_make(-st.c, -st.c));
     }
     st.s += a;
+}
+
+// the exponent reference of a thread: the maximum of its first vector that holds a finite logit
+template <class ROW>
+__device__ __forceinline__ float lean_reference(const ROW &row, int vi, int hi, float k) {
+    for (; vi < hi; vi += 32) {
+        const float m0 = row[vi].max();
+        if (m0 > neg_inf()) return shift_of(m0, k);
+    }
+    return 0.f;
 }
 
 // Pass A over this warp's range of one or two rows.
 // AHEAD: the next vector pair is requested before the current one is consumed (measured per
 // method: it pays for RRS, 1.92 -> 1.82 ms on V = 128256, and costs SpecHub 2 %).
-template <bool BOTH, bool AHEAD = false>
-__device__ __forceinline__ void lean_pass_a(const uint4 *rp, const uint4 *rq, int lo, int hi, int lane,
-                                            float k, LeanAcc &P, LeanAcc &Q) {
-    P.m2 = 0xff80ff80u; P.s = 0.f; P.c = 0.f;
-    Q.m2 = 0xff80ff80u; Q.s = 0.f; Q.c = 0.f;
+template <bool BOTH, bool AHEAD, typename LT, class ROW>
+__device__ __forceinline__ void lean_pass_a(const ROW &rp, const ROW &rq, int lo, int hi, int lane, float k,
+                                            LeanAcc<LT> &P, LeanAcc<LT> &Q) {
+    P.init();
+    Q.init();
     int vi = lo + lane;
-    // the reference comes from the thread's first vector that holds a finite logit
-    for (int vr = vi; vr < hi; vr += 32) {
-        const uint4 a = rp[vr];
-        const float m0 = bf2_hmax(bf2max(bf2max(a.x, a.y), bf2max(a.z, a.w)));
-        if (m0 > neg_inf()) { P.c = shift_of(m0, k); break; }
-    }
-    if (BOTH) {
-        for (int vr = vi; vr < hi; vr += 32) {
-            const uint4 b = rq[vr];
-            const float m0 = bf2_hmax(bf2max(bf2max(b.x, b.y), bf2max(b.z, b.w)));
-            if (m0 > neg_inf()) { Q.c = shift_of(m0, k); break; }
-        }
-    }
+    P.c = lean_reference(rp, vi, hi, k);
+    if (BOTH) Q.c = lean_reference(rq, vi, hi, k);
     if (BOTH && AHEAD) {
-        uint4 na = make_uint4(0, 0, 0, 0), nb = na;
+        Vec8<LT> na = Vec8<LT>::none(), nb = na;
         if (vi < hi) { na = rp[vi]; nb = rq[vi]; }
 #pragma unroll 1
         for (; vi < hi; vi += 32) {
-            const uint4 a = na, b = nb;
+            const Vec8<LT> a = na, b = nb;
             if (vi + 32 < hi) { na = rp[vi + 32]; nb = rq[vi + 32]; }
             lean_push(P, a, k);
             lean_push(Q, b, k);
@@ -161,76 +154,77 @@ __device__ __forceinline__ void lean_pass_a(const uint4 *rp, const uint4 *rq, in
     } else {
 #pragma unroll 2
         for (; vi < hi; vi += 32) {
-            const uint4 a = rp[vi];
-            uint4 b;
+            const Vec8<LT> a = rp[vi];
+            Vec8<LT> b;
             if (BOTH) b = rq[vi];
             lean_push(P, a, k);
             if (BOTH) lean_push(Q, b, k);
         }
     }
 }
+// ... of two rows of any alignment
+template <typename LT>
+__device__ __forceinline__ void lean_pass_a_any(const StreamRow<LT, true> &rp, const StreamRow<LT, true> &rq, int lo, int hi,
+                                                int lane, float k, LeanAcc<LT> &P, LeanAcc<LT> &Q) {
+    P.init();
+    Q.init();
+    P.c = lean_reference(rp, lo + lane, hi, k);
+    Q.c = lean_reference(rq, lo + lane, hi, k);
+    any_pairs<1>(rp, rq, lo, hi, lane, [&](int, const Vec8<LT> &a, const Vec8<LT> &b) {
+        lean_push(P, a, k);
+        lean_push(Q, b, k);
+    });
+}
 
-// Pass A over one row with four vectors per lane in flight: the next four are requested before the current
-// four are consumed.  Same vectors in the same order as lean_pass_a<false>, so the same sums.
-__device__ __forceinline__ void lean_pass_a_deep(const uint4 *rp, int lo, int hi, int lane, float k, LeanAcc &P) {
+// Pass A over one row with 64 bytes per lane in flight: the next vectors (four of bf16, two of fp32) are requested
+// before the current ones are consumed.  Same vectors in the same order as lean_pass_a<false>, so the same sums.
+template <typename LT, class ROW>
+__device__ __forceinline__ void lean_pass_a_deep(const ROW &rp, int lo, int hi, int lane, float k, LeanAcc<LT> &P) {
+    constexpr int D = ROW::kDepth;
     uint64_t pol;   // the row is read again by pass B: L2 is asked to keep it
     asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
-    P.m2 = 0xff80ff80u; P.s = 0.f; P.c = 0.f;
-    for (int vr = lo + lane; vr < hi; vr += 32) {
-        const uint4 a = rp[vr];
-        const float m0 = bf2_hmax(bf2max(bf2max(a.x, a.y), bf2max(a.z, a.w)));
-        if (m0 > neg_inf()) { P.c = shift_of(m0, k); break; }
-    }
+    P.init();
+    P.c = lean_reference(rp, lo + lane, hi, k);
     const int n = (hi - lo - lane + 31) >> 5;   // this lane's vectors (<= 0: none)
-    const uint4 *p = rp + lo + lane;
+    const int v0 = lo + lane;
     int it = 0;
-    uint4 n0 = make_uint4(0, 0, 0, 0), n1 = n0, n2 = n0, n3 = n0;
-    if (4 <= n) { n0 = ld_l2_hint(p, pol); n1 = ld_l2_hint(p + 32, pol); n2 = ld_l2_hint(p + 64, pol); n3 = ld_l2_hint(p + 96, pol); }
-#pragma unroll 1
-    for (; it + 4 <= n; it += 4) {
-        const uint4 a0 = n0, a1 = n1, a2 = n2, a3 = n3;
-        if (it + 8 <= n) {
-            n0 = ld_l2_hint(p + 32 * (it + 4), pol); n1 = ld_l2_hint(p + 32 * (it + 5), pol);
-            n2 = ld_l2_hint(p + 32 * (it + 6), pol); n3 = ld_l2_hint(p + 32 * (it + 7), pol);
-        }
-        lean_push(P, a0, k);
-        lean_push(P, a1, k);
-        lean_push(P, a2, k);
-        lean_push(P, a3, k);
+    Vec8<LT> nx[D] = {};
+    if (D <= n) {
+#pragma unroll
+        for (int i = 0; i < D; ++i) nx[i] = rp.fetch(v0 + 32 * i, pol);
     }
-    for (; it < n; ++it) lean_push(P, p[32 * it], k);
+#pragma unroll 1
+    for (; it + D <= n; it += D) {
+        Vec8<LT> a[D];
+#pragma unroll
+        for (int i = 0; i < D; ++i) a[i] = nx[i];
+        if (it + 2 * D <= n) {
+#pragma unroll
+            for (int i = 0; i < D; ++i) nx[i] = rp.fetch(v0 + 32 * (it + D + i), pol);
+        }
+#pragma unroll
+        for (int i = 0; i < D; ++i) lean_push(P, a[i], k);
+    }
+    for (; it < n; ++it) lean_push(P, rp[v0 + 32 * it], k);
 }
 
 // Pass A over both rows with the vectors coming from the warp's ring (the first pass of its stream, forwards).
-__device__ __forceinline__ void lean_pass_a_ring(WarpRing &R, int lane, float k, LeanAcc &P, LeanAcc &Q) {
-    P.m2 = 0xff80ff80u; P.s = 0.f; P.c = 0.f;
-    Q.m2 = 0xff80ff80u; Q.s = 0.f; Q.c = 0.f;
+template <class ROW>
+__device__ __forceinline__ void lean_pass_a_ring(WarpRing &R, const ROW &vp, const ROW &vq, int lane, float k,
+                                                 LeanAcc<__nv_bfloat16> &P, LeanAcc<__nv_bfloat16> &Q) {
+    P.init();
+    Q.init();
     const int vi0 = R.lo + lane;
     if (R.nc > 0) {
         // the reference comes from the thread's first vector that holds a finite logit: nearly always the
         // very first one, which the first chunk holds; otherwise look further in global memory
         ring_wait(R);
         if (vi0 < R.hi) {
-            uint4 a, b;
+            Vec8<__nv_bfloat16> a, b;
             ring_load(R, 0, lane, a, b);
-            float m0 = bf2_hmax(bf2max(bf2max(a.x, a.y), bf2max(a.z, a.w)));
-            if (m0 > neg_inf()) P.c = shift_of(m0, k);
-            else {
-                for (int vr = vi0 + 32; vr < R.hi; vr += 32) {
-                    const uint4 a2 = R.vp[vr];
-                    m0 = bf2_hmax(bf2max(bf2max(a2.x, a2.y), bf2max(a2.z, a2.w)));
-                    if (m0 > neg_inf()) { P.c = shift_of(m0, k); break; }
-                }
-            }
-            m0 = bf2_hmax(bf2max(bf2max(b.x, b.y), bf2max(b.z, b.w)));
-            if (m0 > neg_inf()) Q.c = shift_of(m0, k);
-            else {
-                for (int vr = vi0 + 32; vr < R.hi; vr += 32) {
-                    const uint4 b2 = R.vq[vr];
-                    m0 = bf2_hmax(bf2max(bf2max(b2.x, b2.y), bf2max(b2.z, b2.w)));
-                    if (m0 > neg_inf()) { Q.c = shift_of(m0, k); break; }
-                }
-            }
+            const float ma = a.max(), mb = b.max();
+            P.c = ma > neg_inf() ? shift_of(ma, k) : lean_reference(vp, vi0 + 32, R.hi, k);
+            Q.c = mb > neg_inf() ? shift_of(mb, k) : lean_reference(vq, vi0 + 32, R.hi, k);
         }
     }
 #pragma unroll 1
@@ -239,7 +233,7 @@ __device__ __forceinline__ void lean_pass_a_ring(WarpRing &R, int lane, float k,
         const int v0 = vi0 + c * kRingChunkVecs;
 #pragma unroll
         for (int j = 0; j < kRingCh; ++j) {
-            uint4 x, y;
+            Vec8<__nv_bfloat16> x, y;
             ring_load(R, j, lane, x, y);
             if (j == kRingCh - 1) ring_release(R, lane);
             if (v0 + j * 32 < R.hi) {
@@ -254,28 +248,27 @@ __device__ __forceinline__ void lean_pass_a_ring(WarpRing &R, int lane, float k,
 // row maximum `val`): lane j takes the j-th vector of that thread, so the rescan costs one load
 // round trip instead of one per vector.  Returns (to every lane) the first index of val among
 // those elements and the sum of 2^(k l - c) over them without that index.
-__device__ __forceinline__ void lean_rescan_warp(const uint4 *row, int lo, int hi, int lane, int src,
+template <class ROW>
+__device__ __forceinline__ void lean_rescan_warp(const ROW &row, int lo, int hi, int lane, int src,
                                                  float val, float k, float c, int &first_idx,
                                                  float &s_excl) {
     int fi = 0x7fffffff;
     // pass 1: first index
     for (int vj = lo + src + 32 * lane; vj < hi; vj += 32 * 32) {
-        float v[8];
-        unpack_bf16x8(row[vj], v);
+        const auto v = row[vj];
 #pragma unroll
         for (int i = 7; i >= 0; --i)
-            if (v[i] == val) fi = min(fi, vj * 8 + i);
+            if (v.get(i) == val) fi = min(fi, vj * 8 + i);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) fi = min(fi, __shfl_xor_sync(kFull, fi, o));
     // pass 2: the sum without it (the vectors are L1/L2 hits now)
     float s = 0.f;
     for (int vj = lo + src + 32 * lane; vj < hi; vj += 32 * 32) {
-        float v[8];
-        unpack_bf16x8(row[vj], v);
+        const auto v = row[vj];
         float e[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) e[i] = (vj * 8 + i == fi) ? 0.f : ex2(__fmaf_rn(v[i], k, -c));
+        for (int i = 0; i < 8; ++i) e[i] = (vj * 8 + i == fi) ? 0.f : ex2(__fmaf_rn(v.get(i), k, -c));
         s += ((e[0] + e[1]) + (e[2] + e[3])) + ((e[4] + e[5]) + (e[6] + e[7]));
     }
     s_excl = warp_sum(s);
@@ -285,11 +278,11 @@ __device__ __forceinline__ void lean_rescan_warp(const uint4 *row, int lo, int h
 // Row-level (max, argmax, sum without the argmax) of the target (r = 0) and, if BOTH, the draft
 // (r = 1) from the per-thread pass-A states.  Leaves the per-warp masses (row scale, argmax left
 // out) in sh.wmass[r] for the samplers.  All threads call it.
-template <bool BOTH>
-__device__ void lean_reduce2(const LeanAcc &tp, const LeanAcc &tq, const uint4 *vp, const uint4 *vq, int lo,
+template <bool BOTH, typename LT, class ROW>
+__device__ void lean_reduce2(const LeanAcc<LT> &tp, const LeanAcc<LT> &tq, const ROW &vp, const ROW &vq, int lo,
                              int hi, float k, LeanShared &sh, ArgMaxSum &P, ArgMaxSum &Q) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    const float mlp = bf2_hmax(tp.m2), mlq = BOTH ? bf2_hmax(tq.m2) : neg_inf();
+    const float mlp = tp.max(), mlq = BOTH ? tq.max() : neg_inf();
     float wp = mlp, wq = mlq;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -549,7 +542,8 @@ __device__ __forceinline__ float slice_mass(const LeanShared &sh, int r, const R
 // Draw inside this CTA's slice from softmax(row) without token `excl`, target t (row scale,
 // relative to the start of the slice).  sh.wmass[r] holds the per-warp sums of the slice on the
 // slice's own scale with the slice argmax left out.
-__device__ inline int lean_sample_slice(const Geo &g, const __nv_bfloat16 *row, float k, const RowStat &st,
+template <class ROW>
+__device__ int lean_sample_slice(const Geo &g, const ROW &row, float k, const RowStat &st,
                                  int excl, float t, int r, LeanShared &sh) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int locarg = sh.x_idx[r];
@@ -569,10 +563,9 @@ __device__ inline int lean_sample_slice(const Geo &g, const __nv_bfloat16 *row, 
         if (warp == wex) {
             float s = 0.f;
             for (int vi = g.seg_lo(warp) + lane; vi < g.seg_hi(warp); vi += 32) {
-                float v[8];
-                load_vec<__nv_bfloat16, true>(row, vi, g.V, v);
+                const auto v = row[vi];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) s += (vi * 8 + i == excl) ? 0.f : ex2(__fmaf_rn(v[i], k, -C));
+                for (int i = 0; i < 8; ++i) s += (vi * 8 + i == excl) ? 0.f : ex2(__fmaf_rn(v.get(i), k, -C));
             }
             s = warp_sum(s);
             if (lane == 0) sh.mass[warp] = s;
@@ -580,10 +573,9 @@ __device__ inline int lean_sample_slice(const Geo &g, const __nv_bfloat16 *row, 
         __syncthreads();
     }
     auto wf = [&](int vi, float(&w)[8]) {
-        float v[8];
-        load_vec<__nv_bfloat16, true>(row, vi, g.V, v);
+        const auto v = row[vi];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) w[i] = (vi * 8 + i == excl) ? 0.f : ex2(__fmaf_rn(v[i], k, -C));
+        for (int i = 0; i < 8; ++i) w[i] = (vi * 8 + i == excl) ? 0.f : ex2(__fmaf_rn(v.get(i), k, -C));
     };
     return block_sample3(g, wf, sh, t);
 }
@@ -591,8 +583,8 @@ __device__ inline int lean_sample_slice(const Geo &g, const __nv_bfloat16 *row, 
 // Draw from softmax(row) without `excl` (the row argmax, a slice argmax, or nothing) over the
 // whole row: every CTA of the row calls it; the CTA whose slice holds the target draws and
 // returns the token, the others return -2.  -1: no mass.
-template <int CS>
-__device__ int lean_sample_row(const Geo &g, const __nv_bfloat16 *row, float k, const RowStat &st, int me,
+template <int CS, class ROW>
+__device__ int lean_sample_row(const Geo &g, const ROW &row, float k, const RowStat &st, int me,
                                int excl, float u, int r, LeanShared &sh) {
     float m[CS];
     float total = 0.f;
@@ -665,16 +657,14 @@ __device__ __forceinline__ int lean_ck_interval(const Geo &g) {
     return 4 * max(1, (iters + 4 * kLeanCk - 1) / (4 * kLeanCk));   // a multiple of the unroll of pass A
 }
 
-__device__ __forceinline__ void lean_pass_a_ck(const uint4 *rq, int lo, int hi, int lane, float k, int CK,
-                                               LeanAcc &Q, float *cks, float *ckc) {
-    LeanAcc st;
-    st.m2 = 0xff80ff80u; st.s = 0.f; st.c = 0.f;
+template <bool SHIFT, typename LT, class ROW>
+__device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, int lane, float k, int CK,
+                                               LeanAcc<LT> &Q, float *cks, float *ckc) {
+    LeanAcc<LT> st;
+    st.init();
     {   // one exponent reference for the whole warp: the maximum of its first vectors
         float m0 = neg_inf();
-        if (lo + lane < hi) {
-            const uint4 a = rq[lo + lane];
-            m0 = bf2_hmax(bf2max(bf2max(a.x, a.y), bf2max(a.z, a.w)));
-        }
+        if (lo + lane < hi) m0 = rq[lo + lane].max();
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) m0 = fmaxf(m0, __shfl_xor_sync(kFull, m0, o));
         if (m0 > neg_inf()) st.c = shift_of(m0, k);
@@ -702,28 +692,30 @@ __device__ __forceinline__ void lean_pass_a_ck(const uint4 *rq, int lo, int hi, 
     };
     const int iters = (hi - lo + 31) >> 5;   // lane-iterations of this warp
     const int nfull = (hi - lo) >> 5;        // those in which every lane has a vector
-    const uint4 *p = rq + lo + lane;
+    const int v0 = lo + lane;
     int it = 0, since = 0;
-    // four vectors per lane in flight; the next four are requested before the current ones are
-    // consumed, so that the checkpoint's shuffle chain overlaps the loads
-    uint4 n0 = make_uint4(0, 0, 0, 0), n1 = n0, n2 = n0, n3 = n0;
-    if (4 <= nfull) { n0 = p[0]; n1 = p[32]; n2 = p[64]; n3 = p[96]; }
-    for (; it + 4 <= nfull; it += 4) {
-        const uint4 a0 = n0, a1 = n1, a2 = n2, a3 = n3;
-        if (it + 8 <= nfull) {
-            n0 = p[32 * (it + 4)]; n1 = p[32 * (it + 5)]; n2 = p[32 * (it + 6)]; n3 = p[32 * (it + 7)];
-        }
-        lean_push(st, a0, k);
-        lean_push(st, a1, k);
-        lean_push(st, a2, k);
-        lean_push(st, a3, k);
-        since += 4;
+    auto push = [&](const Vec8<LT> &v) { lean_push(st, v, k); };
+    auto after = [&](int d) {
+        since += d;
         if (since >= CK) { checkpoint(); since = 0; }
+    };
+    auto slow = [&](int to) {
+#pragma unroll 1
+        for (; it < to; ++it) {
+            if (v0 + 32 * it < hi) push(rq[v0 + 32 * it]);
+            after(1);
+        }
+    };
+    // (the loads of the next vectors also overlap the checkpoint's shuffle chain)
+    if constexpr (SHIFT) {
+        const InsideIters t = inside_iters(rq.src, rq.src, lo, hi);
+        slow(t.i0);
+        if (rq.src.sh == 0) it = inside_ahead(AlignedInside<LT>{rq.src}, v0, it, t.i1, push, after);
+        else it = inside_ahead(ShiftedInside<LT>{rq.src}, v0, it, t.i1, push, after);
+    } else {
+        it = inside_ahead(rq, v0, it, nfull, push, after);
     }
-    for (; it < iters; ++it) {
-        if (lo + lane + 32 * it < hi) lean_push(st, p[32 * it], k);
-        if (++since >= CK) { checkpoint(); since = 0; }
-    }
+    slow(iters);
     if (since > 0) checkpoint();
     if (lane == 0)
         for (; j < kLeanCk; ++j) { cks[j] = 0.f; ckc[j] = 0.f; }
@@ -733,15 +725,15 @@ __device__ __forceinline__ void lean_pass_a_ck(const uint4 *rq, int lo, int hi, 
 // Inverse-CDF draw from softmax(row) without token `excl` (excl < 0: nothing left out) over the
 // checkpoint sub-blocks.  C = the row's exponent shift.  Returns to every thread the token, -1 if
 // nothing has mass.  Called by all threads of the CTA, after the checkpoints are visible.
-__device__ inline int lean_ck_sample(const Geo &g, const __nv_bfloat16 *row, float k, float C, int CK, int excl,
+template <class ROW>
+__device__ int lean_ck_sample(const Geo &g, const ROW &row, float k, float C, int CK, int excl,
                               float u, LeanCkShared &sh) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nslot = g.nwarps * kLeanCk;
     auto wf = [&](int vi, float(&w)[8]) {
-        float v[8];
-        load_vec<__nv_bfloat16, true>(row, vi, g.V, v);
+        const auto v = row[vi];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) w[i] = (vi * 8 + i == excl) ? 0.f : ex2(__fmaf_rn(v[i], k, -C));
+        for (int i = 0; i < 8; ++i) w[i] = (vi * 8 + i == excl) ? 0.f : ex2(__fmaf_rn(v.get(i), k, -C));
     };
     for (int s = threadIdx.x; s < nslot; s += blockDim.x) {
         const float cs = sh.cks[s / kLeanCk][s % kLeanCk];
@@ -824,31 +816,30 @@ __device__ inline int lean_ck_sample(const Geo &g, const __nv_bfloat16 *row, flo
 // pass A over p with checkpoints, then the sub-block sampler.  CTAs of verifying rows leave at
 // once; the verification kernels skip the leaf rows.  Up to three output sets receive the result
 // (the three-method call: the methods share u_res, hence the bonus token).
-template <int THREADS>
-__global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_leaf_kernel(LeafArgs A) {
+template <typename LT, bool SHIFT, int THREADS>
+__global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_leaf_kernel(LeafArgs A) {
     __shared__ LeanCkShared sh;
     const RowArgs &a = A.r;
     const long long r = blockIdx.x;
     const int b = static_cast<int>(r / a.nodes), n = static_cast<int>(r % a.nodes);
     if (!(a.node_kind && a.node_kind[n] == SPECHUB_NODE_LEAF)) return;
-    const __nv_bfloat16 *rowp = static_cast<const __nv_bfloat16 *>(a.target) + b * a.stride_seq + n * a.stride_node;
-    const uint4 *vp = reinterpret_cast<const uint4 *>(rowp);
+    const StreamRow<LT, SHIFT> vp(static_cast<const LT *>(a.target) + b * a.stride_seq + n * a.stride_node, a.vocab);
     const Geo g = make_geo(a.vocab, 8);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int lo = g.seg_lo(warp), hi = g.seg_hi(warp);
     const float k = kLog2e / temperature_of(a, b);
     const float ures = a.uniforms[r * 5 + 4];
     const int CK = lean_ck_interval(g);
-    LeanAcc tp, unused;
-    unused.m2 = 0xff80ff80u; unused.s = 0.f; unused.c = 0.f;
-    lean_pass_a_ck(vp, lo, hi, lane, k, CK, tp, sh.cks[warp], sh.ckc[warp]);
+    LeanAcc<LT> tp, unused;
+    unused.init();
+    lean_pass_a_ck<SHIFT>(vp, lo, hi, lane, k, CK, tp, sh.cks[warp], sh.ckc[warp]);
     ArgMaxSum Ps, unusedq;
     lean_reduce2<false>(tp, unused, vp, vp, lo, hi, k, sh, Ps, unusedq);
     const float Zp = Ps.sx + Ps.own(k);
     uint32_t status = 0;
     int tok = -1;
     if (!(Ps.ml > neg_inf()) || !(Ps.ml < -neg_inf()) || !finite_pos(Zp)) status = SPECHUB_ST_NONFINITE;
-    else tok = lean_ck_sample(g, rowp, k, Ps.c, CK, -1, ures, sh);
+    else tok = lean_ck_sample(g, vp, k, Ps.c, CK, -1, ures, sh);
     if (threadIdx.x == 0) {
         for (int m = 0; m < A.n_out; ++m) {
             const NodeOutPtrs &o = A.out[m];
@@ -875,9 +866,10 @@ __device__ __forceinline__ void lean_terms(float ep, float eq, float rho, float 
 // Sum of a row's exponentials outside id x, from the row's (maximum, argmax, sum without the argmax): RRSw's
 // renormaliser 1 - q(x1) times Z_q without a pass over the row.  The argmax is left out of st.sx already; any
 // other id holds at most half of the mass, so subtracting its own term costs at most one bit.
-__device__ __forceinline__ float sum_without(const RowStat &st, const __nv_bfloat16 *row, int x, float k) {
+template <class ROW>
+__device__ __forceinline__ float sum_without(const RowStat &st, const ROW &row, int x, float k) {
     if (x == st.idx) return st.sx;
-    return __fsub_rn(__fadd_rn(st.sx, st.own), lean_exp(load_one<__nv_bfloat16>(row, x), k, st.C));
+    return __fsub_rn(__fadd_rn(st.sx, st.own), lean_exp(row.one(x), k, st.C));
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -894,8 +886,9 @@ __device__ __forceinline__ float sum_without(const RowStat &st, const __nv_bfloa
 // SPECHUB_ST_STATS.  The passes are register-fed, with L2 eviction hints on the loads (keep the target row
 // after pass A, let the rows go at their last use): with a single row to keep in L2 between passes that
 // beats the rings (RRS 1.53 -> 1.46 ms, RRSw 1.62 -> 1.60 ms on V = 128256, 7936 rows).
-template <int METHOD, int THREADS, int CS, bool RING = false, bool STATS = false>
-__global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_verify_kernel(RowArgs a) {
+template <typename LT, bool SHIFT, int METHOD, int THREADS, int CS, bool RING = false, bool STATS = false>
+__global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_verify_kernel(RowArgs a) {
+    static_assert(!RING || (sizeof(LT) == 2 && !SHIFT), "the ring-fed form: bf16 rows in whole words");
     static_assert(!RING || (CS == 1 && METHOD != kSpecHub), "the ring-fed form: whole rows, RRS and RRSw");
     static_assert(!STATS || (CS == 1 && !RING), "draft statistics: whole rows, register-fed passes");
     __shared__ LeanShared sh;
@@ -904,9 +897,9 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_verify_kernel(Ro
     const int me = RowGroup<CS>::rank();
     const long long r = blockIdx.x / CS;
     const int b = static_cast<int>(r / a.nodes), n = static_cast<int>(r % a.nodes);
-    const __nv_bfloat16 *rowp = static_cast<const __nv_bfloat16 *>(a.target) + b * a.stride_seq + n * a.stride_node;
-    const __nv_bfloat16 *rowq = static_cast<const __nv_bfloat16 *>(a.draft) + b * a.stride_seq + n * a.stride_node;
-    const uint4 *vp = reinterpret_cast<const uint4 *>(rowp), *vq = reinterpret_cast<const uint4 *>(rowq);
+    using V = Vec8<LT>;
+    const StreamRow<LT, SHIFT> vp(static_cast<const LT *>(a.target) + b * a.stride_seq + n * a.stride_node, a.vocab);
+    const StreamRow<LT, SHIFT> vq(static_cast<const LT *>(a.draft) + b * a.stride_seq + n * a.stride_node, a.vocab);
     const Geo g = make_geo(a.vocab, 8, CS, me);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int lo = g.seg_lo(warp), hi = g.seg_hi(warp);
@@ -937,18 +930,25 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_verify_kernel(Ro
         // (a record of a row without a finite maximum or sum needs no look-up: the row is flagged
         // SPECHUB_ST_NONFINITE below, as it is without the record)
         if (ok && ds.ml > neg_inf() && ds.ml < pinf && finite_pos(ds.sx + 1.f))
-            ok = ds.idx >= 0 && ds.idx < a.vocab && load_one<__nv_bfloat16>(rowq, ds.idx) == ds.ml;
+            ok = ds.idx >= 0 && ds.idx < a.vocab && vq.one(ds.idx) == ds.ml;
         sh.stat_ok = ok;
         sh.x_ml[1] = ds.ml; sh.x_sx[1] = ds.sx; sh.x_idx[1] = ok ? ds.idx : 0;
     }
     // the row's stream: pass A forwards, pass B backwards, (RRS, RRSw) pass C forwards
     WarpRing R;
-    if (RING) ring_begin(R, ring_mem + warp * kRingWarpBytes, ring_bars[warp], vp, vq, lo, hi, 3, 2u, lane);
-    LeanAcc tp, tq;
-    if (RING) lean_pass_a_ring(R, lane, k, tp, tq);
-    else if (STATS) lean_pass_a_deep(vp, lo, hi, lane, k, tp);
-    else if (leaf) lean_pass_a<false>(vp, vq, lo, hi, lane, k, tp, tq);
-    else lean_pass_a<true, METHOD == kRRS>(vp, vq, lo, hi, lane, k, tp, tq);
+    LeanAcc<LT> tp, tq;
+    if constexpr (RING) {
+        ring_begin(R, ring_mem + warp * kRingWarpBytes, ring_bars[warp], reinterpret_cast<const uint4 *>(vp.row),
+                   reinterpret_cast<const uint4 *>(vq.row), lo, hi, 3, 2u, lane);
+        lean_pass_a_ring(R, vp, vq, lane, k, tp, tq);
+    } else if constexpr (SHIFT) {
+        lean_pass_a_any(vp, vq, lo, hi, lane, k, tp, tq);
+    } else if constexpr (STATS) {
+        lean_pass_a_deep(vp, lo, hi, lane, k, tp);
+    } else {
+        if (leaf) lean_pass_a<false, false>(vp, vq, lo, hi, lane, k, tp, tq);
+        else lean_pass_a<true, METHOD == kRRS>(vp, vq, lo, hi, lane, k, tp, tq);
+    }
     {
         ArgMaxSum Ps, Qs;
         if (leaf || STATS) lean_reduce2<false>(tp, tq, vp, vq, lo, hi, k, sh, Ps, Qs);
@@ -980,10 +980,10 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_verify_kernel(Ro
         return true;
     };
     const int x1 = a.draft_tokens_in[2 * r], x2 = a.draft_tokens_in[2 * r + 1];
-    auto prob_p = [&](int y) { return prob_of(load_one<__nv_bfloat16>(rowp, y), k, cP, invZp); };
-    auto prob_q = [&](int y) { return prob_of(load_one<__nv_bfloat16>(rowq, y), k, cQ, invZq); };
+    auto prob_p = [&](int y) { return prob_of(vp.one(y), k, cP, invZp); };
+    auto prob_q = [&](int y) { return prob_of(vq.one(y), k, cQ, invZq); };
     auto draw_from_p = [&]() {  // every CTA of the row calls it
-        const int tok = lean_sample_row<CS>(g, rowp, k, P, me, -1, ures, 0, sh);
+        const int tok = lean_sample_row<CS>(g, vp, k, P, me, -1, ures, 0, sh);
         if (tok != -2 && threadIdx.x == 0) a.token[r] = tok;
         token_elsewhere = true;
     };
@@ -1031,23 +1031,15 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_verify_kernel(Ro
             s1 = s2 = rr = f2_make(0.f, 0.f);
             const F2 k2 = f2_make(k, k), ncp2 = f2_make(-cP, -cP), ncq2 = f2_make(-cQ, -cQ);
             const F2 nrho2 = f2_make(-rho, -rho), ncrho2 = f2_make(-crho, -crho);
-            auto vec_b = [&](int vi, const uint4 &cp, const uint4 &cq) {
-                if (STATS) diff |= (cp.x ^ cq.x) | (cp.y ^ cq.y) | (cp.z ^ cq.z) | (cp.w ^ cq.w);
-                unsigned wps[4] = {cp.x, cp.y, cp.z, cp.w}, wqs[4] = {cq.x, cq.y, cq.z, cq.w};
+            auto vec_b = [&](int vi, V cp, V cq) {
+                if (STATS) diff |= cp.differs(cq);
                 if (vi == hubvec) {   // the hub's own pair is no part of the sums over y != a: -inf, mass 0
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        if (i == (hubel >> 1)) {
-                            const unsigned keep = (hubel & 1) ? 0x0000ffffu : 0xffff0000u;
-                            const unsigned ninf = (hubel & 1) ? 0xff800000u : 0x0000ff80u;
-                            wps[i] = (wps[i] & keep) | ninf;
-                            wqs[i] = (wqs[i] & keep) | ninf;
-                        }
-                    }
+                    cp.drop(hubel);
+                    cq.drop(hubel);
                 }
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const F2 ep = f2_exp_word(wps[i], k2, ncp2), eq = f2_exp_word(wqs[i], k2, ncq2);
+                    const F2 ep = f2_exp(cp.pair(i), k2, ncp2), eq = f2_exp(cq.pair(i), k2, ncq2);
                     const F2 d = f2_fma(nrho2, eq, ep);       // Z_p (p - q)
                     const F2 m = f2_max0(d);
                     const F2 t = f2_fma(ncrho2, eq, m);       // Z_p (max(p - q, 0) - c q)
@@ -1057,7 +1049,9 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_verify_kernel(Ro
                     rr = f2_add(rr, w);
                 }
             };
-            {
+            if constexpr (SHIFT) {
+                any_pairs<-1>(vp, vq, lo, hi, lane, vec_b);
+            } else {
                 // software pipeline: the next vector pair is in registers before this one is consumed.
                 // This is the last use of both rows: the loads tell L2 to let these lines go first (one
                 // CTA per row: 1.38 -> 1.30 ms on V = 128256; from draft statistics, where pass A also told
@@ -1066,13 +1060,13 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_verify_kernel(Ro
                 uint64_t polf = 0;
                 constexpr bool kHintB = STATS || CS == 1;
                 if (kHintB) asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(polf));
-                auto ldb = [&](const uint4 *ptr) { return kHintB ? ld_l2_hint(ptr, polf) : *ptr; };
-                uint4 np = make_uint4(0, 0, 0, 0), nq = np;
-                if (last_vi >= lo) { np = ldb(vp + last_vi); nq = ldb(vq + last_vi); }
+                auto ldb = [&](const StreamRow<LT, SHIFT> &row, int vi) { return kHintB ? row.fetch(vi, polf) : row.fetch(vi); };
+                V np = V::none(), nq = np;
+                if (last_vi >= lo) { np = ldb(vp, last_vi); nq = ldb(vq, last_vi); }
 #pragma unroll 1
                 for (int vi = last_vi; vi >= lo; vi -= 32) {
-                    const uint4 cp = np, cq = nq;
-                    if (vi - 32 >= lo) { np = ldb(vp + vi - 32); nq = ldb(vq + vi - 32); }
+                    const V cp = np, cq = nq;
+                    if (vi - 32 >= lo) { np = ldb(vp, vi - 32); nq = ldb(vq, vi - 32); }
                     vec_b(vi, cp, cq);
                 }
             }
@@ -1124,13 +1118,11 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_verify_kernel(Ro
                         if (threadIdx.x < g.nwarps) sh.mass[threadIdx.x] = sh.acc[2][threadIdx.x];
                         __syncthreads();
                         auto wf = [&](int vi, float(&w)[8]) {
-                            float fp[8], fq[8];
-                            unpack_bf16x8(vp[vi], fp);
-                            unpack_bf16x8(vq[vi], fq);
+                            const V fp = vp[vi], fq = vq[vi];
 #pragma unroll
                             for (int i = 0; i < 8; ++i) {
                                 float d, t;
-                                lean_terms(lean_exp(fp[i], k, cP), lean_exp(fq[i], k, cQ), rho, crho, d, t);
+                                lean_terms(lean_exp(fp.get(i), k, cP), lean_exp(fq.get(i), k, cQ), rho, crho, d, t);
                                 w[i] = (vi * 8 + i == hubtok) ? 0.f : fmaxf(t, 0.f);
                             }
                         };
@@ -1159,14 +1151,13 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_verify_kernel(Ro
             // RRSw: the next vector pair is loaded before the current one is consumed (measured:
             // 2.21 -> 2.03 ms on V = 128256; for RRS the plain loop unrolled twice is the faster one)
             constexpr bool PIPE = (METHOD == kRRSw);
-            auto vec_b = [&](int vi, const uint4 &cp, const uint4 &cq) {
-                if (STATS) diff |= (cp.x ^ cq.x) | (cp.y ^ cq.y) | (cp.z ^ cq.z) | (cp.w ^ cq.w);
-                const unsigned wps[4] = {cp.x, cp.y, cp.z, cp.w}, wqs[4] = {cq.x, cq.y, cq.z, cq.w};
+            auto vec_b = [&](int vi, const V &cp, const V &cq) {
+                if (STATS) diff |= cp.differs(cq);
                 F2 eq[4];   // e_q of the vector, by words
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    eq[i] = f2_exp_word(wqs[i], k2, ncq2);
-                    a1 = f2_add(a1, f2_max0(f2_fma(nrho2, eq[i], f2_exp_word(wps[i], k2, ncp2))));
+                    eq[i] = f2_exp(cq.pair(i), k2, ncq2);
+                    a1 = f2_add(a1, f2_max0(f2_fma(nrho2, eq[i], f2_exp(cp.pair(i), k2, ncp2))));
                 }
                 if (METHOD == kRRSw && !STATS) {   // (from draft statistics: sum_without, below)
                     float qq[8];
@@ -1181,28 +1172,34 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_verify_kernel(Ro
                     dnb += (qq[4] + qq[5]) + (qq[6] + qq[7]);
                 }
             };
-            uint4 np = make_uint4(0, 0, 0, 0), nq = np;
+            V np = V::none(), nq = np;
             auto pass_b = [&](bool from_ring) {
             a1 = f2_make(0.f, 0.f); dna = 0.f; dnb = 0.f;
             ncp2 = f2_make(-cP, -cP); nrho2 = f2_make(-rho, -rho);
-            if (RING && from_ring) {
+            if constexpr (RING) {
+            if (from_ring) {
 #pragma unroll 1
                 for (int c = R.nc - 1; c >= 0; --c) {
                     ring_wait(R);
                     const int v0 = lo + lane + c * kRingChunkVecs;
 #pragma unroll
                     for (int j = kRingCh - 1; j >= 0; --j) {
-                        uint4 x, y;
+                        V x, y;
                         ring_load(R, j, lane, x, y);
                         if (j == 0) ring_release(R, lane);
                         if (v0 + j * 32 < hi) vec_b(v0 + j * 32, x, y);
                     }
                 }
+                return;
+            }
+            }
+            if constexpr (SHIFT) {
+                any_pairs<-1>(vp, vq, lo, hi, lane, vec_b);
             } else {
                 if (PIPE && last_vi >= lo) { np = vp[last_vi]; nq = vq[last_vi]; }
 #pragma unroll(PIPE ? 1 : 2)
                 for (int vi = last_vi; vi >= lo; vi -= 32) {
-                    uint4 cp, cq;
+                    V cp, cq;
                     if (PIPE) {
                         cp = np; cq = nq;
                         if (vi - 32 >= lo) { np = vp[vi - 32]; nq = vq[vi - 32]; }
@@ -1220,7 +1217,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_verify_kernel(Ro
             float acc[2] = {a1a + a1b, dna + dnb};
             float part2[2][CS];
             lean_row_sums<CS, 2, 0>(acc, part2, sh);  // [2]
-            if (STATS && METHOD == kRRSw) acc[1] = sum_without(Q, rowq, x1, k);
+            if (STATS && METHOD == kRRSw) acc[1] = sum_without(Q, vq, x1, k);
             const float A1 = acc[0] * invZp, den = acc[1] * invZq;   // the sums are of exponentials
             const bool q1_zero = (METHOD == kRRSw) && !(den > 0.f);
             const float gq = (METHOD == kRRSw) ? (q1_zero ? 0.f : 1.f / den) : 1.f;
@@ -1229,52 +1226,53 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_verify_kernel(Ro
             // pass C: mass of the residual after two rejections
             F2 w2 = f2_make(0.f, 0.f);
             const F2 nsc2 = f2_make(-A1grho, -A1grho);
-            auto vec_c = [&](int vi, const uint4 &cp, const uint4 &cq) {
-                const unsigned wps[4] = {cp.x, cp.y, cp.z, cp.w}, wqs[4] = {cq.x, cq.y, cq.z, cq.w};
+            auto vec_c = [&](int vi, const V &cp, const V &cq) {
                 if (METHOD == kRRSw && vi == x1vec) {   // (one vector of the row) q1(x1) = 0: that lane's scale is 0
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         F2 nsc = nsc2;
                         if (i == (x1el >> 1)) nsc = (x1el & 1) ? f2_make(-A1grho, 0.f) : f2_make(0.f, -A1grho);
-                        const F2 eq = f2_exp_word(wqs[i], k2, ncq2);
-                        const F2 m = f2_max0(f2_fma(nrho2, eq, f2_exp_word(wps[i], k2, ncp2)));
+                        const F2 eq = f2_exp(cq.pair(i), k2, ncq2);
+                        const F2 m = f2_max0(f2_fma(nrho2, eq, f2_exp(cp.pair(i), k2, ncp2)));
                         w2 = f2_add(w2, f2_max0(f2_fma(nsc, eq, m)));
                     }
                     return;
                 }
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const F2 eq = f2_exp_word(wqs[i], k2, ncq2);
-                    const F2 m = f2_max0(f2_fma(nrho2, eq, f2_exp_word(wps[i], k2, ncp2)));
+                    const F2 eq = f2_exp(cq.pair(i), k2, ncq2);
+                    const F2 m = f2_max0(f2_fma(nrho2, eq, f2_exp(cp.pair(i), k2, ncp2)));
                     w2 = f2_add(w2, f2_max0(f2_fma(nsc2, eq, m)));
                 }
             };
-            if (RING) {
+            if constexpr (RING) {
 #pragma unroll 1
                 for (int c = 0; c < R.nc; ++c) {
                     ring_wait(R);
                     const int v0 = lo + lane + c * kRingChunkVecs;
 #pragma unroll
                     for (int j = 0; j < kRingCh; ++j) {
-                        uint4 x, y;
+                        V x, y;
                         ring_load(R, j, lane, x, y);
                         if (j == kRingCh - 1) ring_release(R, lane);
                         if (v0 + j * 32 < hi) vec_c(v0 + j * 32, x, y);
                     }
                 }
+            } else if constexpr (SHIFT) {
+                any_pairs<1>(vp, vq, lo, hi, lane, vec_c);
             } else {
                 uint64_t polc = 0;   // one CTA per row: the rows' last use, L2 may let these lines go first
                 if (CS == 1) asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(polc));
-                auto ldc = [&](const uint4 *ptr) { return CS == 1 ? ld_l2_hint(ptr, polc) : *ptr; };
-                if (PIPE && lo + lane < hi) { np = ldc(vp + lo + lane); nq = ldc(vq + lo + lane); }
+                auto ldc = [&](const StreamRow<LT, SHIFT> &row, int vi) { return CS == 1 ? row.fetch(vi, polc) : row.fetch(vi); };
+                if (PIPE && lo + lane < hi) { np = ldc(vp, lo + lane); nq = ldc(vq, lo + lane); }
 #pragma unroll(PIPE ? 1 : 2)
                 for (int vi = lo + lane; vi < hi; vi += 32) {
-                    uint4 cp, cq;
+                    V cp, cq;
                     if (PIPE) {
                         cp = np; cq = nq;
-                        if (vi + 32 < hi) { np = ldc(vp + vi + 32); nq = ldc(vq + vi + 32); }
+                        if (vi + 32 < hi) { np = ldc(vp, vi + 32); nq = ldc(vq, vi + 32); }
                     } else {
-                        cp = ldc(vp + vi); cq = ldc(vq + vi);
+                        cp = ldc(vp, vi); cq = ldc(vq, vi);
                     }
                     vec_c(vi, cp, cq);
                 }
@@ -1311,14 +1309,12 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_verify_kernel(Ro
                         if (threadIdx.x < g.nwarps) sh.mass[threadIdx.x] = sh.acc[0][threadIdx.x];
                         __syncthreads();
                         auto wf = [&](int vi, float(&w)[8]) {
-                            float fp[8], fq[8];
-                            unpack_bf16x8(vp[vi], fp);
-                            unpack_bf16x8(vq[vi], fq);
+                            const V fp = vp[vi], fq = vq[vi];
 #pragma unroll
                             for (int i = 0; i < 8; ++i) {
                                 float d, t;
                                 const float s = (METHOD == kRRSw && vi * 8 + i == x1) ? 0.f : A1grho;
-                                lean_terms(lean_exp(fp[i], k, cP), lean_exp(fq[i], k, cQ), rho, s, d, t);
+                                lean_terms(lean_exp(fp.get(i), k, cP), lean_exp(fq.get(i), k, cQ), rho, s, d, t);
                                 w[i] = fmaxf(t, 0.f);
                             }
                         };
@@ -1356,7 +1352,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_kernel(Row
     const long long r = blockIdx.x / CS;
     const int b = static_cast<int>(r / a.nodes), n = static_cast<int>(r % a.nodes);
     const __nv_bfloat16 *rowq = static_cast<const __nv_bfloat16 *>(a.draft) + b * a.stride_seq + n * a.stride_node;
-    const uint4 *vq = reinterpret_cast<const uint4 *>(rowq);
+    const StreamRow<__nv_bfloat16, false> vq(rowq, a.vocab);
     const Geo g = make_geo(a.vocab, 8, CS, me);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int lo = g.seg_lo(warp), hi = g.seg_hi(warp);
@@ -1364,8 +1360,8 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_kernel(Row
     const float u1 = a.uniforms[r * 5 + 0], u2 = a.uniforms[r * 5 + 1];
     const bool writer = (me == 0 && threadIdx.x == 0);
 
-    LeanAcc tq, unused;
-    lean_pass_a<false>(vq, vq, lo, hi, lane, k, tq, unused);
+    LeanAcc<__nv_bfloat16> tq, unused;
+    lean_pass_a<false, false>(vq, vq, lo, hi, lane, k, tq, unused);
     {
         ArgMaxSum q, unusedq;
         lean_reduce2<false>(tq, unused, vq, vq, lo, hi, k, sh, q, unusedq);
@@ -1388,7 +1384,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_kernel(Row
         }
     } else {
         // x1 ~ q.  The CTA whose slice holds the target draws it and tells the others.
-        const int t1 = lean_sample_row<CS>(g, rowq, k, Q, me, -1, u1, 0, sh);
+        const int t1 = lean_sample_row<CS>(g, vq, k, Q, me, -1, u1, 0, sh);
         int x1 = t1;
         if (CS > 1) {
             if (t1 != -2 && threadIdx.x == 0) sh.x_tok = t1;
@@ -1412,7 +1408,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_kernel(Row
                 x2 = (hubtok == 0) ? 1 : 0;
                 st |= SPECHUB_ST_DEGENERATE_Q;
             } else {
-                const int t2 = lean_sample_row<CS>(g, rowq, k, Q, me, hubtok, u2, 0, sh);
+                const int t2 = lean_sample_row<CS>(g, vq, k, Q, me, hubtok, u2, 0, sh);
                 x2_elsewhere = true;
                 if (t2 != -2 && threadIdx.x == 0) {
                     a.draft_tokens_out[2 * r + 1] = t2;
@@ -1421,7 +1417,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_kernel(Row
                 }
             }
         } else if (method == kRRS) {
-            const int t2 = lean_sample_row<CS>(g, rowq, k, Q, me, -1, u2, 0, sh);
+            const int t2 = lean_sample_row<CS>(g, vq, k, Q, me, -1, u2, 0, sh);
             x2_elsewhere = true;
             if (t2 != -2 && threadIdx.x == 0) a.draft_tokens_out[2 * r + 1] = t2;
         } else {
@@ -1447,7 +1443,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_kernel(Row
                 st |= SPECHUB_ST_DEGENERATE_Q;
                 if (writer) a.draft_tokens_out[2 * r + 1] = (x1 == 0) ? 1 : 0;
             } else if (sel == me) {
-                const int t2 = lean_sample_slice(g, rowq, k, Q, x1, u2 * total - base, 0, sh);
+                const int t2 = lean_sample_slice(g, vq, k, Q, x1, u2 * total - base, 0, sh);
                 if (threadIdx.x == 0) a.draft_tokens_out[2 * r + 1] = t2;
             }
         }
@@ -1468,13 +1464,12 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_kernel(Row
 // ------------------------------------------------------------------------------------------------
 // Draft step, one CTA per row (checkpointed pass A and sub-block sampler above).
 // ------------------------------------------------------------------------------------------------
-template <int THREADS>
-__global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(RowArgs a, int method) {
+template <typename LT, bool SHIFT, int THREADS>
+__global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_draft_ck_kernel(RowArgs a, int method, bool keep_stats) {
     __shared__ LeanCkShared sh;
     const long long r = blockIdx.x;
     const int b = static_cast<int>(r / a.nodes), n = static_cast<int>(r % a.nodes);
-    const __nv_bfloat16 *rowq = static_cast<const __nv_bfloat16 *>(a.draft) + b * a.stride_seq + n * a.stride_node;
-    const uint4 *vq = reinterpret_cast<const uint4 *>(rowq);
+    const StreamRow<LT, SHIFT> vq(static_cast<const LT *>(a.draft) + b * a.stride_seq + n * a.stride_node, a.vocab);
     const Geo g = make_geo(a.vocab, 8);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int lo = g.seg_lo(warp), hi = g.seg_hi(warp);
@@ -1482,9 +1477,9 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
     const float u1 = a.uniforms[r * 5 + 0], u2 = a.uniforms[r * 5 + 1];
     const int CK = lean_ck_interval(g);
 
-    LeanAcc tq, unused;
-    unused.m2 = 0xff80ff80u; unused.s = 0.f; unused.c = 0.f;
-    lean_pass_a_ck(vq, lo, hi, lane, k, CK, tq, sh.cks[warp], sh.ckc[warp]);
+    LeanAcc<LT> tq, unused;
+    unused.init();
+    lean_pass_a_ck<SHIFT>(vq, lo, hi, lane, k, CK, tq, sh.cks[warp], sh.ckc[warp]);
     {
         ArgMaxSum q, unusedq;
         lean_reduce2<false>(tq, unused, vq, vq, lo, hi, k, sh, q, unusedq);
@@ -1501,23 +1496,23 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
         st = SPECHUB_ST_NONFINITE;
     } else {
         hubtok = Q.idx;
-        x1 = lean_ck_sample(g, rowq, k, Q.C, CK, -1, u1, sh);
+        x1 = lean_ck_sample(g, vq, k, Q.C, CK, -1, u1, sh);
         if (method == kSpecHub) {
             prob0 = Q.own / Zq;
             if (x1 != hubtok) {
                 x2 = hubtok;
-                prob1 = ex2(fmaf(load_one<__nv_bfloat16>(rowq, x1), k, -Q.C)) / Zq;
+                prob1 = ex2(fmaf(vq.one(x1), k, -Q.C)) / Zq;
             } else if (!(Q.sx > 0.f)) {
                 x2 = (hubtok == 0) ? 1 : 0;
                 st |= SPECHUB_ST_DEGENERATE_Q;
             } else {
-                x2 = lean_ck_sample(g, rowq, k, Q.C, CK, hubtok, u2, sh);
-                prob1 = prob0 * ex2(fmaf(load_one<__nv_bfloat16>(rowq, x2), k, -Q.C)) / Q.sx;
+                x2 = lean_ck_sample(g, vq, k, Q.C, CK, hubtok, u2, sh);
+                prob1 = prob0 * ex2(fmaf(vq.one(x2), k, -Q.C)) / Q.sx;
             }
         } else if (method == kRRS) {
-            x2 = lean_ck_sample(g, rowq, k, Q.C, CK, -1, u2, sh);
+            x2 = lean_ck_sample(g, vq, k, Q.C, CK, -1, u2, sh);
         } else {
-            x2 = lean_ck_sample(g, rowq, k, Q.C, CK, x1, u2, sh);
+            x2 = lean_ck_sample(g, vq, k, Q.C, CK, x1, u2, sh);
             if (x2 < 0) {   // nothing left once x1 is removed
                 x2 = (x1 == 0) ? 1 : 0;
                 st |= SPECHUB_ST_DEGENERATE_Q;
@@ -1526,8 +1521,8 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
     }
     if (threadIdx.x == 0) {
         if (a.draft_stats_out) {
-            DraftStat ds;
-            ds.ml = Q.ml; ds.sx = Q.sx; ds.idx = Q.idx; ds.tag = kDraftStatTag ^ __float_as_uint(k);
+            DraftStat ds = {};
+            if (keep_stats) { ds.ml = Q.ml; ds.sx = Q.sx; ds.idx = Q.idx; ds.tag = kDraftStatTag ^ __float_as_uint(k); }
             static_cast<DraftStat *>(a.draft_stats_out)[r] = ds;
         }
         a.draft_tokens_out[2 * r] = x1;

@@ -17,6 +17,8 @@
 
 #include <cstdint>
 
+#include "spechub_vec.cuh"
+
 namespace spechub {
 
 constexpr int kRingCh = 3;       // vectors per lane, row and stage (measured: 1 / 2 / 3 / 4 -> 1.60 / 1.31 / 1.23 / 1.23 ms)
@@ -110,12 +112,12 @@ __device__ __forceinline__ void ring_wait(WarpRing &R) {
 }
 
 // vector j (0 .. kRingCh - 1) of this lane in chunk R.g: target and draft
-__device__ __forceinline__ void ring_load(const WarpRing &R, int j, int lane, uint4 &x, uint4 &y) {
+__device__ __forceinline__ void ring_load(const WarpRing &R, int j, int lane, Vec8<__nv_bfloat16> &x, Vec8<__nv_bfloat16> &y) {
     const uint32_t a = R.data + (static_cast<uint32_t>(R.g) & (kRingStages - 1)) * kRingStageBytes +
                        static_cast<uint32_t>(j * 32 + lane) * 16u;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w) : "r"(a));
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(x.w[0]), "=r"(x.w[1]), "=r"(x.w[2]), "=r"(x.w[3]) : "r"(a));
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(y.x), "=r"(y.y), "=r"(y.z), "=r"(y.w) : "r"(a + kRingChunkVecs * 16));
+                 : "=r"(y.w[0]), "=r"(y.w[1]), "=r"(y.w[2]), "=r"(y.w[3]) : "r"(a + kRingChunkVecs * 16));
 }
 
 // every lane has read chunk R.g: its stage takes the next chunk of the stream

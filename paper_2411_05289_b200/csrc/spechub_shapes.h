@@ -1,17 +1,30 @@
-// CTA shapes of the large-vocabulary kernels (the per-method and the three-method kernels of a step take the
-// same ones: their results are the same bit for bit).
+// CTA shapes of the streaming kernels (the per-method and the three-method kernels of a step take the same ones:
+// their results are the same bit for bit).
 #pragma once
 
 namespace spechub {
 
+constexpr int kSms = 148;
+
+// Threads per row where the rows do not fill the GPU with CTAs of the shape that is best for many rows: one wave of
+// 512 (two per SM) or 256 threads (four per SM).
+constexpr int threads_for_few(unsigned rows, int many) {
+    if (rows <= 2 * kSms) return 512;
+    if (rows <= 4 * kSms) return 256;
+    return many;
+}
 // Draft step and leaf rows: 8 CTAs of 128 threads per SM (64 / 128 / 256 / 512 threads: 0.41 / 0.36 / 0.38 /
-// 0.52 ms on V = 128256; 0.078 / 0.081 / 0.102 / 0.165 ms on V = 32000).
-constexpr int kLeanDraftThreads = 128;
-constexpr int kLeanThreads = 256;  // 4 CTAs per SM measured best (256/512/1024: 1.54/1.65/1.87 ms)
-// Verification from draft statistics on shorter rows: 8 CTAs of 128 threads per SM overlap the fixed work of
-// a row (reductions, tests, draws) better (V = 32000, 3840 rows: SpecHub 0.180 -> 0.158 ms, RRS 0.230 ->
-// 0.205 ms; 64 threads: 0.171 ms; on V = 128256 the 256-thread CTA stays ahead, 1.02 against 1.06 ms).
-constexpr int kLeanSmallThreads = 128;
-constexpr int kLeanSmallVocab = 65536;
+// 0.52 ms on V = 128256; 0.078 / 0.081 / 0.102 / 0.165 ms on V = 32000); rows too short to feed those take 64.
+constexpr int draft_threads(int vocab, unsigned rows) {
+    return vocab < 8192 ? 64 : threads_for_few(rows, 128);
+}
+// Verification: 4 CTAs of 256 threads per SM (256/512/1024: 1.54/1.65/1.87 ms).  From draft statistics and on rows of
+// any alignment shorter rows take 8 CTAs of 128 threads, which overlap the fixed work of a row (reductions, tests,
+// draws) better (V = 32000, 3840 rows: SpecHub 0.180 -> 0.158 ms, RRS 0.230 -> 0.205 ms; 64 threads: 0.171 ms; on
+// V = 128256 the 256-thread CTA stays ahead, 1.02 against 1.06 ms).
+constexpr int verify_threads(int vocab, unsigned rows) {
+    return threads_for_few(rows, vocab <= 65536 ? 128 : 256);
+}
+constexpr int kLeanThreads = 256;   // split rows, and the rings of bulk copies
 
 }  // namespace spechub

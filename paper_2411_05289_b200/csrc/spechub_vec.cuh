@@ -234,4 +234,175 @@ __device__ __forceinline__ Vec8<float> RowVecs<float>::load_shifted(int vi) cons
     return shift_words(p[0], p[1], p[2], sh);
 }
 
+// Loads with an L2 eviction policy (createpolicy).
+__device__ __forceinline__ Vec8<__nv_bfloat16> load_hint(const Vec8<__nv_bfloat16> *p, uint64_t pol) {
+    Vec8<__nv_bfloat16> v;
+    asm volatile("ld.global.L2::cache_hint.v4.b32 {%0, %1, %2, %3}, [%4], %5;"
+                 : "=r"(v.w[0]), "=r"(v.w[1]), "=r"(v.w[2]), "=r"(v.w[3]) : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ Vec8<float> load_hint(const Vec8<float> *p, uint64_t pol) {
+    Vec8<float> v;
+    asm volatile("ld.global.L2::cache_hint.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8], %9;"
+                 : "=f"(v.f[0]), "=f"(v.f[1]), "=f"(v.f[2]), "=f"(v.f[3]), "=f"(v.f[4]), "=f"(v.f[5]), "=f"(v.f[6]), "=f"(v.f[7])
+                 : "l"(p), "l"(pol));
+    return v;
+}
+
+// A row as the streaming kernels read it.  SHIFT = false: every vector is a whole aligned word (bf16: 16 bytes,
+// fp32: 32 bytes); SHIFT = true: any row (see RowVecs).
+template <typename LT, bool SHIFT> struct StreamRow;
+template <typename LT>
+struct StreamRow<LT, false> {
+    using Raw = Vec8<LT>;
+    static constexpr int kDepth = 8 / sizeof(LT);   // vectors per lane that a pass keeps in flight: 64 bytes
+    const LT *row;
+    __device__ __forceinline__ StreamRow(const LT *r, int) : row(r) {}
+    __device__ __forceinline__ const Vec8<LT> *vec(int vi) const { return reinterpret_cast<const Vec8<LT> *>(row) + vi; }
+    __device__ __forceinline__ Vec8<LT> operator[](int vi) const;
+    __device__ __forceinline__ Raw fetch(int vi) const { return (*this)[vi]; }
+    __device__ __forceinline__ Raw fetch(int vi, uint64_t pol) const { return load_hint(vec(vi), pol); }
+    __device__ __forceinline__ Vec8<LT> fix(const Raw &r) const { return r; }
+    __device__ __forceinline__ float one(int y) const { return load_one<LT>(row, y); }
+};
+template <>
+__device__ __forceinline__ Vec8<__nv_bfloat16> StreamRow<__nv_bfloat16, false>::operator[](int vi) const {
+    const uint4 a = reinterpret_cast<const uint4 *>(row)[vi];
+    return {{a.x, a.y, a.z, a.w}};
+}
+template <>
+__device__ __forceinline__ Vec8<float> StreamRow<float, false>::operator[](int vi) const {
+    Vec8<float> v;
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v.f[0]), "=f"(v.f[1]), "=f"(v.f[2]), "=f"(v.f[3]), "=f"(v.f[4]), "=f"(v.f[5]), "=f"(v.f[6]), "=f"(v.f[7])
+                 : "l"(vec(vi)));
+    return v;
+}
+template <typename LT>
+struct StreamRow<LT, true> {
+    RowVecs<LT> src;
+    __device__ __forceinline__ StreamRow(const LT *r, int vocab) : src(r, vocab) {}
+    __device__ __forceinline__ Vec8<LT> operator[](int vi) const {
+        if (!src.whole(vi)) return src.load_slow(vi);
+        return src.sh == 0 ? src.load_aligned(vi) : src.load_shifted(vi);
+    }
+    __device__ __forceinline__ float one(int y) const { return load_one<LT>(src.row, y); }
+};
+
+// The inside of such a row (whole vectors) for the loops that keep loads in flight: they take the words of a vector
+// (fetch) and make the vector of them when it is used (fix).  Shifting is arithmetic on what was loaded: done at
+// once, it would wait for the load.
+template <typename LT> struct ShiftRaw;
+template <> struct ShiftRaw<__nv_bfloat16> { uint4 a, b; };
+template <> struct ShiftRaw<float> { float4 a, b, c; };
+template <typename LT>
+struct AlignedInside {
+    using Raw = Vec8<LT>;
+    static constexpr int kDepth = 8 / sizeof(LT);
+    const RowVecs<LT> &src;
+    __device__ __forceinline__ Raw fetch(int vi) const { return src.load_aligned(vi); }
+    __device__ __forceinline__ Vec8<LT> fix(const Raw &r) const { return r; }
+};
+template <typename LT>
+struct ShiftedInside {
+    using Raw = ShiftRaw<LT>;
+    static constexpr int kDepth = 4 / sizeof(LT);   // (two or three words for one vector)
+    const RowVecs<LT> &src;
+    __device__ __forceinline__ Raw fetch(int vi) const;
+    __device__ __forceinline__ Vec8<LT> fix(const Raw &r) const;
+};
+template <>
+__device__ __forceinline__ ShiftRaw<__nv_bfloat16> ShiftedInside<__nv_bfloat16>::fetch(int vi) const {
+    const uint4 *p = reinterpret_cast<const uint4 *>(src.row - src.sh) + vi;
+    return {p[0], p[1]};
+}
+template <>
+__device__ __forceinline__ Vec8<__nv_bfloat16> ShiftedInside<__nv_bfloat16>::fix(const Raw &r) const {
+    return shift_words(r.a, r.b, src.sh);
+}
+template <>
+__device__ __forceinline__ ShiftRaw<float> ShiftedInside<float>::fetch(int vi) const {
+    const float4 *p = reinterpret_cast<const float4 *>(src.row - src.sh) + 2 * vi;
+    return {p[0], p[1], p[2]};
+}
+template <>
+__device__ __forceinline__ Vec8<float> ShiftedInside<float>::fix(const Raw &r) const {
+    return shift_words(r.a, r.b, r.c, src.sh);
+}
+
+// A warp's range [lo, hi) of such rows: lane-iteration `it` takes the vectors lo + 32 it + lane; the iterations
+// [i0, i1) lie inside the row (or both rows) and need no check per vector.
+struct InsideIters { int i0, i1, n; };
+template <typename LT>
+__device__ __forceinline__ InsideIters inside_iters(const RowVecs<LT> &a, const RowVecs<LT> &b, int lo, int hi) {
+    InsideIters r;
+    r.n = (hi - lo + 31) >> 5;
+    r.i0 = min(r.n, lo < max(a.f0, b.f0) ? 4 : 0);   // (a multiple of every loop's depth)
+    r.i1 = max(r.i0, min(r.n, (min(hi, min(a.f1, b.f1)) - lo) >> 5));
+    return r;
+}
+
+// Loops over the inside of one row, kDepth vectors per lane in flight: the next ones are requested before the
+// current ones are used.  f(vector); after(D) is called after every D iterations.  Returns the iteration reached.
+template <class IN, class F, class AFTER>
+__device__ __forceinline__ int inside_ahead(const IN &row, int v0, int it, int i1, F f, AFTER after) {
+    constexpr int D = IN::kDepth;
+    typename IN::Raw nx[D] = {};
+    if (it + D <= i1) {
+#pragma unroll
+        for (int i = 0; i < D; ++i) nx[i] = row.fetch(v0 + 32 * (it + i));
+    }
+#pragma unroll 1
+    for (; it + D <= i1; it += D) {
+        typename IN::Raw a[D];
+#pragma unroll
+        for (int i = 0; i < D; ++i) a[i] = nx[i];
+        if (it + 2 * D <= i1) {
+#pragma unroll
+            for (int i = 0; i < D; ++i) nx[i] = row.fetch(v0 + 32 * (it + D + i));
+        }
+#pragma unroll
+        for (int i = 0; i < D; ++i) f(row.fix(a[i]));
+        after(D);
+    }
+    return it;
+}
+// ... and over the insides of two rows, the next pair of vectors in flight; STEP = 1 or -1; f(vi, vector, vector)
+template <int STEP, class IN, class F>
+__device__ __forceinline__ void inside_pairs(const IN &p, const IN &q, int v0, int from, int n, F f) {
+    typename IN::Raw np = {}, nq = {};
+    int vi = v0 + 32 * from;
+    if (n > 0) { np = p.fetch(vi); nq = q.fetch(vi); }
+#pragma unroll 1
+    for (; n > 0; --n, vi += 32 * STEP) {
+        const typename IN::Raw cp = np, cq = nq;
+        if (n > 1) { np = p.fetch(vi + 32 * STEP); nq = q.fetch(vi + 32 * STEP); }
+        f(vi, p.fix(cp), q.fix(cq));
+    }
+}
+// All vectors of a warp's range of two rows of any alignment, in ascending (STEP = 1) or descending order.
+template <int STEP, typename LT, class F>
+__device__ __forceinline__ void any_pairs(const StreamRow<LT, true> &p, const StreamRow<LT, true> &q, int lo, int hi, int lane, F f) {
+    const InsideIters t = inside_iters(p.src, q.src, lo, hi);
+    const int v0 = lo + lane;
+    auto slow_run = [&](int from, int n) {
+#pragma unroll 1
+        for (; n > 0; --n, from += STEP) {
+            const int vi = v0 + 32 * from;
+            if (vi < hi) f(vi, p[vi], q[vi]);
+        }
+    };
+    const int from = STEP > 0 ? t.i0 : t.i1 - 1, n = t.i1 - t.i0;
+    if (STEP > 0) slow_run(0, t.i0);
+    else slow_run(t.n - 1, t.n - t.i1);
+    if (p.src.sh == 0 && q.src.sh == 0)
+        inside_pairs<STEP>(AlignedInside<LT>{p.src}, AlignedInside<LT>{q.src}, v0, from, n, f);
+    else if (p.src.sh != 0 && q.src.sh != 0)
+        inside_pairs<STEP>(ShiftedInside<LT>{p.src}, ShiftedInside<LT>{q.src}, v0, from, n, f);
+    else   // (a shifted row beside one that is not: rows of two unlike buffers)
+        slow_run(from, n);
+    if (STEP > 0) slow_run(t.i1, t.n - t.i1);
+    else slow_run(t.i0 - 1, t.i0);
+}
+
 }  // namespace spechub

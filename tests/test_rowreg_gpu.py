@@ -1,4 +1,5 @@
-"""Rows held in registers (calls whose rows do not fill the GPU, short vocabularies): the edges of a lane's vectors,
+"""Rows held in registers (calls whose rows do not fill the GPU, short vocabularies) and streamed rows of any
+alignment: the edges of a lane's vectors,
 of a warp's and a cluster's part, aligned and packed odd rows, both types, against the oracle."""
 import numpy as np
 import pytest
@@ -7,8 +8,10 @@ pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
 
+import parity  # noqa: E402
 import workloads  # noqa: E402
-from test_parity_gpu import random_logits, random_uniforms, run_case, sh  # noqa: E402,F401
+from test_parity_gpu import (METHODS, gpu_draft, gpu_verify, padded, random_logits, random_uniforms,  # noqa: E402,F401
+                             run_case, sh)
 
 
 # one warp of 1 / 2 / 4 / 8 vectors per lane, two warps, a CTA, clusters of 2 / 4 / 8 CTAs, each with its neighbours
@@ -36,3 +39,24 @@ def test_rows_per_cta_and_vectors_per_lane(sh, rows):  # noqa: F811
     V = 384
     lp, lq = random_logits(rng, rows, 1, V, "fp32", sd=3.0)
     run_case(sh, lp, lq, "fp32", 1.0, random_uniforms(rng, rows, 1), False, label="rowreg rows=%d" % rows)
+
+
+# streaming kernels on rows of any alignment: warps' ranges that begin and end inside, at and beyond the whole words
+@pytest.mark.parametrize("pad", [0, 8, 64])
+@pytest.mark.parametrize("V,dtype,B", [(1025, "fp32", 1200), (4105, "bf16", 600), (8199, "fp32", 300), (9001, "bf16", 300)])
+def test_streamed_rows_of_any_alignment(sh, V, dtype, B, pad):  # noqa: F811
+    rng = np.random.default_rng(V + pad)
+    lp, lq = random_logits(rng, B, 3, V, dtype)
+    lq[0, 1] = lp[0, 1]
+    lq[1, 2] = -np.inf; lq[1, 2, V - 1] = 0.0
+    lp, lq = workloads.round_to_storage(lp, dtype), workloads.round_to_storage(lq, dtype)
+    un = random_uniforms(rng, B, 3)
+    pick = np.unique(np.concatenate([[0, 1, B - 1], rng.integers(0, B, 6)]))
+    tp, tq = padded(lp, dtype, pad), padded(lq, dtype, pad)
+    und, tree = torch.from_numpy(un).cuda(), sh.Tree.heap(3)
+    for m in METHODS:
+        d = parity.to_numpy(gpu_draft(sh, m, tq, und, tree, 1.0))
+        parity.check_draft(m, lq[pick], 1.0, un[pick], {k: v[pick] for k, v in d.items()}, label="any")
+        out = parity.to_numpy(gpu_verify(sh, m, tp, tq, torch.from_numpy(d["tokens"]).cuda(), und, tree, 1.0))
+        parity.check_verify(m, lp[pick], lq[pick], 1.0, d["tokens"][pick], un[pick], None,
+                            {k: v[pick] for k, v in out.items()}, label="any")
