@@ -46,10 +46,11 @@ static int leaf_rows(const LeafArgs &la, unsigned rows, cudaStream_t s) {
 }
 
 // The leaf rows of an unsplit call (same CTA shape as the draft step).
-int launch_lean_leaf(int format, const RowArgs &a, const NodeOutPtrs *outs, int n_out, unsigned rows, cudaStream_t s) {
+int launch_lean_leaf(int format, const RowArgs &a, int k, const NodeOutPtrs *outs, int n_out, unsigned rows, cudaStream_t s) {
     LeafArgs la = {};
     la.r = a;
     la.n_out = n_out;
+    la.k = k;
     for (int m = 0; m < n_out; ++m) la.out[m] = outs[m];
     if (format == kBf16) return leaf_rows<__nv_bfloat16, false>(la, rows, s);
     if (format == kBf16Shift) return leaf_rows<__nv_bfloat16, true>(la, rows, s);

@@ -47,7 +47,7 @@ int launch_lean_verify_method(int format, int cs, const RowArgs &a, unsigned row
     if (cs == 2) return verify_split<METHOD, 2>(a, rows, s);
     if (a.node_kind) {
         const NodeOutPtrs o = {a.accept_idx, a.token, a.hub, a.beta, a.rate, a.status};
-        const int lrc = launch_lean_leaf(format, a, &o, 1, rows, s);
+        const int lrc = launch_lean_leaf(format, a, 2, &o, 1, rows, s);
         if (lrc != SPECHUB_OK) return lrc;
     }
     const bool stats = cs == 0 && a.draft_stats_in;

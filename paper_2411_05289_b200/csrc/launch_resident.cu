@@ -84,7 +84,7 @@ int launch_resident(int mask, ResShape sh, const FusedArgs &f, unsigned rows, cu
         int n_out = 0;
         for (int m = 0; m < 3; ++m)
             if (mask & (1 << m)) outs[n_out++] = f.out[m];
-        const int lrc = launch_lean_leaf(kBf16, f.r, outs, n_out, rows, s);
+        const int lrc = launch_lean_leaf(kBf16, f.r, 2, outs, n_out, rows, s);
         if (lrc != SPECHUB_OK) return lrc;
     }
     if (mask == kMaskSpecHub) return launch_resident_mask<kMaskSpecHub>(sh, f, rows, s);

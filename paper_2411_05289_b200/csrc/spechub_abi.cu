@@ -137,7 +137,7 @@ int draft_common(const spechub_desc *d, const void *draft_logits, const float *u
     ka.r = a; ka.k = d->k; ka.without_replacement = (method == kRRSw); ka.keep_stats = keeps_stats(d, fmt);
     RegPlan pl;
     if (use_reg(d, al, rows, &pl)) return launch_reg_draft(pl, d->dtype, ka, method, rows, s);
-    if (d->k > 2) return launch_kary_draft(d->dtype, al, threads_for(d), ka, rows, s);
+    if (d->k > 2) return launch_kary_draft(fmt, ka, rows, s);
     return launch_lean_draft(fmt, method, lean_ok(d, al) ? lean_split(d) : 0, a, ka.keep_stats, rows, s);
 }
 
@@ -200,10 +200,8 @@ int verify_common(const spechub_desc *d, const void *target_logits, const void *
     if (use_reg(d, al, rows, &pl)) {
         lrc = launch_reg_verify(pl, d->dtype, ka, method, rows, s);
     } else if (d->k > 2) {
-        if (!(d->flags & 7u) && resident_fits(d, al, &rs))   // (a split flag asks for the streaming kernel)
-            lrc = launch_resident_kary(rs, ka, rows, s);
-        else
-            lrc = launch_kary_verify(d->dtype, al, threads_for(d), ka, rows, s);
+        if (resident_shape(d, al, &rs)) lrc = launch_resident_kary(rs, ka, rows, s);
+        else lrc = launch_kary_verify(fmt, ka, rows, s);
     } else if (resident_shape(d, al, &rs)) {
         FusedArgs f = {};
         f.r = a;
@@ -299,7 +297,7 @@ int compare_verify(const spechub_desc *d, const void *target_logits, const void 
         lrc = launch_resident(7, rs, f, rows, s);
     } else {
         if (d->node_kind) {
-            const int llrc = launch_lean_leaf(kBf16, f.r, f.out, 3, rows, s);
+            const int llrc = launch_lean_leaf(kBf16, f.r, 2, f.out, 3, rows, s);
             if (llrc != SPECHUB_OK) return llrc;
         }
         if (lean_split(d) == 0) f.r.draft_stats_in = draft_stats;

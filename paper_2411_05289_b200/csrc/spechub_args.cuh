@@ -52,7 +52,7 @@ struct NodeOutPtrs {
 struct LeafArgs {
     RowArgs r;
     NodeOutPtrs out[3];
-    int n_out;
+    int n_out, k;
 };
 
 struct FusedArgs {

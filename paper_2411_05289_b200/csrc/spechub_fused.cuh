@@ -61,31 +61,27 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
     };
 
     if (leaf) return;   // leaf rows belong to lean_leaf_kernel
+    if (STATS && threadIdx.x == THREADS - 1) {   // the draft row's record, checked off the path between the passes
+        const DraftStat ds = static_cast<const DraftStat *>(a.draft_stats_in)[r];
+        bool ok = ds.tag == (kDraftStatTag ^ __float_as_uint(k));
+        if (ok && ds.ml > neg_inf() && ds.ml < pinf && finite_pos(ds.sx + 1.f))
+            ok = ds.idx >= 0 && ds.idx < a.vocab && load_one<__nv_bfloat16>(rowq, ds.idx) == ds.ml;
+        sh.stat_ok = ok;
+        sh.x_ml[1] = ds.ml; sh.x_sx[1] = ds.sx; sh.x_idx[1] = ok ? ds.idx : 0;
+    }
     LeanAcc<__nv_bfloat16> tp, tq;
     if (STATS) lean_pass_a_deep(vp, lo, hi, lane, k, tp);
     else lean_pass_a<true, false>(vp, vq, lo, hi, lane, k, tp, tq);
+    RowStat P, Q;
     {
         ArgMaxSum Ps, Qs;
         if (STATS) lean_reduce2<false>(tp, tq, vp, vq, lo, hi, k, sh, Ps, Qs);
         else lean_reduce2<true>(tp, tq, vp, vq, lo, hi, k, sh, Ps, Qs);
-        if (t0) {
-            sh.x_ml[0] = Ps.ml; sh.x_sx[0] = Ps.sx; sh.x_idx[0] = Ps.idx;
-            if (STATS) {
-                const DraftStat ds = static_cast<const DraftStat *>(a.draft_stats_in)[r];
-                bool ok = ds.tag == (kDraftStatTag ^ __float_as_uint(k));
-                if (ok && ds.ml > neg_inf() && ds.ml < pinf && finite_pos(ds.sx + 1.f))
-                    ok = ds.idx >= 0 && ds.idx < a.vocab && load_one<__nv_bfloat16>(rowq, ds.idx) == ds.ml;
-                sh.stat_ok = ok;
-                sh.x_ml[1] = ds.ml; sh.x_sx[1] = ds.sx; sh.x_idx[1] = ok ? ds.idx : 0;
-            } else {
-                sh.x_ml[1] = Qs.ml; sh.x_sx[1] = Qs.sx; sh.x_idx[1] = Qs.idx;
-            }
-        }
+        if (t0) { sh.x_ml[0] = Ps.ml; sh.x_sx[0] = Ps.sx; sh.x_idx[0] = Ps.idx; }   // (read by a draw from p, after further barriers)
+        if (STATS) { Qs.ml = sh.x_ml[1]; Qs.c = shift_of(Qs.ml, k); Qs.sx = sh.x_sx[1]; Qs.idx = sh.x_idx[1]; }
+        P.set(Ps, k);
+        Q.set(Qs, k);
     }
-    __syncthreads();
-    RowStat P, Q;
-    merge_slices<1>(sh, 0, k, P);
-    merge_slices<1>(sh, 1, k, Q);
     float Zp = P.sx + P.own;
     const float Zq = Q.sx + Q.own;
     float cP = P.C, invZp = 1.f / Zp;
@@ -188,12 +184,16 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
     f2_get(a1, a1a, a1b);
     };
     pass_b();
-    if (STATS && !__syncthreads_or(diff != 0)) {   // the target row is the draft row: Z_p = Z_q exactly
+    float accB[5] = {s1a + s1b, s2a + s2b, ra + rb, a1a + a1b, dna + dnb};
+    lean_block_sums<5, 0, STATS>(accB, sh, &diff);   // per-warp R stays in sh.acc[2]
+    const float *mass_r = sh.acc[2];
+    if (STATS && !diff) {   // the target row is the draft row: Z_p = Z_q exactly
         Zp = Zq; invZp = invZq; cP = cQ; rho = 1.f; crho = c;
         pass_b();
+        accB[0] = s1a + s1b; accB[1] = s2a + s2b; accB[2] = ra + rb; accB[3] = a1a + a1b; accB[4] = dna + dnb;
+        lean_block_sums<5, 8>(accB, sh);
+        mass_r = sh.acc[10];
     }
-    float accB[5] = {s1a + s1b, s2a + s2b, ra + rb, a1a + a1b, dna + dnb};
-    lean_block_sums<5, 0>(accB, sh);   // per-warp R stays in sh.acc[2]
     if (STATS) accB[4] = wx1 >= 0 ? sum_without(Q, vq, wx1, k) : 0.f;
     const float Rraw = accB[2];
     const float S1 = accB[0] * invZp, S2 = degenerate ? qa : accB[1] * invZp, R = Rraw * invZp;
@@ -228,7 +228,6 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
     }
     float accC[2] = {w0a + w0b, w1a + w1b};
     lean_block_sums<2, 5>(accC, sh);   // per-warp W2 stay in sh.acc[5], sh.acc[6]
-    __syncthreads();
 
     // ---- SpecHub decisions (Algorithm 3) ----
     if (ok_s) {
@@ -256,8 +255,6 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
             s.accept_idx = -1;
             int tok;
             if (Rraw > 0.f) {
-                if (threadIdx.x < g.nwarps) sh.mass[threadIdx.x] = sh.acc[2][threadIdx.x];
-                __syncthreads();
                 auto wf = [&](int vi, float(&w)[8]) {
                     const V fp = vp[vi], fq = vq[vi];
 #pragma unroll
@@ -267,7 +264,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
                         w[i] = (vi * 8 + i == hubtok) ? 0.f : fmaxf(t, 0.f);
                     }
                 };
-                tok = block_sample3(g, wf, sh, ures * Rraw);
+                tok = block_sample3(g, wf, mass_r, sh, ures * Rraw);
             } else {
                 s.status |= SPECHUB_ST_ZERO_RESIDUAL;
                 tok = draw_from_p();
@@ -300,8 +297,6 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
             s.accept_idx = -1;
             int tok;
             if (A1 > 0.f && W2raw > 0.f) {
-                if (threadIdx.x < g.nwarps) sh.mass[threadIdx.x] = sh.acc[5 + m][threadIdx.x];
-                __syncthreads();
                 const float coef = A1grho[m];
                 auto wf = [&](int vi, float(&w)[8]) {
                     const V fp = vp[vi], fq = vq[vi];
@@ -313,7 +308,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
                         w[i] = fmaxf(t, 0.f);
                     }
                 };
-                tok = block_sample3(g, wf, sh, ures * W2raw);
+                tok = block_sample3(g, wf, sh.acc[5 + m], sh, ures * W2raw);
             } else {
                 s.status |= SPECHUB_ST_ZERO_RESIDUAL;
                 tok = draw_from_p();
@@ -345,15 +340,13 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
 
     LeanAcc<__nv_bfloat16> tq, unused;
     unused.init();
-    lean_pass_a_ck<false>(vq, lo, hi, lane, k, CK, tq, sh.cks[warp], sh.ckc[warp]);
+    lean_pass_a_ck<false>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * kLeanCk, sh.ckc + warp * kLeanCk);
+    RowStat Q;
     {
         ArgMaxSum q, unusedq;
         lean_reduce2<false>(tq, unused, vq, vq, lo, hi, k, sh, q, unusedq);
-        if (t0) { sh.x_ml[0] = q.ml; sh.x_sx[0] = q.sx; sh.x_idx[0] = q.idx; }
+        Q.set(q, k);
     }
-    __syncthreads();
-    RowStat Q;
-    merge_slices<1>(sh, 0, k, Q);
     const float Zq = Q.sx + Q.own;
     if (t0 && a.draft_stats_out) {   // the record lean_draft_ck_kernel leaves, bit for bit
         DraftStat ds;
@@ -375,6 +368,10 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
     const int x1 = lean_ck_sample(g, vq, k, Q.C, CK, -1, u1, sh);
     uint32_t st[3] = {0, 0, 0};
     int x2[3];
+    // RRS: an independent second draw (before a token is left out of the checkpoints' sums)
+    x2[1] = lean_ck_sample(g, vq, k, Q.C, CK, -1, u2, sh);
+    // RRSw: q with q(x1) set to 0
+    x2[2] = lean_ck_sample(g, vq, k, Q.C, CK, x1, u2, sh);
     // SpecHub (Section 4)
     const float prob0 = Q.own / Zq;
     float prob1 = 0.f;
@@ -385,13 +382,9 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
         x2[0] = (hubtok == 0) ? 1 : 0;
         st[0] |= SPECHUB_ST_DEGENERATE_Q;
     } else {
-        x2[0] = lean_ck_sample(g, vq, k, Q.C, CK, hubtok, u2, sh);
+        x2[0] = x2[2];   // (q without the hub, which is x1: the draw RRSw made)
         prob1 = prob0 * ex2(fmaf(load_one<__nv_bfloat16>(rowq, x2[0]), k, -Q.C)) / Q.sx;
     }
-    // RRS: an independent second draw
-    x2[1] = lean_ck_sample(g, vq, k, Q.C, CK, -1, u2, sh);
-    // RRSw: q with q(x1) set to 0
-    x2[2] = lean_ck_sample(g, vq, k, Q.C, CK, x1, u2, sh);
     if (x2[2] < 0) {
         x2[2] = (x1 == 0) ? 1 : 0;
         st[2] |= SPECHUB_ST_DEGENERATE_Q;

@@ -16,9 +16,6 @@ inline int launch_status() { return cudaGetLastError() == cudaSuccess ? SPECHUB_
 // the caller (one array per kernel).
 int allow_smem(const void *kern, int bytes, bool *configured);
 
-// more than two drafts per node, any shape; th = threads per row
-int launch_kary_draft(int dtype, bool aligned, int th, const KaryArgs &a, unsigned rows, cudaStream_t s);
-int launch_kary_verify(int dtype, bool aligned, int th, const KaryArgs &a, unsigned rows, cudaStream_t s);
 int launch_walk(const WalkKArgs &w, cudaStream_t s);
 
 // Rows held in registers.  reg_plan: false if the row does not fit, or if the streaming kernels are the faster
@@ -32,11 +29,14 @@ int launch_reg_verify(const RegPlan &pl, int dtype, const KaryArgs &a, int metho
 // 32-byte boundaries, vocab % 8 == 0), or shifted into place (any row).
 enum StreamFormat { kBf16, kBf16Shift, kF32, kF32Shift };
 int launch_lean_draft(int format, int method, int cs, const RowArgs &a, bool keep_stats, unsigned rows, cudaStream_t s);
-int launch_lean_leaf(int format, const RowArgs &a, const NodeOutPtrs *outs, int n_out, unsigned rows, cudaStream_t s);
+int launch_lean_leaf(int format, const RowArgs &a, int k, const NodeOutPtrs *outs, int n_out, unsigned rows, cudaStream_t s);
 // cs = CTAs per row asked for (0: the library's choice; other than 0 and 1: kBf16 only)
 int launch_lean_verify_spechub(int format, int cs, const RowArgs &a, unsigned rows, cudaStream_t s);
 int launch_lean_verify_rrs(int format, int cs, const RowArgs &a, unsigned rows, cudaStream_t s);
 int launch_lean_verify_rrsw(int format, int cs, const RowArgs &a, unsigned rows, cudaStream_t s);
+// more than two drafts per node
+int launch_kary_draft(int format, const KaryArgs &a, unsigned rows, cudaStream_t s);
+int launch_kary_verify(int format, const KaryArgs &a, unsigned rows, cudaStream_t s);
 int launch_fused_draft(const FusedArgs &f, int32_t *hub, float *draft_prob, unsigned rows, cudaStream_t s);
 int launch_fused_verify(const FusedArgs &f, unsigned rows, cudaStream_t s);
 

@@ -42,29 +42,56 @@ constexpr int kLeanCk = 8;        // checkpoints per warp in the draft step's pa
 constexpr float kHuge = 1.0e30f;  // ~2^100: partial sums beyond this move the reference
 
 struct LeanShared {
-    float wml[2][kLeanMaxWarps];    // per-warp max logit (0 target, 1 draft)
-    float wmass[2][kLeanMaxWarps];  // per-warp sum of exponentials on the row's scale, argmax left out
-    int cand[2];                    // lowest index attaining the row maximum
-    float acc[8][kLeanMaxWarps];
+    float wml[2][kLeanMaxWarps];     // per-warp max logit (0 target, 1 draft)
+    float wmass[2][kLeanMaxWarps];   // per-warp sum of exponentials on the row's scale
+    float wmassx[2][kLeanMaxWarps];  // the same without the lowest id in that warp that attains the row maximum
+    int widx[2][kLeanMaxWarps];      // that id
+    float acc[16][kLeanMaxWarps];
+    int any[kLeanMaxWarps];
     float mass[kLeanMaxWarps];
-    float part[1024];  // sampler: per-thread block sums of the selected warp range
-    float tt2;
-    int blk;
+    float part[kLeanMaxWarps];  // sampler: per-warp sums of the range drawn from
     int tok;
     // what this CTA tells the other CTAs of its row (read through distributed shared memory)
     float x_ml[2], x_sx[2];  // slice (max logit, sum without the slice argmax), 0 target / 1 draft
     int x_idx[2];            // slice argmax
-    float x_sum[4];          // pass-B / pass-C sums of the slice
+    float x_sum[8];          // pass-B / pass-C sums of the slice
     float x_mass;            // slice mass for a draw from q without a given token
     int x_tok;               // a token drawn by this CTA
-    int stat_ok;             // verification from draft statistics: the row's record was accepted
+    // verification: what the tests need of single ids, fetched by one warp before its pass A
+    int tk[2];               // the drafts
+    float lg[8];             // target logits of the drafts, draft logits of the drafts, -, r1, r2, u_res
+    int stat_ok;             // from draft statistics: the row's record was accepted
 };
-// draft step and leaf rows: also the checkpoint sums of pass A (per warp, every CK lane-iterations), their
-// exponent references, and the masses of those sub-blocks on the row's scale
+// draft step and leaf rows: also the checkpoint sums of pass A (per warp, every CK lane-iterations) and their
+// exponent references
 struct LeanCkShared : LeanShared {
-    float cks[kLeanMaxWarps][kLeanCk], ckc[kLeanMaxWarps][kLeanCk];
-    float ckm[kLeanMaxWarps * kLeanCk];
+    float cks[kLeanMaxWarps * kLeanCk], ckc[kLeanMaxWarps * kLeanCk];
 };
+
+__device__ __forceinline__ float lanes_max(float x) {
+    float m;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(x));
+    return m;
+}
+__device__ __forceinline__ float lanes_prefix(float x) {   // inclusive, over ascending lanes
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const float up = __shfl_up_sync(kFull, x, o);
+        if (lane >= o) x += up;
+    }
+    return x;
+}
+// Inverse-CDF pick over one mass per lane: the lowest lane with mass whose inclusive prefix exceeds t, the last lane
+// with mass if none does; -1: no mass.  t becomes the target within the lane.  The same in every lane.
+__device__ __forceinline__ int lanes_pick(float m, float &t) {
+    const float incl = lanes_prefix(m);
+    const unsigned pos = __ballot_sync(kFull, m > 0.f), hit = __ballot_sync(kFull, m > 0.f && incl > t);
+    if (!pos) return -1;
+    const int L = hit ? __ffs(hit) - 1 : 31 - __clz(pos);
+    t = __shfl_sync(kFull, t - (incl - m), L);
+    return L;
+}
 
 // The CTAs of one row.  CS = 1 compiles to no cluster instruction at all.
 template <int CS>
@@ -84,10 +111,11 @@ struct RowGroup {
     }
 };
 
-// CTAs of THREADS threads per SM.  bf16 rows in whole words: 64 registers per thread (1024 threads per SM) measured
-// best; wider vectors, and the two words of a shifted one, take 80 (768 threads per SM).
-template <typename LT, bool SHIFT>
-constexpr int lean_ctas(int threads) { return (sizeof(LT) == 2 && !SHIFT ? 1024 : 768) / threads; }
+// CTAs of THREADS threads per SM.  64 registers per thread (1024 threads per SM) measured best on rows in whole words
+// and for the draft step; verification of shifted rows holds two or three words per vector and row: 80 registers
+// (V = 50257, 896 rows, fp32: 87 -> 78 us, RRSw in bf16 69 -> 63 us; the draft step there 23.5 us with 80, 22 us with 64).
+template <bool SHIFT>
+constexpr int lean_ctas(int threads) { return (SHIFT ? 768 : 1024) / threads; }
 
 template <typename LT>
 struct LeanAcc {  // one thread's pass-A state for one row
@@ -276,215 +304,135 @@ __device__ __forceinline__ void lean_rescan_warp(const ROW &row, int lo, int hi,
 }
 
 // Row-level (max, argmax, sum without the argmax) of the target (r = 0) and, if BOTH, the draft
-// (r = 1) from the per-thread pass-A states.  Leaves the per-warp masses (row scale, argmax left
-// out) in sh.wmass[r] for the samplers.  All threads call it.
+// (r = 1) from the per-thread pass-A states.  Leaves the per-warp masses in sh.wmass[r] / wmassx[r] for the
+// samplers.  All threads call it; two barriers, and every warp merges the warps' values by itself.
+template <int R, typename LT, class ROW>
+__device__ __forceinline__ void lean_publish(const LeanAcc<LT> &t, const ROW &row, int lo, int hi, float k, float rm,
+                                             LeanShared &sh) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const float ml = t.max();
+    int best = 0x7fffffff, best_lane = -1;
+    float best_sx = 0.f;
+    unsigned cm = __ballot_sync(kFull, ml == rm && rm > neg_inf() && rm < -neg_inf());
+    while (cm) {   // (one lane of the CTA, or a few on ties)
+        const int src = __ffs(cm) - 1;
+        cm &= cm - 1;
+        int fi; float sx;
+        lean_rescan_warp(row, lo, hi, lane, src, rm, k, __shfl_sync(kFull, t.c, src), fi, sx);
+        if (fi < best) { best = fi; best_lane = src; best_sx = sx; }
+    }
+    const float f = ml > neg_inf() ? ex2(t.c - shift_of(rm, k)) : 0.f;
+    const float all = warp_sum(__fmul_rn(t.s, f));
+    const float without = best_lane < 0 ? all : warp_sum(__fmul_rn(lane == best_lane ? best_sx : t.s, f));
+    if (lane == 0) { sh.wmass[R][warp] = all; sh.wmassx[R][warp] = without; sh.widx[R][warp] = best; }
+}
+template <int R>
+__device__ __forceinline__ void lean_merge_warps(const LeanShared &sh, float rm, float k, ArgMaxSum &o) {
+    const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+    const int mine = lane < nwarps ? sh.widx[R][lane] : 0x7fffffff;
+    o.ml = rm;
+    o.c = shift_of(rm, k);
+    o.idx = __reduce_min_sync(kFull, mine);
+    const float m = lane < nwarps ? (mine == o.idx ? sh.wmassx[R][lane] : sh.wmass[R][lane]) : 0.f;
+    o.sx = warp_sum(m);
+}
 template <bool BOTH, typename LT, class ROW>
 __device__ void lean_reduce2(const LeanAcc<LT> &tp, const LeanAcc<LT> &tq, const ROW &vp, const ROW &vq, int lo,
                              int hi, float k, LeanShared &sh, ArgMaxSum &P, ArgMaxSum &Q) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    const float mlp = tp.max(), mlq = BOTH ? tq.max() : neg_inf();
-    float wp = mlp, wq = mlq;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        wp = fmaxf(wp, __shfl_xor_sync(kFull, wp, o));
-        if (BOTH) wq = fmaxf(wq, __shfl_xor_sync(kFull, wq, o));
-    }
-    if (lane == 0) { sh.wml[0][warp] = wp; sh.wml[1][warp] = wq; }
-    if (threadIdx.x == 0) { sh.cand[0] = 0x7fffffff; sh.cand[1] = 0x7fffffff; }
+    const float wp = lanes_max(tp.max()), wq = BOTH ? lanes_max(tq.max()) : neg_inf();
+    if (lane == 0) { sh.wml[0][warp] = wp; if (BOTH) sh.wml[1][warp] = wq; }
     __syncthreads();
-    float rmp = sh.wml[0][0], rmq = sh.wml[1][0];
-    for (int w = 1; w < nwarps; ++w) { rmp = fmaxf(rmp, sh.wml[0][w]); rmq = fmaxf(rmq, sh.wml[1][w]); }
-    const float pinf = -neg_inf();
-    int idxp_mine = 0x7fffffff, idxq_mine = 0x7fffffff;
-    float sxp = 0.f, sxq = 0.f;
-    {
-        const bool cand = (mlp == rmp) && rmp > neg_inf() && rmp < pinf;
-        unsigned cm = __ballot_sync(kFull, cand);
-        while (cm) {
-            const int src = __ffs(cm) - 1;
-            cm &= cm - 1;
-            int fi; float sx;
-            lean_rescan_warp(vp, lo, hi, lane, src, rmp, k, __shfl_sync(kFull, tp.c, src), fi, sx);
-            if (lane == src) { idxp_mine = fi; sxp = sx; atomicMin(&sh.cand[0], fi); }
-        }
-    }
-    if (BOTH) {
-        const bool cand = (mlq == rmq) && rmq > neg_inf() && rmq < pinf;
-        unsigned cm = __ballot_sync(kFull, cand);
-        while (cm) {
-            const int src = __ffs(cm) - 1;
-            cm &= cm - 1;
-            int fi; float sx;
-            lean_rescan_warp(vq, lo, hi, lane, src, rmq, k, __shfl_sync(kFull, tq.c, src), fi, sx);
-            if (lane == src) { idxq_mine = fi; sxq = sx; atomicMin(&sh.cand[1], fi); }
-        }
-    }
+    const float rmp = lanes_max(lane < nwarps ? sh.wml[0][lane] : neg_inf());
+    const float rmq = BOTH ? lanes_max(lane < nwarps ? sh.wml[1][lane] : neg_inf()) : neg_inf();
+    lean_publish<0>(tp, vp, lo, hi, k, rmp, sh);
+    if (BOTH) lean_publish<1>(tq, vq, lo, hi, k, rmq, sh);
     __syncthreads();
-    const int idxp = sh.cand[0], idxq = sh.cand[1];
-    const float Cp = shift_of(rmp, k), Cq = shift_of(rmq, k);
-    {
-        const float mine = (idxp_mine != 0x7fffffff && idxp_mine == idxp) ? sxp : tp.s;
-        float v = (mlp > neg_inf()) ? mine * ex2(tp.c - Cp) : 0.f;
-        v = warp_sum(v);
-        if (lane == 0) sh.wmass[0][warp] = v;
-    }
-    if (BOTH) {
-        const float mine = (idxq_mine != 0x7fffffff && idxq_mine == idxq) ? sxq : tq.s;
-        float v = (mlq > neg_inf()) ? mine * ex2(tq.c - Cq) : 0.f;
-        v = warp_sum(v);
-        if (lane == 0) sh.wmass[1][warp] = v;
-    }
-    __syncthreads();
-    float t0 = 0.f, t1 = 0.f;
-    for (int w = 0; w < nwarps; ++w) { t0 += sh.wmass[0][w]; if (BOTH) t1 += sh.wmass[1][w]; }
-    P.ml = rmp; P.c = Cp; P.idx = idxp; P.sx = t0;
-    Q.ml = rmq; Q.c = Cq; Q.idx = idxq; Q.sx = t1;
+    lean_merge_warps<0>(sh, rmp, k, P);
+    if (BOTH) lean_merge_warps<1>(sh, rmq, k, Q);
+    else { Q.ml = neg_inf(); Q.c = 0.f; Q.idx = 0x7fffffff; Q.sx = 0.f; }
 }
 
-// CTA-wide inverse-CDF draw over this CTA's part of a row.  sh.mass[w] = total weight of warp w's
-// range (the coarse CDF); weights(vi, w[8]) the weights of vector vi; t = target prefix within
-// this part.  Every thread knows the selected warp range; pass 1 cuts it into one contiguous
-// block of vectors per thread of the CTA and sums the blocks in parallel, warp 0 scans the block
-// sums; pass 2 spreads the chosen block's vectors over the lanes of warp 0.  Two load round trips
-// in all.  Returns to every thread the lowest id whose inclusive prefix exceeds t; when rounding
-// leaves none inside the selected range, the last id with positive weight there; -1 when this
-// part has no mass.  Called by all threads of the CTA.
-// The two passes of the CTA-wide draw over the vectors [lo, hi): tt = target prefix within the
-// range.  Called by all threads of the CTA; returns the id to every thread (-1: no mass in range).
+// CTA-wide inverse-CDF draw over the vectors [lo, hi): weights(vi, w[8]) the weights of vector vi, tt = target prefix
+// within the range.  One block of consecutive vectors per thread is summed, every warp picks the warp that holds the
+// target from the warps' sums, and that warp spreads the picked thread's vectors over its lanes: two load round
+// trips, two barriers.  Called by all threads of the CTA; returns to every thread the lowest id whose inclusive prefix
+// exceeds tt; when rounding leaves none, the last id with positive weight of the picked block; -1: no mass.
 template <class WF>
 __device__ int range_sample3(int lo, int hi, WF weights, LeanShared &sh, float tt) {
-    const int lane = threadIdx.x & 31, nth = blockDim.x;
-    const int Bv = (hi - lo + nth - 1) / nth;  // vectors per thread block
-    {   // pass 1
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nth = blockDim.x;
+    const int Bv = (hi - lo + nth - 1) / nth;  // vectors per thread
+    float tot = 0.f;
+    {
         const int b0 = lo + threadIdx.x * Bv, b1 = min(hi, b0 + Bv);
-        float tot = 0.f;
 #pragma unroll 4
         for (int vi = b0; vi < b1; ++vi) {
             float w[8];
             weights(vi, w);
             tot += ((w[0] + w[1]) + (w[2] + w[3])) + ((w[4] + w[5]) + (w[6] + w[7]));
         }
-        sh.part[threadIdx.x] = tot;
     }
+    const float wt = warp_sum(tot);
+    if (lane == 0) sh.part[warp] = wt;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        const int per = nth >> 5;  // block sums per lane
-        float ls = 0.f;
-        for (int i = 0; i < per; ++i) ls += sh.part[lane * per + i];
-        float incl = ls;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const float up = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += up;
-        }
-        const unsigned pos = __ballot_sync(kFull, ls > 0.f);
-        const unsigned hit = __ballot_sync(kFull, ls > 0.f && incl > tt);
-        int blk = -1;
-        float tt2 = 0.f;
-        if (pos) {
-            const int L = hit ? (__ffs(hit) - 1) : (31 - __clz(pos));
-            if (lane == L) {
-                float acc = incl - ls;
-                int lastb = -1;
-                float lastacc = 0.f;
-                for (int i = 0; i < per; ++i) {
-                    const float m = sh.part[lane * per + i];
-                    if (m > 0.f) {
-                        lastb = lane * per + i;
-                        lastacc = acc;
-                        if (blk < 0 && acc + m > tt) { blk = lastb; tt2 = tt - acc; }
-                    }
-                    acc += m;
-                }
-                if (blk < 0) { blk = lastb; tt2 = tt - lastacc; }
-                sh.blk = blk;
-                sh.tt2 = tt2;
-            }
-        } else if (lane == 0) {
-            sh.blk = -1;
-        }
-        __syncwarp();
-        blk = sh.blk;
-        tt2 = sh.tt2;
+    const int W = lanes_pick(lane < (nth >> 5) ? sh.part[lane] : 0.f, tt);
+    if (W < 0) { __syncthreads(); return -1; }
+    if (warp == W) {
+        const int L = lanes_pick(tot, tt);
         int found = -1;
-        if (blk >= 0) {   // pass 2: the block's vectors over the lanes
-            const int c0 = lo + blk * Bv, c1 = min(hi, c0 + Bv);
-            float prefix = 0.f;
-            int lastpos = -1;
-            for (int v0 = c0; v0 < c1 && found < 0; v0 += 32) {
-                const int vi = v0 + lane;
-                float w[8];
-                if (vi < c1) {
-                    weights(vi, w);
-                } else {
+        const int c0 = lo + (W * 32 + max(L, 0)) * Bv, c1 = min(hi, c0 + Bv);
+        float prefix = 0.f;
+        int lastpos = -1;
+        for (int v0 = c0; v0 < c1 && found < 0; v0 += 32) {
+            const int vi = v0 + lane;
+            float w[8];
+            if (vi < c1) {
+                weights(vi, w);
+            } else {
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) w[i] = 0.f;
-                }
-                float lsum = 0.f;
-                int lp = -1;
+                for (int i = 0; i < 8; ++i) w[i] = 0.f;
+            }
+            float lsum = 0.f;
+            int lp = -1;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                lsum += w[i];
+                if (w[i] > 0.f) lp = vi * 8 + i;
+            }
+            const float in2 = lanes_prefix(lsum);
+            const unsigned hit2 = __ballot_sync(kFull, lsum > 0.f && prefix + in2 > tt);
+            if (hit2) {
+                float acc = prefix + (in2 - lsum);
+                int cand = -1, lastin = -1;
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    lsum += w[i];
-                    if (w[i] > 0.f) lp = vi * 8 + i;
-                }
-                float in2 = lsum;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const float up = __shfl_up_sync(kFull, in2, o);
-                    if (lane >= o) in2 += up;
-                }
-                const float tot2 = __shfl_sync(kFull, in2, 31);
-                const unsigned hit2 = __ballot_sync(kFull, lsum > 0.f && prefix + in2 > tt2);
-                if (hit2) {
-                    const int M = __ffs(hit2) - 1;
-                    int cand = -1;
-                    if (lane == M) {
-                        float acc = prefix + (in2 - lsum);
-                        int lastin = -1;
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            acc += w[i];
-                            if (w[i] > 0.f) {
-                                lastin = vi * 8 + i;
-                                if (cand < 0 && acc > tt2) cand = lastin;
-                            }
-                        }
-                        if (cand < 0) cand = lastin;
+                    acc += w[i];
+                    if (w[i] > 0.f) {
+                        lastin = vi * 8 + i;
+                        if (cand < 0 && acc > tt) cand = lastin;
                     }
-                    found = __shfl_sync(kFull, cand, M);
-                } else {
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) lp = max(lp, __shfl_xor_sync(kFull, lp, o));
-                    lastpos = max(lastpos, lp);
-                    prefix += tot2;
                 }
+                found = __shfl_sync(kFull, cand < 0 ? lastin : cand, __ffs(hit2) - 1);
+            } else {
+                lastpos = max(lastpos, __reduce_max_sync(kFull, lp));
+                prefix += __shfl_sync(kFull, in2, 31);
             }
-            if (found < 0) found = lastpos;
         }
+        if (found < 0) found = lastpos;
         if (lane == 0) sh.tok = found;
     }
     __syncthreads();
-    const int tok = sh.tok;
-    __syncthreads();
-    return tok;
+    return sh.tok;   // (written again only after the first barrier of a later draw)
 }
 
+// ... over this CTA's part of a row: mass[w] = total weight of warp w's range (the coarse CDF), t = target prefix
+// within this part
 template <class WF>
-__device__ int block_sample3(const Geo &g, WF weights, LeanShared &sh, float t) {
-    int wsel = -1, lastw = -1;
-    float base = 0.f, lastbase = 0.f, run = 0.f;
-    for (int w = 0; w < g.nwarps; ++w) {
-        const float m = sh.mass[w];
-        if (m > 0.f) {
-            lastw = w;
-            lastbase = run;
-            if (wsel < 0 && run + m > t) { wsel = w; base = run; }
-        }
-        run += m;
-    }
-    if (lastw < 0) return -1;
-    if (wsel < 0) { wsel = lastw; base = lastbase; }
-    return range_sample3(g.seg_lo(wsel), g.seg_hi(wsel), weights, sh, t - base);
+__device__ int block_sample3(const Geo &g, WF weights, const float *mass, LeanShared &sh, float t) {
+    const int lane = threadIdx.x & 31;
+    const int w = lanes_pick(lane < g.nwarps ? mass[lane] : 0.f, t);
+    if (w < 0) return -1;
+    return range_sample3(g.seg_lo(w), g.seg_hi(w), weights, sh, t);
 }
 
 // Pick the CTA of a row whose part holds the target t of an inverse-CDF draw over per-CTA masses
@@ -510,6 +458,7 @@ struct RowStat {
     float ml, C, sx;  // row max logit, its shift, sum without the row argmax
     float own;        // the row argmax's own term 2^(k ml - C) (1 up to the rounding of C)
     int idx;          // row argmax
+    __device__ __forceinline__ void set(const ArgMaxSum &o, float k) { ml = o.ml; C = o.c; sx = o.sx; idx = o.idx; own = o.own(k); }
 };
 
 // Merge the slices' (max, argmax, sum without argmax) in rank order (Section 4: a = argmax q).
@@ -541,7 +490,7 @@ __device__ __forceinline__ float slice_mass(const LeanShared &sh, int r, const R
 
 // Draw inside this CTA's slice from softmax(row) without token `excl`, target t (row scale,
 // relative to the start of the slice).  sh.wmass[r] holds the per-warp sums of the slice on the
-// slice's own scale with the slice argmax left out.
+// slice's own scale.
 template <class ROW>
 __device__ int lean_sample_slice(const Geo &g, const ROW &row, float k, const RowStat &st,
                                  int excl, float t, int r, LeanShared &sh) {
@@ -552,9 +501,7 @@ __device__ int lean_sample_slice(const Geo &g, const ROW &row, float k, const Ro
     const float C = st.C;
     if (threadIdx.x < g.nwarps) {
         const int w = threadIdx.x;
-        const int lv = locarg >> 3;
-        const bool holds = lml > neg_inf() && lv >= g.seg_lo(w) && lv < g.seg_hi(w);
-        sh.mass[w] = (sh.wmass[r][w] + ((holds && excl != locarg) ? own_term(lml, k) : 0.f)) * f;
+        sh.mass[w] = (excl >= 0 && excl == locarg && sh.widx[r][w] == locarg ? sh.wmassx[r][w] : sh.wmass[r][w]) * f;
     }
     __syncthreads();
     if (excl >= 0 && excl != locarg && g.holds_vec(excl >> 3)) {
@@ -577,7 +524,7 @@ __device__ int lean_sample_slice(const Geo &g, const ROW &row, float k, const Ro
 #pragma unroll
         for (int i = 0; i < 8; ++i) w[i] = (vi * 8 + i == excl) ? 0.f : ex2(__fmaf_rn(v.get(i), k, -C));
     };
-    return block_sample3(g, wf, sh, t);
+    return block_sample3(g, wf, sh.mass, sh, t);
 }
 
 // Draw from softmax(row) without `excl` (the row argmax, a slice argmax, or nothing) over the
@@ -597,36 +544,37 @@ __device__ int lean_sample_row(const Geo &g, const ROW &row, float k, const RowS
     return lean_sample_slice(g, row, k, st, excl, u * total - base, r, sh);
 }
 
-// CTA sums of NACC per-thread accumulators; the per-warp sums stay in sh.acc[OFF + i][w].
-template <int NACC, int OFF = 0>
-__device__ __forceinline__ void lean_block_sums(float (&x)[NACC], LeanShared &sh) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// CTA sums of NACC per-thread accumulators; the per-warp sums stay in sh.acc[OFF + i][w].  ANY: also whether `any` is
+// set in some thread.  One barrier; a second call in the same kernel takes other rows of sh.acc.
+template <int NACC, int OFF, bool ANY = false>
+__device__ __forceinline__ void lean_block_sums(float (&x)[NACC], LeanShared &sh, unsigned *any = nullptr) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
 #pragma unroll
     for (int i = 0; i < NACC; ++i) {
         const float s = warp_sum(x[i]);
         if (lane == 0) sh.acc[OFF + i][warp] = s;
     }
-    __syncthreads();
-    const int nwarps = blockDim.x >> 5;
-#pragma unroll
-    for (int i = 0; i < NACC; ++i) {
-        float t = 0.f;
-        for (int w = 0; w < nwarps; ++w) t += sh.acc[OFF + i][w];
-        x[i] = t;
+    if (ANY) {
+        const int a = __any_sync(kFull, *any != 0);
+        if (lane == 0) sh.any[warp] = a;
     }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < NACC; ++i) x[i] = warp_sum(lane < nwarps ? sh.acc[OFF + i][lane] : 0.f);
+    if (ANY) *any = __any_sync(kFull, lane < nwarps && sh.any[lane]);
 }
 
 // Sum NACC per-thread accumulators over the whole row: CTA sums, then the slices in rank order.
-// part[i][c] receives slice c's sum of accumulator i; sh.acc[i][w] keeps this CTA's per-warp sums.
+// part[i][c] receives slice c's sum of accumulator i; sh.acc[OFF + i][w] keeps this CTA's per-warp sums.
 // Contains one row-group barrier.  OFF: first exchange slot used (a second call in the same
 // kernel takes other slots, so no CTA overwrites what a slower one has not read yet).
-template <int CS, int NACC, int OFF>
-__device__ __forceinline__ void lean_row_sums(float (&x)[NACC], float (&part)[NACC][CS], LeanShared &sh) {
-    lean_block_sums<NACC>(x, sh);
+template <int CS, int NACC, int OFF, bool ANY = false>
+__device__ __forceinline__ void lean_row_sums(float (&x)[NACC], float (&part)[NACC][CS], LeanShared &sh,
+                                              unsigned *any = nullptr) {
+    lean_block_sums<NACC, OFF, ANY>(x, sh, any);
     if (CS == 1) {
 #pragma unroll
         for (int i = 0; i < NACC; ++i) part[i][0] = x[i];
-        __syncthreads();  // sh.acc may be rewritten by a later sum only after all have read it
         return;
     }
     if (threadIdx.x == 0) {
@@ -722,93 +670,78 @@ __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, in
     Q.m2 = st.m2; Q.c = st.c; Q.s = tot;
 }
 
-// Inverse-CDF draw from softmax(row) without token `excl` (excl < 0: nothing left out) over the
-// checkpoint sub-blocks.  C = the row's exponent shift.  Returns to every thread the token, -1 if
-// nothing has mass.  Called by all threads of the CTA, after the checkpoints are visible.
-template <class ROW>
-__device__ int lean_ck_sample(const Geo &g, const ROW &row, float k, float C, int CK, int excl,
-                              float u, LeanCkShared &sh) {
+// The sub-block that holds id y is summed again without the ids that `left_out` names: subtracting their own terms
+// would cancel when they carry most of the sub-block's mass.  Called by all threads of the CTA; the new sum is
+// visible to all on return.  C = the row's exponent shift.
+template <class ROW, class EX>
+__device__ void lean_ck_drop(const Geo &g, const ROW &row, float k, float C, int CK, EX left_out, int y, LeanCkShared &sh) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nslot = g.nwarps * kLeanCk;
-    auto wf = [&](int vi, float(&w)[8]) {
+    const int w = g.warp_of_vec(y >> 3), j = ((y >> 3) - g.seg_lo(w)) / (32 * CK);
+    const int b0 = g.seg_lo(w) + 32 * CK * j, b1 = min(g.seg_hi(w), b0 + 32 * CK);
+    float s = 0.f;
+    for (int vi = b0 + threadIdx.x; vi < b1; vi += blockDim.x) {
         const auto v = row[vi];
+        float e[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) w[i] = (vi * 8 + i == excl) ? 0.f : ex2(__fmaf_rn(v.get(i), k, -C));
+        for (int i = 0; i < 8; ++i) e[i] = left_out(vi * 8 + i) ? 0.f : ex2(__fmaf_rn(v.get(i), k, -C));
+        s += ((e[0] + e[1]) + (e[2] + e[3])) + ((e[4] + e[5]) + (e[6] + e[7]));
+    }
+    s = warp_sum(s);
+    if (lane == 0) sh.mass[warp] = s;
+    __syncthreads();
+    if (warp == 0) {
+        s = warp_sum(lane < g.nwarps ? sh.mass[lane] : 0.f);
+        if (lane == 0) { sh.cks[w * kLeanCk + j] = s; sh.ckc[w * kLeanCk + j] = C; }
+    }
+    __syncthreads();
+}
+
+// Inverse-CDF draw from softmax(row) over the checkpoint sub-blocks, ids that `left_out` names having no weight (their
+// sub-blocks' sums say so already).  C = the row's exponent shift.  Returns to every thread the token, -1 if nothing has
+// mass.  Called by all threads of the CTA, after the checkpoints are visible.
+template <class ROW, class EX>
+__device__ int lean_ck_draw(const Geo &g, const ROW &row, float k, float C, int CK, EX left_out, float u, LeanCkShared &sh) {
+    const int lane = threadIdx.x & 31;
+    const int nslot = g.nwarps * kLeanCk, per = (nslot + 31) >> 5;   // (consecutive sub-blocks per lane)
+    // every warp picks the sub-block by itself
+    auto slot_mass = [&](int s) {
+        const float cs = s < nslot ? sh.cks[s] : 0.f;
+        return cs > 0.f ? cs * ex2(sh.ckc[s] - C) : 0.f;
     };
-    for (int s = threadIdx.x; s < nslot; s += blockDim.x) {
-        const float cs = sh.cks[s / kLeanCk][s % kLeanCk];
-        sh.ckm[s] = cs > 0.f ? cs * ex2(sh.ckc[s / kLeanCk][s % kLeanCk] - C) : 0.f;
+    float ls = 0.f;
+    for (int i = 0; i < per; ++i) ls += slot_mass(lane * per + i);
+    const float total = __shfl_sync(kFull, lanes_prefix(ls), 31);
+    if (!(total > 0.f)) return -1;
+    float t = u * total;
+    const int L = lanes_pick(ls, t);
+    int slot = -1, last = -1;
+    float acc = 0.f, tt = 0.f, lastacc = 0.f;
+    for (int i = 0; i < per; ++i) {
+        const int s = L * per + i;
+        const float m = slot_mass(s);
+        if (m > 0.f) {
+            last = s;
+            lastacc = acc;
+            if (slot < 0 && acc + m > t) { slot = s; tt = t - acc; }
+        }
+        acc += m;
     }
-    __syncthreads();
-    if (excl >= 0) {
-        // the sub-block that holds the excluded token is summed again without it: subtracting the
-        // token's own term would cancel when that token carries most of the sub-block's mass
-        const int ev = excl >> 3;
-        const int w = g.warp_of_vec(ev), j = (ev - g.seg_lo(w)) / (32 * CK);
-        const int b0 = g.seg_lo(w) + 32 * CK * j, b1 = min(g.seg_hi(w), b0 + 32 * CK);
-        float s = 0.f;
-        for (int vi = b0 + threadIdx.x; vi < b1; vi += blockDim.x) {
-            float wt[8];
-            wf(vi, wt);
-            s += ((wt[0] + wt[1]) + (wt[2] + wt[3])) + ((wt[4] + wt[5]) + (wt[6] + wt[7]));
-        }
-        s = warp_sum(s);
-        if (lane == 0) sh.mass[warp] = s;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            float t = 0.f;
-            for (int x = 0; x < g.nwarps; ++x) t += sh.mass[x];
-            sh.ckm[w * kLeanCk + j] = t;
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x < 32) {   // warp 0: prefix sums over the sub-blocks, in id order
-        const int per = (nslot + 31) >> 5;
-        float ls = 0.f;
-        for (int i = 0; i < per; ++i) {
-            const int s = lane * per + i;
-            if (s < nslot) ls += sh.ckm[s];
-        }
-        float incl = ls;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const float up = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += up;
-        }
-        const float total = __shfl_sync(kFull, incl, 31);
-        const float t = u * total;
-        const unsigned pos = __ballot_sync(kFull, ls > 0.f);
-        const unsigned hit = __ballot_sync(kFull, ls > 0.f && incl > t);
-        if (!pos || !(total > 0.f)) {
-            if (lane == 0) sh.blk = -1;
-        } else {
-            const int L = hit ? (__ffs(hit) - 1) : (31 - __clz(pos));
-            if (lane == L) {
-                float acc = incl - ls, lastacc = 0.f;
-                int sel = -1, last = -1;
-                for (int i = 0; i < per; ++i) {
-                    const int s = lane * per + i;
-                    const float m = s < nslot ? sh.ckm[s] : 0.f;
-                    if (m > 0.f) {
-                        last = s;
-                        lastacc = acc;
-                        if (sel < 0 && acc + m > t) { sel = s; sh.tt2 = t - acc; }
-                    }
-                    acc += m;
-                }
-                if (sel < 0) { sel = last; sh.tt2 = t - lastacc; }
-                sh.blk = sel;
-            }
-        }
-    }
-    __syncthreads();
-    const int slot = sh.blk;
-    const float tt = sh.tt2;
-    __syncthreads();   // range_sample3 reuses blk / tt2
-    if (slot < 0) return -1;
+    if (slot < 0) { slot = last; tt = t - lastacc; }
     const int w = slot / kLeanCk, j = slot % kLeanCk;
     const int b0 = g.seg_lo(w) + 32 * CK * j, b1 = min(g.seg_hi(w), b0 + 32 * CK);
-    return range_sample3(b0, b1, wf, sh, tt);
+    return range_sample3(b0, b1, [&](int vi, float(&wt)[8]) {
+        const auto v = row[vi];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) wt[i] = left_out(vi * 8 + i) ? 0.f : ex2(__fmaf_rn(v.get(i), k, -C));
+    }, sh, tt);
+}
+
+// ... without token `excl` (excl < 0: nothing left out; later draws leave it out too)
+template <class ROW>
+__device__ int lean_ck_sample(const Geo &g, const ROW &row, float k, float C, int CK, int excl, float u, LeanCkShared &sh) {
+    auto left_out = [&](int y) { return y == excl; };
+    if (excl >= 0) lean_ck_drop(g, row, k, C, CK, left_out, excl, sh);
+    return lean_ck_draw(g, row, k, C, CK, left_out, u, sh);
 }
 
 // Leaf rows (Figure 2: after the last accepted draft the bonus token is a draw from p) of a call
@@ -817,7 +750,7 @@ __device__ int lean_ck_sample(const Geo &g, const ROW &row, float k, float C, in
 // once; the verification kernels skip the leaf rows.  Up to three output sets receive the result
 // (the three-method call: the methods share u_res, hence the bonus token).
 template <typename LT, bool SHIFT, int THREADS>
-__global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_leaf_kernel(LeafArgs A) {
+__global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_leaf_kernel(LeafArgs A) {
     __shared__ LeanCkShared sh;
     const RowArgs &a = A.r;
     const long long r = blockIdx.x;
@@ -828,11 +761,12 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_l
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int lo = g.seg_lo(warp), hi = g.seg_hi(warp);
     const float k = kLog2e / temperature_of(a, b);
-    const float ures = a.uniforms[r * 5 + 4];
+    const int K = A.k;
+    const float ures = a.uniforms[r * (2 * K + 1) + 2 * K];
     const int CK = lean_ck_interval(g);
     LeanAcc<LT> tp, unused;
     unused.init();
-    lean_pass_a_ck<SHIFT>(vp, lo, hi, lane, k, CK, tp, sh.cks[warp], sh.ckc[warp]);
+    lean_pass_a_ck<SHIFT>(vp, lo, hi, lane, k, CK, tp, sh.cks + warp * kLeanCk, sh.ckc + warp * kLeanCk);
     ArgMaxSum Ps, unusedq;
     lean_reduce2<false>(tp, unused, vp, vp, lo, hi, k, sh, Ps, unusedq);
     const float Zp = Ps.sx + Ps.own(k);
@@ -846,8 +780,11 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_l
             o.accept_idx[r] = -1;
             o.token[r] = tok;
             if (o.hub) o.hub[r] = -1;
-            if (o.beta) { o.beta[2 * r] = 0.f; o.beta[2 * r + 1] = 0.f; }
-            if (o.rate) { o.rate[3 * r] = 0.f; o.rate[3 * r + 1] = 0.f; o.rate[3 * r + 2] = status ? 0.f : 1.f; }
+            for (int i = 0; i < K; ++i) {
+                if (o.beta) o.beta[K * r + i] = 0.f;
+                if (o.rate) o.rate[(K + 1) * r + i] = 0.f;
+            }
+            if (o.rate) o.rate[(K + 1) * r + K] = status ? 0.f : 1.f;
             if (o.status) o.status[r] = status;
         }
     }
@@ -887,7 +824,7 @@ __device__ __forceinline__ float sum_without(const RowStat &st, const ROW &row, 
 // after pass A, let the rows go at their last use): with a single row to keep in L2 between passes that
 // beats the rings (RRS 1.53 -> 1.46 ms, RRSw 1.62 -> 1.60 ms on V = 128256, 7936 rows).
 template <typename LT, bool SHIFT, int METHOD, int THREADS, int CS, bool RING = false, bool STATS = false>
-__global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_verify_kernel(RowArgs a) {
+__global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verify_kernel(RowArgs a) {
     static_assert(!RING || (sizeof(LT) == 2 && !SHIFT), "the ring-fed form: bf16 rows in whole words");
     static_assert(!RING || (CS == 1 && METHOD != kSpecHub), "the ring-fed form: whole rows, RRS and RRSw");
     static_assert(!STATS || (CS == 1 && !RING), "draft statistics: whole rows, register-fed passes");
@@ -907,7 +844,6 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_v
     // the tail of the row is still in L2 even when the rows in flight exceed its capacity.
     const int last_vi = (lo + lane < hi) ? lo + lane + ((hi - 1 - lo - lane) / 32) * 32 : lo - 1;
     const float k = kLog2e / temperature_of(a, b);
-    const float r1 = a.uniforms[r * 5 + 2], r2 = a.uniforms[r * 5 + 3], ures = a.uniforms[r * 5 + 4];
     const float pinf = -neg_inf();
     // leaf rows of an unsplit call belong to lean_leaf_kernel
     if (CS == 1 && a.node_kind && a.node_kind[n] == SPECHUB_NODE_LEAF) return;
@@ -921,18 +857,29 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_v
     // a flagged row, the CTA that draws for a residual / leaf token.
     bool token_elsewhere = false;
 
-    if (STATS && threadIdx.x == THREADS - 1) {
-        // The draft row's record, fetched and checked by one thread before it starts on pass A: its two
-        // dependent look-ups (the record, then the draft logit at the recorded argmax) are off the path
-        // between pass A and pass B.  (Nothing else writes these fields; they are read after barriers.)
-        const DraftStat ds = static_cast<const DraftStat *>(a.draft_stats_in)[r];
-        bool ok = ds.tag == (kDraftStatTag ^ __float_as_uint(k));
-        // (a record of a row without a finite maximum or sum needs no look-up: the row is flagged
-        // SPECHUB_ST_NONFINITE below, as it is without the record)
-        if (ok && ds.ml > neg_inf() && ds.ml < pinf && finite_pos(ds.sx + 1.f))
-            ok = ds.idx >= 0 && ds.idx < a.vocab && vq.one(ds.idx) == ds.ml;
-        sh.stat_ok = ok;
-        sh.x_ml[1] = ds.ml; sh.x_sx[1] = ds.sx; sh.x_idx[1] = ok ? ds.idx : 0;
+    // What the tests need of single ids -- the drafts, their logits, the uniforms, the draft row's record -- is fetched
+    // by the last warp before it starts on pass A: two dependent look-ups that are off the path between the passes.
+    // (Nothing else writes these fields; they are read after barriers.)
+    if (warp == THREADS / 32 - 1) {
+        const int t1 = a.draft_tokens_in[2 * r], t2 = a.draft_tokens_in[2 * r + 1];
+        DraftStat ds = {};
+        if (STATS) ds = static_cast<const DraftStat *>(a.draft_stats_in)[r];
+        int y = lane > 4 ? -1 : lane == 4 ? (STATS ? ds.idx : -1) : (lane & 1) ? t2 : t1;
+        if (leaf) y = -1;
+        float l = neg_inf();
+        if (y >= 0 && y < a.vocab) l = lane < 2 ? vp.one(y) : vq.one(y);
+        if (lane > 4 && lane < 8) l = a.uniforms[r * 5 + lane - 3];
+        if (lane < 8) sh.lg[lane] = l;
+        if (lane == 0) { sh.tk[0] = t1; sh.tk[1] = t2; }
+        if (STATS && lane == 4) {
+            bool ok = ds.tag == (kDraftStatTag ^ __float_as_uint(k));
+            // (a record of a row without a finite maximum or sum needs no look-up: the row is flagged
+            // SPECHUB_ST_NONFINITE below, as it is without the record)
+            if (ok && ds.ml > neg_inf() && ds.ml < pinf && finite_pos(ds.sx + 1.f))
+                ok = ds.idx >= 0 && ds.idx < a.vocab && l == ds.ml;
+            sh.stat_ok = ok;
+            sh.x_ml[1] = ds.ml; sh.x_sx[1] = ds.sx; sh.x_idx[1] = ok ? ds.idx : 0;
+        }
     }
     // the row's stream: pass A forwards, pass B backwards, (RRS, RRSw) pass C forwards
     WarpRing R;
@@ -949,6 +896,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_v
         if (leaf) lean_pass_a<false, false>(vp, vq, lo, hi, lane, k, tp, tq);
         else lean_pass_a<true, METHOD == kRRS>(vp, vq, lo, hi, lane, k, tp, tq);
     }
+    RowStat P, Q;
     {
         ArgMaxSum Ps, Qs;
         if (leaf || STATS) lean_reduce2<false>(tp, tq, vp, vq, lo, hi, k, sh, Ps, Qs);
@@ -957,11 +905,18 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_v
             sh.x_ml[0] = Ps.ml; sh.x_sx[0] = Ps.sx; sh.x_idx[0] = Ps.idx;
             if (!STATS) { sh.x_ml[1] = Qs.ml; sh.x_sx[1] = Qs.sx; sh.x_idx[1] = Qs.idx; }
         }
+        if (CS == 1) {   // (the published values are read by a draw from p only, after further barriers)
+            if (STATS) { Qs.ml = sh.x_ml[1]; Qs.c = shift_of(Qs.ml, k); Qs.sx = sh.x_sx[1]; Qs.idx = sh.x_idx[1]; }
+            P.set(Ps, k);
+            Q.set(Qs, k);
+        }
     }
-    RowGroup<CS>::sync();  // [1] slices published
-    RowStat P, Q;
-    merge_slices<CS>(sh, 0, k, P);
-    merge_slices<CS>(sh, 1, k, Q);
+    if (CS > 1) {
+        RowGroup<CS>::sync();  // [1] slices published
+        merge_slices<CS>(sh, 0, k, P);
+        merge_slices<CS>(sh, 1, k, Q);
+    }
+    const float r1 = sh.lg[5], r2 = sh.lg[6], ures = sh.lg[7];
     // (Z_p, its shift and rho change only in verification from draft statistics, when the two rows turn
     // out to be the same row: see below)
     float Zp = P.sx + P.own;
@@ -974,14 +929,10 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_v
     // the sums S1, R, A1 are exactly 0, which a rho of 1 +- 1e-7 would turn into noise that the tests then
     // divide by.  Pass B sees both rows and notices; the row is then redone with p's normaliser set to q's.
     unsigned diff = 0;
-    auto rows_identical = [&]() {
-        if (__syncthreads_or(diff != 0)) return false;
-        Zp = Zq; invZp = invZq; cP = cQ; rho = 1.f;
-        return true;
-    };
-    const int x1 = a.draft_tokens_in[2 * r], x2 = a.draft_tokens_in[2 * r + 1];
-    auto prob_p = [&](int y) { return prob_of(vp.one(y), k, cP, invZp); };
-    auto prob_q = [&](int y) { return prob_of(vq.one(y), k, cQ, invZq); };
+    auto take_q_normaliser = [&]() { Zp = Zq; invZp = invZq; cP = cQ; rho = 1.f; };
+    const int x1 = sh.tk[0], x2 = sh.tk[1];
+    auto prob_p = [&](int i) { return prob_of(sh.lg[i], k, cP, invZp); };       // of draft i
+    auto prob_q = [&](int i) { return prob_of(sh.lg[2 + i], k, cQ, invZq); };
     auto draw_from_p = [&]() {  // every CTA of the row calls it
         const int tok = lean_sample_row<CS>(g, vp, k, P, me, -1, ures, 0, sh);
         if (tok != -2 && threadIdx.x == 0) a.token[r] = tok;
@@ -1009,8 +960,9 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_v
             float crho = c * rho;
             const float qa = Q.own * invZq, rest = Q.sx * invZq;
             const int hubvec = hubtok >> 3, hubel = hubtok & 7;
-            float px = prob_p(x);
-            const float qx = prob_q(x);
+            const int ix = pair_xa ? 0 : 1;   // the draft that is not the hub
+            float px = prob_p(ix);
+            const float qx = prob_q(ix);
             if (!a.beta && !a.rate) {
                 // No probability is asked for: the first test needs scalars only, and if it accepts
                 // the transport sums decide nothing.
@@ -1072,22 +1024,23 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_v
             }
             };
             pass_b();
-            if (STATS && rows_identical()) {
+            float acc[3] = {f2_sum(s1), f2_sum(s2), f2_sum(rr)};
+            float part[3][CS];
+            lean_row_sums<CS, 3, 0, STATS>(acc, part, sh, &diff);  // [2]
+            const float *mass_r = sh.acc[2];
+            if (STATS && !diff) {
+                take_q_normaliser();
                 crho = c;
                 px = qx;
                 pass_b();
+                acc[0] = f2_sum(s1); acc[1] = f2_sum(s2); acc[2] = f2_sum(rr);
+                lean_row_sums<CS, 3, 3>(acc, part, sh);
+                mass_r = sh.acc[5];
             }
-            float s1a, s1b, s2a, s2b, ra, rb;
-            f2_get(s1, s1a, s1b);
-            f2_get(s2, s2a, s2b);
-            f2_get(rr, ra, rb);
-            float acc[3] = {s1a + s1b, s2a + s2b, ra + rb};
-            float part[3][CS];
-            lean_row_sums<CS, 3, 0>(acc, part, sh);  // [2]
             // the sums are in units of 1 / Z_p; Rraw stays in them for the residual draw
             const float Rraw = acc[2];
             const float S1 = acc[0] * invZp, S2 = degenerate ? qa : acc[1] * invZp, R = Rraw * invZp;
-            const float pa = prob_p(hubtok);
+            const float pa = prob_p(1 - ix);
             const float hub_left = fmaxf(pa - S2, 0.f);
             o.rate[0] = fmaxf(rest - S1, 0.f) + fminf(pa, S2);
             o.rate[1] = (degenerate ? 0.f : fmaxf(qa - S2, 0.f)) + fminf(hub_left, S1);
@@ -1115,8 +1068,6 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_v
                 } else {
                     token_elsewhere = true;
                     if (sel == me) {
-                        if (threadIdx.x < g.nwarps) sh.mass[threadIdx.x] = sh.acc[2][threadIdx.x];
-                        __syncthreads();
                         auto wf = [&](int vi, float(&w)[8]) {
                             const V fp = vp[vi], fq = vq[vi];
 #pragma unroll
@@ -1126,7 +1077,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_v
                                 w[i] = (vi * 8 + i == hubtok) ? 0.f : fmaxf(t, 0.f);
                             }
                         };
-                        const int tok = block_sample3(g, wf, sh, ures * Rraw - base);
+                        const int tok = block_sample3(g, wf, mass_r, sh, ures * Rraw - base);
                         if (threadIdx.x == 0) a.token[r] = tok;
                     }
                 }
@@ -1135,7 +1086,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_v
             if (x1 < 0 || x1 >= a.vocab || x2 < 0 || x2 >= a.vocab) { o.status = SPECHUB_ST_TOKEN_RANGE; break; }
             if (!a.beta && !a.rate) {
                 // no probability asked for: an accepted first draft needs no sum at all
-                if (accept_test(r1, prob_p(x1), prob_q(x1), o.beta[0], true, o.status)) {
+                if (accept_test(r1, prob_p(0), prob_q(0), o.beta[0], true, o.status)) {
                     o.accept_idx = 0;
                     o.token = x1;
                     break;
@@ -1211,12 +1162,15 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_v
             }
             };
             pass_b(true);
-            if (STATS && rows_identical()) pass_b(false);
-            float a1a, a1b;
-            f2_get(a1, a1a, a1b);
-            float acc[2] = {a1a + a1b, dna + dnb};
+            float acc[2] = {f2_sum(a1), dna + dnb};
             float part2[2][CS];
-            lean_row_sums<CS, 2, 0>(acc, part2, sh);  // [2]
+            lean_row_sums<CS, 2, 0, STATS>(acc, part2, sh, &diff);  // [2]
+            if (STATS && !diff) {
+                take_q_normaliser();
+                pass_b(false);
+                acc[0] = f2_sum(a1); acc[1] = dna + dnb;
+                lean_row_sums<CS, 2, 4>(acc, part2, sh);
+            }
             if (STATS && METHOD == kRRSw) acc[1] = sum_without(Q, vq, x1, k);
             const float A1 = acc[0] * invZp, den = acc[1] * invZq;   // the sums are of exponentials
             const bool q1_zero = (METHOD == kRRSw) && !(den > 0.f);
@@ -1286,7 +1240,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_v
             o.rate[0] = fmaxf(1.f - A1, 0.f);
             o.rate[1] = fmaxf(A1 - W2, 0.f);
             o.rate[2] = W2;
-            const float px1 = prob_p(x1), qx1 = prob_q(x1), px2 = prob_p(x2), qx2 = prob_q(x2);
+            const float px1 = prob_p(0), qx1 = prob_q(0), px2 = prob_p(1), qx2 = prob_q(1);
             const bool acc1 = accept_test(r1, px1, qx1, o.beta[0], true, o.status);
             if (acc1) { o.accept_idx = 0; o.token = x1; }
             if (!acc1 && q1_zero) o.status |= SPECHUB_ST_DEGENERATE_Q;
@@ -1306,8 +1260,6 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_v
                 } else {
                     token_elsewhere = true;
                     if (sel == me) {
-                        if (threadIdx.x < g.nwarps) sh.mass[threadIdx.x] = sh.acc[0][threadIdx.x];
-                        __syncthreads();
                         auto wf = [&](int vi, float(&w)[8]) {
                             const V fp = vp[vi], fq = vq[vi];
 #pragma unroll
@@ -1318,7 +1270,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_v
                                 w[i] = fmaxf(t, 0.f);
                             }
                         };
-                        const int tok = block_sample3(g, wf, sh, ures * W2raw - base);
+                        const int tok = block_sample3(g, wf, sh.acc[2], sh, ures * W2raw - base);
                         if (threadIdx.x == 0) a.token[r] = tok;
                     }
                 }
@@ -1465,7 +1417,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_kernel(Row
 // Draft step, one CTA per row (checkpointed pass A and sub-block sampler above).
 // ------------------------------------------------------------------------------------------------
 template <typename LT, bool SHIFT, int THREADS>
-__global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_draft_ck_kernel(RowArgs a, int method, bool keep_stats) {
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(RowArgs a, int method, bool keep_stats) {
     __shared__ LeanCkShared sh;
     const long long r = blockIdx.x;
     const int b = static_cast<int>(r / a.nodes), n = static_cast<int>(r % a.nodes);
@@ -1479,15 +1431,13 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<LT, SHIFT>(THREADS)) lean_d
 
     LeanAcc<LT> tq, unused;
     unused.init();
-    lean_pass_a_ck<SHIFT>(vq, lo, hi, lane, k, CK, tq, sh.cks[warp], sh.ckc[warp]);
+    lean_pass_a_ck<SHIFT>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * kLeanCk, sh.ckc + warp * kLeanCk);
+    RowStat Q;
     {
         ArgMaxSum q, unusedq;
         lean_reduce2<false>(tq, unused, vq, vq, lo, hi, k, sh, q, unusedq);
-        if (threadIdx.x == 0) { sh.x_ml[0] = q.ml; sh.x_sx[0] = q.sx; sh.x_idx[0] = q.idx; }
+        Q.set(q, k);
     }
-    __syncthreads();
-    RowStat Q;
-    merge_slices<1>(sh, 0, k, Q);
     const float Zq = Q.sx + Q.own;
     uint32_t st = 0;
     int x1 = -1, x2 = -1, hubtok = -1;

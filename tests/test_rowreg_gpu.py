@@ -1,6 +1,6 @@
 """Rows held in registers (calls whose rows do not fill the GPU, short vocabularies) and streamed rows of any
-alignment: the edges of a lane's vectors,
-of a warp's and a cluster's part, aligned and packed odd rows, both types, against the oracle."""
+alignment: the edges of a lane's vectors, of a warp's and a cluster's part, aligned and packed odd rows, both types,
+against the oracle."""
 import numpy as np
 import pytest
 
