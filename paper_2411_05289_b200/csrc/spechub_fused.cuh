@@ -347,6 +347,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
         lean_reduce2<false>(tq, unused, vq, vq, lo, hi, k, sh, q, unusedq);
         Q.set(q, k);
     }
+    if (warp != 0) return;
     const float Zq = Q.sx + Q.own;
     if (t0 && a.draft_stats_out) {   // the record lean_draft_ck_kernel leaves, bit for bit
         DraftStat ds;
@@ -365,29 +366,33 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
         return;
     }
     const int hubtok = Q.idx;
-    const int x1 = lean_ck_sample(g, vq, k, Q.C, CK, -1, u1, sh);
+    int x1 = lean_ck_draw(g, vq, k, Q.C, CK, NoneOut{}, u1, sh);
+    if (x1 < 0) x1 = hubtok;   // (as in lean_draft_ck_kernel)
     uint32_t st[3] = {0, 0, 0};
     int x2[3];
     // RRS: an independent second draw (before a token is left out of the checkpoints' sums)
-    x2[1] = lean_ck_sample(g, vq, k, Q.C, CK, -1, u2, sh);
+    x2[1] = lean_ck_draw(g, vq, k, Q.C, CK, NoneOut{}, u2, sh);
     // RRSw: q with q(x1) set to 0
-    x2[2] = lean_ck_sample(g, vq, k, Q.C, CK, x1, u2, sh);
+    lean_ck_drop(g, vq, k, Q.C, CK, OneOut{x1}, x1, sh);
+    x2[2] = lean_ck_draw(g, vq, k, Q.C, CK, OneOut{x1}, u2, sh);
+    if (x2[2] < 0) {
+        x2[2] = (x1 == 0) ? 1 : 0;
+        st[2] |= SPECHUB_ST_DEGENERATE_Q;
+    }
     // SpecHub (Section 4)
     const float prob0 = Q.own / Zq;
     float prob1 = 0.f;
     if (x1 != hubtok) {
         x2[0] = hubtok;
         prob1 = ex2(fmaf(load_one<__nv_bfloat16>(rowq, x1), k, -Q.C)) / Zq;
-    } else if (!(Q.sx > 0.f)) {
-        x2[0] = (hubtok == 0) ? 1 : 0;
-        st[0] |= SPECHUB_ST_DEGENERATE_Q;
-    } else {
-        x2[0] = x2[2];   // (q without the hub, which is x1: the draw RRSw made)
-        prob1 = prob0 * ex2(fmaf(load_one<__nv_bfloat16>(rowq, x2[0]), k, -Q.C)) / Q.sx;
-    }
-    if (x2[2] < 0) {
-        x2[2] = (x1 == 0) ? 1 : 0;
-        st[2] |= SPECHUB_ST_DEGENERATE_Q;
+    } else {   // q without the hub, which is x1: the draw RRSw made
+        x2[0] = x2[2];
+        if (!(Q.sx > 0.f) || st[2]) {
+            x2[0] = (hubtok == 0) ? 1 : 0;
+            st[0] |= SPECHUB_ST_DEGENERATE_Q;
+        } else {
+            prob1 = prob0 * ex2(fmaf(load_one<__nv_bfloat16>(rowq, x2[0]), k, -Q.C)) / Q.sx;
+        }
     }
     if (t0) {
         for (int m = 0; m < 3; ++m) {

@@ -670,40 +670,65 @@ __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, in
     Q.m2 = st.m2; Q.c = st.c; Q.s = tot;
 }
 
-// The sub-block that holds id y is summed again without the ids that `left_out` names: subtracting their own terms
-// would cancel when they carry most of the sub-block's mass.  Called by all threads of the CTA; the new sum is
-// visible to all on return.  C = the row's exponent shift.
-template <class ROW, class EX>
-__device__ void lean_ck_drop(const Geo &g, const ROW &row, float k, float C, int CK, EX left_out, int y, LeanCkShared &sh) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int w = g.warp_of_vec(y >> 3), j = ((y >> 3) - g.seg_lo(w)) / (32 * CK);
-    const int b0 = g.seg_lo(w) + 32 * CK * j, b1 = min(g.seg_hi(w), b0 + 32 * CK);
+// The draws are made by one warp, the others are done: a sub-block is a few vectors per lane, and a CTA-wide draw costs
+// every warp its barriers and its share of the picking (V = 32000: 5800 of the 12000 warp instructions of a row).
+struct NoneOut {   // ids that a draw leaves out: none, one, the first n of a list
+    template <class V> __device__ __forceinline__ void apply(int, V &) const {}
+};
+struct OneOut {
+    int y;
+    template <class V> __device__ __forceinline__ void apply(int vi, V &v) const { if (vi == (y >> 3)) v.drop(y & 7); }
+};
+struct ListOut {
+    const int *x;
+    int n;
+    template <class V> __device__ __forceinline__ void apply(int vi, V &v) const {
+        for (int i = 0; i < n; ++i)
+            if (vi == (x[i] >> 3)) v.drop(x[i] & 7);
+    }
+};
+// this lane's share of a sub-block: its consecutive vectors [b0 + lane * Bv, ...), summed without the ids left out
+template <class ROW, class OUT>
+__device__ __forceinline__ float ck_lane_sum(const ROW &row, float k, float C, int v0, int v1, OUT out) {
     float s = 0.f;
-    for (int vi = b0 + threadIdx.x; vi < b1; vi += blockDim.x) {
-        const auto v = row[vi];
-        float e[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) e[i] = left_out(vi * 8 + i) ? 0.f : ex2(__fmaf_rn(v.get(i), k, -C));
-        s += ((e[0] + e[1]) + (e[2] + e[3])) + ((e[4] + e[5]) + (e[6] + e[7]));
+#pragma unroll 4
+    for (int vi = v0; vi < v1; ++vi) {
+        auto v = row[vi];
+        out.apply(vi, v);
+        s += vec_sum(v, f2_make(k, k), f2_make(-C, -C));
     }
-    s = warp_sum(s);
-    if (lane == 0) sh.mass[warp] = s;
-    __syncthreads();
-    if (warp == 0) {
-        s = warp_sum(lane < g.nwarps ? sh.mass[lane] : 0.f);
-        if (lane == 0) { sh.cks[w * kLeanCk + j] = s; sh.ckc[w * kLeanCk + j] = C; }
-    }
-    __syncthreads();
+    return s;
+}
+struct CkBlock { int b0, b1, Bv; };
+__device__ __forceinline__ CkBlock ck_block(const Geo &g, int CK, int slot) {
+    const int w = slot / kLeanCk, j = slot % kLeanCk;
+    CkBlock o;
+    o.b0 = g.seg_lo(w) + 32 * CK * j;
+    o.b1 = min(g.seg_hi(w), o.b0 + 32 * CK);
+    o.Bv = (o.b1 - o.b0 + 31) >> 5;
+    return o;
 }
 
-// Inverse-CDF draw from softmax(row) over the checkpoint sub-blocks, ids that `left_out` names having no weight (their
-// sub-blocks' sums say so already).  C = the row's exponent shift.  Returns to every thread the token, -1 if nothing has
-// mass.  Called by all threads of the CTA, after the checkpoints are visible.
-template <class ROW, class EX>
-__device__ int lean_ck_draw(const Geo &g, const ROW &row, float k, float C, int CK, EX left_out, float u, LeanCkShared &sh) {
+// The sub-block that holds id y is summed again without the ids left out: subtracting their own terms would cancel
+// when they carry most of the sub-block's mass.  C = the row's exponent shift.
+template <class ROW, class OUT>
+__device__ __forceinline__ void lean_ck_drop(const Geo &g, const ROW &row, float k, float C, int CK, OUT out, int y, LeanCkShared &sh) {
+    const int lane = threadIdx.x & 31, w = g.warp_of_vec(y >> 3);
+    const int slot = w * kLeanCk + ((y >> 3) - g.seg_lo(w)) / (32 * CK);
+    const CkBlock b = ck_block(g, CK, slot);
+    const int v0 = b.b0 + lane * b.Bv;
+    const float s = warp_sum(ck_lane_sum(row, k, C, v0, min(b.b1, v0 + b.Bv), out));
+    if (lane == 0) { sh.cks[slot] = s; sh.ckc[slot] = C; }
+    __syncwarp();
+}
+
+// Inverse-CDF draw from softmax(row) over the checkpoint sub-blocks, the ids left out having no weight (their
+// sub-blocks' sums say so already).  C = the row's exponent shift.  Returns the token, -1 if nothing has mass.  Called
+// by one warp, after the checkpoints are visible.
+template <class ROW, class OUT>
+__device__ __forceinline__ int lean_ck_draw(const Geo &g, const ROW &row, float k, float C, int CK, OUT out, float u, const LeanCkShared &sh) {
     const int lane = threadIdx.x & 31;
     const int nslot = g.nwarps * kLeanCk, per = (nslot + 31) >> 5;   // (consecutive sub-blocks per lane)
-    // every warp picks the sub-block by itself
     auto slot_mass = [&](int s) {
         const float cs = s < nslot ? sh.cks[s] : 0.f;
         return cs > 0.f ? cs * ex2(sh.ckc[s] - C) : 0.f;
@@ -713,35 +738,61 @@ __device__ int lean_ck_draw(const Geo &g, const ROW &row, float k, float C, int 
     const float total = __shfl_sync(kFull, lanes_prefix(ls), 31);
     if (!(total > 0.f)) return -1;
     float t = u * total;
-    const int L = lanes_pick(ls, t);
-    int slot = -1, last = -1;
-    float acc = 0.f, tt = 0.f, lastacc = 0.f;
-    for (int i = 0; i < per; ++i) {
-        const int s = L * per + i;
-        const float m = slot_mass(s);
-        if (m > 0.f) {
-            last = s;
-            lastacc = acc;
-            if (slot < 0 && acc + m > t) { slot = s; tt = t - acc; }
+    int slot = lanes_pick(ls, t);
+    if (per > 1) {   // the sub-block within the lane's
+        const int first = slot * per;
+        int last = -1;
+        slot = -1;
+        float acc = 0.f, tt = 0.f, lastacc = 0.f;
+        for (int i = 0; i < per; ++i) {
+            const float m = slot_mass(first + i);
+            if (m > 0.f) {
+                last = first + i;
+                lastacc = acc;
+                if (slot < 0 && acc + m > t) { slot = first + i; tt = t - acc; }
+            }
+            acc += m;
         }
-        acc += m;
+        if (slot < 0) { slot = last; tt = t - lastacc; }
+        t = tt;
     }
-    if (slot < 0) { slot = last; tt = t - lastacc; }
-    const int w = slot / kLeanCk, j = slot % kLeanCk;
-    const int b0 = g.seg_lo(w) + 32 * CK * j, b1 = min(g.seg_hi(w), b0 + 32 * CK);
-    return range_sample3(b0, b1, [&](int vi, float(&wt)[8]) {
-        const auto v = row[vi];
+    const CkBlock b = ck_block(g, CK, slot);
+    const int v0 = b.b0 + lane * b.Bv;
+    const int L = lanes_pick(ck_lane_sum(row, k, C, v0, min(b.b1, v0 + b.Bv), out), t);
+    if (L < 0) return -1;
+    // the picked lane's vectors over the lanes
+    const int c0 = b.b0 + L * b.Bv, c1 = min(b.b1, c0 + b.Bv);
+    float prefix = 0.f;
+    int lastpos = -1;
+    for (int vb = c0; vb < c1; vb += 32) {
+        const int vi = vb + lane;
+        float w[8], lsum = 0.f;
+        auto v = row[min(vi, c1 - 1)];
+        out.apply(vi, v);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) wt[i] = left_out(vi * 8 + i) ? 0.f : ex2(__fmaf_rn(v.get(i), k, -C));
-    }, sh, tt);
-}
-
-// ... without token `excl` (excl < 0: nothing left out; later draws leave it out too)
-template <class ROW>
-__device__ int lean_ck_sample(const Geo &g, const ROW &row, float k, float C, int CK, int excl, float u, LeanCkShared &sh) {
-    auto left_out = [&](int y) { return y == excl; };
-    if (excl >= 0) lean_ck_drop(g, row, k, C, CK, left_out, excl, sh);
-    return lean_ck_draw(g, row, k, C, CK, left_out, u, sh);
+        for (int i = 0; i < 8; ++i) {
+            w[i] = vi < c1 ? ex2(__fmaf_rn(v.get(i), k, -C)) : 0.f;
+            lsum += w[i];
+        }
+        const float incl = lanes_prefix(lsum);
+        const unsigned pos = __ballot_sync(kFull, lsum > 0.f), hit = __ballot_sync(kFull, lsum > 0.f && prefix + incl > t);
+        if (!pos) continue;
+        const int M = hit ? __ffs(hit) - 1 : 31 - __clz(pos);
+        float acc = prefix + (incl - lsum);
+        int cand = -1, lastin = -1;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            acc += w[i];
+            if (w[i] > 0.f) {
+                lastin = vi * 8 + i;
+                if (cand < 0 && acc > t) cand = lastin;
+            }
+        }
+        lastpos = __shfl_sync(kFull, cand < 0 ? lastin : cand, M);
+        if (hit) return lastpos;
+        prefix += __shfl_sync(kFull, incl, 31);
+    }
+    return lastpos;
 }
 
 // Leaf rows (Figure 2: after the last accepted draft the bonus token is a draw from p) of a call
@@ -770,10 +821,11 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_leaf_
     ArgMaxSum Ps, unusedq;
     lean_reduce2<false>(tp, unused, vp, vp, lo, hi, k, sh, Ps, unusedq);
     const float Zp = Ps.sx + Ps.own(k);
+    if (warp != 0) return;
     uint32_t status = 0;
     int tok = -1;
     if (!(Ps.ml > neg_inf()) || !(Ps.ml < -neg_inf()) || !finite_pos(Zp)) status = SPECHUB_ST_NONFINITE;
-    else tok = lean_ck_sample(g, vp, k, Ps.c, CK, -1, ures, sh);
+    else tok = lean_ck_draw(g, vp, k, Ps.c, CK, NoneOut{}, ures, sh);
     if (threadIdx.x == 0) {
         for (int m = 0; m < A.n_out; ++m) {
             const NodeOutPtrs &o = A.out[m];
@@ -1438,6 +1490,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
         lean_reduce2<false>(tq, unused, vq, vq, lo, hi, k, sh, q, unusedq);
         Q.set(q, k);
     }
+    if (warp != 0) return;
     const float Zq = Q.sx + Q.own;
     uint32_t st = 0;
     int x1 = -1, x2 = -1, hubtok = -1;
@@ -1446,7 +1499,8 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
         st = SPECHUB_ST_NONFINITE;
     } else {
         hubtok = Q.idx;
-        x1 = lean_ck_sample(g, vq, k, Q.C, CK, -1, u1, sh);
+        x1 = lean_ck_draw(g, vq, k, Q.C, CK, NoneOut{}, u1, sh);
+        if (x1 < 0) x1 = hubtok;   // (a sub-block of exponentials below the smallest normal number)
         if (method == kSpecHub) {
             prob0 = Q.own / Zq;
             if (x1 != hubtok) {
@@ -1455,17 +1509,18 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
             } else if (!(Q.sx > 0.f)) {
                 x2 = (hubtok == 0) ? 1 : 0;
                 st |= SPECHUB_ST_DEGENERATE_Q;
-            } else {
-                x2 = lean_ck_sample(g, vq, k, Q.C, CK, hubtok, u2, sh);
-                prob1 = prob0 * ex2(fmaf(vq.one(x2), k, -Q.C)) / Q.sx;
             }
         } else if (method == kRRS) {
-            x2 = lean_ck_sample(g, vq, k, Q.C, CK, -1, u2, sh);
-        } else {
-            x2 = lean_ck_sample(g, vq, k, Q.C, CK, x1, u2, sh);
+            x2 = lean_ck_draw(g, vq, k, Q.C, CK, NoneOut{}, u2, sh);
+        }
+        if (x2 < 0 && method != kRRS) {   // q without x1 (SpecHub: x1 is the hub)
+            lean_ck_drop(g, vq, k, Q.C, CK, OneOut{x1}, x1, sh);
+            x2 = lean_ck_draw(g, vq, k, Q.C, CK, OneOut{x1}, u2, sh);
             if (x2 < 0) {   // nothing left once x1 is removed
                 x2 = (x1 == 0) ? 1 : 0;
                 st |= SPECHUB_ST_DEGENERATE_Q;
+            } else if (method == kSpecHub) {
+                prob1 = prob0 * ex2(fmaf(vq.one(x2), k, -Q.C)) / Q.sx;
             }
         }
     }

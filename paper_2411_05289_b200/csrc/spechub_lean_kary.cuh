@@ -56,31 +56,29 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_kary_draft_kerne
     lean_reduce2<false>(tq, unused, vq, vq, lo, hi, k, sh, Q, unusedq);
     const float Zq = Q.sx + Q.own(k);
     uint32_t st = 0;
+    if (warp != 0) return;
     const bool bad = !(Q.ml > neg_inf()) || !finite_pos(Zq) || !(Q.ml < -neg_inf());
     if (bad) st = SPECHUB_ST_NONFINITE;
     for (int i = 0; i < K; ++i) {
         int t = -1;
         if (!bad) {
             const int out = A.without_replacement ? i : 0;   // x[0..out) are left out
-            t = lean_ck_draw(g, vq, k, Q.c, CK, [&](int y) { return one_of(sh.x, out, y); }, un[i], sh);
+            t = lean_ck_draw(g, vq, k, Q.c, CK, ListOut{sh.x, out}, un[i], sh);
             if (t < 0) {   // nothing left to draw from: lowest id not drawn yet
                 st |= SPECHUB_ST_DEGENERATE_Q;
-                __syncthreads();
                 for (t = 0; t < a.vocab && one_of(sh.x, i, t); ++t) {}
                 if (t >= a.vocab) t = 0;
             }
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
+        if (lane == 0) {
             sh.x[i] = t;
             a.draft_tokens_out[K * r + i] = t;
         }
-        if (!bad && A.without_replacement && i + 1 < K) {
-            __syncthreads();
-            lean_ck_drop(g, vq, k, Q.c, CK, [&](int y) { return one_of(sh.x, i + 1, y); }, t, sh);
-        }
+        __syncwarp();
+        if (!bad && A.without_replacement && i + 1 < K)
+            lean_ck_drop(g, vq, k, Q.c, CK, ListOut{sh.x, i + 1}, t, sh);
     }
-    if (threadIdx.x == 0) {
+    if (lane == 0) {
         void_draft_stat(a, r);
         if (a.status) a.status[r] = st;
     }
