@@ -7,19 +7,17 @@ namespace spechub {
 
 int launch_fused_draft(const FusedArgs &f, int32_t *hub, float *draft_prob, unsigned rows, cudaStream_t s) {
     const int th = draft_threads(f.r.vocab, rows);
-    if (th == 512) fused_draft_kernel<512><<<rows, 512, 0, s>>>(f, hub, draft_prob);
-    else if (th == 256) fused_draft_kernel<256><<<rows, 256, 0, s>>>(f, hub, draft_prob);
-    else fused_draft_kernel<128><<<rows, 128, 0, s>>>(f, hub, draft_prob);
-    return launch_status();
+    if (th == 512) return launch_grid(fused_draft_kernel<512>, rows, 512, 0, 1, s, f, hub, draft_prob);
+    if (th == 256) return launch_grid(fused_draft_kernel<256>, rows, 256, 0, 1, s, f, hub, draft_prob);
+    return launch_grid(fused_draft_kernel<128>, rows, 128, 0, 1, s, f, hub, draft_prob);
 }
 
 int launch_fused_verify(const FusedArgs &f, unsigned rows, cudaStream_t s) {
-    const int th = verify_threads(f.r.vocab, rows);
-    if (!f.r.draft_stats_in) fused_verify_kernel<kLeanThreads><<<rows, kLeanThreads, 0, s>>>(f);
-    else if (th == 512) fused_verify_kernel<512, true><<<rows, 512, 0, s>>>(f);
-    else if (th == 256) fused_verify_kernel<256, true><<<rows, 256, 0, s>>>(f);
-    else fused_verify_kernel<128, true><<<rows, 128, 0, s>>>(f);
-    return launch_status();
+    if (!f.r.draft_stats_in) return launch_grid(fused_verify_kernel<kLeanThreads>, rows, kLeanThreads, 0, 1, s, f);
+    const int th = verify_threads(f.r.vocab, rows, 1024);
+    if (th == 512) return launch_grid(fused_verify_kernel<512, true>, rows, 512, 0, 1, s, f);
+    if (th == 256) return launch_grid(fused_verify_kernel<256, true>, rows, 256, 0, 1, s, f);
+    return launch_grid(fused_verify_kernel<128, true>, rows, 128, 0, 1, s, f);
 }
 
 }  // namespace spechub

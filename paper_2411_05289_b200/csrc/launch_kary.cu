@@ -9,19 +9,17 @@ namespace spechub {
 template <typename LT, bool SHIFT>
 static int kary_draft(const KaryArgs &a, unsigned rows, cudaStream_t s) {
     const int th = draft_threads(a.r.vocab, rows);
-    if (th == 512) lean_kary_draft_kernel<LT, SHIFT, 512><<<rows, 512, 0, s>>>(a);
-    else if (th == 256) lean_kary_draft_kernel<LT, SHIFT, 256><<<rows, 256, 0, s>>>(a);
-    else if (th == 128) lean_kary_draft_kernel<LT, SHIFT, 128><<<rows, 128, 0, s>>>(a);
-    else lean_kary_draft_kernel<LT, SHIFT, 64><<<rows, 64, 0, s>>>(a);
-    return launch_status();
+    if (th == 512) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 512>, rows, 512, 0, 1, s, a);
+    if (th == 256) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 256>, rows, 256, 0, 1, s, a);
+    if (th == 128) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 128>, rows, 128, 0, 1, s, a);
+    return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 64>, rows, 64, 0, 1, s, a);
 }
 template <typename LT, bool SHIFT>
 static int kary_verify(const KaryArgs &a, unsigned rows, cudaStream_t s) {
-    const int th = verify_threads(a.r.vocab, rows);
-    if (th == 512) lean_kary_verify_kernel<LT, SHIFT, 512><<<rows, 512, 0, s>>>(a);
-    else if (th == 256) lean_kary_verify_kernel<LT, SHIFT, 256><<<rows, 256, 0, s>>>(a);
-    else lean_kary_verify_kernel<LT, SHIFT, 128><<<rows, 128, 0, s>>>(a);
-    return launch_status();
+    const int th = verify_threads(a.r.vocab, rows, SHIFT ? 768 : 1024);
+    if (th == 512) return launch_grid(lean_kary_verify_kernel<LT, SHIFT, 512>, rows, 512, 0, 1, s, a);
+    if (th == 256) return launch_grid(lean_kary_verify_kernel<LT, SHIFT, 256>, rows, 256, 0, 1, s, a);
+    return launch_grid(lean_kary_verify_kernel<LT, SHIFT, 128>, rows, 128, 0, 1, s, a);
 }
 
 int launch_kary_draft(int format, const KaryArgs &a, unsigned rows, cudaStream_t s) {
@@ -44,10 +42,8 @@ int launch_kary_verify(int format, const KaryArgs &a, unsigned rows, cudaStream_
 }
 
 int launch_walk(const WalkKArgs &wk, cudaStream_t s) {
-    const int blocks = (wk.w.batch + 127) / 128;
-    if (wk.k > 2) walk_k_kernel<<<blocks, 128, 0, s>>>(wk);
-    else walk_kernel<<<blocks, 128, 0, s>>>(wk.w);
-    return launch_status();
+    const int warp_per_seq = wk.w.nodes <= kWalkNodes, per = warp_per_seq ? kWalkThreads / 32 : kWalkThreads;
+    return launch_grid(walk_kernel, (wk.w.batch + per - 1) / per, kWalkThreads, 0, 1, s, wk, warp_per_seq);
 }
 
 }  // namespace spechub

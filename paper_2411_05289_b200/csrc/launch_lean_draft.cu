@@ -7,23 +7,16 @@ namespace spechub {
 
 template <int CS>
 static int draft_group(const RowArgs &a, int method, unsigned rows, cudaStream_t s) {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at; cfg.numAttrs = 1;
-    cfg.gridDim = dim3(rows * CS); cfg.blockDim = dim3(kLeanThreads); cfg.stream = s;
-    return cudaLaunchKernelEx(&cfg, lean_draft_kernel<kLeanThreads, CS>, a, method) == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH;
+    return launch_grid(lean_draft_kernel<kLeanThreads, CS>, rows * CS, kLeanThreads, 0, CS, s, a, method);
 }
 
 template <typename LT, bool SHIFT>
 static int draft_rows(const RowArgs &a, int method, bool keep_stats, unsigned rows, cudaStream_t s) {
     const int th = draft_threads(a.vocab, rows);
-    if (th == 512) lean_draft_ck_kernel<LT, SHIFT, 512><<<rows, 512, 0, s>>>(a, method, keep_stats);
-    else if (th == 256) lean_draft_ck_kernel<LT, SHIFT, 256><<<rows, 256, 0, s>>>(a, method, keep_stats);
-    else if (th == 128) lean_draft_ck_kernel<LT, SHIFT, 128><<<rows, 128, 0, s>>>(a, method, keep_stats);
-    else lean_draft_ck_kernel<LT, SHIFT, 64><<<rows, 64, 0, s>>>(a, method, keep_stats);
-    return launch_status();
+    if (th == 512) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 512>, rows, 512, 0, 1, s, a, method, keep_stats);
+    if (th == 256) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 256>, rows, 256, 0, 1, s, a, method, keep_stats);
+    if (th == 128) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 128>, rows, 128, 0, 1, s, a, method, keep_stats);
+    return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 64>, rows, 64, 0, 1, s, a, method, keep_stats);
 }
 
 int launch_lean_draft(int format, int method, int cs, const RowArgs &a, bool keep_stats, unsigned rows, cudaStream_t s) {
@@ -38,11 +31,10 @@ int launch_lean_draft(int format, int method, int cs, const RowArgs &a, bool kee
 template <typename LT, bool SHIFT>
 static int leaf_rows(const LeafArgs &la, unsigned rows, cudaStream_t s) {
     const int th = draft_threads(la.r.vocab, rows);
-    if (th == 512) lean_leaf_kernel<LT, SHIFT, 512><<<rows, 512, 0, s>>>(la);
-    else if (th == 256) lean_leaf_kernel<LT, SHIFT, 256><<<rows, 256, 0, s>>>(la);
-    else if (th == 128) lean_leaf_kernel<LT, SHIFT, 128><<<rows, 128, 0, s>>>(la);
-    else lean_leaf_kernel<LT, SHIFT, 64><<<rows, 64, 0, s>>>(la);
-    return launch_status();
+    if (th == 512) return launch_grid(lean_leaf_kernel<LT, SHIFT, 512>, rows, 512, 0, 1, s, la);
+    if (th == 256) return launch_grid(lean_leaf_kernel<LT, SHIFT, 256>, rows, 256, 0, 1, s, la);
+    if (th == 128) return launch_grid(lean_leaf_kernel<LT, SHIFT, 128>, rows, 128, 0, 1, s, la);
+    return launch_grid(lean_leaf_kernel<LT, SHIFT, 64>, rows, 64, 0, 1, s, la);
 }
 
 // The leaf rows of an unsplit call (same CTA shape as the draft step).

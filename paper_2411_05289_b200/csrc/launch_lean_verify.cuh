@@ -9,14 +9,7 @@ namespace spechub {
 
 template <int METHOD, int CS>
 int verify_split(const RowArgs &a, unsigned rows, cudaStream_t s) {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at; cfg.numAttrs = CS > 1 ? 1 : 0;
-    cfg.gridDim = dim3(rows * CS); cfg.blockDim = dim3(kLeanThreads); cfg.stream = s;
-    return cudaLaunchKernelEx(&cfg, lean_verify_kernel<__nv_bfloat16, false, METHOD, kLeanThreads, CS>, a) == cudaSuccess
-               ? SPECHUB_OK : SPECHUB_ERR_LAUNCH;
+    return launch_grid(lean_verify_kernel<__nv_bfloat16, false, METHOD, kLeanThreads, CS>, rows * CS, kLeanThreads, 0, CS, s, a);
 }
 
 // One CTA per row, the passes fed by per-warp rings of bulk copies (spechub_ring.cuh).
@@ -27,28 +20,27 @@ int verify_ring(const RowArgs &a, unsigned rows, cudaStream_t s) {
     static bool configured[kMaxDevices] = {};
     const int rc = allow_smem(reinterpret_cast<const void *>(kern), smem, configured);
     if (rc != SPECHUB_OK) return rc;
-    kern<<<rows, kLeanThreads, smem, s>>>(a);
-    return launch_status();
+    return launch_grid(kern, rows, kLeanThreads, smem, 1, s, a);
 }
 
 // One CTA per row.  STATS: the draft row's statistics come from the draft step.
 template <typename LT, bool SHIFT, int METHOD, bool STATS>
 int verify_rows(const RowArgs &a, unsigned rows, cudaStream_t s) {
-    const int th = verify_threads(a.vocab, rows);
-    if (th == 512) lean_verify_kernel<LT, SHIFT, METHOD, 512, 1, false, STATS><<<rows, 512, 0, s>>>(a);
-    else if (th == 256) lean_verify_kernel<LT, SHIFT, METHOD, 256, 1, false, STATS><<<rows, 256, 0, s>>>(a);
-    else lean_verify_kernel<LT, SHIFT, METHOD, 128, 1, false, STATS><<<rows, 128, 0, s>>>(a);
-    return launch_status();
+    const int th = verify_threads(a.vocab, rows, SHIFT ? 768 : 1024);
+    if (th == 512) return launch_grid(lean_verify_kernel<LT, SHIFT, METHOD, 512, 1, false, STATS>, rows, 512, 0, 1, s, a);
+    if (th == 256) return launch_grid(lean_verify_kernel<LT, SHIFT, METHOD, 256, 1, false, STATS>, rows, 256, 0, 1, s, a);
+    return launch_grid(lean_verify_kernel<LT, SHIFT, METHOD, 128, 1, false, STATS>, rows, 128, 0, 1, s, a);
 }
 
 template <int METHOD>
-int launch_lean_verify_method(int format, int cs, const RowArgs &a, unsigned rows, cudaStream_t s) {
+int launch_lean_verify_method(int format, int cs, RowArgs a, unsigned rows, cudaStream_t s) {
     if (cs == 4) return verify_split<METHOD, 4>(a, rows, s);
     if (cs == 2) return verify_split<METHOD, 2>(a, rows, s);
     if (a.node_kind) {
         const NodeOutPtrs o = {a.accept_idx, a.token, a.hub, a.beta, a.rate, a.status};
         const int lrc = launch_lean_leaf(format, a, 2, &o, 1, rows, s);
         if (lrc != SPECHUB_OK) return lrc;
+        a.after_leaves = 1;
     }
     const bool stats = cs == 0 && a.draft_stats_in;
     if (format == kBf16Shift) return verify_rows<__nv_bfloat16, true, METHOD, false>(a, rows, s);

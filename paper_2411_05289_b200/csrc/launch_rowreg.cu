@@ -34,16 +34,9 @@ bool reg_plan(int dtype, int vocab, long long rows, RegPlan *out) {
 
 template <class K, class... Args>
 static int launch(const RegPlan &pl, K kern, unsigned rows, cudaStream_t s, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = pl.cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at; cfg.numAttrs = pl.cs > 1 ? 1 : 0;
-    cfg.gridDim = dim3(pl.cs > 1 ? rows * pl.cs : (rows + pl.rows_per_cta - 1) / pl.rows_per_cta);
-    cfg.blockDim = dim3(pl.w * pl.rows_per_cta * 32);
-    cfg.stream = s;
     const RegGeo geo = {pl.w, pl.cs, pl.rows_per_cta, pl.seg};
-    return cudaLaunchKernelEx(&cfg, kern, args..., rows, geo) == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH;
+    return launch_grid(kern, pl.cs > 1 ? rows * pl.cs : (rows + pl.rows_per_cta - 1) / pl.rows_per_cta,
+                       pl.w * pl.rows_per_cta * 32, 0, pl.cs, s, args..., rows, geo);
 }
 
 template <typename LT, int NV>

@@ -30,6 +30,7 @@ __device__ __forceinline__ void write_node3(const NodeOutPtrs &p, long long r, c
 template <int THREADS, bool STATS = false>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(FusedArgs A) {
     __shared__ LeanShared sh;
+    pdl_begin();
     const RowArgs &a = A.r;
     const long long r = blockIdx.x;
     const int b = static_cast<int>(r / a.nodes), n = static_cast<int>(r % a.nodes);
@@ -325,6 +326,7 @@ template <int THREADS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(FusedArgs A, int32_t *hub_out,
                                                                             float *draft_prob) {
     __shared__ LeanCkShared sh;
+    pdl_begin();
     const RowArgs &a = A.r;
     const long long r = blockIdx.x;
     const int b = static_cast<int>(r / a.nodes), n = static_cast<int>(r % a.nodes);
@@ -336,11 +338,11 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
     const float k = kLog2e / temperature_of(a, b);
     const float u1 = a.uniforms[r * 5 + 0], u2 = a.uniforms[r * 5 + 1];
     const bool t0 = threadIdx.x == 0;
-    const int CK = lean_ck_interval(g);
+    const int CK = lean_ck_interval(g), CS = lean_ck_slots(g, CK);
 
     LeanAcc<__nv_bfloat16> tq, unused;
     unused.init();
-    lean_pass_a_ck<false>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * kLeanCk, sh.ckc + warp * kLeanCk);
+    lean_pass_a_ck<false>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * CS, sh.ckc + warp * CS, CS);
     RowStat Q;
     {
         ArgMaxSum q, unusedq;

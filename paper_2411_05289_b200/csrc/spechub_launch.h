@@ -12,6 +12,21 @@ constexpr int kMaxDevices = 64;
 
 inline int launch_status() { return cudaGetLastError() == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH; }
 
+// One launch: `cs` CTAs per cluster (1: none), as a programmatic dependent of the stream's last kernel.  Only for
+// kernels that begin with pdl_begin() (or keep its promise otherwise).
+template <class K, class... Args>
+int launch_grid(K kern, unsigned grid, int threads, int smem, int cs, cudaStream_t s, const Args &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = cs; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = cs > 1 ? 2 : 1;
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    return cudaLaunchKernelEx(&cfg, kern, args...) == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH;
+}
+
 // Raise a kernel's dynamic shared memory limit once per device.  `configured`: one flag per device, kept by
 // the caller (one array per kernel).
 int allow_smem(const void *kern, int bytes, bool *configured);

@@ -38,7 +38,7 @@ namespace spechub {
 namespace cg = cooperative_groups;
 
 constexpr int kLeanMaxWarps = 32;
-constexpr int kLeanCk = 8;        // checkpoints per warp in the draft step's pass A
+constexpr int kLeanCk = 16;       // checkpoints per warp in the draft step's pass A, at most
 constexpr float kHuge = 1.0e30f;  // ~2^100: partial sums beyond this move the reference
 
 struct LeanShared {
@@ -604,10 +604,13 @@ __device__ __forceinline__ int lean_ck_interval(const Geo &g) {
     const int iters = (g.seg + 31) >> 5;
     return 4 * max(1, (iters + 4 * kLeanCk - 1) / (4 * kLeanCk));   // a multiple of the unroll of pass A
 }
+__device__ __forceinline__ int lean_ck_slots(const Geo &g, int CK) {   // sub-blocks per warp
+    return (((g.seg + 31) >> 5) + CK - 1) / CK;
+}
 
 template <bool SHIFT, typename LT, class ROW>
 __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, int lane, float k, int CK,
-                                               LeanAcc<LT> &Q, float *cks, float *ckc) {
+                                               LeanAcc<LT> &Q, float *cks, float *ckc, int slots) {
     LeanAcc<LT> st;
     st.init();
     {   // one exponent reference for the whole warp: the maximum of its first vectors
@@ -666,7 +669,7 @@ __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, in
     slow(iters);
     if (since > 0) checkpoint();
     if (lane == 0)
-        for (; j < kLeanCk; ++j) { cks[j] = 0.f; ckc[j] = 0.f; }
+        for (; j < slots; ++j) { cks[j] = 0.f; ckc[j] = 0.f; }
     Q.m2 = st.m2; Q.c = st.c; Q.s = tot;
 }
 
@@ -701,7 +704,7 @@ __device__ __forceinline__ float ck_lane_sum(const ROW &row, float k, float C, i
 }
 struct CkBlock { int b0, b1, Bv; };
 __device__ __forceinline__ CkBlock ck_block(const Geo &g, int CK, int slot) {
-    const int w = slot / kLeanCk, j = slot % kLeanCk;
+    const int slots = lean_ck_slots(g, CK), w = slot / slots, j = slot - w * slots;
     CkBlock o;
     o.b0 = g.seg_lo(w) + 32 * CK * j;
     o.b1 = min(g.seg_hi(w), o.b0 + 32 * CK);
@@ -714,7 +717,7 @@ __device__ __forceinline__ CkBlock ck_block(const Geo &g, int CK, int slot) {
 template <class ROW, class OUT>
 __device__ __forceinline__ void lean_ck_drop(const Geo &g, const ROW &row, float k, float C, int CK, OUT out, int y, LeanCkShared &sh) {
     const int lane = threadIdx.x & 31, w = g.warp_of_vec(y >> 3);
-    const int slot = w * kLeanCk + ((y >> 3) - g.seg_lo(w)) / (32 * CK);
+    const int slot = w * lean_ck_slots(g, CK) + ((y >> 3) - g.seg_lo(w)) / (32 * CK);
     const CkBlock b = ck_block(g, CK, slot);
     const int v0 = b.b0 + lane * b.Bv;
     const float s = warp_sum(ck_lane_sum(row, k, C, v0, min(b.b1, v0 + b.Bv), out));
@@ -728,7 +731,7 @@ __device__ __forceinline__ void lean_ck_drop(const Geo &g, const ROW &row, float
 template <class ROW, class OUT>
 __device__ __forceinline__ int lean_ck_draw(const Geo &g, const ROW &row, float k, float C, int CK, OUT out, float u, const LeanCkShared &sh) {
     const int lane = threadIdx.x & 31;
-    const int nslot = g.nwarps * kLeanCk, per = (nslot + 31) >> 5;   // (consecutive sub-blocks per lane)
+    const int nslot = g.nwarps * lean_ck_slots(g, CK), per = (nslot + 31) >> 5;   // (consecutive sub-blocks per lane)
     auto slot_mass = [&](int s) {
         const float cs = s < nslot ? sh.cks[s] : 0.f;
         return cs > 0.f ? cs * ex2(sh.ckc[s] - C) : 0.f;
@@ -803,6 +806,7 @@ __device__ __forceinline__ int lean_ck_draw(const Geo &g, const ROW &row, float 
 template <typename LT, bool SHIFT, int THREADS>
 __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_leaf_kernel(LeafArgs A) {
     __shared__ LeanCkShared sh;
+    pdl_begin();
     const RowArgs &a = A.r;
     const long long r = blockIdx.x;
     const int b = static_cast<int>(r / a.nodes), n = static_cast<int>(r % a.nodes);
@@ -814,10 +818,10 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_leaf_
     const float k = kLog2e / temperature_of(a, b);
     const int K = A.k;
     const float ures = a.uniforms[r * (2 * K + 1) + 2 * K];
-    const int CK = lean_ck_interval(g);
+    const int CK = lean_ck_interval(g), CS = lean_ck_slots(g, CK);
     LeanAcc<LT> tp, unused;
     unused.init();
-    lean_pass_a_ck<SHIFT>(vp, lo, hi, lane, k, CK, tp, sh.cks + warp * kLeanCk, sh.ckc + warp * kLeanCk);
+    lean_pass_a_ck<SHIFT>(vp, lo, hi, lane, k, CK, tp, sh.cks + warp * CS, sh.ckc + warp * CS, CS);
     ArgMaxSum Ps, unusedq;
     lean_reduce2<false>(tp, unused, vp, vp, lo, hi, k, sh, Ps, unusedq);
     const float Zp = Ps.sx + Ps.own(k);
@@ -883,6 +887,10 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
     __shared__ LeanShared sh;
     extern __shared__ __align__(128) unsigned char ring_mem[];
     __shared__ __align__(8) uint64_t ring_bars[RING ? THREADS / 32 : 1][kRingStages];
+    // After the leaf kernel of the same call, whose rows are others, this one need not wait: the leaf kernel let it be
+    // launched when it had waited itself.  One CTA waits at its end, so that this grid ends after the leaf kernel's.
+    if (!a.after_leaves) pdl_wait();
+    pdl_trigger();
     const int me = RowGroup<CS>::rank();
     const long long r = blockIdx.x / CS;
     const int b = static_cast<int>(r / a.nodes), n = static_cast<int>(r % a.nodes);
@@ -898,7 +906,10 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
     const float k = kLog2e / temperature_of(a, b);
     const float pinf = -neg_inf();
     // leaf rows of an unsplit call belong to lean_leaf_kernel
-    if (CS == 1 && a.node_kind && a.node_kind[n] == SPECHUB_NODE_LEAF) return;
+    if (CS == 1 && a.node_kind && a.node_kind[n] == SPECHUB_NODE_LEAF) {
+        if (a.after_leaves && blockIdx.x == 0) pdl_wait();
+        return;
+    }
     const bool leaf = CS > 1 && a.node_kind && a.node_kind[n] == SPECHUB_NODE_LEAF;
     const bool writer = (me == 0 && threadIdx.x == 0);
 
@@ -913,9 +924,13 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
     // by the last warp before it starts on pass A: two dependent look-ups that are off the path between the passes.
     // (Nothing else writes these fields; they are read after barriers.)
     if (warp == THREADS / 32 - 1) {
-        const int t1 = a.draft_tokens_in[2 * r], t2 = a.draft_tokens_in[2 * r + 1];
+        // (from L2: with the leaf kernel between them the draft step's kernel is not the one waited for)
+        const int t1 = __ldcg(a.draft_tokens_in + 2 * r), t2 = __ldcg(a.draft_tokens_in + 2 * r + 1);
         DraftStat ds = {};
-        if (STATS) ds = static_cast<const DraftStat *>(a.draft_stats_in)[r];
+        if (STATS) {
+            const int4 rec = __ldcg(static_cast<const int4 *>(a.draft_stats_in) + r);
+            ds.ml = __int_as_float(rec.x); ds.sx = __int_as_float(rec.y); ds.idx = rec.z; ds.tag = static_cast<unsigned>(rec.w);
+        }
         int y = lane > 4 ? -1 : lane == 4 ? (STATS ? ds.idx : -1) : (lane & 1) ? t2 : t1;
         if (leaf) y = -1;
         float l = neg_inf();
@@ -1344,6 +1359,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
         if (a.status) a.status[r] = o.status;
     }
     if (CS > 1) RowGroup<CS>::sync();  // no CTA leaves while another may still read its shared memory
+    if (a.after_leaves && blockIdx.x == 0) pdl_wait();
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1352,6 +1368,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
 template <int THREADS, int CS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_kernel(RowArgs a, int method) {
     __shared__ LeanShared sh;
+    pdl_begin();
     const int me = RowGroup<CS>::rank();
     const long long r = blockIdx.x / CS;
     const int b = static_cast<int>(r / a.nodes), n = static_cast<int>(r % a.nodes);
@@ -1471,6 +1488,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_kernel(Row
 template <typename LT, bool SHIFT, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(RowArgs a, int method, bool keep_stats) {
     __shared__ LeanCkShared sh;
+    pdl_begin();
     const long long r = blockIdx.x;
     const int b = static_cast<int>(r / a.nodes), n = static_cast<int>(r % a.nodes);
     const StreamRow<LT, SHIFT> vq(static_cast<const LT *>(a.draft) + b * a.stride_seq + n * a.stride_node, a.vocab);
@@ -1479,11 +1497,11 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
     const int lo = g.seg_lo(warp), hi = g.seg_hi(warp);
     const float k = kLog2e / temperature_of(a, b);
     const float u1 = a.uniforms[r * 5 + 0], u2 = a.uniforms[r * 5 + 1];
-    const int CK = lean_ck_interval(g);
+    const int CK = lean_ck_interval(g), CS = lean_ck_slots(g, CK);
 
     LeanAcc<LT> tq, unused;
     unused.init();
-    lean_pass_a_ck<SHIFT>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * kLeanCk, sh.ckc + warp * kLeanCk);
+    lean_pass_a_ck<SHIFT>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * CS, sh.ckc + warp * CS, CS);
     RowStat Q;
     {
         ArgMaxSum q, unusedq;

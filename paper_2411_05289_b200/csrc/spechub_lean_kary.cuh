@@ -37,6 +37,7 @@ __device__ __forceinline__ bool one_of(const int *x, int n, int y) {
 template <typename LT, bool SHIFT, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_kary_draft_kernel(KaryArgs A) {
     __shared__ LeanKaryShared sh;
+    pdl_begin();
     const RowArgs &a = A.r;
     const int K = A.k;
     const long long r = blockIdx.x;
@@ -47,11 +48,11 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_kary_draft_kerne
     const int lo = g.seg_lo(warp), hi = g.seg_hi(warp);
     const float k = kLog2e / temperature_of(a, b);
     const float *un = a.uniforms + r * (2 * K + 1);
-    const int CK = lean_ck_interval(g);
+    const int CK = lean_ck_interval(g), CS = lean_ck_slots(g, CK);
 
     LeanAcc<LT> tq, unused;
     unused.init();
-    lean_pass_a_ck<SHIFT>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * kLeanCk, sh.ckc + warp * kLeanCk);
+    lean_pass_a_ck<SHIFT>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * CS, sh.ckc + warp * CS, CS);
     ArgMaxSum Q, unusedq;
     lean_reduce2<false>(tq, unused, vq, vq, lo, hi, k, sh, Q, unusedq);
     const float Zq = Q.sx + Q.own(k);
@@ -99,6 +100,7 @@ __device__ __forceinline__ void stream_pairs(const StreamRow<LT, SHIFT> &p, cons
 template <typename LT, bool SHIFT, int THREADS>
 __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_kary_verify_kernel(KaryArgs A) {
     __shared__ LeanKaryShared sh;
+    pdl_begin();
     using V = Vec8<LT>;
     const RowArgs &a = A.r;
     const int K = A.k;

@@ -393,6 +393,7 @@ __device__ __forceinline__ void clean_masses(PerPart &mass) {
 template <typename LT, int NV, int KK>
 __global__ void __launch_bounds__(kRegThreads) reg_draft_kernel(KaryArgs A, int method, unsigned rows, RegGeo geo) {
     __shared__ RegShared sh;
+    pdl_begin();
     const RowArgs &a = A.r;
     const RegRow g(geo, a.vocab);
     if (g.r >= rows) return;
@@ -549,6 +550,7 @@ __device__ __forceinline__ bool draft_stat_ok(const RowArgs &a, long long r, con
 template <typename LT, int NV>
 __global__ void __launch_bounds__(kRegThreads) reg_verify_spechub_kernel(RowArgs a, unsigned rows, RegGeo geo) {
     __shared__ RegShared sh;
+    pdl_begin();
     const RegRow g(geo, a.vocab);
     if (g.r >= rows) return;
     g.arrive_start();
@@ -689,6 +691,7 @@ template <typename LT, int NV, int KK>
 __global__ void __launch_bounds__(kRegThreads) reg_verify_rrs_kernel(KaryArgs A, unsigned rows, RegGeo geo) {
     constexpr int MK = KK ? KK : kMaxK;
     __shared__ RegShared sh;
+    pdl_begin();
     const RowArgs &a = A.r;
     const RegRow g(geo, a.vocab);
     if (g.r >= rows) return;

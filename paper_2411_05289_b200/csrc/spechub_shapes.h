@@ -18,12 +18,11 @@ constexpr int threads_for_few(unsigned rows, int many) {
 constexpr int draft_threads(int vocab, unsigned rows) {
     return vocab < 8192 ? 64 : threads_for_few(rows, 128);
 }
-// Verification: 4 CTAs of 256 threads per SM (256/512/1024: 1.54/1.65/1.87 ms).  From draft statistics and on rows of
-// any alignment shorter rows take 8 CTAs of 128 threads, which overlap the fixed work of a row (reductions, tests,
-// draws) better (V = 32000, 3840 rows: SpecHub 0.180 -> 0.158 ms, RRS 0.230 -> 0.205 ms; 64 threads: 0.171 ms; on
-// V = 128256 the 256-thread CTA stays ahead, 1.02 against 1.06 ms).
-constexpr int verify_threads(int vocab, unsigned rows) {
-    return threads_for_few(rows, vocab <= 65536 ? 128 : 256);
+// Verification: 4 CTAs of 256 threads per SM (256/512/1024: 1.54/1.65/1.87 ms on V = 128256); 128 threads on rows too
+// short to feed those (V = 8192, 1792 rows: SpecHub 28.6 -> 23.3 us, RRSw 30.7 -> 26.2 us).
+// (`per_sm`: threads of these kernels that fit an SM)
+constexpr int verify_threads(int vocab, unsigned rows, int per_sm) {
+    return rows <= unsigned(per_sm / 512 * kSms) ? 512 : rows <= unsigned(per_sm / 256 * kSms) || vocab >= 16384 ? 256 : 128;
 }
 constexpr int kLeanThreads = 256;   // split rows, and the rings of bulk copies
 
