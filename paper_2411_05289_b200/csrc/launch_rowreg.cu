@@ -14,10 +14,8 @@ bool reg_plan(int dtype, int vocab, long long rows, RegPlan *out) {
     // as many warps per row as one wave holds (16 per SM): the fewest vectors per lane that allow it
     for (p.nv = 1;; p.nv *= 2) {
         const int parts = (nvec + 32 * p.nv - 1) / (32 * p.nv);
-        if (parts > kRegMaxParts) {
-            if (p.nv == max_nv) return false;
-            continue;
-        }
+        if (parts > kRegMaxParts && p.nv == max_nv) return false;
+        if (parts > 64 && p.nv < max_nv) continue;   // (fewer records to merge)
         p.cs = 1;
         while (p.cs * 8 < parts && p.cs < 8) p.cs *= 2;   // CTAs of up to 8 warps measured as good as 4 and better than 16
         p.w = (parts + p.cs - 1) / p.cs;

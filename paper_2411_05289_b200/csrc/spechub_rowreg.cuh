@@ -1,14 +1,14 @@
-// Rows held in registers: each row is read from memory once, every lane keeps up to NV consecutive logical vectors
-// (8 ids each) of it, and all passes of a step run over those registers.
+// Rows held in registers: each row is read from memory once, every lane keeps up to NV logical vectors (8 ids each)
+// of it, and all passes of a step run over those registers.
 //
 // A row is cut into contiguous parts, one per warp: W warps of a CTA, on CS CTAs of a cluster when one CTA's
 // warps do not hold it.  Short rows take one warp or a few, several rows per CTA, and never meet a CTA-wide
-// barrier.  After each pass every warp posts a small record into the shared memory of all CTAs of its row,
-// one barrier follows (a warp barrier, a named barrier, or the cluster's), and every warp merges the records
-// for itself in the same order: all warps hold bit-identical row values, take the same decisions, and pick the
-// same part in an inverse-CDF draw.  The picked part's warp picks a lane from the lanes' own sums and spreads
-// that lane's few ids over the warp, read again from the cache: no register is indexed, and the code stays small
-// (a first pass over 5000 instructions costs more in instruction fetches than in execution).
+// barrier.  Vector j of a part's lane l is the part's (32 j + l)-th: a load is one contiguous request.  (Consecutive
+// vectors per lane would make draws simpler, but each load then touches up to 32 lines: 31 rows of 128256 ids, 8000
+// cycles for the loads alone.)  After each pass every warp posts a small record into the shared memory of all CTAs of
+// its row, one barrier follows (a warp barrier, a named barrier, or the cluster's), and every warp merges the records
+// for itself in the same order: all warps hold bit-identical row values, take the same decisions, and pick the same
+// part in an inverse-CDF draw, whose warp draws from its registers.
 //
 // What bounds these kernels is the chain load -> reduce -> barrier -> reduce -> draw, a few microseconds, not
 // bandwidth.  They take the calls whose rows do not fill the GPU: a row spread over many warps instead of one
@@ -36,13 +36,13 @@ struct RegShared {
     float2 p[kRegMaxParts];        // (max logit, sum of exponentials on that maximum's scale)
     float4 q[kRegMaxParts];        // the same, the sum without the part's argmax, the argmax
     float4 sum[2][kRegMaxParts];   // sums of a pass, two buffers
-    float2 drawn[2][4];            // draft step: a drawn id and what its part weighs without it, per row of the CTA
+    float2 drawn[kMaxK][4];        // draft step: a drawn id and what its part weighs without it, per row of the CTA
 };
 
 struct RegRow {   // this warp's place in its row
     int part, parts, slot0;    // its part, the parts of the row, the row's first record
     int lo, hi, seg;           // its vectors; vectors per part
-    int nj, lv;                // vectors per lane, this lane's first
+    int nj, lv;                // vectors per lane, this lane's first (the others follow at distances of 32)
     int w, cs, rows_per_cta, group;
     unsigned r;                // the row
 
@@ -59,11 +59,10 @@ struct RegRow {   // this warp's place in its row
         lo = min(part * seg, nvec);
         hi = min(lo + seg, nvec);
         nj = (seg + 31) >> 5;
-        lv = lo + static_cast<int>(threadIdx.x & 31) * nj;
+        lv = lo + static_cast<int>(threadIdx.x & 31);
     }
-    __device__ __forceinline__ bool has(int j) const { return j < nj && lv + j < hi; }
+    __device__ __forceinline__ bool has(int j) const { return lv + 32 * j < hi; }
     __device__ __forceinline__ bool holds(int y) const { return (y >> 3) >= lo && (y >> 3) < hi; }   // id y, the warp
-    __device__ __forceinline__ int lane_of(int y) const { return ((y >> 3) - lo) / nj; }               // (holds(y))
     __device__ __forceinline__ int part_of(int y) const { return (y >> 3) / seg; }
     // a value into the same place of every CTA of the row (lane c writes CTA c's copy)
     template <class T>
@@ -121,23 +120,23 @@ struct RegVecs {
         if (src.sh == 0) {
 #pragma unroll
             for (int j = 0; j < NV; ++j)
-                if (g.has(j) && src.whole(g.lv + j)) v[j] = src.load_aligned(g.lv + j);
+                if (g.has(j) && src.whole(g.lv + 32 * j)) v[j] = src.load_aligned(g.lv + 32 * j);
         } else {
 #pragma unroll
             for (int j = 0; j < NV; ++j)
-                if (g.has(j) && src.whole(g.lv + j)) v[j] = src.load_shifted(g.lv + j);
+                if (g.has(j) && src.whole(g.lv + 32 * j)) v[j] = src.load_shifted(g.lv + 32 * j);
         }
         if (g.lo < src.f0 || g.hi > src.f1) {   // the vectors at the edges of the row
 #pragma unroll
             for (int j = 0; j < NV; ++j)
-                if (g.has(j) && !src.whole(g.lv + j)) v[j] = src.load_slow(g.lv + j);
+                if (g.has(j) && !src.whole(g.lv + 32 * j)) v[j] = src.load_slow(g.lv + 32 * j);
         }
     }
     __device__ __forceinline__ void drop(const RegRow &g, int y) {   // id y becomes -inf
         if (!g.holds(y)) return;
 #pragma unroll
         for (int j = 0; j < NV; ++j)
-            if (g.lv + j == (y >> 3)) v[j].drop(y & 7);
+            if (g.lv + 32 * j == (y >> 3)) v[j].drop(y & 7);
     }
 };
 
@@ -158,24 +157,13 @@ __device__ __forceinline__ void forget(RegVecs<float, NV> &x) {
         for (int i = 0; i < 8; ++i) asm volatile("" : "+f"(x.v[j].f[i]));
 }
 
-// The ids of one lane of the warp, spread over the warp: f(id, in range) for rounds of 32 ids until it returns true.
-template <class F>
-__device__ __forceinline__ void lane_ids(const RegRow &g, int src, int vocab, F f) {
-    const int first = (g.lo + src * g.nj) * 8;
-    const int end = min(vocab, min(g.hi, g.lo + (src + 1) * g.nj) * 8);
-#pragma unroll 1
-    for (int y0 = first; y0 < end; y0 += 32) {
-        const int y = y0 + static_cast<int>(threadIdx.x & 31);
-        if (f(y, y < end)) return;
-    }
-}
-
 // ---- pass A of a part: maximum, sum of exponentials, (argmax and the sum without it) ----------------
 // Both rows of a pair go through the same arithmetic with pinned roundings: equal rows give equal bits.
-struct PartStat { float ml, s, sx, mine; int idx; };   // mine: this lane's own sum
+struct PartStat { float ml, s, sx; int idx; };
 
 template <bool ARG, typename LT, int NV>
 __device__ __forceinline__ PartStat part_stat(const RegRow &g, const RegVecs<LT, NV> &x, const LT *row, int vocab, float k) {
+    const int lane = threadIdx.x & 31;
     auto m2 = x.v[0].packed_max();
 #pragma unroll
     for (int j = 1; j < NV; ++j)
@@ -185,33 +173,35 @@ __device__ __forceinline__ PartStat part_stat(const RegRow &g, const RegVecs<LT,
     o.ml = warp_max(m);
     const float c = shift_of(o.ml, k);
     const F2 k2 = f2_make(k, k), nc2 = f2_make(-c, -c);
-    F2 s2 = f2_make(0.f, 0.f);
+    float vs[NV], mine = 0.f;
 #pragma unroll
-    for (int j = 0; j < NV; ++j)
+    for (int j = 0; j < NV; ++j) {
+        vs[j] = 0.f;
         if (j < g.nj)
-            s2 = f2_add(s2, f2_add(f2_add(f2_exp(x.v[j].pair(0), k2, nc2), f2_exp(x.v[j].pair(1), k2, nc2)),
-                                   f2_add(f2_exp(x.v[j].pair(2), k2, nc2), f2_exp(x.v[j].pair(3), k2, nc2))));
-    o.mine = f2_sum(s2);
-    o.s = warp_sum(o.mine);
+            vs[j] = f2_sum(f2_add(f2_add(f2_exp(x.v[j].pair(0), k2, nc2), f2_exp(x.v[j].pair(1), k2, nc2)),
+                                  f2_add(f2_exp(x.v[j].pair(2), k2, nc2), f2_exp(x.v[j].pair(3), k2, nc2))));
+        mine += vs[j];
+    }
+    o.s = warp_sum(mine);
     o.sx = 0.f;
     o.idx = 0x7fffffff;
     if (ARG && o.ml > neg_inf()) {
-        // lanes hold ascending ids: the lowest lane with the maximum has its first id
-        const int L = __ffs(__ballot_sync(kFull, m == o.ml)) - 1;
-        int first = 0x7fffffff;
-        float rest = 0.f;
-        lane_ids(g, L, vocab, [&](int y, bool in) {
-            const float l = in ? load_one<LT>(row, y) : neg_inf();
-            if (first == 0x7fffffff) {
-                const unsigned at = __ballot_sync(kFull, in && l == o.ml);
-                if (at) first = y - static_cast<int>(threadIdx.x & 31) + __ffs(at) - 1;
-            }
-            rest += (in && y != first) ? ex2(__fmaf_rn(l, k, -c)) : 0.f;
-            return false;
-        });
+        // the lowest vector that holds the maximum, its ids over the lanes
+        int jm = NV;
+#pragma unroll
+        for (int j = NV - 1; j >= 0; --j)
+            if (j < g.nj && x.v[j].max() == o.ml) jm = j;
+        const int at = __reduce_min_sync(kFull, jm * 32 + lane);   // (jm < NV in some lane)
+        const int y = (g.lo + at) * 8 + lane;
+        const float l = lane < 8 && y < vocab ? load_one<LT>(row, y) : neg_inf();
+        const int first = __ffs(__ballot_sync(kFull, lane < 8 && l == o.ml)) - 1;
+        o.idx = (g.lo + at) * 8 + first;
+        float rest = lane == first ? 0.f : ex2(__fmaf_rn(l, k, -c));   // that vector without it
         rest = warp_sum(rest);
-        o.idx = first;
-        o.sx = warp_sum(static_cast<int>(threadIdx.x & 31) == L ? rest : o.mine);
+        float other = 0.f;
+#pragma unroll
+        for (int j = 0; j < NV; ++j) other += lane == (at & 31) && j == (at >> 5) ? rest : vs[j];
+        o.sx = warp_sum(other);
     }
     return o;
 }
@@ -351,39 +341,53 @@ __device__ __forceinline__ float4 sum_parts(const RegRow &g, const float4 *rec, 
     return s;
 }
 
-// The draw inside a part, by its warp: `mine` = what this lane's ids weigh, weight(y) the weight of id y.  Lowest id
-// whose inclusive prefix exceeds t; the last id with mass when rounding leaves none; -1: no mass.
-template <class WF>
-__device__ __forceinline__ int draw_in_part(const RegRow &g, int vocab, float mine, WF weight, float t) {
+// The draw inside a part, by its warp: vec(j) = what this lane's j-th vector weighs (registers), weight(y) the weight of
+// id y (memory).  Lowest id whose inclusive prefix exceeds t; the last id with mass of the picked vector when rounding
+// leaves none; -1: no mass.
+template <int NV, class VF, class WF>
+__device__ __forceinline__ int draw_in_part(const RegRow &g, int vocab, VF vec, WF weight, float t) {
+    const int lane = threadIdx.x & 31;
+    float s[NV], tot[NV];
+#pragma unroll
+    for (int j = 0; j < NV; ++j) s[j] = j < g.nj ? vec(j) : 0.f;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) tot[j] = warp_sum(s[j]);
+    float run = 0.f, base = 0.f, mine = 0.f;
+    int row = -1;
+    bool found = false;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+        if (tot[j] > 0.f && !found) {
+            row = j; base = run; mine = s[j];
+            found = run + tot[j] > t;
+        }
+        run += tot[j];
+    }
+    if (row < 0) return -1;
+    t -= base;
     const float incl = warp_prefix(mine);
     const unsigned pos = __ballot_sync(kFull, mine > 0.f), hit = __ballot_sync(kFull, mine > 0.f && incl > t);
-    if (!pos) return -1;
     const int L = hit ? __ffs(hit) - 1 : 31 - __clz(pos);
     t = __shfl_sync(kFull, t - (incl - mine), L);
-    float prefix = 0.f;
-    int tok = -1, last = -1;
-    lane_ids(g, L, vocab, [&](int y, bool in) {
-        const float w = in ? weight(y) : 0.f;
-        const float inc = prefix + warp_prefix(w);
-        const int y0 = y - static_cast<int>(threadIdx.x & 31);
-        const unsigned p2 = __ballot_sync(kFull, w > 0.f), h2 = __ballot_sync(kFull, w > 0.f && inc > t);
-        if (h2) { tok = y0 + __ffs(h2) - 1; return true; }
-        if (p2) last = y0 + 31 - __clz(p2);
-        prefix = __shfl_sync(kFull, inc, 31);
-        return false;
-    });
-    return tok < 0 ? last : tok;
+    const int y = (g.lo + row * 32 + L) * 8 + lane;
+    const float w = lane < 8 && y < vocab ? weight(y) : 0.f;
+    const float inc = warp_prefix(w);
+    const unsigned p2 = __ballot_sync(kFull, w > 0.f), h2 = __ballot_sync(kFull, w > 0.f && inc > t);
+    if (!p2) return -1;
+    return y - lane + (h2 ? __ffs(h2) - 1 : 31 - __clz(p2));
 }
 
-// A lane's or a part's sum brought from its own scale to the row's: sums that may consist of exponentials below the
-// smallest normal number on the row's scale (zero there) count as zero, so that a picked lane has an id to give.
-__device__ __forceinline__ float lane_mass(float mine, float f) {
-    const float m = mine * f;
-    return m < 1e-36f ? 0.f : m;   // (64 ids of 2^-126)
-}
+// Parts' sums brought to the row's scale: those that may consist of exponentials below the smallest normal number there
+// (zero) count as zero, so that a picked part has an id to give.
 __device__ __forceinline__ void clean_masses(PerPart &mass) {
 #pragma unroll
-    for (int i = 0; i < kRegPer; ++i) mass.m[i] = mass.m[i] < 3.2e-35f ? 0.f : mass.m[i];
+    for (int i = 0; i < kRegPer; ++i) mass.m[i] = mass.m[i] < 2.5e-35f ? 0.f : mass.m[i];   // (2048 ids of 2^-126)
+}
+// What a vector of a row weighs: its exponentials on the row's scale.
+template <typename LT>
+__device__ __forceinline__ float vec_mass(const Vec8<LT> &v, F2 k2, F2 nc2) {
+    return f2_sum(f2_add(f2_add(f2_exp(v.pair(0), k2, nc2), f2_exp(v.pair(1), k2, nc2)),
+                         f2_add(f2_exp(v.pair(2), k2, nc2), f2_exp(v.pair(3), k2, nc2))));
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -429,79 +433,73 @@ __global__ void __launch_bounds__(kRegThreads) reg_draft_kernel(KaryArgs A, int 
         return;
     }
     clean_masses(mass);
-    float mine = lane_mass(ps.mine, rescale(ps.ml, shift_of(ps.ml, k), Q.C));
+    forget(q);
     uint32_t st = 0;
-    int x[KK ? KK : kMaxK];
+    const F2 k2 = f2_make(k, k), nc2 = f2_make(-Q.C, -Q.C);
+    auto vec = [&](int j) { return vec_mass(q.v[j], k2, nc2); };
     auto expo = [&](int y) { return ex2(__fmaf_rn(load_one<LT>(rowq, y), k, -Q.C)); };
+    auto drawn = [&](int i) { return __float_as_int(sh.drawn[i][g.group].x); };
     if (method == kRRS) {   // independent draws: the parts that hold them write them
 #pragma unroll 1
         for (int i = 0; i < K; ++i) {
             float t;
             const int s = pick_part_of(g, mass, un[i], t);
             if (s == g.part) {
-                const int tok = draw_in_part(g, a.vocab, mine, expo, t);
+                const int tok = draw_in_part<NV>(g, a.vocab, vec, expo, t);
                 if (lane == 0) a.draft_tokens_out[K * r + i] = tok;
             }
         }
-        x[0] = 0;
     } else {
-        // Draw i leaves out what was drawn before (RRSw), or the hub once it was drawn (SpecHub's second draw).
-        // The part that holds a drawn id tells the row the id and, for the next draw, its mass without all ids
-        // drawn so far, summed directly.
+        // Draw i leaves out what was drawn before (RRSw), or the hub once it was drawn (SpecHub's second draw): the part
+        // that holds a drawn id takes it out of its registers and tells the row the id and its own new mass, summed
+        // directly.
         const int draws = method == kSpecHub ? 2 : K;
-#pragma unroll
-        for (int i = 0; i < (KK ? KK : kMaxK); ++i) {
-            if (i >= draws) break;
-            if (method == kSpecHub && i == 1) {
-                if (x[0] != Q.idx) { x[1] = Q.idx; break; }
-                if (!(Q.sx > 0.f)) { x[1] = Q.idx == 0 ? 1 : 0; st |= SPECHUB_ST_DEGENERATE_Q; break; }
-            }
-            auto weight = [&](int y) {
-                bool out = false;
-#pragma unroll
-                for (int l = 0; l < (KK ? KK : kMaxK); ++l) out |= l < i && x[l] == y;
-                return out ? 0.f : expo(y);
-            };
+#pragma unroll 1
+        for (int i = 0; i < draws; ++i) {
             float t;
-            const int s = pick_part_of(g, mass, un[i], t);
-            if (s < 0) {   // nothing left to draw from: lowest id not drawn yet
-                st |= SPECHUB_ST_DEGENERATE_Q;
-                int tok = 0;
-                for (bool again = true; again && tok < a.vocab;) {
-                    again = false;
-#pragma unroll
-                    for (int l = 0; l < (KK ? KK : kMaxK); ++l)
-                        if (l < i && x[l] == tok) { ++tok; again = true; break; }
+            int known = -2;
+            if (method == kSpecHub && i == 1) {
+                if (drawn(0) != Q.idx) known = Q.idx;
+                else if (!(Q.sx > 0.f)) { known = Q.idx == 0 ? 1 : 0; st |= SPECHUB_ST_DEGENERATE_Q; }
+            }
+            const int s = known >= 0 ? -1 : pick_part_of(g, mass, un[i], t);
+            if (s < 0) {
+                if (known < 0) {   // nothing left to draw from: lowest id not drawn yet
+                    st |= SPECHUB_ST_DEGENERATE_Q;
+                    known = 0;
+                    for (bool again = true; again && known < a.vocab;) {
+                        again = false;
+                        for (int l = 0; l < i; ++l)
+                            if (drawn(l) == known) { ++known; again = true; break; }
+                    }
+                    if (known >= a.vocab) known = 0;
                 }
-                x[i] = tok >= a.vocab ? 0 : tok;
+                __syncwarp();
+                if (lane == 0) sh.drawn[i][g.group] = make_float2(__int_as_float(known), 0.f);   // (every warp the same)
+                __syncwarp();
                 continue;
             }
             if (s == g.part) {
-                const int tok = draw_in_part(g, a.vocab, mine, weight, t);
-                x[i] = tok;
+                const int tok = draw_in_part<NV>(g, a.vocab, vec, [&](int y) {
+                    bool out = false;
+                    for (int l = 0; l < i; ++l) out |= drawn(l) == y;
+                    return out ? 0.f : expo(y);
+                }, t);
                 float rest = 0.f;
-                if (i + 1 < draws && tok >= 0) {   // the lane that holds it, summed again without it
-                    const int L = g.lane_of(tok);
-                    lane_ids(g, L, a.vocab, [&](int y, bool in) {
-                        rest += in && y != tok ? weight(y) : 0.f;
-                        return false;
-                    });
+                if (i + 1 < draws) {
+                    q.drop(g, tok);
+#pragma unroll
+                    for (int j = 0; j < NV; ++j)
+                        if (j < g.nj) rest += vec(j);
                     rest = warp_sum(rest);
-                    if (lane == L) mine = rest;
-                    rest = warp_sum(mine);
                 }
-                g.post(&sh.drawn[i & 1][g.group], make_float2(__int_as_float(x[i]), rest));
+                g.post(&sh.drawn[i][g.group], make_float2(__int_as_float(tok), rest));
             }
             g.sync();
-            const float2 d = sh.drawn[i & 1][g.group];
-            x[i] = __float_as_int(d.x);
-            mass.set(s, d.y);
+            mass.set(s, sh.drawn[i][g.group].y);
         }
-        if (lead) {
-#pragma unroll
-            for (int i = 0; i < (KK ? KK : kMaxK); ++i)
-                if (i < K) a.draft_tokens_out[K * r + i] = x[i];
-        }
+        if (lead)
+            for (int i = 0; i < K; ++i) a.draft_tokens_out[K * r + i] = drawn(i);
     }
     if (!lead) return;
     if (a.hub) a.hub[r] = method == kSpecHub ? Q.idx : -1;
@@ -509,8 +507,8 @@ __global__ void __launch_bounds__(kRegThreads) reg_draft_kernel(KaryArgs A, int 
         float prob0 = 0.f, prob1 = 0.f;
         if (method == kSpecHub) {
             prob0 = Q.own / Q.Z;
-            if (x[0] != Q.idx) prob1 = expo(x[0]) / Q.Z;
-            else if (Q.sx > 0.f) prob1 = prob0 * expo(x[1]) / Q.sx;
+            if (drawn(0) != Q.idx) prob1 = expo(drawn(0)) / Q.Z;
+            else if (Q.sx > 0.f) prob1 = prob0 * expo(drawn(1)) / Q.sx;
         }
         a.draft_prob[2 * r] = prob0;
         a.draft_prob[2 * r + 1] = prob1;
@@ -521,18 +519,25 @@ __global__ void __launch_bounds__(kRegThreads) reg_draft_kernel(KaryArgs A, int 
 // ------------------------------------------------------------------------------------------------
 // Verification
 // ------------------------------------------------------------------------------------------------
-// Bonus token of a leaf row, and the fallback of a rejection without residual mass: a draw from p.  `pp` = this
-// part's statistics of the whole row; the records are in sh.p.
-template <typename LT>
-__device__ __forceinline__ void reg_draw_from_p(const RegRow &g, const RegShared &sh, const PartStat &pp, const LT *rowp,
-                                                int vocab, float k, float u, int32_t *token) {
-    PerPart mass;
-    const RegStat P = merge_parts<false, true>(g, sh.p, k, neg_inf(), &mass);
+// A draw from p by the row's warps: bonus token of a leaf row, fallback of a rejection without residual mass.  `mass` =
+// the parts' masses of p; out[i], i in the set `which`, are ids that were taken out of p's registers (their masses are
+// in `mass`).
+template <typename LT, int NV>
+__device__ __forceinline__ void reg_draw_from_p(const RegRow &g, PerPart mass, const RegVecs<LT, NV> &p, const LT *rowp, int vocab,
+                                                float k, float C, const int *out, unsigned which, float u, int32_t *token) {
     clean_masses(mass);
     float t;
     if (pick_part_of(g, mass, u, t) != g.part) return;
-    const float mine = lane_mass(pp.mine, rescale(pp.ml, shift_of(pp.ml, k), P.C));
-    const int tok = draw_in_part(g, vocab, mine, [&](int y) { return ex2(__fmaf_rn(load_one<LT>(rowp, y), k, -P.C)); }, t);
+    const F2 k2 = f2_make(k, k), nc2 = f2_make(-C, -C);
+    auto weight = [&](int y) { return ex2(__fmaf_rn(load_one<LT>(rowp, y), k, -C)); };
+    const int tok = draw_in_part<NV>(g, vocab, [&](int j) {
+        float s = vec_mass(p.v[j], k2, nc2);
+        for (unsigned m = which; m; m &= m - 1) {
+            const int y = out[__ffs(m) - 1];
+            if (g.lv + 32 * j == (y >> 3)) s += weight(y);
+        }
+        return s;
+    }, weight, t);
     if ((threadIdx.x & 31) == 0) *token = tok;
 }
 
@@ -600,13 +605,15 @@ __global__ void __launch_bounds__(kRegThreads) reg_verify_spechub_kernel(RowArgs
     if (!leaf) g.post(&sh.q[g.slot0 + g.part], make_float4(pq.ml, pq.s, pq.sx, __int_as_float(pq.idx)));
     g.sync();
     const RegStat P = merge_parts<false, false>(g, sh.p, k, neg_inf(), nullptr);
-    auto draw_from_p = [&]() {
-        reg_draw_from_p(g, sh, pp, rowp, a.vocab, k, ures, a.token + r);
+    auto draw_from_p = [&](int hub, unsigned taken_out) {
+        PerPart mp;
+        merge_parts<false, true>(g, sh.p, k, neg_inf(), &mp);
+        reg_draw_from_p(g, mp, p, rowp, a.vocab, k, P.C, &hub, taken_out, ures, a.token + r);
         elsewhere = true;
     };
     if (!stat_ok) { o.status = SPECHUB_ST_STATS; write(); return; }
     if (!(P.ml > neg_inf()) || !(P.ml < pinf) || !finite_pos(P.Z)) { o.status = SPECHUB_ST_NONFINITE; write(); return; }
-    if (leaf) { draw_from_p(); o.rate[2] = 1.f; write(); return; }
+    if (leaf) { draw_from_p(0, 0u); o.rate[2] = 1.f; write(); return; }
     const RegStat Q = merge_parts<true, false>(g, sh.q, k, neg_inf(), nullptr);
     if (!(Q.ml > neg_inf()) || !(Q.ml < pinf) || !finite_pos(Q.Z)) { o.status = SPECHUB_ST_NONFINITE; write(); return; }
 
@@ -648,8 +655,7 @@ __global__ void __launch_bounds__(kRegThreads) reg_verify_spechub_kernel(RowArgs
             rr = f2_add(rr, w);
         }
     }
-    const float mine = f2_sum(rr);
-    const float w1 = warp_sum(f2_sum(s1)), w2 = warp_sum(f2_sum(s2)), wr = warp_sum(mine);
+    const float w1 = warp_sum(f2_sum(s1)), w2 = warp_sum(f2_sum(s2)), wr = warp_sum(f2_sum(rr));
     g.post(&sh.sum[0][g.slot0 + g.part], make_float4(w1, w2, wr, 0.f));
     g.sync();
     PerPart mass;
@@ -664,12 +670,22 @@ __global__ void __launch_bounds__(kRegThreads) reg_verify_spechub_kernel(RowArgs
     if (!(acc1 || acc2)) {
         if (!(Rraw > 0.f)) {
             o.status |= SPECHUB_ST_ZERO_RESIDUAL;
-            draw_from_p();
+            draw_from_p(hubtok, 1u);
         } else {
             elsewhere = true;
             float t;
             if (pick_part_of(g, mass, ures, t) == g.part) {
-                const int tok = draw_in_part(g, a.vocab, mine, [&](int y) {
+                forget(p);
+                forget(q);
+                const int tok = draw_in_part<NV>(g, a.vocab, [&](int j) {
+                    F2 w = f2_make(0.f, 0.f);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const F2 ep = f2_exp(p.v[j].pair(i), k2, ncp2), eq = f2_exp(q.v[j].pair(i), k2, ncq2);
+                        w = f2_add(w, f2_max0(f2_fma(ncrho2, eq, f2_max0(f2_fma(nrho2, eq, ep)))));
+                    }
+                    return f2_sum(w);
+                }, [&](int y) {
                     const float ep = ex2(__fmaf_rn(load_one<LT>(rowp, y), k, -P.C)), eq = ex2(__fmaf_rn(load_one<LT>(rowq, y), k, -Q.C));
                     const float d = __fmaf_rn(-rho, eq, ep);
                     return y == hubtok ? 0.f : fmaxf(__fmaf_rn(-crho, eq, fmaxf(d, 0.f)), 0.f);
@@ -786,7 +802,9 @@ __global__ void __launch_bounds__(kRegThreads) reg_verify_rrs_kernel(KaryArgs A,
     if (!stat_ok) { status = SPECHUB_ST_STATS; write(); return; }
     if (!(P.ml > neg_inf()) || !(P.ml < pinf) || !finite_pos(P.Z)) { status = SPECHUB_ST_NONFINITE; write(); return; }
     if (leaf) {
-        reg_draw_from_p(g, sh, pp, rowp, a.vocab, k, ures, a.token + r);
+        PerPart mp;
+        merge_parts<false, true>(g, sh.p, k, neg_inf(), &mp);
+        reg_draw_from_p(g, mp, p, rowp, a.vocab, k, P.C, x, 0u, ures, a.token + r);
         elsewhere = true;
         rate[MK] = 1.f;
         write();
@@ -800,7 +818,6 @@ __global__ void __launch_bounds__(kRegThreads) reg_verify_rrs_kernel(KaryArgs A,
 
     float m = 1.f, C = 0.f;   // m_{j-1}, C_{j-1}
     float Cx[MK];             // what C came to for x_i: stops growing once x_i is drawn (RRSw)
-    float mine = 0.f;
     PerPart mass;             // of P_j
     bool accepted = false;
 #pragma unroll
@@ -847,8 +864,7 @@ __global__ void __launch_bounds__(kRegThreads) reg_verify_rrs_kernel(KaryArgs A,
             for (int i = 0; i < 4; ++i)
                 s = f2_add(s, f2_max0(f2_fma(nc, f2_exp(q.v[jj].pair(i), k2, ncq2), f2_exp(p.v[jj].pair(i), k2, ncp2))));
         }
-        mine = f2_sum(s);
-        g.post(&sh.sum[j & 1][g.slot0 + g.part], make_float4(0.f, 0.f, warp_sum(mine), 0.f));
+        g.post(&sh.sum[j & 1][g.slot0 + g.part], make_float4(0.f, 0.f, warp_sum(f2_sum(s)), 0.f));
         g.sync();
         float m_next = sum_parts(g, sh.sum[j & 1], mass).z;
 #pragma unroll
@@ -857,7 +873,6 @@ __global__ void __launch_bounds__(kRegThreads) reg_verify_rrs_kernel(KaryArgs A,
                 const float v = fmaxf(__fmaf_rn(-(i <= j ? Cx[i] : C) * rho, eq1[i], ep1[i]), 0.f);
                 m_next += v;
                 mass.add(g.part_of(x[i]), v);
-                if (g.holds(x[i]) && lane == g.lane_of(x[i])) mine += v;
             }
         m_next *= invZp;
         rate[j] = alive ? fmaxf(m - m_next, 0.f) : 0.f;
@@ -869,24 +884,42 @@ __global__ void __launch_bounds__(kRegThreads) reg_verify_rrs_kernel(KaryArgs A,
         if (m > 0.f) {
             float t;
             if (pick_part_of(g, mass, ures, t) == g.part) {
-                const int tok = draw_in_part(g, a.vocab, mine, [&](int y) {
+                auto weight = [&](int y) {
                     float Cy = C;
 #pragma unroll
                     for (int i = 0; i < MK; ++i)
                         if (single[i] && x[i] == y) Cy = Cx[i];
                     const float ep = ex2(__fmaf_rn(load_one<LT>(rowp, y), k, -P.C)), eq = ex2(__fmaf_rn(load_one<LT>(rowq, y), k, -Q.C));
                     return fmaxf(__fmaf_rn(-Cy * rho, eq, ep), 0.f);
-                }, t);
+                };
+                const F2 nc = f2_make(-C * rho, -C * rho);
+                forget(p);
+                forget(q);
+                const int tok = draw_in_part<NV>(g, a.vocab, [&](int j) {
+                    F2 w = f2_make(0.f, 0.f);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        w = f2_add(w, f2_max0(f2_fma(nc, f2_exp(q.v[j].pair(i), k2, ncq2), f2_exp(p.v[j].pair(i), k2, ncp2))));
+                    float s = f2_sum(w);
+#pragma unroll
+                    for (int i = 0; i < MK; ++i)
+                        if (single[i] && g.lv + 32 * j == (x[i] >> 3)) s += weight(x[i]);
+                    return s;
+                }, weight, t);
                 if (lane == 0) a.token[r] = tok;
             }
-        } else {   // (rare) a draw from the whole of p
+        } else {   // (rare) a draw from p
             status |= SPECHUB_ST_ZERO_RESIDUAL;
-            p.load(g, rowp, a.vocab);
-            const PartStat whole = part_stat<false>(g, p, rowp, a.vocab, k);
-            g.sync();
-            g.post(&sh.p[g.slot0 + g.part], make_float2(whole.ml, whole.s));
-            g.sync();
-            reg_draw_from_p(g, sh, whole, rowp, a.vocab, k, ures, a.token + r);
+            PerPart mp;
+            merge_parts<false, true>(g, sh.p, k, floor_p, &mp);
+            unsigned which = 0;
+#pragma unroll
+            for (int i = 0; i < MK; ++i)
+                if (single[i]) {
+                    which |= 1u << i;
+                    mp.add(g.part_of(x[i]), ep1[i]);
+                }
+            reg_draw_from_p(g, mp, p, rowp, a.vocab, k, P.C, x, which, ures, a.token + r);
         }
     }
     write();
