@@ -4,11 +4,17 @@
 
 namespace spechub {
 
-// Warps of the whole call from which the streaming kernels are faster, on rows of several warps: about 24 per SM, or
-// one and a half waves of these kernels (V = 32000: 224 rows, V = 128256: 56 rows; measured for each step, both types).
-constexpr long long kRegMaxWarps = 24 * 148;
+// Warps of the whole call up to which these kernels are the faster ones, on rows of several warps (V = 2056 .. 128256,
+// both types).  Draft step: one wave, 16 per SM (7 x batch rows of 32000 bf16 ids: 56 rows 8.7 us, streaming 9.7; 112
+// rows 10.9, 9.3).  Verification: 20 per SM (32000 fp32 ids, 56 rows 12.3 us, streaming 14.3; 112 rows 18.3, 14.3), and
+// 25 while the streaming kernels, one CTA per row, leave half of the SMs without a row (128256 bf16 ids, 56 rows: SpecHub
+// 22.6 us, streaming 27.7; RRSw 24.6, 35.3); 24 with more than two drafts, whose streaming kernels read the rows more
+// often (k = 3, 208 rows of 32000 bf16 ids: RRSw 27.9 us, streaming 35.7).
+constexpr long long max_warps(bool verify, int k, long long rows) {
+    return 148 * (!verify ? 16 : rows <= 148 / 2 ? 25 : k > 2 ? 24 : 20);
+}
 
-bool reg_plan(int dtype, int vocab, long long rows, RegPlan *out) {
+bool reg_plan(bool verify, int dtype, int k, int vocab, long long rows, RegPlan *out) {
     const int nvec = (vocab + 7) / 8, max_nv = dtype == SPECHUB_BF16 ? 8 : 4;
     RegPlan p = {};
     // as many warps per row as one wave holds (16 per SM): the fewest vectors per lane that allow it
@@ -25,9 +31,10 @@ bool reg_plan(int dtype, int vocab, long long rows, RegPlan *out) {
     p.rows_per_cta = p.w <= 2 ? 4 / p.w : 1;
     p.seg = (nvec + p.w * p.cs - 1) / (p.w * p.cs);
     *out = p;
-    // rows of one warp (bf16: of two) are the faster ones here however many they are (7168 rows, fp32 V = 1000: draft
-    // step 27.7 -> 17.9 us, verification 50.4 -> 29.6 us; bf16 V = 4096: 45.6 -> 40.5, 92.6 -> 75.9 us)
-    return p.w * p.cs <= (dtype == SPECHUB_BF16 ? 2 : 1) || rows * p.w * p.cs <= kRegMaxWarps;
+    // rows of one warp (verification of bf16 rows: of two) are the faster ones here however many they are (7168 rows,
+    // bf16 V = 2056, verification: SpecHub 65.9 us, streaming 85.8; V = 4096: 86.9, 99.3)
+    const int few = verify && dtype == SPECHUB_BF16 ? 2 : 1, warps = p.w * p.cs;
+    return warps <= few || rows * warps <= max_warps(verify, k, rows);
 }
 
 template <class K, class... Args>

@@ -105,8 +105,8 @@ bool keeps_stats(const spechub_desc *d, int format) {
 }
 
 // Rows held in registers: no flag asks for another kernel.
-bool use_reg(const spechub_desc *d, bool aligned, long long rows, RegPlan *pl) {
-    return (d->flags == 0 || !lean_ok(d, aligned)) && reg_plan(d->dtype, d->vocab, rows, pl);
+bool use_reg(bool verify, const spechub_desc *d, bool aligned, long long rows, RegPlan *pl) {
+    return (d->flags == 0 || !lean_ok(d, aligned)) && reg_plan(verify, d->dtype, d->k, d->vocab, rows, pl);
 }
 
 int draft_common(const spechub_desc *d, const void *draft_logits, const float *uniforms, int method,
@@ -136,7 +136,7 @@ int draft_common(const spechub_desc *d, const void *draft_logits, const float *u
     KaryArgs ka;
     ka.r = a; ka.k = d->k; ka.without_replacement = (method == kRRSw); ka.keep_stats = keeps_stats(d, fmt);
     RegPlan pl;
-    if (use_reg(d, al, rows, &pl)) return launch_reg_draft(pl, d->dtype, ka, method, rows, s);
+    if (use_reg(false, d, al, rows, &pl)) return launch_reg_draft(pl, d->dtype, ka, method, rows, s);
     if (d->k > 2) return launch_kary_draft(fmt, ka, rows, s);
     return launch_lean_draft(fmt, method, lean_ok(d, al) ? lean_split(d) : 0, a, ka.keep_stats, rows, s);
 }
@@ -197,7 +197,7 @@ int verify_common(const spechub_desc *d, const void *target_logits, const void *
     KaryArgs ka;
     ka.r = a; ka.k = d->k; ka.without_replacement = (method == kRRSw);
     const int cs = lean_ok(d, al) ? lean_split(d) : 0;
-    if (use_reg(d, al, rows, &pl)) {
+    if (use_reg(true, d, al, rows, &pl)) {
         lrc = launch_reg_verify(pl, d->dtype, ka, method, rows, s);
     } else if (d->k > 2) {
         if (resident_shape(d, al, &rs)) lrc = launch_resident_kary(rs, ka, rows, s);
@@ -233,7 +233,7 @@ int compare_draft(const spechub_desc *d, const void *draft_logits, const float *
     const unsigned rows = (unsigned)(d->batch * (int64_t)d->nodes);
     RegPlan pl;
     const bool al = rows_aligned(d, draft_logits);
-    if (!lean_ok(d, al) || use_reg(d, al, rows, &pl)) {
+    if (!lean_ok(d, al) || use_reg(false, d, al, rows, &pl)) {
         for (int m = 0; m < 3; ++m) {
             const int mrc = draft_common(d, draft_logits, uniforms, m, draft_tokens[m], m == 0 ? hub : nullptr,
                                          m == 0 ? draft_prob : nullptr, status ? status[m] : nullptr, stream,
@@ -273,7 +273,7 @@ int compare_verify(const spechub_desc *d, const void *target_logits, const void 
     const bool al = rows_aligned(d, target_logits) && rows_aligned(d, draft_logits);
     const unsigned rows = (unsigned)(d->batch * (int64_t)d->nodes);
     RegPlan pl;
-    if (!lean_ok(d, al) || use_reg(d, al, rows, &pl)) {
+    if (!lean_ok(d, al) || use_reg(true, d, al, rows, &pl)) {
         for (int m = 0; m < 3; ++m) {
             const int mrc = verify_common(d, target_logits, draft_logits, draft_tokens[m], uniforms, m, &no[m],
                                           so ? &so[m] : nullptr, workspace, workspace_bytes, stream, draft_stats);

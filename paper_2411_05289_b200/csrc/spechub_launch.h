@@ -36,7 +36,7 @@ int launch_walk(const WalkKArgs &w, cudaStream_t s);
 // Rows held in registers.  reg_plan: false if the row does not fit, or if the streaming kernels are the faster
 // ones for so many rows.
 struct RegPlan { int nv, w, cs, rows_per_cta, seg; };
-bool reg_plan(int dtype, int vocab, long long rows, RegPlan *out);
+bool reg_plan(bool verify, int dtype, int k, int vocab, long long rows, RegPlan *out);
 int launch_reg_draft(const RegPlan &pl, int dtype, const KaryArgs &a, int method, unsigned rows, cudaStream_t s);
 int launch_reg_verify(const RegPlan &pl, int dtype, const KaryArgs &a, int method, unsigned rows, cudaStream_t s);
 

@@ -10,7 +10,7 @@ torch = pytest.importorskip("torch")
 
 import parity  # noqa: E402
 import workloads  # noqa: E402
-from test_parity_gpu import (METHODS, gpu_draft, gpu_verify, padded, random_logits, random_uniforms,  # noqa: E402,F401
+from test_parity_gpu import (METHODS, gpu_draft, gpu_draft_stats, gpu_verify, gpu_verify_stats, padded, random_logits, random_uniforms,  # noqa: E402,F401
                              run_case, sh)
 
 
@@ -43,7 +43,7 @@ def test_rows_per_cta_and_vectors_per_lane(sh, rows):  # noqa: F811
 
 # streaming kernels on rows of any alignment: warps' ranges that begin and end inside, at and beyond the whole words
 @pytest.mark.parametrize("pad", [0, 8, 64])
-@pytest.mark.parametrize("V,dtype,B", [(1025, "fp32", 1200), (4105, "bf16", 600), (8199, "fp32", 300), (9001, "bf16", 300)])
+@pytest.mark.parametrize("V,dtype,B", [(1025, "fp32", 1200), (2049, "bf16", 500), (4105, "bf16", 600), (8199, "fp32", 300), (9001, "bf16", 300)])
 def test_streamed_rows_of_any_alignment(sh, V, dtype, B, pad):  # noqa: F811
     rng = np.random.default_rng(V + pad)
     lp, lq = random_logits(rng, B, 3, V, dtype)
@@ -60,3 +60,23 @@ def test_streamed_rows_of_any_alignment(sh, V, dtype, B, pad):  # noqa: F811
         out = parity.to_numpy(gpu_verify(sh, m, tp, tq, torch.from_numpy(d["tokens"]).cuda(), und, tree, 1.0))
         parity.check_verify(m, lp[pick], lq[pick], 1.0, d["tokens"][pick], un[pick], None,
                             {k: v[pick] for k, v in out.items()}, label="any")
+
+
+@pytest.mark.parametrize("V,dtype,B", [(8192, "bf16", 199), (8192, "fp32", 101), (128256, "bf16", 13)])
+def test_records_of_streamed_draft_rows_read_by_registers(sh, V, dtype, B):  # noqa: F811
+    """Between the two steps' limits: the draft step streams its rows and leaves records, the verification holds them
+    in registers."""
+    rng = np.random.default_rng(V + B)
+    lp, lq = random_logits(rng, B, 3, V, dtype)
+    lp, lq = workloads.round_to_storage(lp, dtype), workloads.round_to_storage(lq, dtype)
+    un = random_uniforms(rng, B, 3)
+    pick = np.unique(np.concatenate([[0, B - 1], rng.integers(0, B, 6)]))
+    tp, tq = padded(lp, dtype, 0), padded(lq, dtype, 0)
+    und, tree = torch.from_numpy(un).cuda(), sh.Tree.heap(3)
+    for m in METHODS:
+        d = gpu_draft_stats(sh, m, tq, und, tree, 1.0)
+        out = parity.to_numpy(gpu_verify_stats(sh, m, tp, tq, d["stats"], d["tokens"], und, tree, 1.0))
+        d = parity.to_numpy(d)
+        parity.check_draft(m, lq[pick], 1.0, un[pick], {k: v[pick] for k, v in d.items()}, label="records")
+        parity.check_verify(m, lp[pick], lq[pick], 1.0, d["tokens"][pick], un[pick], None,
+                            {k: v[pick] for k, v in out.items()}, label="records")
