@@ -27,6 +27,11 @@ __device__ __forceinline__ void write_node3(const NodeOutPtrs &p, long long r, c
 // STATS: as in lean_verify_kernel -- the draft row's maximum, argmax and sum come from the record the draft
 // step left, pass A reads the target row only, and a row pair that turns out to be one row twice is redone
 // with p's normaliser set to q's.
+// Bound by DRAM (three passes over rows that L2 holds a third of), by ex2 (five per vocabulary pair) and by issue slots
+// at about 60 % each.  The loops of passes B and C keep one pair of vectors in flight ahead, and are not unrolled: what
+// is live across them fills the 64 registers, and the kernel's code should fit the instruction cache (7936 rows, V =
+// 32000 / 128256 / 152064: two pairs loaded when needed 626 / 2019 / 2368 us; ahead, unrolled twice 602 / 1806 / 2147;
+// not unrolled, drafts read again for the tests 531 / 1768 / 2095; 512 threads 758 / 2150 / 2487).
 template <int THREADS, bool STATS = false>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(FusedArgs A) {
     __shared__ LeanShared sh;
@@ -141,9 +146,12 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
     dna = dnb = 0.f;
     const F2 k2 = f2_make(k, k), ncp2 = f2_make(-cP, -cP), ncq2 = f2_make(-cQ, -cQ);
     const F2 nrho2 = f2_make(-rho, -rho), ncrho2 = f2_make(-crho, -crho);
-#pragma unroll 2
+    V np, nq;
+    if (last_vi >= lo) { np = vp[last_vi]; nq = vq[last_vi]; }
+#pragma unroll 1
     for (int vi = last_vi; vi >= lo; vi -= 32) {
-        const V cp = vp[vi], cq = vq[vi];
+        const V cp = np, cq = nq;
+        if (vi - 32 >= lo) { np = vp[vi - 32]; nq = vq[vi - 32]; }
         if (STATS) diff |= cp.differs(cq);
         float qw[8];
 #pragma unroll
@@ -211,17 +219,25 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
         const F2 nsc0 = f2_make(-A1grho[0], -A1grho[0]), nsc1 = f2_make(-A1grho[1], -A1grho[1]);
         uint64_t polf;   // the rows' last use: L2 may let these lines go first
         asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(polf));
-#pragma unroll 2
+        V mp, mq;
+        if (lo + lane < hi) { mp = vp.fetch(lo + lane, polf); mq = vq.fetch(lo + lane, polf); }
+#pragma unroll 1
         for (int vi = lo + lane; vi < hi; vi += 32) {
-            const V cp = vp.fetch(vi, polf), cq = vq.fetch(vi, polf);
+            const V cp = mp, cq = mq;
+            if (vi + 32 < hi) { mp = vp.fetch(vi + 32, polf); mq = vq.fetch(vi + 32, polf); }
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                F2 nsc = nsc1;
-                if (vi == wvec && i == (wel >> 1)) nsc = (wel & 1) ? f2_make(-A1grho[1], 0.f) : f2_make(0.f, -A1grho[1]);
                 const F2 eq = f2_exp(cq.pair(i), k2, ncq2);
                 const F2 m = f2_max0(f2_fma(nrho2, eq, f2_exp(cp.pair(i), k2, ncp2)));
                 w0 = f2_add(w0, f2_max0(f2_fma(nsc0, eq, m)));
-                w1 = f2_add(w1, f2_max0(f2_fma(nsc, eq, m)));
+                F2 t1 = f2_fma(nsc1, eq, m);
+                if (vi == wvec && i == (wel >> 1)) {   // RRSw's x1 is no part of its second draft
+                    float u0, u1, m0, m1;
+                    f2_get(t1, u0, u1);
+                    f2_get(m, m0, m1);
+                    t1 = (wel & 1) ? f2_make(u0, m1) : f2_make(m0, u1);
+                }
+                w1 = f2_add(w1, f2_max0(t1));
             }
         }
         f2_get(w0, w0a, w0b);
@@ -276,11 +292,11 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
     // ---- RRS / RRSw decisions (Algorithm 1) ----
 #pragma unroll
     for (int m = 0; m < 2; ++m) {
-        if (!ok_r[m]) continue;
         NodeResult &s = o[1 + m];
+        if (s.status) continue;
         const bool wo = (m == 1);
         const float W2raw = accC[m], W2 = W2raw * invZp;
-        const int x1 = rx1[m], x2 = rx2[m];
+        const int x1 = A.tok[1 + m][2 * r], x2 = A.tok[1 + m][2 * r + 1];
         s.rate[0] = fmaxf(1.f - A1, 0.f);
         s.rate[1] = fmaxf(A1 - W2, 0.f);
         s.rate[2] = W2;
