@@ -13,8 +13,12 @@ int launch_fused_draft(const FusedArgs &f, int32_t *hub, float *draft_prob, unsi
 }
 
 int launch_fused_verify(const FusedArgs &f, unsigned rows, cudaStream_t s) {
-    if (!f.r.draft_stats_in) return launch_grid(fused_verify_kernel<kLeanThreads>, rows, kLeanThreads, 0, 1, s, f);
     const int th = verify_threads(f.r.vocab, rows, 1024);
+    if (!f.r.draft_stats_in) {
+        if (th == 512) return launch_grid(fused_verify_kernel<512>, rows, 512, 0, 1, s, f);
+        if (th == 256) return launch_grid(fused_verify_kernel<256>, rows, 256, 0, 1, s, f);
+        return launch_grid(fused_verify_kernel<128>, rows, 128, 0, 1, s, f);
+    }
     if (th == 512) return launch_grid(fused_verify_kernel<512, true>, rows, 512, 0, 1, s, f);
     if (th == 256) return launch_grid(fused_verify_kernel<256, true>, rows, 256, 0, 1, s, f);
     return launch_grid(fused_verify_kernel<128, true>, rows, 128, 0, 1, s, f);

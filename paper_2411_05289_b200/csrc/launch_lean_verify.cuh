@@ -12,6 +12,8 @@ int verify_split(const RowArgs &a, unsigned rows, cudaStream_t s) {
     return launch_grid(lean_verify_kernel<__nv_bfloat16, false, METHOD, kLeanThreads, CS>, rows * CS, kLeanThreads, 0, CS, s, a);
 }
 
+constexpr int kRingVocab = 65536;
+
 // One CTA per row, the passes fed by per-warp rings of bulk copies (spechub_ring.cuh).
 template <int METHOD>
 int verify_ring(const RowArgs &a, unsigned rows, cudaStream_t s) {
@@ -48,10 +50,13 @@ int launch_lean_verify_method(int format, int cs, RowArgs a, unsigned rows, cuda
     if (format == kF32)
         return stats ? verify_rows<float, false, METHOD, true>(a, rows, s) : verify_rows<float, false, METHOD, false>(a, rows, s);
     if (stats) return verify_rows<__nv_bfloat16, false, METHOD, true>(a, rows, s);
-    // (the plain calls and the three-method kernel: always 256 threads)
+    if (cs == 1) return verify_split<METHOD, 1>(a, rows, s);
+    // Rings of bulk copies: rows that L2 does not hold from pass to pass, enough of them for CTAs of 256 threads (1984
+    // rows, V = 128256: RRS 468 us, without rings 537, RRSw 489, 530; V = 32000: 478, 459, 499, 455; 112 rows, V =
+    // 128256: RRS 68 us, CTAs of 512 threads without rings 39).
     if constexpr (METHOD != kSpecHub)
-        if (cs == 0) return verify_ring<METHOD>(a, rows, s);
-    return verify_split<METHOD, 1>(a, rows, s);
+        if (a.vocab >= kRingVocab && verify_threads(a.vocab, rows, 1024) == kLeanThreads) return verify_ring<METHOD>(a, rows, s);
+    return verify_rows<__nv_bfloat16, false, METHOD, false>(a, rows, s);
 }
 
 }  // namespace spechub

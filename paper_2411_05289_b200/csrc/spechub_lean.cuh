@@ -160,7 +160,8 @@ __device__ __forceinline__ float lean_reference(const ROW &row, int vi, int hi, 
 
 // Pass A over this warp's range of one or two rows.
 // AHEAD: the next vector pair is requested before the current one is consumed (measured per
-// method: it pays for RRS, 1.92 -> 1.82 ms on V = 128256, and costs SpecHub 2 %).
+// method: it pays for RRS, 1.92 -> 1.82 ms on V = 128256, and RRSw, 468 -> 455 us on 7936 rows of 32000 ids; SpecHub
+// gains 3 % on those and on few rows, and loses 5 % on 7936 rows of 128256: there it is for CTAs of 512 threads, few rows).
 template <bool BOTH, bool AHEAD, typename LT, class ROW>
 __device__ __forceinline__ void lean_pass_a(const ROW &rp, const ROW &rq, int lo, int hi, int lane, float k,
                                             LeanAcc<LT> &P, LeanAcc<LT> &Q) {
@@ -961,7 +962,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
         lean_pass_a_deep(vp, lo, hi, lane, k, tp);
     } else {
         if (leaf) lean_pass_a<false, false>(vp, vq, lo, hi, lane, k, tp, tq);
-        else lean_pass_a<true, METHOD == kRRS>(vp, vq, lo, hi, lane, k, tp, tq);
+        else lean_pass_a<true, METHOD != kSpecHub || THREADS == 512>(vp, vq, lo, hi, lane, k, tp, tq);
     }
     RowStat P, Q;
     {
