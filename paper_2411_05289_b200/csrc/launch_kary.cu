@@ -41,9 +41,10 @@ int launch_kary_verify(int format, const KaryArgs &a, unsigned rows, cudaStream_
     return kary_verify<float, true>(a, rows, s);
 }
 
-int launch_walk(const WalkKArgs &wk, cudaStream_t s) {
-    const int warp_per_seq = wk.w.nodes <= kWalkNodes, per = warp_per_seq ? kWalkThreads / 32 : kWalkThreads;
-    return launch_grid(walk_kernel, (wk.w.batch + per - 1) / per, kWalkThreads, 0, 1, s, wk, warp_per_seq);
+int launch_walk(const WalkKArgs &wk, int n, cudaStream_t s) {
+    const int warp_per_seq = wk.w[0].nodes <= kWalkNodes, per = warp_per_seq ? kWalkThreads / 32 : kWalkThreads;
+    const unsigned blocks = (wk.w[0].batch + per - 1) / per;
+    return launch_grid(walk_kernel, n * blocks, kWalkThreads, 0, 1, s, wk, warp_per_seq, blocks);
 }
 
 }  // namespace spechub

@@ -141,23 +141,27 @@ int draft_common(const spechub_desc *d, const void *draft_logits, const float *u
     return launch_lean_draft(fmt, method, lean_ok(d, al) ? lean_split(d) : 0, a, ka.keep_stats, rows, s);
 }
 
-int launch_walk(const spechub_desc *d, const spechub_node_out *no, const spechub_seq_out *so, cudaStream_t s) {
-    if (!(so && (so->n_accepted || so->n_emitted || so->path_nodes || so->path_tokens))) return SPECHUB_OK;
-    WalkArgs w;
-    w.accept_idx = no->accept_idx;
-    w.token = no->token;
-    w.child = d->child;
-    w.node_kind = d->node_kind;
-    w.n_accepted = so->n_accepted;
-    w.n_emitted = so->n_emitted;
-    w.path_nodes = so->path_nodes;
-    w.path_tokens = so->path_tokens;
-    w.batch = d->batch;
-    w.nodes = d->nodes;
-    w.levels = d->levels;
+// The walks of n methods over the same trees, in one launch (so = nullptr: none).
+int launch_walks(const spechub_desc *d, const spechub_node_out *no, const spechub_seq_out *so, int n, cudaStream_t s) {
     WalkKArgs wk;
-    wk.w = w; wk.k = d->k;
-    return launch_walk(wk, s);
+    wk.k = d->k;
+    int walks = 0;
+    for (int m = 0; m < n && so; ++m) {
+        if (!(so[m].n_accepted || so[m].n_emitted || so[m].path_nodes || so[m].path_tokens)) continue;
+        WalkArgs &w = wk.w[walks++];
+        w.accept_idx = no[m].accept_idx;
+        w.token = no[m].token;
+        w.child = d->child;
+        w.node_kind = d->node_kind;
+        w.n_accepted = so[m].n_accepted;
+        w.n_emitted = so[m].n_emitted;
+        w.path_nodes = so[m].path_nodes;
+        w.path_tokens = so[m].path_tokens;
+        w.batch = d->batch;
+        w.nodes = d->nodes;
+        w.levels = d->levels;
+    }
+    return walks ? launch_walk(wk, walks, s) : SPECHUB_OK;
 }
 
 int verify_common(const spechub_desc *d, const void *target_logits, const void *draft_logits,
@@ -216,7 +220,7 @@ int verify_common(const spechub_desc *d, const void *target_logits, const void *
         lrc = launch_lean_verify_rrsw(fmt, cs, a, rows, s);
     }
     if (lrc != SPECHUB_OK) return lrc;
-    return launch_walk(d, no, so, s);
+    return launch_walks(d, no, so, 1, s);
 }
 
 // One kernel for the three methods where the lean kernels apply, the three separate paths otherwise.
@@ -276,10 +280,10 @@ int compare_verify(const spechub_desc *d, const void *target_logits, const void 
     if (!lean_ok(d, al) || use_reg(true, d, al, rows, &pl)) {
         for (int m = 0; m < 3; ++m) {
             const int mrc = verify_common(d, target_logits, draft_logits, draft_tokens[m], uniforms, m, &no[m],
-                                          so ? &so[m] : nullptr, workspace, workspace_bytes, stream, draft_stats);
+                                          nullptr, workspace, workspace_bytes, stream, draft_stats);
             if (mrc != SPECHUB_OK) return mrc;
         }
-        return SPECHUB_OK;
+        return launch_walks(d, no, so, 3, static_cast<cudaStream_t>(stream));
     }
     FusedArgs f = {};
     f.r = base_args(d);
@@ -303,8 +307,7 @@ int compare_verify(const spechub_desc *d, const void *target_logits, const void 
         if (lean_split(d) == 0) f.r.draft_stats_in = draft_stats;
         lrc = launch_fused_verify(f, rows, s);
     }
-    for (int m = 0; m < 3 && lrc == SPECHUB_OK && so; ++m) lrc = launch_walk(d, &no[m], &so[m], s);
-    return lrc;
+    return lrc == SPECHUB_OK ? launch_walks(d, no, so, 3, s) : lrc;
 }
 
 // ---- vocabulary-sharded phases ------------------------------------------------------------------
@@ -470,7 +473,7 @@ int spechub_walk_tree(const spechub_desc *desc, const int32_t *accept_idx, const
     spechub_node_out no = {};
     no.accept_idx = const_cast<int32_t *>(accept_idx);
     no.token = const_cast<int32_t *>(token);
-    return launch_walk(desc, &no, seq_out, static_cast<cudaStream_t>(stream));
+    return launch_walks(desc, &no, seq_out, 1, static_cast<cudaStream_t>(stream));
 }
 
 int spechub_shard_stats(const spechub_desc *desc, const spechub_shard *shard, const void *target_slice,
@@ -701,5 +704,5 @@ extern "C" int spechub_verify_tree_static(const spechub_desc *desc, const void *
     a.r.beta = no->beta; a.r.rate = no->rate; a.r.status = no->status;
     prc = run_shard_phase(kPhaseDecide, desc, a, stream);
     if (prc != SPECHUB_OK) return prc;
-    return launch_walk(desc, no, so, static_cast<cudaStream_t>(stream));
+    return launch_walks(desc, no, so, 1, static_cast<cudaStream_t>(stream));
 }

@@ -97,7 +97,7 @@ struct WalkArgs {
 };
 
 struct WalkKArgs {
-    WalkArgs w;
+    WalkArgs w[3];
     int k;
 };
 }  // namespace spechub

@@ -31,7 +31,7 @@ int launch_grid(K kern, unsigned grid, int threads, int smem, int cs, cudaStream
 // the caller (one array per kernel).
 int allow_smem(const void *kern, int bytes, bool *configured);
 
-int launch_walk(const WalkKArgs &w, cudaStream_t s);
+int launch_walk(const WalkKArgs &w, int n, cudaStream_t s);   // the first n
 
 // Rows held in registers.  reg_plan: false if the row does not fit, or if the streaming kernels are the faster
 // ones for so many rows.

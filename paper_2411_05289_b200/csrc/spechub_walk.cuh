@@ -12,12 +12,14 @@ constexpr int kWalkNodes = 128;   // trees of up to so many nodes: one warp per 
 
 // One warp per sequence: the lanes fetch all nodes' results at once (one round trip to memory instead of two or three
 // per level), and the path is followed in shared memory.  Larger trees: one thread per sequence.
-__global__ void __launch_bounds__(kWalkThreads) walk_kernel(WalkKArgs A, int warp_per_seq) {
+// `blocks`: those of one walk; the three methods side by side walk in one launch.
+__global__ void __launch_bounds__(kWalkThreads) walk_kernel(WalkKArgs A, int warp_per_seq, unsigned blocks) {
     __shared__ int sh_tok[kWalkThreads / 32][kWalkNodes], sh_acc[kWalkThreads / 32][kWalkNodes];
     pdl_begin();
-    const WalkArgs &a = A.w;
+    const unsigned which = blockIdx.x / blocks, block = blockIdx.x - which * blocks;
+    const WalkArgs &a = A.w[which];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int b = warp_per_seq ? blockIdx.x * (kWalkThreads / 32) + warp : blockIdx.x * kWalkThreads + threadIdx.x;
+    const int b = warp_per_seq ? block * (kWalkThreads / 32) + warp : block * kWalkThreads + threadIdx.x;
     if (b >= a.batch) return;
     const long long r0 = static_cast<long long>(b) * a.nodes;
     if (warp_per_seq) {
