@@ -91,9 +91,10 @@ extern "C" {
 
 /* descriptor flags: how many CTAs of a thread-block cluster share one row in the large-vocabulary
  * bf16 kernels (a tuning hint; results do not depend on it beyond fp32 summation order).  At most
- * one of the three may be set; none = the library chooses: one CTA per row, and for RRS / RRSw the
- * verification passes read the rows through per-warp rings of bulk copies into shared memory
- * (cp.async.bulk) -- same results, bit for bit, as SPECHUB_FLAG_SPLIT_1, whose loads go to registers. */
+ * one of the three may be set; none = the library chooses by rows, length and type: rows held in
+ * registers, one CTA per row of 64 to 512 threads, or (RRS / RRSw on many long rows) rings of bulk
+ * copies into shared memory.  SPECHUB_FLAG_SPLIT_1 asks for one CTA of 256 threads per row whose loads
+ * go to registers. */
 #define SPECHUB_FLAG_SPLIT_1 1u
 #define SPECHUB_FLAG_SPLIT_2 2u
 #define SPECHUB_FLAG_SPLIT_4 4u
@@ -278,10 +279,9 @@ int rrs_verify_tree_stats(const spechub_desc *desc, const void *target_logits, c
  * q_j = q (RRS) or q with q(x_1..x_{j-1}) zeroed and renormalised (RRSw),
  * P_j = max(P_{j-1} - m_{j-1} q_j, 0) and m_j = sum P_j; the residual token is
  * drawn from P_k; rate[j] = m_j - m_{j+1} (j < k), rate[k] = m_k.
- * For desc->k > 2 on bf16 rows that are 16-byte aligned with 8192 <= vocab <=
- * 262144, vocab % 8 == 0 and no split flag, the stages run over exponentials
- * kept in the SMs' tensor memory and shared memory (see SPECHUB_FLAG_RESIDENT
- * for what that means for other work on the GPU).
+ * For desc->k > 2 the stages re-read the rows (from L2 as far as it holds them);
+ * with SPECHUB_FLAG_RESIDENT, on the shapes named there, they run over
+ * exponentials kept in the SMs' tensor memory and shared memory.
  */
 int rrs_verify_tree(const spechub_desc *desc, const void *target_logits, const void *draft_logits,
                     const int32_t *draft_tokens, const float *uniforms, int without_replacement,

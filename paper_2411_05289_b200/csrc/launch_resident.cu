@@ -1,6 +1,5 @@
 // Verification with the exponentials resident on chip.
 #include "spechub_launch.h"
-#include "spechub_kary.cuh"
 #include "spechub_resident.cuh"
 #include "spechub_resident_kary.cuh"
 

@@ -68,8 +68,8 @@ RowArgs base_args(const spechub_desc *d) {
 // CTAs per row.  With 4 CTAs per SM and 148 SMs, 592/CS rows are between their first and second
 // read at any time; at CS = 4 on V = 128256 that fits L2 (DRAM reads drop from 2.0x to 1.0x the
 // algorithmic bytes) but the per-CTA fixed work grows 4x, and the two cancel (1.6 vs 1.8 ms).
-// 0 = no flag: one CTA per row (measured on B200: the per-CTA fixed work of a split row still outweighs
-// the L2 hits), and the verification of RRS / RRSw takes its vectors from per-warp rings of bulk copies.
+// 0 = no flag: one CTA per row (the per-CTA fixed work of a split row outweighs the L2 hits), whose shape
+// and loads the launches choose.
 int lean_split(const spechub_desc *d) {
     if (d->flags & SPECHUB_FLAG_SPLIT_1) return 1;
     if (d->flags & SPECHUB_FLAG_SPLIT_2) return 2;

@@ -253,11 +253,10 @@ __device__ __forceinline__ float warp_sum(float x) {
 // mass[w] (shared memory) = total weight of warp w's range.  weights(vi, w[]) must
 // return the VW weights of vector vi (0 for ids that carry no mass or lie past V)
 // and must be the same arithmetic that produced mass[].  Returns to every thread
-// the lowest id whose inclusive prefix exceeds u * total; when rounding leaves
+// the lowest id whose inclusive prefix exceeds t; when rounding leaves
 // none inside the selected range, the last id with positive weight there; -1 when
 // the total is 0.  Must be called by all threads of the CTA.
-// block_sample_at takes the target prefix t itself (a draw whose total spans more than this CTA's
-// range); block_sample draws with u * (this range's total).
+// t is the target prefix itself (a draw's total spans more than this CTA's range).
 template <int VW, class WF>
 __device__ int block_sample_at(const Geo &g, WF weights, const float *mass, float t, int *sh_tok) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -334,14 +333,6 @@ __device__ int block_sample_at(const Geo &g, WF weights, const float *mass, floa
     const int tok = *sh_tok;
     __syncthreads();
     return tok;
-}
-
-template <int VW, class WF>
-__device__ int block_sample(const Geo &g, WF weights, const float *mass, float u, int *sh_tok) {
-    float total = 0.f;
-    for (int w = 0; w < g.nwarps; ++w) total += mass[w];
-    if (!(total > 0.f)) return -1;
-    return block_sample_at<VW>(g, weights, mass, u * total, sh_tok);
 }
 
 }  // namespace spechub

@@ -1,15 +1,8 @@
-// Lean streaming kernels for bf16 rows with 16-byte aligned starts and V % 8 == 0
-// (the shapes of the large-vocabulary workloads).  A (sequence, node) row is
-// worked on by a cluster of CS CTAs (CS = 1, 2 or 4), each owning a contiguous
-// slice of the vocabulary; several CTAs of different rows share an SM so that one
-// row's reductions overlap another row's streaming.  Splitting a row keeps the
-// number of rows in flight -- and with it the bytes between a row's first and
-// second read -- small enough that pass B hits L2 instead of HBM, without giving
-// up the thread count that hides latency.  The CTAs of a row meet at two or three
-// hardware cluster barriers and read each other's few partial results through
-// distributed shared memory.  Compared with the general kernels in
-// spechub_stream.cuh the inner loops are branch-free and carry no index
-// bookkeeping:
+// Streaming kernels: bf16 or fp32 rows of any alignment, read as logical vectors of 8 ids (spechub_vec.cuh); two or
+// three passes, the later ones from L2 as far as it holds the rows.
+// One CTA per row; long bf16 rows in whole words can also be split over a cluster of 2 or 4 CTAs, which meet at two or
+// three cluster barriers and read each other's partial results through distributed shared memory.  Several CTAs of
+// different rows share an SM, so that one row's reductions overlap another row's streaming.
 //
 //   pass A  per 16-byte vector: a packed bf16 max tree (4 ops), 8 x (unpack, FMA,
 //           ex2, add).  The exponent reference c of a thread is the maximum of the

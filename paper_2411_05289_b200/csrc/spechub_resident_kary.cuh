@@ -13,10 +13,30 @@
 // the records up by itself, in the same order: no CTA waits for one warp to broadcast.
 #pragma once
 
-#include "spechub_kary.cuh"
+#include "spechub_common.cuh"
+#include "spechub_stream.cuh"
 #include "spechub_resident.cuh"
 
 namespace spechub {
+
+// Is token y one of x[0..n)?
+__device__ __forceinline__ bool in_set(const int *x, int n, int y) {
+    bool f = false;
+    for (int i = 0; i < n; ++i) f |= (x[i] == y);
+    return f;
+}
+
+// P_j(y) from p(y), q(y): j subtractions with the stage coefficients; for RRSw a token already
+// drawn before stage l carries no draft mass there.
+__device__ __forceinline__ float stage_value(float pp, float qq, int y, int j, const float *coef, const int *x,
+                                             bool wo, bool check_set) {
+    float v = pp;
+    for (int l = 0; l < j; ++l) {
+        const float ql = (wo && check_set && in_set(x, l, y)) ? 0.f : qq;
+        v = fmaxf(__fmaf_rn(-coef[l], ql, v), 0.f);
+    }
+    return v;
+}
 
 struct __align__(16) ResKaryShared {
     float recA[kResMaxParts][8];      // c_p, s_p, c_q, s_q, s_q without the drafts x_1..x_{k-1}

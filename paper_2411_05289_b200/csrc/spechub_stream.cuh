@@ -1,8 +1,5 @@
-// General streaming kernels: one CTA per (sequence, node) row, any vocabulary
-// size, fp32 or bf16 logits, aligned or not.  Pass A reads the row(s) from HBM;
-// the later passes re-read them, which hit L2 while the row pair is still
-// there.  Large bf16 vocabularies with aligned rows take the kernels of
-// spechub_lean.cuh instead; these remain the path for every other shape.
+// Pieces that the kernels share: pass A of the vocabulary-sharded phases (any row, fp32 or bf16), probabilities with
+// pinned rounding, the acceptance test, a row's outputs.
 #pragma once
 
 #include "spechub.h"
@@ -74,47 +71,6 @@ __device__ __forceinline__ void transport_terms(float pp, float qq, float s, flo
 
 __device__ __forceinline__ bool finite_pos(float x) { return x > 0.f && x < __int_as_float(0x7f800000); }
 
-// Draw from softmax(row) with token `excl` removed (excl < 0: nothing removed).
-// Uses the per-warp partials of pass_a; `hubtok` is the row's argmax, cQ its shift.
-template <typename LT, bool AL>
-__device__ int sample_row(const Geo &g, const LT *row, float k, float cQ, int hubtok, int excl,
-                          float u, const WarpPart &wp, Partials &sh) {
-    constexpr int VW = VecOf<LT>::W;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x < g.nwarps) {
-        const int w = threadIdx.x;
-        const float ml = wp.ml[w];
-        const bool holds_hub = (wp.idx[w] == hubtok);
-        // the warp's partial leaves out its own argmax: add it back unless it is the excluded hub
-        const float own = (holds_hub && excl == hubtok) ? 0.f : own_term(ml, k);
-        sh.mass[w] = (wp.sx[w] + own) * rescale(ml, shift_of(ml, k), cQ);
-    }
-    __syncthreads();
-    if (excl >= 0 && excl != hubtok) {
-        // an arbitrary token is removed (RRS without replacement): its warp re-sums its range
-        const int wex = (excl / VW) / g.seg;
-        if (warp == wex) {
-            float s = 0.f;
-            for (int vi = g.seg_lo(warp) + lane; vi < g.seg_hi(warp); vi += 32) {
-                float v[VW];
-                load_vec<LT, AL>(row, vi, g.V, v);
-#pragma unroll
-                for (int i = 0; i < VW; ++i) s += (vi * VW + i == excl) ? 0.f : ex2(fmaf(v[i], k, -cQ));
-            }
-            s = warp_sum(s);
-            if (lane == 0) sh.mass[warp] = s;
-        }
-        __syncthreads();
-    }
-    auto wf = [&](int vi, float(&w)[VW]) {
-        float v[VW];
-        load_vec<LT, AL>(row, vi, g.V, v);
-#pragma unroll
-        for (int i = 0; i < VW; ++i) w[i] = (vi * VW + i == excl) ? 0.f : ex2(fmaf(v[i], k, -cQ));
-    };
-    return block_sample<VW>(g, wf, sh.mass, u, &sh.tok);
-}
-
 // ------------------------------------------------------------------------------------------------
 // Verification of one row.
 // ------------------------------------------------------------------------------------------------
@@ -159,7 +115,5 @@ __device__ __forceinline__ void block_sums(const Geo &g, float (&x)[NACC], Parti
         x[i] = t;
     }
 }
-// sh.acc may be rewritten only after every thread has read it
-__device__ __forceinline__ void release_sums() { __syncthreads(); }
 
 }  // namespace spechub
