@@ -14,9 +14,12 @@ constexpr int threads_for_few(unsigned rows, int many) {
     return many;
 }
 // Draft step and leaf rows: 8 CTAs of 128 threads per SM (64 / 128 / 256 / 512 threads: 0.41 / 0.36 / 0.38 /
-// 0.52 ms on V = 128256; 0.078 / 0.081 / 0.102 / 0.165 ms on V = 32000); rows too short to feed those take 64.
+// 0.52 ms on V = 128256).  Rows too short to feed those take 64, and so do rows below 40960 ids in more than one wave of
+// 64 threads: one warp draws while the others' registers idle, which weighs more the shorter the row and the more draws
+// it makes (3584 rows: RRSw V = 16384 44.0 -> 37.9 us, V = 32000 67.7 -> 61.8, SpecHub 58.6 -> 59.1; three drafts, 10240
+// rows of 32000 216 -> 199; but V = 65472 106 -> 109, SpecHub 95 -> 105, and 1400 rows of 32000 27.8 -> 31.8).
 constexpr int draft_threads(int vocab, unsigned rows) {
-    return vocab < 8192 ? 64 : threads_for_few(rows, 128);
+    return vocab < 8192 || (vocab < 40960 && rows > 16 * kSms) ? 64 : threads_for_few(rows, 128);
 }
 // Verification: 4 CTAs of 256 threads per SM (256/512/1024: 1.54/1.65/1.87 ms on V = 128256); 128 threads on rows too
 // short to feed those (V = 8192, 1792 rows: SpecHub 28.6 -> 23.3 us, RRSw 30.7 -> 26.2 us).

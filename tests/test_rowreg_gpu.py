@@ -43,7 +43,8 @@ def test_rows_per_cta_and_vectors_per_lane(sh, rows):  # noqa: F811
 
 # streaming kernels on rows of any alignment: warps' ranges that begin and end inside, at and beyond the whole words
 @pytest.mark.parametrize("pad", [0, 8, 64])
-@pytest.mark.parametrize("V,dtype,B", [(1025, "fp32", 1200), (2049, "bf16", 500), (4105, "bf16", 600), (8199, "fp32", 300), (9001, "bf16", 300)])
+@pytest.mark.parametrize("V,dtype,B", [(1025, "fp32", 1200), (2049, "bf16", 500), (4105, "bf16", 600), (8199, "fp32", 300), (9001, "bf16", 300),
+                                       (8201, "bf16", 790), (8192, "fp32", 790)])
 def test_streamed_rows_of_any_alignment(sh, V, dtype, B, pad):  # noqa: F811
     rng = np.random.default_rng(V + pad)
     lp, lq = random_logits(rng, B, 3, V, dtype)
@@ -80,3 +81,17 @@ def test_records_of_streamed_draft_rows_read_by_registers(sh, V, dtype, B):  # n
         parity.check_draft(m, lq[pick], 1.0, un[pick], {k: v[pick] for k, v in d.items()}, label="records")
         parity.check_verify(m, lp[pick], lq[pick], 1.0, d["tokens"][pick], un[pick], None,
                             {k: v[pick] for k, v in out.items()}, label="records")
+
+
+def test_three_methods_on_more_than_a_wave_of_rows(sh):  # noqa: F811
+    """Draft step in CTAs of 64 threads: the three-method call gives the per-method calls' results bit for bit."""
+    rng = np.random.default_rng(5)
+    B, N, V = 793, 3, 8192
+    lp, lq = random_logits(rng, B, N, V, "bf16")
+    un = random_uniforms(rng, B, N)
+    tq, und, tree = padded(workloads.round_to_storage(lq, "bf16"), "bf16", 0), torch.from_numpy(un).cuda(), sh.Tree.heap(N)
+    out = sh.mdsd_compare_draft_sample_stats(tq, und, tree, 1.0)
+    for m in METHODS:
+        one = gpu_draft_stats(sh, m, tq, und, tree, 1.0)
+        assert torch.equal(one["tokens"], out[m]["tokens"]), m
+        assert torch.equal(one["stats"], out["stats"]), m
