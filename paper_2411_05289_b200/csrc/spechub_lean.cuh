@@ -607,12 +607,11 @@ __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, in
                                                LeanAcc<LT> &Q, float *cks, float *ckc, int slots) {
     LeanAcc<LT> st;
     st.init();
-    {   // one exponent reference for the whole warp: the maximum of its first vectors
-        float m0 = neg_inf();
-        if (lo + lane < hi) m0 = rq[lo + lane].max();
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m0 = fmaxf(m0, __shfl_xor_sync(kFull, m0, o));
-        if (m0 > neg_inf()) st.c = shift_of(m0, k);
+    // one exponent reference for the whole warp: the maximum of its first 32 vectors that hold a finite logit (nearly
+    // always the very first ones; a warp whose range begins with masked ids looks further)
+    for (int v0 = lo; v0 < hi; v0 += 32) {
+        const float m0 = lanes_max(v0 + lane < hi ? rq[v0 + lane].max() : neg_inf());
+        if (m0 > neg_inf()) { st.c = shift_of(m0, k); break; }
     }
     float cref = st.c;              // the reference every lane is expected to hold
     float tot = 0.f, ctot = st.c;   // this thread's sum over all checkpoints, on the scale ctot

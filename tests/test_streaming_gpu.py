@@ -1,0 +1,117 @@
+"""Streaming kernels, on calls with more rows than the kernels that hold rows in registers take: rows that are hard on
+their sums and draws, in all row formats, with and without leaf rows, two and more drafts, against the oracle on a
+sample of the rows."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+import oracle  # noqa: E402
+import parity  # noqa: E402
+import workloads  # noqa: E402
+from test_kary_gpu import close  # noqa: E402
+from test_parity_gpu import (METHODS, gpu_draft, gpu_draft_stats, gpu_verify, gpu_verify_stats, padded, random_logits,  # noqa: E402,F401
+                             random_uniforms, sh)
+
+# (V, dtype, ids between row starts are a multiple of pad): whole words and rows of any alignment, both types
+FORMATS = [(8192, "bf16", 0), (9001, "bf16", 0), (8192, "fp32", 0), (8201, "fp32", 0)]
+
+
+def batch_that_streams(nodes, V, dtype):
+    """Sequences whose rows are certain to be streamed: a warp holds at most 2048 bf16 or 1024 fp32 ids in registers,
+    rows of one or two warps are always held so, and no more than 25 warps per SM are."""
+    warps = -(-V // (2048 if dtype == "bf16" else 1024))
+    assert warps > 2
+    return 25 * 148 // (warps * nodes) + 2
+
+
+def sample(rng, B, first=8, n=12):
+    return np.unique(np.concatenate([np.arange(first), [B - 1], rng.integers(0, B, n)]))
+
+
+def check_two_drafts(sh, lp, lq, dtype, pad, T, un, leaves, pick, label, stats=False):  # noqa: F811
+    """Both steps on all rows, the sequences `pick` against the oracle."""
+    N = lp.shape[1]
+    tp, tq, und = padded(lp, dtype, pad), padded(lq, dtype, pad), torch.from_numpy(un).cuda()
+    tree, kind = sh.Tree.heap(N, leaves_sample=leaves), workloads.paper_node_kind(N) if leaves else None
+    for m in METHODS:
+        d = (gpu_draft_stats if stats else gpu_draft)(sh, m, tq, und, tree, T)
+        if stats:
+            out = gpu_verify_stats(sh, m, tp, tq, d["stats"], d["tokens"], und, tree, T)
+        else:
+            out = gpu_verify(sh, m, tp, tq, d["tokens"], und, tree, T)
+        d, out = parity.to_numpy(d), parity.to_numpy(out)
+        parity.check_draft(m, lq[pick], T, un[pick], {k: v[pick] for k, v in d.items() if k != "stats"}, label=label)
+        parity.check_verify(m, lp[pick], lq[pick], T, d["tokens"][pick], un[pick], kind,
+                            {k: v[pick] for k, v in out.items()}, label=label)
+
+
+def check_more_drafts(sh, k, wo, lp, lq, dtype, pad, T, un, leaves, pick, label):  # noqa: F811
+    """RRS / RRSw with k drafts per node, complete k-ary tree of two levels (as test_kary_gpu.check, on a sample)."""
+    N = lp.shape[1]
+    tree = sh.Tree.kary(k, 2, leaves_sample=leaves)
+    kind = np.array([0] + [1] * k, np.uint8) if leaves else None
+    tp, tq, und = padded(lp, dtype, pad), padded(lq, dtype, pad), torch.from_numpy(un).cuda()
+    d = sh.rrs_draft_sample(tq, und, tree, wo, T)
+    out = parity.to_numpy(sh.rrs_verify_tree(tp, tq, d["tokens"], und, tree, wo, T))
+    d = {key: v[pick] for key, v in parity.to_numpy(d).items()}
+    out = {key: v[pick] for key, v in out.items()}
+    lp, lq, un = lp[pick], lq[pick], un[pick]
+    od = oracle.rrs_k_draft_batch(k, wo, lq, T, un)
+    ov = oracle.rrs_k_verify_batch(k, wo, lp, lq, T, d["tokens"], un, kind)
+    for b in range(len(pick)):
+        for n in range(N):
+            ctx = "%s k=%d wo=%s b=%d n=%d V=%d" % (label, k, wo, pick[b], n, lp.shape[2])
+            if tuple(d["tokens"][b, n]) == tuple(od["tokens"][b, n]):
+                assert d["status"][b, n] == od["status"][b, n], ctx
+            else:   # every draw admissible given the earlier ones
+                w, _ = oracle.softmax(lq[b, n], T)
+                for i, x in enumerate(d["tokens"][b, n]):
+                    lo, hi = oracle.cdf_interval(w, int(x))
+                    assert lo - parity.NEAR <= un[b, n, i] <= hi + parity.NEAR, ("draft", ctx, i)
+                    if wo:
+                        w[x] = 0.0
+            token, o_token = int(out["token"][b, n]), int(ov["token"][b, n])
+            if kind is not None and kind[n] == 1:
+                if token != o_token:
+                    lo, hi = oracle.cdf_interval(oracle.softmax(lp[b, n], T)[0], token)
+                    assert lo - parity.NEAR <= un[b, n, 2 * k] <= hi + parity.NEAR, ctx
+                assert out["status"][b, n] == 0, ctx
+                continue
+            close(out["beta"][b, n], ov["beta"][b, n], ov["cond"][b, n], "beta", ctx)
+            close(out["rate"][b, n], ov["rate"][b, n], 0.0, "rate", ctx)
+            if token == o_token and out["accept_idx"][b, n] == ov["accept_idx"][b, n]:
+                assert out["status"][b, n] | 16 == ov["status"][b, n] | 16, ctx
+                continue
+            bands = [max(parity.NEAR, parity.EPS * c) for c in ov["cond"][b, n]] + [parity.NEAR]
+            assert any(m <= bd for m, bd in zip(ov["margin"][b, n], bands)), (ctx, token, o_token, ov["margin"][b, n])
+
+
+def mask_starts(x, V):
+    """-inf on the first 300 ids of every 128 vectors and more: whatever CTA shape, some warps' ranges begin with
+    ids that are all masked."""
+    for s in range(0, V, max(1024, V // 64 // 8 * 8)):
+        x[..., s:s + 300] = -np.inf
+
+
+@pytest.mark.parametrize("leaves", [False, True])
+@pytest.mark.parametrize("V,dtype,pad", FORMATS + [(32000, "bf16", 0)])
+def test_rows_that_begin_with_masked_ids_and_lie_low(sh, V, dtype, pad, leaves):  # noqa: F811
+    """The first ids of warps' ranges are masked and the others lie far below 0: exponentials on the scale of 0 would
+    all be 0."""
+    rng = np.random.default_rng(V + leaves)
+    B = batch_that_streams(3, V, dtype)
+    lp, lq = random_logits(rng, B, 3, V, dtype)
+    shift = np.float32([-200.0, -85.0])[np.arange(B) % 2][:, None, None]
+    lp, lq = lp + shift, lq + shift
+    mask_starts(lp, V)
+    mask_starts(lq, V)
+    lp, lq = workloads.round_to_storage(lp, dtype), workloads.round_to_storage(lq, dtype)
+    check_two_drafts(sh, lp, lq, dtype, pad, 1.0, random_uniforms(rng, B, 3), leaves, sample(rng, B), "masked")
+    B = batch_that_streams(4, V, dtype)
+    lp, lq = np.resize(lp, (B, 4, V)), np.resize(lq, (B, 4, V))
+    un = rng.integers(0, 1 << 24, (B, 4, 7)).astype(np.float32) * np.float32(2.0 ** -24)
+    for wo in (False, True):
+        check_more_drafts(sh, 3, wo, lp, lq, dtype, pad, 1.0, un, leaves, sample(rng, B), "masked")
