@@ -251,6 +251,47 @@ __device__ __forceinline__ float warp_sum(float x) {
     return x;
 }
 
+// ---- a row's mass in twice the precision ------------------------------------------------------
+// The coarse pick of an inverse-CDF draw compares a prefix of the row's masses with a target.  Both are as large as the
+// row's mass, and an id may be 1e-6 of it: in fp32 the roundings of prefix and target decide some draws (share that take
+// another id than fp64 throughout, rows of 128256 fp32 ids, T = 1: 0.0030; so 0.0016, what is left are the roundings of
+// the masses).  Unevaluated sums of two floats: fp64 took more registers than the passes of some kernels leave (a step on
+// 480 rows of 128256 fp32 ids 154 us, in fp64 156 to 165).
+struct Pair { float hi, lo; };
+__device__ __forceinline__ Pair pair_add(Pair a, Pair b) {   // Knuth's two-sum
+    const float s = __fadd_rn(a.hi, b.hi), t = __fsub_rn(s, a.hi);
+    const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, t)), __fsub_rn(b.hi, t));
+    return {s, __fadd_rn(e, __fadd_rn(a.lo, b.lo))};
+}
+__device__ __forceinline__ Pair pair_times(float u, Pair a) {
+    const float p = __fmul_rn(u, a.hi);
+    return {p, __fmaf_rn(u, a.lo, __fmaf_rn(u, a.hi, -p))};
+}
+__device__ __forceinline__ float pair_diff(Pair a, Pair b) { return __fadd_rn(__fsub_rn(a.hi, b.hi), __fsub_rn(a.lo, b.lo)); }
+__device__ __forceinline__ Pair pair_shfl(Pair a, int lane) { return {__shfl_sync(kFull, a.hi, lane), __shfl_sync(kFull, a.lo, lane)}; }
+__device__ __forceinline__ Pair pair_prefix(float m) {   // inclusive, over ascending lanes
+    const int lane = threadIdx.x & 31;
+    Pair x = {m, 0.f};
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const Pair up = {__shfl_up_sync(kFull, x.hi, o), __shfl_up_sync(kFull, x.lo, o)};
+        if (lane >= o) x = pair_add(up, x);
+    }
+    return x;
+}
+// Inverse-CDF pick over one mass per lane with the target u times the lanes' total: the lowest lane with mass whose
+// inclusive prefix exceeds the target, the last lane with mass if none does; -1: no mass.  t_in = the target within the
+// lane.  The same in every lane.
+__device__ __forceinline__ int pair_pick(float m, float u, float &t_in) {
+    const Pair incl = pair_prefix(m);
+    const float beyond = pair_diff(incl, pair_times(u, pair_shfl(incl, 31)));
+    const unsigned pos = __ballot_sync(kFull, m > 0.f), hit = __ballot_sync(kFull, m > 0.f && beyond > 0.f);
+    if (!pos) return -1;
+    const int L = hit ? __ffs(hit) - 1 : 31 - __clz(pos);
+    t_in = __shfl_sync(kFull, m - beyond, L);
+    return L;
+}
+
 // ---- inverse-CDF draw over a row, CTA-wide ----------------------------------------------------
 // mass[w] (shared memory) = total weight of warp w's range.  weights(vi, w[]) must
 // return the VW weights of vector vi (0 for ids that carry no mass or lie past V)

@@ -419,22 +419,24 @@ __device__ int range_sample3(int lo, int hi, WF weights, LeanShared &sh, float t
     return sh.tok;   // (written again only after the first barrier of a later draw)
 }
 
-// ... over this CTA's part of a row: mass[w] = total weight of warp w's range (the coarse CDF), t = target prefix
-// within this part
-template <class WF>
-__device__ int block_sample3(const Geo &g, WF weights, const float *mass, LeanShared &sh, float t) {
+// ... over this CTA's part of a row: mass[w] = total weight of warp w's range (the coarse CDF).  WHOLE: the part is the
+// row and u the uniform; else u is the target prefix within the part.
+template <bool WHOLE, class WF>
+__device__ int block_sample3(const Geo &g, WF weights, const float *mass, LeanShared &sh, float u) {
     const int lane = threadIdx.x & 31;
-    const int w = lanes_pick(lane < g.nwarps ? mass[lane] : 0.f, t);
+    const float m = lane < g.nwarps ? mass[lane] : 0.f;
+    float t = u;
+    const int w = WHOLE ? pair_pick(m, u, t) : lanes_pick(m, t);
     if (w < 0) return -1;
     return range_sample3(g.seg_lo(w), g.seg_hi(w), weights, sh, t);
 }
 
 // Pick the CTA of a row whose part holds the target t of an inverse-CDF draw over per-CTA masses
 // m[0..n) (ascending token ranges).  Returns the rank (-1 if no mass) and the mass before it.
-__device__ __forceinline__ int pick_part(const float *m, int n, float t, float &base) {
+__device__ __forceinline__ int pick_part(const float *m, int n, double t, double &base) {
     int sel = -1, last = -1;
-    float lastbase = 0.f, run = 0.f;
-    base = 0.f;
+    double lastbase = 0., run = 0.;
+    base = 0.;
     for (int r = 0; r < n; ++r) {
         if (m[r] > 0.f) {
             last = r;
@@ -482,12 +484,12 @@ __device__ __forceinline__ float slice_mass(const LeanShared &sh, int r, const R
     return (ps->x_sx[r] + own) * rescale(ml, shift_of(ml, k), st.C);
 }
 
-// Draw inside this CTA's slice from softmax(row) without token `excl`, target t (row scale,
-// relative to the start of the slice).  sh.wmass[r] holds the per-warp sums of the slice on the
+// Draw inside this CTA's slice from softmax(row) without token `excl`.  u: target (row scale, relative to the start of
+// the slice); CS = 1: the uniform.  sh.wmass[r] holds the per-warp sums of the slice on the
 // slice's own scale.
-template <class ROW>
+template <int CS, class ROW>
 __device__ int lean_sample_slice(const Geo &g, const ROW &row, float k, const RowStat &st,
-                                 int excl, float t, int r, LeanShared &sh) {
+                                 int excl, float u, int r, LeanShared &sh) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int locarg = sh.x_idx[r];
     const float lml = sh.x_ml[r];
@@ -518,7 +520,7 @@ __device__ int lean_sample_slice(const Geo &g, const ROW &row, float k, const Ro
 #pragma unroll
         for (int i = 0; i < 8; ++i) w[i] = (vi * 8 + i == excl) ? 0.f : ex2(__fmaf_rn(v.get(i), k, -C));
     };
-    return block_sample3(g, wf, sh.mass, sh, t);
+    return block_sample3<CS == 1>(g, wf, sh.mass, sh, u);
 }
 
 // Draw from softmax(row) without `excl` (the row argmax, a slice argmax, or nothing) over the
@@ -528,14 +530,15 @@ template <int CS, class ROW>
 __device__ int lean_sample_row(const Geo &g, const ROW &row, float k, const RowStat &st, int me,
                                int excl, float u, int r, LeanShared &sh) {
     float m[CS];
-    float total = 0.f;
+    double total = 0.;
 #pragma unroll
     for (int c = 0; c < CS; ++c) { m[c] = slice_mass<CS>(sh, r, st, c, excl, k); total += m[c]; }
-    if (!(total > 0.f)) return -1;
-    float base;
+    if (!(total > 0.)) return -1;
+    if (CS == 1) return lean_sample_slice<1>(g, row, k, st, excl, u, r, sh);
+    double base;
     const int sel = pick_part(m, CS, u * total, base);
     if (sel != me) return -2;
-    return lean_sample_slice(g, row, k, st, excl, u * total - base, r, sh);
+    return lean_sample_slice<CS>(g, row, k, st, excl, static_cast<float>(u * total - base), r, sh);
 }
 
 // CTA sums of NACC per-thread accumulators; the per-warp sums stay in sh.acc[OFF + i][w].  ANY: also whether `any` is
@@ -731,10 +734,9 @@ __device__ __forceinline__ int lean_ck_draw(const Geo &g, const ROW &row, float 
     };
     float ls = 0.f;
     for (int i = 0; i < per; ++i) ls += slot_mass(lane * per + i);
-    const float total = __shfl_sync(kFull, lanes_prefix(ls), 31);
-    if (!(total > 0.f)) return -1;
-    float t = u * total;
-    int slot = lanes_pick(ls, t);
+    float t;
+    int slot = pair_pick(ls, u, t);
+    if (slot < 0) return -1;
     if (per > 1) {   // the sub-block within the lane's
         const int first = slot * per;
         int last = -1;
@@ -1120,8 +1122,9 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
             }
             if (!(acc1 || acc2)) {
                 o.accept_idx = -1;
-                float base = 0.f;
-                const int sel = (Rraw > 0.f) ? pick_part(part[2], CS, ures * Rraw, base) : -1;
+                const double target = static_cast<double>(ures) * Rraw;   // (CS > 1)
+                double base = 0.;
+                const int sel = (Rraw > 0.f) ? pick_part(part[2], CS, target, base) : -1;
                 if (sel < 0) {
                     o.status |= SPECHUB_ST_ZERO_RESIDUAL;
                     draw_from_p();
@@ -1137,7 +1140,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
                                 w[i] = (vi * 8 + i == hubtok) ? 0.f : fmaxf(t, 0.f);
                             }
                         };
-                        const int tok = block_sample3(g, wf, mass_r, sh, ures * Rraw - base);
+                        const int tok = block_sample3<CS == 1>(g, wf, mass_r, sh, CS == 1 ? ures : static_cast<float>(target - base));
                         if (threadIdx.x == 0) a.token[r] = tok;
                     }
                 }
@@ -1312,8 +1315,9 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
             if (!acc1 && acc2) { o.accept_idx = 1; o.token = x2; }
             if (!(acc1 || acc2)) {
                 o.accept_idx = -1;
-                float base = 0.f;
-                const int sel = (A1 > 0.f && W2raw > 0.f) ? pick_part(part1[0], CS, ures * W2raw, base) : -1;
+                const double target = static_cast<double>(ures) * W2raw;   // (CS > 1)
+                double base = 0.;
+                const int sel = (A1 > 0.f && W2raw > 0.f) ? pick_part(part1[0], CS, target, base) : -1;
                 if (sel < 0) {
                     o.status |= SPECHUB_ST_ZERO_RESIDUAL;
                     draw_from_p();
@@ -1330,7 +1334,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
                                 w[i] = fmaxf(t, 0.f);
                             }
                         };
-                        const int tok = block_sample3(g, wf, sh.acc[2], sh, ures * W2raw - base);
+                        const int tok = block_sample3<CS == 1>(g, wf, sh.acc[2], sh, CS == 1 ? ures : static_cast<float>(target - base));
                         if (threadIdx.x == 0) a.token[r] = tok;
                     }
                 }
@@ -1442,7 +1446,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_kernel(Row
             const int ox = min((x1 >> 3) / per, CS - 1);
             const float lx1 = load_one<__nv_bfloat16>(rowq, x1);
             float m[CS];
-            float total = 0.f;
+            double total = 0.;
 #pragma unroll
             for (int c = 0; c < CS; ++c) {
                 m[c] = slice_mass<CS>(sh, 0, Q, c, x1, k);
@@ -1451,13 +1455,13 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_kernel(Row
                 total += m[c];
             }
             x2_elsewhere = true;
-            float base = 0.f;
-            const int sel = (total > 0.f) ? pick_part(m, CS, u2 * total, base) : -1;
+            double base = 0.;
+            const int sel = (total > 0.) ? pick_part(m, CS, u2 * total, base) : -1;
             if (sel < 0) {
                 st |= SPECHUB_ST_DEGENERATE_Q;
                 if (writer) a.draft_tokens_out[2 * r + 1] = (x1 == 0) ? 1 : 0;
             } else if (sel == me) {
-                const int t2 = lean_sample_slice(g, vq, k, Q, x1, u2 * total - base, 0, sh);
+                const int t2 = lean_sample_slice<CS>(g, vq, k, Q, x1, static_cast<float>(u2 * total - base), 0, sh);
                 if (threadIdx.x == 0) a.draft_tokens_out[2 * r + 1] = t2;
             }
         }

@@ -272,8 +272,8 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_kary_
             const int i = __ffs(sg) - 1;
             if (g.warp_of_vec(sh.x[i] >> 3) == lane) wm += zero ? ep(i) : fmaxf(__fmaf_rn(-sh.cx[i] * rho, eq(i), ep(i)), 0.f);
         }
-        float t = sh.u[K] * warp_sum(wm);
-        const int w = lanes_pick(wm, t);
+        float t;
+        const int w = pair_pick(wm, sh.u[K], t);
         if (w >= 0)
             token = range_sample3(g.seg_lo(w), g.seg_hi(w), [&](int vi, float(&out)[8]) {
                 const V x = vp[vi], y = vq[vi];

@@ -28,7 +28,7 @@ namespace cg = cooperative_groups;
 
 constexpr int kRegMaxParts = 128;   // warps per row: 16 x a cluster of 8
 constexpr int kRegThreads = 512;    // threads of a CTA, at most
-constexpr int kRegPer = kRegMaxParts / 32;   // records per lane: lane l holds those of the parts l, 32 + l, ...
+constexpr int kRegPer = kRegMaxParts / 32;   // records per lane, at most: consecutive parts
 
 struct RegGeo { int w, cs, rows_per_cta, seg; };   // warps per row and CTA, CTAs per row, rows per CTA, vectors per part
 
@@ -43,6 +43,7 @@ struct RegRow {   // this warp's place in its row
     int part, parts, slot0;    // its part, the parts of the row, the row's first record
     int lo, hi, seg;           // its vectors; vectors per part
     int nj, lv;                // vectors per lane, this lane's first (the others follow at distances of 32)
+    int per;                   // records per lane
     int w, cs, rows_per_cta, group;
     unsigned r;                // the row
 
@@ -55,6 +56,7 @@ struct RegRow {   // this warp's place in its row
         r = cs > 1 ? blockIdx.x / cs : blockIdx.x * rows_per_cta + group;
         part = rank * w + (warp - slot0);
         parts = w * cs;
+        per = (parts + 31) >> 5;
         const int nvec = (vocab + 7) / 8;
         lo = min(part * seg, nvec);
         hi = min(lo + seg, nvec);
@@ -208,18 +210,20 @@ __device__ __forceinline__ PartStat part_stat(const RegRow &g, const RegVecs<LT,
 
 // ---- row values from the parts' records -------------------------------------------------------------
 struct RegStat { float ml, C, Z, sx, own; int idx; };
-// One value per part: lane l holds those of the parts l, 32 + l, ...
+// One value per part: lane l holds those of the parts l * per, l * per + 1, ...
 struct PerPart {
     float m[kRegPer];
-    __device__ __forceinline__ void set(int s, float v) {
+    __device__ __forceinline__ void set(const RegRow &g, int s, float v) {
+        s -= static_cast<int>(threadIdx.x & 31) * g.per;
 #pragma unroll
         for (int i = 0; i < kRegPer; ++i)
-            if (s == i * 32 + static_cast<int>(threadIdx.x & 31)) m[i] = v;
+            if (i < g.per && s == i) m[i] = v;
     }
-    __device__ __forceinline__ void add(int s, float v) {
+    __device__ __forceinline__ void add(const RegRow &g, int s, float v) {
+        s -= static_cast<int>(threadIdx.x & 31) * g.per;
 #pragma unroll
         for (int i = 0; i < kRegPer; ++i)
-            if (s == i * 32 + static_cast<int>(threadIdx.x & 31)) m[i] += v;
+            if (i < g.per && s == i) m[i] += v;
     }
 };
 
@@ -251,7 +255,7 @@ __device__ __forceinline__ RegStat merge_parts(const RegRow &g, const REC *rec, 
     for (int i = 0; i < kRegPer; ++i) {
         a[i] = REC{};
         a[i].x = neg_inf();
-        if (i * 32 + lane < g.parts) a[i] = rec[g.slot0 + i * 32 + lane];
+        if (i < g.per && lane * g.per + i < g.parts) a[i] = rec[g.slot0 + lane * g.per + i];
         ml = fmaxf(ml, a[i].x);
     }
     o.ml = warp_max(ml);
@@ -267,7 +271,7 @@ __device__ __forceinline__ RegStat merge_parts(const RegRow &g, const REC *rec, 
 #pragma unroll
     for (int i = 0; i < kRegPer; ++i) {
         if (MASS) mass->m[i] = 0.f;
-        if (i * 32 < g.parts) {
+        if (i < g.per) {
             const float f = rescale(a[i].x, shift_of(a[i].x, k), o.C);
             const float m = __fmul_rn(a[i].y, f);
             z = __fadd_rn(z, m);
@@ -291,31 +295,23 @@ __device__ __forceinline__ int pick_part_of(const RegRow &g, const PerPart &mass
         t_in = u * m;
         return m > 0.f ? 0 : -1;
     }
-    float tot[kRegPer], total = 0.f;
-#pragma unroll
-    for (int i = 0; i < kRegPer; ++i) {
-        tot[i] = i * 32 < g.parts ? warp_sum(mass.m[i]) : 0.f;
-        total += tot[i];
-    }
-    if (!(total > 0.f)) return -1;
-    const float t = u * total;
-    // the group of 32 parts
-    float run = 0.f, base = 0.f, m = 0.f;
-    int grp = -1;
+    static_assert(kRegPer == 4, "a lane's masses");
+    const int L = pair_pick((mass.m[0] + mass.m[1]) + (mass.m[2] + mass.m[3]), u, t_in);
+    if (L < 0 || g.per == 1) return L;
+    // the part within the lane's
+    float run = 0.f, base = 0.f;
+    int at = 0;
     bool found = false;
 #pragma unroll
     for (int i = 0; i < kRegPer; ++i) {
-        if (tot[i] > 0.f && !found) {
-            grp = i; base = run; m = mass.m[i];
-            found = run + tot[i] > t;
+        if (mass.m[i] > 0.f && !found) {
+            at = i; base = run;
+            found = run + mass.m[i] > t_in;
         }
-        run += tot[i];
+        run += mass.m[i];
     }
-    const float incl = warp_prefix(m);
-    const unsigned pos = __ballot_sync(kFull, m > 0.f), hit = __ballot_sync(kFull, m > 0.f && incl > t - base);
-    const int L = hit ? __ffs(hit) - 1 : 31 - __clz(pos);
-    t_in = __shfl_sync(kFull, (t - base) - (incl - m), L);
-    return grp * 32 + L;
+    t_in -= __shfl_sync(kFull, base, L);
+    return L * g.per + __shfl_sync(kFull, at, L);
 }
 
 // The sums of a pass from the parts' records; the third one's parts are kept for a draw.
@@ -331,8 +327,8 @@ __device__ __forceinline__ float4 sum_parts(const RegRow &g, const float4 *rec, 
 #pragma unroll
     for (int i = 0; i < kRegPer; ++i) {
         third.m[i] = 0.f;
-        if (i * 32 + lane < g.parts) {
-            const float4 a = rec[g.slot0 + i * 32 + lane];
+        if (i < g.per && lane * g.per + i < g.parts) {
+            const float4 a = rec[g.slot0 + lane * g.per + i];
             s.x += a.x; s.y += a.y; s.z += a.z;
             third.m[i] = a.z;
         }
@@ -496,7 +492,7 @@ __global__ void __launch_bounds__(kRegThreads) reg_draft_kernel(KaryArgs A, int 
                 g.post(&sh.drawn[i][g.group], make_float2(__int_as_float(tok), rest));
             }
             g.sync();
-            mass.set(s, sh.drawn[i][g.group].y);
+            mass.set(g, s, sh.drawn[i][g.group].y);
         }
         if (lead)
             for (int i = 0; i < K; ++i) a.draft_tokens_out[K * r + i] = drawn(i);
@@ -872,7 +868,7 @@ __global__ void __launch_bounds__(kRegThreads) reg_verify_rrs_kernel(KaryArgs A,
             if (single[i]) {   // (a draft that is still in q has the C of all ids)
                 const float v = fmaxf(__fmaf_rn(-(i <= j ? Cx[i] : C) * rho, eq1[i], ep1[i]), 0.f);
                 m_next += v;
-                mass.add(g.part_of(x[i]), v);
+                mass.add(g, g.part_of(x[i]), v);
             }
         m_next *= invZp;
         rate[j] = alive ? fmaxf(m - m_next, 0.f) : 0.f;
@@ -917,7 +913,7 @@ __global__ void __launch_bounds__(kRegThreads) reg_verify_rrs_kernel(KaryArgs A,
             for (int i = 0; i < MK; ++i)
                 if (single[i]) {
                     which |= 1u << i;
-                    mp.add(g.part_of(x[i]), ep1[i]);
+                    mp.add(g, g.part_of(x[i]), ep1[i]);
                 }
             reg_draw_from_p(g, mp, p, rowp, a.vocab, k, P.C, x, which, ures, a.token + r);
         }

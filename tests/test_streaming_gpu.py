@@ -115,3 +115,29 @@ def test_rows_that_begin_with_masked_ids_and_lie_low(sh, V, dtype, pad, leaves):
     un = rng.integers(0, 1 << 24, (B, 4, 7)).astype(np.float32) * np.float32(2.0 ** -24)
     for wo in (False, True):
         check_more_drafts(sh, 3, wo, lp, lq, dtype, pad, 1.0, un, leaves, sample(rng, B), "masked")
+
+
+@pytest.mark.parametrize("V,dtype,rows,calls,most", [(128256, "fp32", 1024, 8, 0.0022), (50257, "bf16", 2048, 8, 0.0006)])
+def test_draws_take_the_ids_that_fp64_takes(sh, V, dtype, rows, calls, most):  # noqa: F811
+    """Draws by the prefix sums of whole rows: an id of the flat tail weighs 1e-6 of its row, a few fp32 roundings of the
+    row's mass.  What is left are the roundings of the masses themselves (0.0016 and 0.0003 of the draws; with prefixes
+    and targets in fp32 too, 0.0030 and 0.0012): the limits lie between the two."""
+    leaf = sh.Tree.heap(1)
+    leaf.node_kind = torch.ones(1, dtype=torch.uint8, device="cuda")
+    off = n = 0
+    for call in range(calls):
+        gen = torch.Generator(device="cuda")
+        gen.manual_seed(1000 + call * rows)
+        prior = -1.2 * torch.log1p(torch.randperm(V, generator=gen, device="cuda").float())
+        logits = torch.randn((rows, V), generator=gen, device="cuda") + prior
+        logits = logits.to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+        un = torch.randint(0, 1 << 24, (rows, 1, 5), generator=gen, device="cuda").float() * 2.0 ** -24
+        cdf = logits.double().softmax(1).cumsum(1)
+        x = logits[:, None, :]
+        drafts = sh.rrs_draft_sample(x, un, sh.Tree.heap(1), False)["tokens"][:, 0]
+        bonus = sh.rrs_verify_tree(x, x, drafts[:, None].contiguous(), un, leaf, False)["token"][:, 0]
+        for u, got in ((0, drafts[:, 0]), (1, drafts[:, 1]), (4, bonus)):
+            want = torch.searchsorted(cdf, un[:, 0, u:u + 1].double() * cdf[:, -1:], right=True)[:, 0].clamp(max=V - 1)
+            off += int((got != want).sum())
+            n += rows
+    assert off <= most * n, (off, n)
