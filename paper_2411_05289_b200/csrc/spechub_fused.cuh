@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
                         w[i] = (vi * 8 + i == hubtok) ? 0.f : fmaxf(t, 0.f);
                     }
                 };
-                tok = block_sample3<true>(g, wf, mass_r, sh, ures);
+                tok = block_sample3<true, true>(g, wf, mass_r, sh, ures);
             } else {
                 s.status |= SPECHUB_ST_ZERO_RESIDUAL;
                 tok = draw_from_p();
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
                         w[i] = fmaxf(t, 0.f);
                     }
                 };
-                tok = block_sample3<true>(g, wf, sh.acc[5 + m], sh, ures);
+                tok = block_sample3<true, true>(g, wf, sh.acc[5 + m], sh, ures);
             } else {
                 s.status |= SPECHUB_ST_ZERO_RESIDUAL;
                 tok = draw_from_p();

@@ -419,14 +419,28 @@ __device__ int range_sample3(int lo, int hi, WF weights, LeanShared &sh, float t
     return sh.tok;   // (written again only after the first barrier of a later draw)
 }
 
+// (a call instead of inlined code: where a kernel draws several times, that takes registers from its passes)
+struct LanePick { int lane; float t; };
+static __device__ __noinline__ LanePick pair_pick_call(float m, float u) {
+    LanePick o;
+    o.lane = pair_pick(m, u, o.t);
+    return o;
+}
 // ... over this CTA's part of a row: mass[w] = total weight of warp w's range (the coarse CDF).  WHOLE: the part is the
-// row and u the uniform; else u is the target prefix within the part.
-template <bool WHOLE, class WF>
+// row and u the uniform; else u is the target prefix within the part.  CALL: pick by pair_pick_call.
+template <bool WHOLE, bool CALL = false, class WF>
 __device__ int block_sample3(const Geo &g, WF weights, const float *mass, LeanShared &sh, float u) {
     const int lane = threadIdx.x & 31;
     const float m = lane < g.nwarps ? mass[lane] : 0.f;
     float t = u;
-    const int w = WHOLE ? pair_pick(m, u, t) : lanes_pick(m, t);
+    int w;
+    if (WHOLE && CALL) {
+        const LanePick x = pair_pick_call(m, u);
+        w = x.lane;
+        t = x.t;
+    } else {
+        w = WHOLE ? pair_pick(m, u, t) : lanes_pick(m, t);
+    }
     if (w < 0) return -1;
     return range_sample3(g.seg_lo(w), g.seg_hi(w), weights, sh, t);
 }
@@ -610,15 +624,19 @@ __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, in
                                                LeanAcc<LT> &Q, float *cks, float *ckc, int slots) {
     LeanAcc<LT> st;
     st.init();
-    // one exponent reference for the whole warp: the maximum of its first 32 vectors that hold a finite logit (nearly
-    // always the very first ones; a warp whose range begins with masked ids looks further)
-    for (int v0 = lo; v0 < hi; v0 += 32) {
-        const float m0 = lanes_max(v0 + lane < hi ? rq[v0 + lane].max() : neg_inf());
-        if (m0 > neg_inf()) { st.c = shift_of(m0, k); break; }
-    }
-    float cref = st.c;              // the reference every lane is expected to hold
-    float tot = 0.f, ctot = st.c;   // this thread's sum over all checkpoints, on the scale ctot
+    float cref = 0.f;               // the reference every lane is expected to hold
+    float tot = 0.f, ctot = 0.f;    // this thread's sum over all checkpoints, on the scale ctot
     int j = 0;
+    // One exponent reference for the whole warp: the maximum of its first 32 vectors that hold a finite logit (nearly
+    // always the very first ones; a warp whose range begins with masked ids looks further).  Behind the pass's first
+    // loads (a step on 448 rows of 32000 ids: 44.9 us, 46.0 where they wait for the search).
+    auto reference = [&]() {
+        float m0 = lanes_max(lo + lane < hi ? rq[lo + lane].max() : neg_inf());
+#pragma unroll 1
+        for (int vb = lo + 32; !(m0 > neg_inf()) && vb < hi; vb += 32)
+            m0 = lanes_max(vb + lane < hi ? rq[vb + lane].max() : neg_inf());
+        st.c = cref = ctot = shift_of(m0, k);
+    };
     // checkpoint: the warp's sum since the last one.  A lane that had to move its reference (sums
     // beyond 2^100, rare) is brought to the warp's largest reference first.
     auto checkpoint = [&]() {
@@ -656,11 +674,12 @@ __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, in
     // (the loads of the next vectors also overlap the checkpoint's shuffle chain)
     if constexpr (SHIFT) {
         const InsideIters t = inside_iters(rq.src, rq.src, lo, hi);
+        reference();
         slow(t.i0);
-        if (rq.src.sh == 0) it = inside_ahead(AlignedInside<LT>{rq.src}, v0, it, t.i1, push, after);
-        else it = inside_ahead(ShiftedInside<LT>{rq.src}, v0, it, t.i1, push, after);
+        if (rq.src.sh == 0) it = inside_ahead(AlignedInside<LT>{rq.src}, v0, it, t.i1, [] {}, push, after);
+        else it = inside_ahead(ShiftedInside<LT>{rq.src}, v0, it, t.i1, [] {}, push, after);
     } else {
-        it = inside_ahead(rq, v0, it, nfull, push, after);
+        it = inside_ahead(rq, v0, it, nfull, reference, push, after);
     }
     slow(iters);
     if (since > 0) checkpoint();

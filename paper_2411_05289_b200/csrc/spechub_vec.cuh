@@ -343,15 +343,17 @@ __device__ __forceinline__ InsideIters inside_iters(const RowVecs<LT> &a, const 
 }
 
 // Loops over the inside of one row, kDepth vectors per lane in flight: the next ones are requested before the
-// current ones are used.  f(vector); after(D) is called after every D iterations.  Returns the iteration reached.
-template <class IN, class F, class AFTER>
-__device__ __forceinline__ int inside_ahead(const IN &row, int v0, int it, int i1, F f, AFTER after) {
+// current ones are used.  begin() is called once, with the first ones requested; f(vector); after(D) is called after
+// every D iterations.  Returns the iteration reached.
+template <class IN, class BEGIN, class F, class AFTER>
+__device__ __forceinline__ int inside_ahead(const IN &row, int v0, int it, int i1, BEGIN begin, F f, AFTER after) {
     constexpr int D = IN::kDepth;
     typename IN::Raw nx[D] = {};
     if (it + D <= i1) {
 #pragma unroll
         for (int i = 0; i < D; ++i) nx[i] = row.fetch(v0 + 32 * (it + i));
     }
+    begin();
 #pragma unroll 1
     for (; it + D <= i1; it += D) {
         typename IN::Raw a[D];
