@@ -35,14 +35,13 @@ int verify_rows(const RowArgs &a, unsigned rows, cudaStream_t s) {
 }
 
 template <int METHOD>
-int launch_lean_verify_method(int format, int cs, RowArgs a, unsigned rows, cudaStream_t s) {
+int launch_lean_verify_method(int format, int cs, const RowArgs &a, unsigned rows, cudaStream_t s) {
     if (cs == 4) return verify_split<METHOD, 4>(a, rows, s);
     if (cs == 2) return verify_split<METHOD, 2>(a, rows, s);
     if (a.node_kind) {
         const NodeOutPtrs o = {a.accept_idx, a.token, a.hub, a.beta, a.rate, a.status};
         const int lrc = launch_lean_leaf(format, a, 2, &o, 1, rows, s);
         if (lrc != SPECHUB_OK) return lrc;
-        a.after_leaves = 1;
     }
     const bool stats = cs == 0 && a.draft_stats_in;
     if (format == kBf16Shift) return verify_rows<__nv_bfloat16, true, METHOD, false>(a, rows, s);

@@ -32,7 +32,6 @@ struct RowArgs {
     // per-row statistics of the draft logits, handed from the draft step to verification: [B][N] DraftStat
     void *draft_stats_out;       // draft step, may be NULL
     const void *draft_stats_in;  // verification through a *_stats entry point
-    int after_leaves;            // verification launched right behind the leaf rows' kernel of the same call
 };
 
 // What the draft step knows about a row of draft logits once it has read it, and what verification would

@@ -13,7 +13,7 @@ constexpr int kMaxDevices = 64;
 inline int launch_status() { return cudaGetLastError() == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH; }
 
 // One launch: `cs` CTAs per cluster (1: none), as a programmatic dependent of the stream's last kernel.  Only for
-// kernels that begin with pdl_begin() (or keep its promise otherwise).
+// kernels that begin with pdl_begin().
 template <class K, class... Args>
 int launch_grid(K kern, unsigned grid, int threads, int smem, int cs, cudaStream_t s, const Args &...args) {
     cudaLaunchConfig_t cfg = {};

@@ -901,10 +901,10 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
     __shared__ LeanShared sh;
     extern __shared__ __align__(128) unsigned char ring_mem[];
     __shared__ __align__(8) uint64_t ring_bars[RING ? THREADS / 32 : 1][kRingStages];
-    // After the leaf kernel of the same call, whose rows are others, this one need not wait: the leaf kernel let it be
-    // launched when it had waited itself.  One CTA waits at its end, so that this grid ends after the leaf kernel's.
-    if (!a.after_leaves) pdl_wait();
-    pdl_trigger();
+    // (Behind the leaf kernel of the same call, too: its rows are others, but what the kernels before it wrote is promised
+    // only to a grid that waits itself.  Without
+    // the wait a step with leaf rows took 163 us instead of 173 on 3840 rows of 32000 ids, 119 instead of 130 on 960 of 50257.)
+    pdl_begin();
     const int me = RowGroup<CS>::rank();
     const long long r = blockIdx.x / CS;
     const int b = static_cast<int>(r / a.nodes), n = static_cast<int>(r % a.nodes);
@@ -920,10 +920,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
     const float k = kLog2e / temperature_of(a, b);
     const float pinf = -neg_inf();
     // leaf rows of an unsplit call belong to lean_leaf_kernel
-    if (CS == 1 && a.node_kind && a.node_kind[n] == SPECHUB_NODE_LEAF) {
-        if (a.after_leaves && blockIdx.x == 0) pdl_wait();
-        return;
-    }
+    if (CS == 1 && a.node_kind && a.node_kind[n] == SPECHUB_NODE_LEAF) return;
     const bool leaf = CS > 1 && a.node_kind && a.node_kind[n] == SPECHUB_NODE_LEAF;
     const bool writer = (me == 0 && threadIdx.x == 0);
 
@@ -938,13 +935,9 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
     // by the last warp before it starts on pass A: two dependent look-ups that are off the path between the passes.
     // (Nothing else writes these fields; they are read after barriers.)
     if (warp == THREADS / 32 - 1) {
-        // (from L2: with the leaf kernel between them the draft step's kernel is not the one waited for)
-        const int t1 = __ldcg(a.draft_tokens_in + 2 * r), t2 = __ldcg(a.draft_tokens_in + 2 * r + 1);
+        const int t1 = a.draft_tokens_in[2 * r], t2 = a.draft_tokens_in[2 * r + 1];
         DraftStat ds = {};
-        if (STATS) {
-            const int4 rec = __ldcg(static_cast<const int4 *>(a.draft_stats_in) + r);
-            ds.ml = __int_as_float(rec.x); ds.sx = __int_as_float(rec.y); ds.idx = rec.z; ds.tag = static_cast<unsigned>(rec.w);
-        }
+        if (STATS) ds = static_cast<const DraftStat *>(a.draft_stats_in)[r];
         int y = lane > 4 ? -1 : lane == 4 ? (STATS ? ds.idx : -1) : (lane & 1) ? t2 : t1;
         if (leaf) y = -1;
         float l = neg_inf();
@@ -1375,7 +1368,6 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
         if (a.status) a.status[r] = o.status;
     }
     if (CS > 1) RowGroup<CS>::sync();  // no CTA leaves while another may still read its shared memory
-    if (a.after_leaves && blockIdx.x == 0) pdl_wait();
 }
 
 // ------------------------------------------------------------------------------------------------

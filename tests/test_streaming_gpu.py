@@ -141,3 +141,28 @@ def test_draws_take_the_ids_that_fp64_takes(sh, V, dtype, rows, calls, most):  #
             off += int((got != want).sum())
             n += rows
     assert off <= most * n, (off, n)
+
+
+@pytest.mark.parametrize("V,dtype", [(8192, "bf16"), (9001, "bf16"), (8192, "fp32")])
+def test_verification_with_leaf_rows_reads_what_the_kernel_before_it_wrote(sh, V, dtype):  # noqa: F811
+    """Logits, drafts and uniforms overwritten by kernels of the same stream right before the call, in buffers that the
+    call before it read: every call sees the new values."""
+    rng = np.random.default_rng(V)
+    B, tree = batch_that_streams(3, V, dtype), sh.Tree.heap(3, leaves_sample=True)
+    sets = []
+    for _ in range(3):
+        lp, lq = random_logits(rng, B, 3, V, dtype)
+        tp, tq, un = padded(lp, dtype, 0), padded(lq, dtype, 0), torch.from_numpy(random_uniforms(rng, B, 3)).cuda()
+        sets.append((tp, tq, un))
+    for m in METHODS:
+        drafts = [gpu_draft(sh, m, tq, un, tree, 1.0)["tokens"] for _, tq, un in sets]
+        want = [parity.to_numpy(gpu_verify(sh, m, tp, tq, d, un, tree, 1.0)) for (tp, tq, un), d in zip(sets, drafts)]
+        tp, tq, un, d = *(t.clone() for t in sets[0]), drafts[0].clone()
+        got = []
+        for i in range(9):
+            for buf, new in zip((tq, un, d, tp), (sets[i % 3][1], sets[i % 3][2], drafts[i % 3], sets[i % 3][0])):
+                buf.copy_(new)
+            got.append(gpu_verify(sh, m, tp, tq, d, un, tree, 1.0))
+        for i, out in enumerate(got):
+            for key, v in parity.to_numpy(out).items():
+                np.testing.assert_array_equal(v.view(np.int32), want[i % 3][key].view(np.int32), err_msg="%s %s" % (m, key))
