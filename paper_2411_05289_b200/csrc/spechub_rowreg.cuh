@@ -228,7 +228,8 @@ struct PerPart {
 };
 
 // `floor_ml`: a logit that the row's maximum is not below (ids left out of the parts); -inf if none.
-// MASS: also the parts' masses on the row's scale, for a draw.
+// MASS: also the parts' masses on the row's scale, for a draw: 0 for a part whose exponentials are all below the smallest
+// normal number there, 0, so that a picked part has an id to give.
 template <bool ARG, bool MASS, class REC>
 __device__ __forceinline__ RegStat merge_parts(const RegRow &g, const REC *rec, float k, float floor_ml, PerPart *mass) {
     const int lane = threadIdx.x & 31;
@@ -275,7 +276,7 @@ __device__ __forceinline__ RegStat merge_parts(const RegRow &g, const REC *rec, 
             const float f = rescale(a[i].x, shift_of(a[i].x, k), o.C);
             const float m = __fmul_rn(a[i].y, f);
             z = __fadd_rn(z, m);
-            if (MASS) mass->m[i] = m;
+            if (MASS) mass->m[i] = ex2(__fmaf_rn(a[i].x, k, -o.C)) > 0.f ? m : 0.f;
             if constexpr (ARG)
                 zx = __fadd_rn(zx, (a[i].x == o.ml && __float_as_int(a[i].w) == o.idx) ? __fmul_rn(a[i].z, f) : m);
         }
@@ -373,12 +374,6 @@ __device__ __forceinline__ int draw_in_part(const RegRow &g, int vocab, VF vec, 
     return y - lane + (h2 ? __ffs(h2) - 1 : 31 - __clz(p2));
 }
 
-// Parts' sums brought to the row's scale: those that may consist of exponentials below the smallest normal number there
-// (zero) count as zero, so that a picked part has an id to give.
-__device__ __forceinline__ void clean_masses(PerPart &mass) {
-#pragma unroll
-    for (int i = 0; i < kRegPer; ++i) mass.m[i] = mass.m[i] < 2.5e-35f ? 0.f : mass.m[i];   // (2048 ids of 2^-126)
-}
 // What a vector of a row weighs: its exponentials on the row's scale.
 template <typename LT>
 __device__ __forceinline__ float vec_mass(const Vec8<LT> &v, F2 k2, F2 nc2) {
@@ -428,7 +423,6 @@ __global__ void __launch_bounds__(kRegThreads) reg_draft_kernel(KaryArgs A, int 
         }
         return;
     }
-    clean_masses(mass);
     forget(q);
     uint32_t st = 0;
     const F2 k2 = f2_make(k, k), nc2 = f2_make(-Q.C, -Q.C);
@@ -521,7 +515,6 @@ __global__ void __launch_bounds__(kRegThreads) reg_draft_kernel(KaryArgs A, int 
 template <typename LT, int NV>
 __device__ __forceinline__ void reg_draw_from_p(const RegRow &g, PerPart mass, const RegVecs<LT, NV> &p, const LT *rowp, int vocab,
                                                 float k, float C, const int *out, unsigned which, float u, int32_t *token) {
-    clean_masses(mass);
     float t;
     if (pick_part_of(g, mass, u, t) != g.part) return;
     const F2 k2 = f2_make(k, k), nc2 = f2_make(-C, -C);

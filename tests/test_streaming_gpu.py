@@ -166,3 +166,20 @@ def test_verification_with_leaf_rows_reads_what_the_kernel_before_it_wrote(sh, V
         for i, out in enumerate(got):
             for key, v in parity.to_numpy(out).items():
                 np.testing.assert_array_equal(v.view(np.int32), want[i % 3][key].view(np.int32), err_msg="%s %s" % (m, key))
+
+
+@pytest.mark.parametrize("B", [2, 600])
+@pytest.mark.parametrize("V,dtype", [(8192, "bf16"), (8201, "fp32")])
+def test_second_drafts_from_next_to_nothing(sh, V, dtype, B):  # noqa: F811
+    """Nearly all mass on one id and 2^-120 of it on three others: they are what is left to draw from."""
+    rng = np.random.default_rng(V + B)
+    lq = np.full((B, 3, V), -np.inf, np.float32)
+    lq[:, :, 6000] = 4.0
+    lq[:, :, [100, 3000, 8000]] = 4.0 - 83.2
+    lq = workloads.round_to_storage(lq, dtype)
+    un, pick = random_uniforms(rng, B, 3), sample(rng, B, first=2)
+    tq, und = padded(lq, dtype, 0), torch.from_numpy(un).cuda()
+    for m in METHODS:
+        d = parity.to_numpy(gpu_draft(sh, m, tq, und, sh.Tree.heap(3), 1.0))
+        parity.check_draft(m, lq[pick], 1.0, un[pick], {k: v[pick] for k, v in d.items()}, label="next to nothing")
+        assert int(d["status"].max()) == 0, m
