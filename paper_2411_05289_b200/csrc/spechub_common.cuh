@@ -281,10 +281,12 @@ __device__ __forceinline__ Pair pair_prefix(float m) {   // inclusive, over asce
 }
 // Inverse-CDF pick over one mass per lane with the target u times the lanes' total: the lowest lane with mass whose
 // inclusive prefix exceeds the target, the last lane with mass if none does; -1: no mass.  t_in = the target within the
-// lane.  The same in every lane.
-__device__ __forceinline__ int pair_pick(float m, float u, float &t_in) {
-    const Pair incl = pair_prefix(m);
-    const float beyond = pair_diff(incl, pair_times(u, pair_shfl(incl, 31)));
+// lane.  The same in every lane.  `least`: targets are kept above it, unless the total is as small as that.
+__device__ __forceinline__ int pair_pick(float m, float u, float &t_in, float least = 0.f) {
+    const Pair incl = pair_prefix(m), total = pair_shfl(incl, 31);
+    Pair target = pair_times(u, total);
+    if (least > 0.f && target.hi < least && total.hi > least * 1e9f) target = {least, 0.f};
+    const float beyond = pair_diff(incl, target);
     const unsigned pos = __ballot_sync(kFull, m > 0.f), hit = __ballot_sync(kFull, m > 0.f && beyond > 0.f);
     if (!pos) return -1;
     const int L = hit ? __ffs(hit) - 1 : 31 - __clz(pos);

@@ -390,6 +390,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
     int x2[3];
     // RRS: an independent second draw (before a token is left out of the checkpoints' sums)
     x2[1] = lean_ck_draw(g, vq, k, Q.C, CK, NoneOut{}, u2, sh);
+    if (x2[1] < 0) x2[1] = hubtok;
     // RRSw: q with q(x1) set to 0
     lean_ck_drop(g, vq, k, Q.C, CK, OneOut{x1}, x1, sh);
     x2[2] = lean_ck_draw(g, vq, k, Q.C, CK, OneOut{x1}, u2, sh);

@@ -32,6 +32,7 @@ namespace cg = cooperative_groups;
 
 constexpr int kLeanMaxWarps = 32;
 constexpr int kLeanCk = 16;       // checkpoints per warp in the draft step's pass A, at most
+constexpr float kNoIds = 6.2e-33f;  // 2^-107
 constexpr float kHuge = 1.0e30f;  // ~2^100: partial sums beyond this move the reference
 
 struct LeanShared {
@@ -486,6 +487,10 @@ __device__ __forceinline__ void merge_slices(const LeanShared &sh, int r, float 
     st.ml = tot.ml; st.C = tot.c; st.sx = tot.sx; st.idx = tot.idx; st.own = tot.own(k);
 }
 
+// Does a part of a row with the maximum logit ml have an exponential above 0 on the row's scale?  (Its sum, made on its
+// own scale, may be above 0 there although all of its exponentials are below the smallest normal number.)
+__device__ __forceinline__ bool gives_id(float ml, float k, float C) { return ml > neg_inf() && ex2(__fmaf_rn(ml, k, -C)) > 0.f; }
+
 // Mass of slice c of a row (row scale) for a draw from softmax(row) without token `excl`
 // (excl < 0: none; only a slice's own argmax can be left out here).  The slices' published
 // partials stay valid until the kernel ends.
@@ -494,6 +499,7 @@ __device__ __forceinline__ float slice_mass(const LeanShared &sh, int r, const R
                                             float k) {
     const LeanShared *ps = RowGroup<CS>::peer(&sh, c);
     const float ml = ps->x_ml[r];
+    if (!gives_id(ml, k, st.C)) return 0.f;
     const float own = (ps->x_idx[r] != excl) ? own_term(ml, k) : 0.f;
     return (ps->x_sx[r] + own) * rescale(ml, shift_of(ml, k), st.C);
 }
@@ -511,7 +517,8 @@ __device__ int lean_sample_slice(const Geo &g, const ROW &row, float k, const Ro
     const float C = st.C;
     if (threadIdx.x < g.nwarps) {
         const int w = threadIdx.x;
-        sh.mass[w] = (excl >= 0 && excl == locarg && sh.widx[r][w] == locarg ? sh.wmassx[r][w] : sh.wmass[r][w]) * f;
+        const float m = (excl >= 0 && excl == locarg && sh.widx[r][w] == locarg ? sh.wmassx[r][w] : sh.wmass[r][w]) * f;
+        sh.mass[w] = gives_id(sh.wml[r][w], k, C) ? m : 0.f;
     }
     __syncthreads();
     if (excl >= 0 && excl != locarg && g.holds_vec(excl >> 3)) {
@@ -743,6 +750,9 @@ __device__ __forceinline__ void lean_ck_drop(const Geo &g, const ROW &row, float
 // Inverse-CDF draw from softmax(row) over the checkpoint sub-blocks, the ids left out having no weight (their
 // sub-blocks' sums say so already).  C = the row's exponent shift.  Returns the token, -1 if nothing has mass.  Called
 // by one warp, after the checkpoints are visible.
+// A sub-block's sum is of its own scale: brought to the row's it may be above 0 where all its exponentials are below the
+// smallest normal number, 0, and it has no id to give.  All of those together stay below kNoIds (2^19 ids), which targets
+// are kept above where the draw's mass is not itself that small.
 template <class ROW, class OUT>
 __device__ __forceinline__ int lean_ck_draw(const Geo &g, const ROW &row, float k, float C, int CK, OUT out, float u, const LeanCkShared &sh) {
     const int lane = threadIdx.x & 31;
@@ -754,7 +764,7 @@ __device__ __forceinline__ int lean_ck_draw(const Geo &g, const ROW &row, float 
     float ls = 0.f;
     for (int i = 0; i < per; ++i) ls += slot_mass(lane * per + i);
     float t;
-    int slot = pair_pick(ls, u, t);
+    int slot = pair_pick(ls, u, t, kNoIds);
     if (slot < 0) return -1;
     if (per > 1) {   // the sub-block within the lane's
         const int first = slot * per;
@@ -843,7 +853,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_leaf_
     uint32_t status = 0;
     int tok = -1;
     if (!(Ps.ml > neg_inf()) || !(Ps.ml < -neg_inf()) || !finite_pos(Zp)) status = SPECHUB_ST_NONFINITE;
-    else tok = lean_ck_draw(g, vp, k, Ps.c, CK, NoneOut{}, ures, sh);
+    else if ((tok = lean_ck_draw(g, vp, k, Ps.c, CK, NoneOut{}, ures, sh)) < 0) tok = Ps.idx;   // (as in the draft step)
     if (threadIdx.x == 0) {
         for (int m = 0; m < A.n_out; ++m) {
             const NodeOutPtrs &o = A.out[m];
@@ -1437,7 +1447,8 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_kernel(Row
                 x2 = (hubtok == 0) ? 1 : 0;
                 st |= SPECHUB_ST_DEGENERATE_Q;
             } else {
-                const int t2 = lean_sample_row<CS>(g, vq, k, Q, me, hubtok, u2, 0, sh);
+                int t2 = lean_sample_row<CS>(g, vq, k, Q, me, hubtok, u2, 0, sh);
+                if (t2 == -1) t2 = hubtok == 0 ? 1 : 0;   // (what is left is below the smallest normal number)
                 x2_elsewhere = true;
                 if (t2 != -2 && threadIdx.x == 0) {
                     a.draft_tokens_out[2 * r + 1] = t2;
@@ -1526,7 +1537,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
     } else {
         hubtok = Q.idx;
         x1 = lean_ck_draw(g, vq, k, Q.C, CK, NoneOut{}, u1, sh);
-        if (x1 < 0) x1 = hubtok;   // (a sub-block of exponentials below the smallest normal number)
+        if (x1 < 0) x1 = hubtok;   // (a sub-block without an id, by rounding at its edge)
         if (method == kSpecHub) {
             prob0 = Q.own / Zq;
             if (x1 != hubtok) {
@@ -1538,6 +1549,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
             }
         } else if (method == kRRS) {
             x2 = lean_ck_draw(g, vq, k, Q.C, CK, NoneOut{}, u2, sh);
+            if (x2 < 0) x2 = hubtok;
         }
         if (x2 < 0 && method != kRRS) {   // q without x1 (SpecHub: x1 is the hub)
             lean_ck_drop(g, vq, k, Q.C, CK, OneOut{x1}, x1, sh);

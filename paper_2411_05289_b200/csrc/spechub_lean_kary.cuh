@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_kary_draft_kerne
         if (!bad) {
             const int out = A.without_replacement ? i : 0;   // x[0..out) are left out
             t = lean_ck_draw(g, vq, k, Q.c, CK, ListOut{sh.x, out}, un[i], sh);
+            if (t < 0 && out == 0) t = Q.idx;   // (as in lean_draft_ck_kernel)
             if (t < 0) {   // nothing left to draw from: lowest id not drawn yet
                 st |= SPECHUB_ST_DEGENERATE_Q;
                 for (t = 0; t < a.vocab && one_of(sh.x, i, t); ++t) {}
@@ -267,7 +268,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_kary_
         // residual: every warp picks the warp whose range holds the target, single terms counted where they lie
         const bool zero = !(m > 0.f);
         if (zero) status |= SPECHUB_ST_ZERO_RESIDUAL;   // a draw from p: C = 0 for every id
-        float wm = lane < nwarps ? (zero ? sh.wmass[0][lane] : sh.acc[K - 1][lane]) : 0.f;
+        float wm = lane < nwarps ? (zero ? (gives_id(sh.wml[0][lane], k, Cp) ? sh.wmass[0][lane] : 0.f) : sh.acc[K - 1][lane]) : 0.f;
         for (unsigned sg = singles; sg; sg &= sg - 1) {
             const int i = __ffs(sg) - 1;
             if (g.warp_of_vec(sh.x[i] >> 3) == lane) wm += zero ? ep(i) : fmaxf(__fmaf_rn(-sh.cx[i] * rho, eq(i), ep(i)), 0.f);

@@ -183,3 +183,30 @@ def test_second_drafts_from_next_to_nothing(sh, V, dtype, B):  # noqa: F811
         d = parity.to_numpy(gpu_draft(sh, m, tq, und, sh.Tree.heap(3), 1.0))
         parity.check_draft(m, lq[pick], 1.0, un[pick], {k: v[pick] for k, v in d.items()}, label="next to nothing")
         assert int(d["status"].max()) == 0, m
+
+
+def test_draws_from_rows_with_ids_of_no_normal_exponential(sh):  # noqa: F811
+    """Uniforms of 0 on rows whose first ids lie just below 2^-126 of the top: together they have mass, each alone has
+    none in fp32.  Draws go to an id that has some, and no row is flagged."""
+    rng = np.random.default_rng(77)
+    for V, dtype, B in ((8192, "bf16", batch_that_streams(3, 8192, "bf16")), (9001, "fp32", batch_that_streams(3, 9001, "fp32")),
+                        (8192, "bf16", 4), (9001, "fp32", 4)):
+        lp, lq = random_logits(rng, B, 3, V, dtype)
+        for x in (lp, lq):
+            x[...] = np.minimum(x, 7.0)
+            x[:, :, :4096] = -80.0     # log2(e) * -80 = -115.4; the reference of the row is 11 = rint(log2(e) * 7.5)
+            x[:, :, 5000] = 7.5        # the maximum
+        lp, lq = workloads.round_to_storage(lp, dtype), workloads.round_to_storage(lq, dtype)
+        un = random_uniforms(rng, B, 3)
+        un[:, :, [0, 1, 4]] = 0.0
+        for leaves in (False, True):
+            check_two_drafts(sh, lp, lq, dtype, 0, 1.0, un, leaves, sample(rng, B, first=min(B, 8)), "below normal")
+        tq, und = padded(lq, dtype, 0), torch.from_numpy(un).cuda()
+        all3 = sh.mdsd_compare_draft_sample(tq, und, sh.Tree.heap(3), 1.0)
+        assert all(int(all3[m]["tokens"].min()) >= 0 and int(all3[m]["status"].max()) == 0 for m in METHODS)
+        un = np.zeros((B, 4, 7), np.float32)
+        un[:, :, 3:6] = 0.5
+        lp, lq = np.resize(lp, (B, 4, V)), np.resize(lq, (B, 4, V))
+        for wo in (False, True):
+            for leaves in (False, True):
+                check_more_drafts(sh, 3, wo, lp, lq, dtype, 0, 1.0, un, leaves, sample(rng, B, first=min(B, 8)), "below normal")
