@@ -45,8 +45,18 @@ struct Names {  // interned attribute and key names
     PyObject *spechub, *rrs, *rrsw;
 } N;
 
-int check(int code) {
-    if (code == SPECHUB_OK) return code;
+// Without the interpreter's lock: other Python threads run while a call waits for a place in a full launch queue or for
+// memory.  (Among them may be the callback that the queue waits for.)
+struct Unlocked {
+    PyThreadState *state = PyEval_SaveThread();
+    Unlocked() = default;
+    Unlocked(const Unlocked &) = delete;
+    Unlocked &operator=(const Unlocked &) = delete;
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
+
+void check(int code) {
+    if (code == SPECHUB_OK) return;
     Ref e(PyObject_CallFunction(g_error, "is", code, spechub_status_string(code)));
     if (e.o) PyErr_SetObject(g_error, e.o);
     fail();
@@ -112,9 +122,12 @@ struct Desc {
         d.stride_node = Nn > 1 ? s1 : std::max(s1, V);
         if (THPVariable_Check(temp)) {
             temperature = THPVariable_Unpack(temp);
-            if (temperature.device() != dev || temperature.scalar_type() != at::kFloat)
-                temperature = temperature.to(dev, at::kFloat);
-            temperature = temperature.contiguous();
+            {
+                Unlocked u;
+                if (temperature.device() != dev || temperature.scalar_type() != at::kFloat)
+                    temperature = temperature.to(dev, at::kFloat);
+                temperature = temperature.contiguous();
+            }
             if (temperature.dim() != 1 || temperature.size(0) != B) value_error("temperature tensor must be [batch]");
             d.temperature = 1.0f;
             d.temperature_per_seq = temperature.const_data_ptr<float>();
@@ -206,21 +219,44 @@ void hold_values(PyObject *stream, PyObject *mapping) {
 }
 
 // ---- outputs of a verify call --------------------------------------------------------------------
-PyObject *new_outputs(int64_t B, int64_t Nn, int64_t levels, int64_t k, const at::Device &dev) {
-    Ref o(PyDict_New());
-    if (!o.o) fail();
-    put(o.o, N.accept_idx, make({B, Nn}, at::kInt, dev));
-    put(o.o, N.token, make({B, Nn}, at::kInt, dev));
-    put(o.o, N.hub, make({B, Nn}, at::kInt, dev));
-    put(o.o, N.beta, make({B, Nn, k}, at::kFloat, dev));
-    put(o.o, N.rate, make({B, Nn, k + 1}, at::kFloat, dev));
-    put(o.o, N.status, make({B, Nn}, at::kInt, dev));
-    put(o.o, N.n_accepted, make({B}, at::kInt, dev));
-    put(o.o, N.n_emitted, make({B}, at::kInt, dev));
-    put(o.o, N.path_nodes, make({B, levels}, at::kInt, dev));
-    put(o.o, N.path_tokens, make({B, levels}, at::kInt, dev));
-    return o.release();
-}
+struct NewOutputs {
+    Tensor accept_idx, token, hub, beta, rate, status, n_accepted, n_emitted, path_nodes, path_tokens;
+    void allocate(const Desc &d, int64_t levels, int64_t k, bool probabilities, spechub_node_out &no, spechub_seq_out &so) {
+        for (Tensor *t : {&accept_idx, &token, &hub, &status}) *t = make({d.B, d.Nn}, at::kInt, d.dev);
+        beta = make({d.B, d.Nn, k}, at::kFloat, d.dev);
+        rate = make({d.B, d.Nn, k + 1}, at::kFloat, d.dev);
+        for (Tensor *t : {&n_accepted, &n_emitted}) *t = make({d.B}, at::kInt, d.dev);
+        for (Tensor *t : {&path_nodes, &path_tokens}) *t = make({d.B, levels}, at::kInt, d.dev);
+        no = {};
+        no.accept_idx = static_cast<int32_t *>(accept_idx.data_ptr());
+        no.token = static_cast<int32_t *>(token.data_ptr());
+        no.hub = static_cast<int32_t *>(hub.data_ptr());
+        if (probabilities) {
+            no.beta = static_cast<float *>(beta.data_ptr());
+            no.rate = static_cast<float *>(rate.data_ptr());
+        }
+        no.status = static_cast<uint32_t *>(status.data_ptr());
+        so.n_accepted = static_cast<int32_t *>(n_accepted.data_ptr());
+        so.n_emitted = static_cast<int32_t *>(n_emitted.data_ptr());
+        so.path_nodes = static_cast<int32_t *>(path_nodes.data_ptr());
+        so.path_tokens = static_cast<int32_t *>(path_tokens.data_ptr());
+    }
+    PyObject *dict() const {
+        Ref o(PyDict_New());
+        if (!o.o) fail();
+        put(o.o, N.accept_idx, accept_idx);
+        put(o.o, N.token, token);
+        put(o.o, N.hub, hub);
+        put(o.o, N.beta, beta);
+        put(o.o, N.rate, rate);
+        put(o.o, N.status, status);
+        put(o.o, N.n_accepted, n_accepted);
+        put(o.o, N.n_emitted, n_emitted);
+        put(o.o, N.path_nodes, path_nodes);
+        put(o.o, N.path_tokens, path_tokens);
+        return o.release();
+    }
+};
 
 template <class T>
 T *field(PyObject *out, PyObject *key) {
@@ -284,28 +320,33 @@ PyObject *draft_impl(PyObject *const *a, Py_ssize_t n) {
     const float *un = uniforms_of(a[2], d);
     const bool with_stats = truth(a[7]);
     void *s = stream_of(a[5]);
+    Tensor tokens, status, hub, prob, stats;
+    const void *xp = x.const_data_ptr();
+    int rc;
+    {
+        Unlocked u;
+        tokens = make({d.B, d.Nn, tree.k}, at::kInt, d.dev);
+        status = make({d.B, d.Nn}, at::kInt, d.dev);
+        if (with_stats) stats = make_stats(d);
+        void *stp = with_stats ? stats.data_ptr() : nullptr;
+        int32_t *tp = static_cast<int32_t *>(tokens.data_ptr());
+        uint32_t *sp = static_cast<uint32_t *>(status.data_ptr());
+        if (method == kSpecHub) {
+            hub = make({d.B, d.Nn}, at::kInt, d.dev);
+            prob = make({d.B, d.Nn, 2}, at::kFloat, d.dev);
+            int32_t *hp = static_cast<int32_t *>(hub.data_ptr());
+            float *pp = static_cast<float *>(prob.data_ptr());
+            rc = with_stats ? spechub_draft_sample_stats(&d.d, xp, un, tp, hp, pp, sp, stp, s)
+                            : spechub_draft_sample(&d.d, xp, un, tp, hp, pp, sp, s);
+        } else {
+            const int wo = method == kRRSw;
+            rc = with_stats ? rrs_draft_sample_stats(&d.d, xp, un, wo, tp, sp, stp, s)
+                            : rrs_draft_sample(&d.d, xp, un, wo, tp, sp, s);
+        }
+    }
+    check(rc);
     Ref out(PyDict_New());
     if (!out.o) fail();
-    const Tensor tokens = make({d.B, d.Nn, tree.k}, at::kInt, d.dev), status = make({d.B, d.Nn}, at::kInt, d.dev);
-    Tensor hub, prob, stats;
-    if (method == kSpecHub) {
-        hub = make({d.B, d.Nn}, at::kInt, d.dev);
-        prob = make({d.B, d.Nn, 2}, at::kFloat, d.dev);
-    }
-    if (with_stats) stats = make_stats(d);
-    const void *xp = x.const_data_ptr();
-    int32_t *tp = static_cast<int32_t *>(tokens.data_ptr());
-    uint32_t *sp = static_cast<uint32_t *>(status.data_ptr());
-    if (method == kSpecHub) {
-        int32_t *hp = static_cast<int32_t *>(hub.data_ptr());
-        float *pp = static_cast<float *>(prob.data_ptr());
-        check(with_stats ? spechub_draft_sample_stats(&d.d, xp, un, tp, hp, pp, sp, stats.data_ptr(), s)
-                         : spechub_draft_sample(&d.d, xp, un, tp, hp, pp, sp, s));
-    } else {
-        const int wo = method == kRRSw;
-        check(with_stats ? rrs_draft_sample_stats(&d.d, xp, un, wo, tp, sp, stats.data_ptr(), s)
-                         : rrs_draft_sample(&d.d, xp, un, wo, tp, sp, s));
-    }
     put(out.o, N.tokens, tokens);
     if (method == kSpecHub) {
         put(out.o, N.hub, hub);
@@ -335,22 +376,32 @@ PyObject *verify_impl(PyObject *const *a, Py_ssize_t n) {
     if (method == kSpecHub) need_k2(tree);
     const float *un = uniforms_of(a[5], d);
     const int32_t *tok = tokens_of(a[4], d, "draft_tokens must be a contiguous int32 [batch][nodes][k] tensor");
-    Ref out(a[9] == Py_None ? new_outputs(d.B, d.Nn, tree.levels, tree.k, d.dev) : Py_NewRef(a[9]));
+    Ref out(a[9] == Py_None ? nullptr : Py_NewRef(a[9]));
+    const bool probabilities = truth(a[10]), with_stats = truth(a[12]);
     spechub_node_out no;
     spechub_seq_out so;
-    output_pointers(out.o, truth(a[10]), no, so);
-    size_t wsb;
-    const Tensor ws = make_workspace(d, wsb);
-    void *wp = wsb ? ws.data_ptr() : nullptr, *s = stream_of(a[8]);
+    if (out.o) output_pointers(out.o, probabilities, no, so);
+    const void *st = with_stats ? stats_of(a[3], d) : nullptr;
+    void *s = stream_of(a[8]);
     const void *tp = tl.const_data_ptr(), *dp = dl.const_data_ptr();
-    if (truth(a[12])) {
-        const void *st = stats_of(a[3], d);
-        check(method == kSpecHub ? spechub_verify_tree_stats(&d.d, tp, dp, st, tok, un, &no, &so, wp, wsb, s)
-                                 : rrs_verify_tree_stats(&d.d, tp, dp, st, tok, un, method == kRRSw, &no, &so, wp, wsb, s));
-    } else {
-        check(method == kSpecHub ? spechub_verify_tree(&d.d, tp, dp, tok, un, &no, &so, wp, wsb, s)
-                                 : rrs_verify_tree(&d.d, tp, dp, tok, un, method == kRRSw, &no, &so, wp, wsb, s));
+    NewOutputs fresh;
+    Tensor ws;
+    int rc;
+    {
+        Unlocked u;
+        if (!out.o) fresh.allocate(d, tree.levels, tree.k, probabilities, no, so);
+        size_t wsb;
+        ws = make_workspace(d, wsb);
+        void *wp = wsb ? ws.data_ptr() : nullptr;
+        if (with_stats)
+            rc = method == kSpecHub ? spechub_verify_tree_stats(&d.d, tp, dp, st, tok, un, &no, &so, wp, wsb, s)
+                                    : rrs_verify_tree_stats(&d.d, tp, dp, st, tok, un, method == kRRSw, &no, &so, wp, wsb, s);
+        else
+            rc = method == kSpecHub ? spechub_verify_tree(&d.d, tp, dp, tok, un, &no, &so, wp, wsb, s)
+                                    : rrs_verify_tree(&d.d, tp, dp, tok, un, method == kRRSw, &no, &so, wp, wsb, s);
     }
+    check(rc);
+    if (!out.o) out.o = fresh.dict();
     hold(a[8], d.temperature);
     hold(a[8], ws);
     hold(a[8], a[3]);
@@ -368,21 +419,28 @@ PyObject *compare_draft_impl(PyObject *const *a, Py_ssize_t n) {
     const float *un = uniforms_of(a[1], d);
     const bool with_stats = truth(a[6]);
     void *s = stream_of(a[4]);
-    Tensor tokens[3], status[3], stats;
-    int32_t *tp[3];
-    uint32_t *sp[3];
-    for (int m = 0; m < 3; ++m) {
-        tokens[m] = make({d.B, d.Nn, 2}, at::kInt, d.dev);
-        status[m] = make({d.B, d.Nn}, at::kInt, d.dev);
-        tp[m] = static_cast<int32_t *>(tokens[m].data_ptr());
-        sp[m] = static_cast<uint32_t *>(status[m].data_ptr());
+    Tensor tokens[3], status[3], stats, hub, prob;
+    const void *xp = x.const_data_ptr();
+    int rc;
+    {
+        Unlocked u;
+        int32_t *tp[3];
+        uint32_t *sp[3];
+        for (int m = 0; m < 3; ++m) {
+            tokens[m] = make({d.B, d.Nn, 2}, at::kInt, d.dev);
+            status[m] = make({d.B, d.Nn}, at::kInt, d.dev);
+            tp[m] = static_cast<int32_t *>(tokens[m].data_ptr());
+            sp[m] = static_cast<uint32_t *>(status[m].data_ptr());
+        }
+        hub = make({d.B, d.Nn}, at::kInt, d.dev);
+        prob = make({d.B, d.Nn, 2}, at::kFloat, d.dev);
+        if (with_stats) stats = make_stats(d);
+        int32_t *hp = static_cast<int32_t *>(hub.data_ptr());
+        float *pp = static_cast<float *>(prob.data_ptr());
+        rc = with_stats ? mdsd_compare_draft_sample_stats(&d.d, xp, un, tp, hp, pp, sp, stats.data_ptr(), s)
+                        : mdsd_compare_draft_sample(&d.d, xp, un, tp, hp, pp, sp, s);
     }
-    const Tensor hub = make({d.B, d.Nn}, at::kInt, d.dev), prob = make({d.B, d.Nn, 2}, at::kFloat, d.dev);
-    if (with_stats) stats = make_stats(d);
-    int32_t *hp = static_cast<int32_t *>(hub.data_ptr());
-    float *pp = static_cast<float *>(prob.data_ptr());
-    check(with_stats ? mdsd_compare_draft_sample_stats(&d.d, x.const_data_ptr(), un, tp, hp, pp, sp, stats.data_ptr(), s)
-                     : mdsd_compare_draft_sample(&d.d, x.const_data_ptr(), un, tp, hp, pp, sp, s));
+    check(rc);
     Ref out(PyDict_New());
     if (!out.o) fail();
     PyObject *names[3] = {N.spechub, N.rrs, N.rrsw};
@@ -423,28 +481,39 @@ PyObject *compare_verify_impl(PyObject *const *a, Py_ssize_t n) {
                                 "] must be a contiguous int32 [batch][nodes][2] tensor";
         tok[m] = tokens_of(t.o, d, msg.c_str());
     }
-    Ref out(a[8] == Py_None ? PyDict_New() : Py_NewRef(a[8]));
-    if (!out.o) fail();
+    Ref out(a[8] == Py_None ? nullptr : Py_NewRef(a[8]));
     spechub_node_out no[3];
     spechub_seq_out so[3];
-    const bool probabilities = truth(a[9]);
-    for (int m = 0; m < 3; ++m) {
-        if (a[8] == Py_None) {
-            Ref one(new_outputs(d.B, d.Nn, tree.levels, 2, d.dev));
-            if (PyDict_SetItem(out.o, names[m], one.o) < 0) fail();
-        }
+    const bool probabilities = truth(a[9]), with_stats = truth(a[11]);
+    for (int m = 0; m < 3 && out.o; ++m) {
         Ref one(PyObject_GetItem(out.o, names[m]));
         if (!one.o) fail();
         output_pointers(one.o, probabilities, no[m], so[m]);
     }
-    size_t wsb;
-    const Tensor ws = make_workspace(d, wsb);
-    void *wp = wsb ? ws.data_ptr() : nullptr, *s = stream_of(a[7]);
+    const void *st = with_stats ? stats_of(a[2], d) : nullptr;
+    void *s = stream_of(a[7]);
     const void *tp = tl.const_data_ptr(), *dp = dl.const_data_ptr();
-    if (truth(a[11]))
-        check(mdsd_compare_verify_tree_stats(&d.d, tp, dp, stats_of(a[2], d), tok, un, no, so, wp, wsb, s));
-    else
-        check(mdsd_compare_verify_tree(&d.d, tp, dp, tok, un, no, so, wp, wsb, s));
+    NewOutputs fresh[3];
+    Tensor ws;
+    int rc;
+    {
+        Unlocked u;
+        for (int m = 0; m < 3 && !out.o; ++m) fresh[m].allocate(d, tree.levels, 2, probabilities, no[m], so[m]);
+        size_t wsb;
+        ws = make_workspace(d, wsb);
+        void *wp = wsb ? ws.data_ptr() : nullptr;
+        rc = with_stats ? mdsd_compare_verify_tree_stats(&d.d, tp, dp, st, tok, un, no, so, wp, wsb, s)
+                        : mdsd_compare_verify_tree(&d.d, tp, dp, tok, un, no, so, wp, wsb, s);
+    }
+    check(rc);
+    if (!out.o) {
+        out.o = PyDict_New();
+        if (!out.o) fail();
+        for (int m = 0; m < 3; ++m) {
+            Ref one(fresh[m].dict());
+            if (PyDict_SetItem(out.o, names[m], one.o) < 0) fail();
+        }
+    }
     hold(a[7], d.temperature);
     hold(a[7], ws);
     hold(a[7], a[2]);
@@ -467,11 +536,21 @@ PyObject *verify_static_impl(PyObject *const *a, Py_ssize_t n) {
     const Desc d(tl, tree, a[5], flags_of(a[8]));
     const float *un = uniforms_of(a[3], d);
     const int32_t *tok = tokens_of(a[2], d, "draft_tokens must be a contiguous int32 [batch][nodes][2] tensor");
-    Ref out(a[7] == Py_None ? new_outputs(d.B, d.Nn, tree.levels, 2, d.dev) : Py_NewRef(a[7]));
+    Ref out(a[7] == Py_None ? nullptr : Py_NewRef(a[7]));
     spechub_node_out no;
     spechub_seq_out so;
-    output_pointers(out.o, true, no, so);
-    check(spechub_verify_tree_static(&d.d, tl.const_data_ptr(), dl.const_data_ptr(), tok, un, &no, &so, stream_of(a[6])));
+    if (out.o) output_pointers(out.o, true, no, so);
+    void *s = stream_of(a[6]);
+    const void *tp = tl.const_data_ptr(), *dp = dl.const_data_ptr();
+    NewOutputs fresh;
+    int rc;
+    {
+        Unlocked u;
+        if (!out.o) fresh.allocate(d, tree.levels, 2, true, no, so);
+        rc = spechub_verify_tree_static(&d.d, tp, dp, tok, un, &no, &so, s);
+    }
+    check(rc);
+    if (!out.o) out.o = fresh.dict();
     hold(a[6], d.temperature);
     hold_values(a[6], out.o);
     return out.release();
