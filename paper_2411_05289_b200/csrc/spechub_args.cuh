@@ -38,11 +38,11 @@ struct RowArgs {
 // otherwise have to read the row for a second time to find out (Section 4: a = argmax q; q(a); 1 - q(a)).
 struct DraftStat {
     float ml;       // the row's maximum logit
-    float sx;       // sum over ids != argmax of 2^(k l - k ml), k = log2(e) / T
+    float sx;       // sum over ids != argmax of 2^(k l - rint(k ml)), k = log2(e) / T
     int idx;        // argmax, lowest id on ties
-    unsigned tag;   // kDraftStatTag ^ bits of k: a record of another library version or temperature is refused
+    unsigned tag;   // kDraftStatTag ^ bits of k: a record of another kind or temperature is refused
 };
-constexpr unsigned kDraftStatTag = 0x51a75u << 12;
+constexpr unsigned kDraftStatTag = 0x51a76u << 12;   // (another number whenever the record's meaning changes)
 
 struct NodeOutPtrs {
     int32_t *accept_idx, *token, *hub;

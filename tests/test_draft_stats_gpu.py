@@ -167,3 +167,18 @@ def test_more_than_two_drafts_neither_write_nor_read_records(sh):
         torch.cuda.synchronize()
         for k in a:
             assert torch.equal(a[k], b[k]), (wo, k)
+
+
+@pytest.mark.parametrize("B", [4, 300])
+def test_records_of_another_scale_are_refused(sh, B):
+    """A record of the form whose sum is relative to k * ml itself (tag 0x51a75)."""
+    tp, tq, un = problem(16384, "bf16", 17, B=B)
+    tree = sh.Tree.heap(7)
+    d = draft(sh, "spechub", tq, un, tree)
+    k = np.float32(1.4426950408889634)
+    old = d["stats"].clone().view(-1, 4)
+    old[:, 3] = int(((0x51a75 << 12) ^ int(k.view(np.uint32))) - (1 << 32) if ((0x51a75 << 12) ^ int(k.view(np.uint32))) >> 31
+                    else (0x51a75 << 12) ^ int(k.view(np.uint32)))
+    out = verify(sh, "spechub", tp, tq, d, un, tree, stats=old.view(-1))
+    torch.cuda.synchronize()
+    assert bool(((out["status"] & ST_STATS) != 0).all())
