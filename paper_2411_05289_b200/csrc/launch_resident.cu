@@ -38,7 +38,7 @@ static int launch_resident_one(int nb, const FusedArgs &f, unsigned rows, cudaSt
     at[0].val.clusterDim.x = CS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at; cfg.numAttrs = CS > 1 ? 1 : 0;
     cfg.gridDim = dim3(rows * CS); cfg.blockDim = dim3(kResThreads); cfg.dynamicSmemBytes = smem; cfg.stream = s;
-    return cudaLaunchKernelEx(&cfg, kern, f, nb, cols) == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH;
+    return launch_status(cudaLaunchKernelEx(&cfg, kern, f, nb, cols));
 }
 
 template <int MASK>
@@ -66,7 +66,7 @@ static int launch_resident_kary_one(int nb, const KaryArgs &ka, unsigned rows, c
     at[0].val.clusterDim.x = CS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at; cfg.numAttrs = CS > 1 ? 1 : 0;
     cfg.gridDim = dim3(rows * CS); cfg.blockDim = dim3(kResThreads); cfg.dynamicSmemBytes = smem; cfg.stream = s;
-    return cudaLaunchKernelEx(&cfg, kern, ka, nb, cols) == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH;
+    return launch_status(cudaLaunchKernelEx(&cfg, kern, ka, nb, cols));
 }
 
 int launch_resident_kary(ResShape sh, const KaryArgs &ka, unsigned rows, cudaStream_t s) {

@@ -11,6 +11,11 @@ namespace spechub {
 constexpr int kMaxDevices = 64;
 
 inline int launch_status() { return cudaGetLastError() == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH; }
+// ... of a launch that says itself how it went; a refused one leaves no error behind for a later call to find
+inline int launch_status(cudaError_t e) {
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH;
+}
 
 // One launch: `cs` CTAs per cluster (1: none), as a programmatic dependent of the stream's last kernel.  Only for
 // kernels that begin with pdl_begin().
@@ -24,7 +29,7 @@ int launch_grid(K kern, unsigned grid, int threads, int smem, int cs, cudaStream
     at[1].val.clusterDim.x = cs; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
     cfg.attrs = at; cfg.numAttrs = cs > 1 ? 2 : 1;
     cfg.gridDim = dim3(grid); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = s;
-    return cudaLaunchKernelEx(&cfg, kern, args...) == cudaSuccess ? SPECHUB_OK : SPECHUB_ERR_LAUNCH;
+    return launch_status(cudaLaunchKernelEx(&cfg, kern, args...));
 }
 
 // Raise a kernel's dynamic shared memory limit once per device.  `configured`: one flag per device, kept by

@@ -36,3 +36,22 @@ def test_other_threads_run_while_a_call_waits_for_the_launch_queue(sh):  # noqa:
     gap = max(b - a for a, b in zip(ticks, ticks[1:]))
     assert took[0] > 0.5, took    # (the calls did wait)
     assert gap < 0.25, (gap, took)
+
+
+def test_a_refused_launch_leaves_no_error_for_later_calls(sh):  # noqa: F811
+    """More CTAs than a grid may have (2^29 + 1 rows on four each) is refused by the host; the next call, whose launches
+    are checked by the last error, is not told of it."""
+    import ctypes
+
+    from paper_2411_05289_b200 import binding
+
+    lib, x = sh.load_library(), torch.randn((2, 3, 64), device="cuda")
+    un, tree, word = torch.rand((2, 3, 5), device="cuda"), sh.Tree.heap(3), torch.zeros(64, device="cuda")
+    d, _ = binding._desc(x, tree, 1.0)
+    d.batch, d.nodes, d.vocab, d.levels, d.dtype, d.flags = (1 << 29) + 1, 1, 8192, 1, binding.BF16, 4
+    d.stride_seq = d.stride_node = 8192
+    at = ctypes.c_void_p(word.data_ptr())   # (no kernel runs: nothing is read)
+    assert lib.spechub_draft_sample(ctypes.byref(d), at, at, at, None, None, None, None) == -8
+    tokens = sh.spechub_draft_sample(x, un, tree)["tokens"]
+    sh.spechub_verify_tree_static(x, x, tokens, un, tree)
+    torch.cuda.synchronize()
