@@ -8,6 +8,7 @@
 #include <ATen/cuda/EmptyTensor.h>
 #include <ATen/ops/empty.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <cmath>
@@ -562,8 +563,8 @@ PyObject *guarded(PyObject *, PyObject *const *a, Py_ssize_t n) {
         return IMPL(a, n);
     } catch (const PyFail &) {
         return nullptr;
-    } catch (const std::exception &e) {   // torch: out of memory and the like
-        if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, e.what());
+    } catch (...) {   // torch's, as torch's own functions raise them (OutOfMemoryError and the like)
+        if (!PyErr_Occurred()) torch::translate_exception_to_python(std::current_exception());
         return nullptr;
     }
 }

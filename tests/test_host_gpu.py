@@ -55,3 +55,15 @@ def test_a_refused_launch_leaves_no_error_for_later_calls(sh):  # noqa: F811
     tokens = sh.spechub_draft_sample(x, un, tree)["tokens"]
     sh.spechub_verify_tree_static(x, x, tokens, un, tree)
     torch.cuda.synchronize()
+
+
+def test_out_of_memory_is_torch_s_own_error(sh):  # noqa: F811
+    x, un, tree = torch.zeros((1 << 21, 1, 2), device="cuda"), torch.zeros((1 << 21, 1, 5), device="cuda"), sh.Tree.heap(1)
+    torch.cuda.empty_cache()
+    torch.cuda.set_per_process_memory_fraction(1e-5)   # no new segment is given out
+    try:
+        with pytest.raises(torch.cuda.OutOfMemoryError):
+            sh.spechub_draft_sample(x, un, tree)
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    assert sh.spechub_draft_sample(x, un, tree)["tokens"].shape == (1 << 21, 1, 2)
