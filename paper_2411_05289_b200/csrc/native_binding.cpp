@@ -133,9 +133,9 @@ struct Desc {
             d.temperature = 1.0f;
             d.temperature_per_seq = temperature.const_data_ptr<float>();
         } else {
-            const double t = PyFloat_AsDouble(temp);
-            if (t == -1.0 && PyErr_Occurred()) fail();
-            d.temperature = static_cast<float>(t);
+            const Ref f(PyNumber_Float(temp));   // whatever float() takes
+            if (!f.o) fail();
+            d.temperature = static_cast<float>(PyFloat_AS_DOUBLE(f.o));
         }
         if (tree.child.o != Py_None) {
             const Tensor &c = tensor(tree.child.o, "child must be a tensor");

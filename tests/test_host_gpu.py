@@ -67,3 +67,11 @@ def test_out_of_memory_is_torch_s_own_error(sh):  # noqa: F811
     finally:
         torch.cuda.set_per_process_memory_fraction(1.0)
     assert sh.spechub_draft_sample(x, un, tree)["tokens"].shape == (1 << 21, 1, 2)
+
+
+def test_temperature_is_whatever_float_takes(sh):  # noqa: F811
+    x, un, tree = torch.randn((4, 1, 64), device="cuda"), torch.rand((4, 1, 5), device="cuda"), sh.Tree.heap(1)
+    want = sh.spechub_draft_sample(x, un, tree, 0.5)
+    for t in ("0.5", b"0.5"):
+        got = sh.spechub_draft_sample(x, un, tree, t)
+        assert all(torch.equal(want[k], got[k]) for k in want)
