@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
     using V = Vec8<__nv_bfloat16>;
     const StreamRow<__nv_bfloat16, false> vp(rowp, a.vocab), vq(rowq, a.vocab);
     const Geo g = make_geo(a.vocab, 8);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int lo = g.seg_lo(warp), hi = g.seg_hi(warp);
     const int last_vi = (lo + lane < hi) ? lo + lane + ((hi - 1 - lo - lane) / 32) * 32 : lo - 1;
     const float k = kLog2e / temperature_of(a, b);
@@ -76,8 +76,8 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
         sh.x_ml[1] = ds.ml; sh.x_sx[1] = ds.sx; sh.x_idx[1] = ok ? ds.idx : 0;
     }
     LeanAcc<__nv_bfloat16> tp, tq;
-    if (STATS) lean_pass_a_deep(vp, lo, hi, lane, k, tp);
-    else lean_pass_a<true, false>(vp, vq, lo, hi, lane, k, tp, tq);
+    if constexpr (STATS) lean_pass_a1<true>(vp, lo, hi, lane, k, tp);
+    else lean_pass_a2<false>(vp, vq, lo, hi, lane, k, tp, tq);
     RowStat P, Q;
     {
         ArgMaxSum Ps, Qs;
@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
     const __nv_bfloat16 *rowq = static_cast<const __nv_bfloat16 *>(a.draft) + b * a.stride_seq + n * a.stride_node;
     const StreamRow<__nv_bfloat16, false> vq(rowq, a.vocab);
     const Geo g = make_geo(a.vocab, 8);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int lo = g.seg_lo(warp), hi = g.seg_hi(warp);
     const float k = kLog2e / temperature_of(a, b);
     const float u1 = a.uniforms[r * 5 + 0], u2 = a.uniforms[r * 5 + 1];

@@ -21,6 +21,8 @@
 
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "spechub.h"
 #include "spechub_common.cuh"
 #include "spechub_stream.cuh"
@@ -30,7 +32,7 @@
 namespace spechub {
 namespace cg = cooperative_groups;
 
-constexpr int kLeanMaxWarps = 32;
+constexpr int kLeanMaxWarps = 16;
 constexpr int kLeanCk = 16;       // checkpoints per warp in the draft step's pass A, at most
 constexpr float kNoIds = 6.2e-33f;  // 2^-107
 constexpr float kHuge = 1.0e30f;  // ~2^100: partial sums beyond this move the reference
@@ -142,6 +144,34 @@ __device__ __forceinline__ void lean_push(LeanAcc<LT> &st, const Vec8<LT> &v, fl
     st.s += a;
 }
 
+// ... of a batch of vectors: the same sums in the same order, with one look at their size.  (Where that fails the vectors,
+// vi, vi + 32, ..., are read again: kept for it, they would not fit the registers.)
+template <typename LT>
+struct LeanBatch {
+    LeanAcc<LT> &st;
+    F2 k2, nc2;
+    float s;
+    typename Vec8<LT>::Max m2;
+    __device__ __forceinline__ LeanBatch(LeanAcc<LT> &a) : st(a) {}
+    __device__ __forceinline__ void begin(float k) { k2 = f2_make(k, k); again(); }
+    __device__ __forceinline__ void again() { nc2 = f2_make(-st.c, -st.c); s = st.s; m2 = st.m2; }
+    __device__ __forceinline__ void push(const Vec8<LT> &v) {
+        m2 = Vec8<LT>::max_of(m2, v.packed_max());
+        s += vec_sum(v, k2, nc2);
+    }
+    template <int D, class IN>
+    __device__ __forceinline__ void commit(const IN &in, float k, int vi, int hi) {
+        if (s < kHuge) {
+            st.m2 = m2;
+            st.s = s;
+        } else {
+#pragma unroll 1
+            for (int d = 0; d < D; ++d) lean_push(st, in.fix(in.checked(vi + 32 * d, hi)), k);
+            again();
+        }
+    }
+};
+
 // the exponent reference of a thread: the maximum of its first vector that holds a finite logit
 template <class ROW>
 __device__ __forceinline__ float lean_reference(const ROW &row, int vi, int hi, float k) {
@@ -152,83 +182,78 @@ __device__ __forceinline__ float lean_reference(const ROW &row, int vi, int hi, 
     return 0.f;
 }
 
-// Pass A over this warp's range of one or two rows.
+// ... whose first vector is at hand
+template <typename LT, class ROW>
+__device__ __forceinline__ float lean_reference(const Vec8<LT> &first, const ROW &row, int v0, int hi, float k) {
+    const float m0 = first.max();
+    return m0 > neg_inf() ? shift_of(m0, k) : lean_reference(row, v0 + 32, hi, k);
+}
+
+// This warp's range of two rows: f(vector index, target vector, draft vector), as in pair_turns
+template <int STEP, typename LT, bool SHIFT, class F>
+__device__ __forceinline__ void stream_pairs(const StreamRow<LT, SHIFT> &p, const StreamRow<LT, SHIFT> &q, int lo, int hi, int lane, F f) {
+    if constexpr (SHIFT) {
+        any_pairs<STEP>(p, q, lo, hi, lane, f);
+    } else {
+        const int n = (hi - lo - lane + 31) >> 5;   // this lane's vectors
+        pair_turns<STEP>(WholeIn<LT>{p}, WholeIn<LT>{q}, lo + lane, STEP > 0 ? 0 : n - 1, n, f);
+    }
+}
+// ... for the last time: L2 may let these lines go first
+template <int STEP, typename LT, bool SHIFT, class F>
+__device__ __forceinline__ void stream_pairs_last(const StreamRow<LT, SHIFT> &p, const StreamRow<LT, SHIFT> &q, int lo, int hi, int lane, F f) {
+    if constexpr (SHIFT) {
+        any_pairs<STEP>(p, q, lo, hi, lane, f);
+    } else {
+        uint64_t pol;
+        asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+        const int n = (hi - lo - lane + 31) >> 5;
+        pair_turns<STEP>(HintedIn<LT>{p, pol}, HintedIn<LT>{q, pol}, lo + lane, STEP > 0 ? 0 : n - 1, n, f);
+    }
+}
+
+// Pass A over this warp's range of two rows.
 // AHEAD: the next vector pair is requested before the current one is consumed (measured per
 // method: it pays for RRS, 1.92 -> 1.82 ms on V = 128256, and RRSw, 468 -> 455 us on 7936 rows of 32000 ids; SpecHub
 // gains 3 % on those and on few rows, and loses 5 % on 7936 rows of 128256: there it is for CTAs of 512 threads, few rows).
-template <bool BOTH, bool AHEAD, typename LT, class ROW>
-__device__ __forceinline__ void lean_pass_a(const ROW &rp, const ROW &rq, int lo, int hi, int lane, float k,
-                                            LeanAcc<LT> &P, LeanAcc<LT> &Q) {
+template <bool AHEAD, typename LT, bool SHIFT>
+__device__ __forceinline__ void lean_pass_a2(const StreamRow<LT, SHIFT> &rp, const StreamRow<LT, SHIFT> &rq, int lo, int hi, int lane, float k,
+                                             LeanAcc<LT> &P, LeanAcc<LT> &Q) {
     P.init();
     Q.init();
     int vi = lo + lane;
     P.c = lean_reference(rp, vi, hi, k);
-    if (BOTH) Q.c = lean_reference(rq, vi, hi, k);
-    if (BOTH && AHEAD) {
-        Vec8<LT> na = Vec8<LT>::none(), nb = na;
-        if (vi < hi) { na = rp[vi]; nb = rq[vi]; }
-#pragma unroll 1
-        for (; vi < hi; vi += 32) {
-            const Vec8<LT> a = na, b = nb;
-            if (vi + 32 < hi) { na = rp[vi + 32]; nb = rq[vi + 32]; }
-            lean_push(P, a, k);
-            lean_push(Q, b, k);
-        }
-    } else {
-#pragma unroll 2
-        for (; vi < hi; vi += 32) {
-            const Vec8<LT> a = rp[vi];
-            Vec8<LT> b;
-            if (BOTH) b = rq[vi];
-            lean_push(P, a, k);
-            if (BOTH) lean_push(Q, b, k);
-        }
-    }
-}
-// ... of two rows of any alignment
-template <typename LT>
-__device__ __forceinline__ void lean_pass_a_any(const StreamRow<LT, true> &rp, const StreamRow<LT, true> &rq, int lo, int hi,
-                                                int lane, float k, LeanAcc<LT> &P, LeanAcc<LT> &Q) {
-    P.init();
-    Q.init();
-    P.c = lean_reference(rp, lo + lane, hi, k);
-    Q.c = lean_reference(rq, lo + lane, hi, k);
-    any_pairs<1>(rp, rq, lo, hi, lane, [&](int, const Vec8<LT> &a, const Vec8<LT> &b) {
+    Q.c = lean_reference(rq, vi, hi, k);
+    auto push = [&](int, const Vec8<LT> &a, const Vec8<LT> &b) {
         lean_push(P, a, k);
         lean_push(Q, b, k);
-    });
+    };
+    if constexpr (AHEAD || SHIFT) {
+        stream_pairs<1>(rp, rq, lo, hi, lane, push);
+    } else {
+#pragma unroll 2
+        for (; vi < hi; vi += 32) push(vi, rp[vi], rq[vi]);
+    }
 }
 
-// Pass A over one row with 64 bytes per lane in flight: the next vectors (four of bf16, two of fp32) are requested
-// before the current ones are consumed.  Same vectors in the same order as lean_pass_a<false>, so the same sums.
-template <typename LT, class ROW>
-__device__ __forceinline__ void lean_pass_a_deep(const ROW &rp, int lo, int hi, int lane, float k, LeanAcc<LT> &P) {
-    constexpr int D = ROW::kDepth;
-    uint64_t pol;   // the row is read again by pass B: L2 is asked to keep it
-    asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
+// Pass A over one row.  KEEP: the row is read again by pass B, and L2 is asked to keep it.
+template <bool KEEP, typename LT>
+__device__ __forceinline__ void lean_pass_a1(const StreamRow<LT, false> &rp, int lo, int hi, int lane, float k, LeanAcc<LT> &P) {
     P.init();
-    P.c = lean_reference(rp, lo + lane, hi, k);
-    const int n = (hi - lo - lane + 31) >> 5;   // this lane's vectors (<= 0: none)
-    const int v0 = lo + lane;
-    int it = 0;
-    Vec8<LT> nx[D] = {};
-    if (D <= n) {
-#pragma unroll
-        for (int i = 0; i < D; ++i) nx[i] = rp.fetch(v0 + 32 * i, pol);
+    LeanBatch<LT> B(P);
+    auto run = [&](const auto &in) {
+        constexpr int D = std::decay_t<decltype(in)>::kDepth;
+        row_batches<D, true>(in, lo + lane, hi, whole_iters(lo, hi),
+                             [&](const Vec8<LT> &first) { P.c = lean_reference(first, rp, lo + lane, hi, k); B.begin(k); },
+                             [&](const Vec8<LT> &v) { B.push(v); }, [&](int vi) { B.template commit<D>(in, k, vi, hi); });
+    };
+    if constexpr (KEEP) {
+        uint64_t pol;
+        asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
+        run(HintedIn<LT>{rp, pol});
+    } else {
+        run(WholeIn<LT>{rp});
     }
-#pragma unroll 1
-    for (; it + D <= n; it += D) {
-        Vec8<LT> a[D];
-#pragma unroll
-        for (int i = 0; i < D; ++i) a[i] = nx[i];
-        if (it + 2 * D <= n) {
-#pragma unroll
-            for (int i = 0; i < D; ++i) nx[i] = rp.fetch(v0 + 32 * (it + D + i), pol);
-        }
-#pragma unroll
-        for (int i = 0; i < D; ++i) lean_push(P, a[i], k);
-    }
-    for (; it < n; ++it) lean_push(P, rp[v0 + 32 * it], k);
 }
 
 // Pass A over both rows with the vectors coming from the warp's ring (the first pass of its stream, forwards).
@@ -276,24 +301,31 @@ __device__ __forceinline__ void lean_rescan_warp(const ROW &row, int lo, int hi,
                                                  float val, float k, float c, int &first_idx,
                                                  float &s_excl) {
     int fi = 0x7fffffff;
-    // pass 1: first index
-    for (int vj = lo + src + 32 * lane; vj < hi; vj += 32 * 32) {
-        const auto v = row[vj];
+    const int v0 = lo + src + 32 * lane;
+    // the first round's vector stays in registers for the sum (ranges of up to 1024 vectors: all of them)
+    auto first = Vec8<typename ROW::Elem>::none();
+    if (v0 < hi) first = row[v0];
+    auto find = [&](const auto &v, int vj) {
 #pragma unroll
         for (int i = 7; i >= 0; --i)
             if (v.get(i) == val) fi = min(fi, vj * 8 + i);
-    }
+    };
+    if (v0 < hi) find(first, v0);
+#pragma unroll 1
+    for (int vj = v0 + 32 * 32; vj < hi; vj += 32 * 32) find(row[vj], vj);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) fi = min(fi, __shfl_xor_sync(kFull, fi, o));
-    // pass 2: the sum without it (the vectors are L1/L2 hits now)
+    // the sum without it
     float s = 0.f;
-    for (int vj = lo + src + 32 * lane; vj < hi; vj += 32 * 32) {
-        const auto v = row[vj];
+    auto add = [&](const auto &v, int vj) {
         float e[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) e[i] = (vj * 8 + i == fi) ? 0.f : ex2(__fmaf_rn(v.get(i), k, -c));
         s += ((e[0] + e[1]) + (e[2] + e[3])) + ((e[4] + e[5]) + (e[6] + e[7]));
-    }
+    };
+    if (v0 < hi) add(first, v0);
+#pragma unroll 1
+    for (int vj = v0 + 32 * 32; vj < hi; vj += 32 * 32) add(row[vj], vj);
     s_excl = warp_sum(s);
     first_idx = fi;
 }
@@ -637,8 +669,8 @@ __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, in
     // One exponent reference for the whole warp: the maximum of its first 32 vectors that hold a finite logit (nearly
     // always the very first ones; a warp whose range begins with masked ids looks further).  Behind the pass's first
     // loads (a step on 448 rows of 32000 ids: 44.9 us, 46.0 where they wait for the search).
-    auto reference = [&]() {
-        float m0 = lanes_max(lo + lane < hi ? rq[lo + lane].max() : neg_inf());
+    auto reference = [&](const Vec8<LT> &first) {
+        float m0 = lanes_max(first.max());
 #pragma unroll 1
         for (int vb = lo + 32; !(m0 > neg_inf()) && vb < hi; vb += 32)
             m0 = lanes_max(vb + lane < hi ? rq[vb + lane].max() : neg_inf());
@@ -662,33 +694,25 @@ __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, in
         tot += st.s;
         st.s = 0.f;
     };
-    const int iters = (hi - lo + 31) >> 5;   // lane-iterations of this warp
-    const int nfull = (hi - lo) >> 5;        // those in which every lane has a vector
-    const int v0 = lo + lane;
-    int it = 0, since = 0;
-    auto push = [&](const Vec8<LT> &v) { lean_push(st, v, k); };
-    auto after = [&](int d) {
-        since += d;
-        if (since >= CK) { checkpoint(); since = 0; }
+    int since = 0;
+    LeanBatch<LT> B(st);
+    auto run = [&](const auto &in, const Iters &t) {   // (the loads of the next vectors also overlap the checkpoint's shuffle chain)
+        constexpr int D = std::decay_t<decltype(in)>::kDepth;
+        row_batches<D, false>(in, lo + lane, hi, t, [&](const Vec8<LT> &first) { reference(first); B.begin(k); },
+                       [&](const Vec8<LT> &v) { B.push(v); },
+                       [&](int vi) {
+                           B.template commit<D>(in, k, vi, hi);
+                           since += D;
+                           if (since >= CK) { checkpoint(); since = 0; B.again(); }
+                       });
     };
-    auto slow = [&](int to) {
-#pragma unroll 1
-        for (; it < to; ++it) {
-            if (v0 + 32 * it < hi) push(rq[v0 + 32 * it]);
-            after(1);
-        }
-    };
-    // (the loads of the next vectors also overlap the checkpoint's shuffle chain)
     if constexpr (SHIFT) {
-        const InsideIters t = inside_iters(rq.src, rq.src, lo, hi);
-        reference();
-        slow(t.i0);
-        if (rq.src.sh == 0) it = inside_ahead(AlignedInside<LT>{rq.src}, v0, it, t.i1, [] {}, push, after);
-        else it = inside_ahead(ShiftedInside<LT>{rq.src}, v0, it, t.i1, [] {}, push, after);
+        const Iters t = inside_iters(rq.src, rq.src, lo, hi);
+        if (rq.src.sh == 0) run(AlignedIn<LT>{rq.src}, t);
+        else run(ShiftedIn<LT>{rq.src}, t);
     } else {
-        it = inside_ahead(rq, v0, it, nfull, reference, push, after);
+        run(WholeIn<LT>{rq}, whole_iters(lo, hi));
     }
-    slow(iters);
     if (since > 0) checkpoint();
     if (lane == 0)
         for (; j < slots; ++j) { cks[j] = 0.f; ckc[j] = 0.f; }
@@ -837,7 +861,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_leaf_
     if (!(a.node_kind && a.node_kind[n] == SPECHUB_NODE_LEAF)) return;
     const StreamRow<LT, SHIFT> vp(static_cast<const LT *>(a.target) + b * a.stride_seq + n * a.stride_node, a.vocab);
     const Geo g = make_geo(a.vocab, 8);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int lo = g.seg_lo(warp), hi = g.seg_hi(warp);
     const float k = kLog2e / temperature_of(a, b);
     const int K = A.k;
@@ -922,11 +946,10 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
     const StreamRow<LT, SHIFT> vp(static_cast<const LT *>(a.target) + b * a.stride_seq + n * a.stride_node, a.vocab);
     const StreamRow<LT, SHIFT> vq(static_cast<const LT *>(a.draft) + b * a.stride_seq + n * a.stride_node, a.vocab);
     const Geo g = make_geo(a.vocab, 8, CS, me);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int lo = g.seg_lo(warp), hi = g.seg_hi(warp);
-    // Pass B walks this lane's vectors backwards: what pass A read last is read again first, so
-    // the tail of the row is still in L2 even when the rows in flight exceed its capacity.
-    const int last_vi = (lo + lane < hi) ? lo + lane + ((hi - 1 - lo - lane) / 32) * 32 : lo - 1;
+    // (Pass B walks this lane's vectors backwards: what pass A read last is read again first, so
+    // the tail of the row is still in L2 even when the rows in flight exceed its capacity.)
     const float k = kLog2e / temperature_of(a, b);
     const float pinf = -neg_inf();
     // leaf rows of an unsplit call belong to lean_leaf_kernel
@@ -972,13 +995,13 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
         ring_begin(R, ring_mem + warp * kRingWarpBytes, ring_bars[warp], reinterpret_cast<const uint4 *>(vp.row),
                    reinterpret_cast<const uint4 *>(vq.row), lo, hi, 3, 2u, lane);
         lean_pass_a_ring(R, vp, vq, lane, k, tp, tq);
-    } else if constexpr (SHIFT) {
-        lean_pass_a_any(vp, vq, lo, hi, lane, k, tp, tq);
     } else if constexpr (STATS) {
-        lean_pass_a_deep(vp, lo, hi, lane, k, tp);
+        lean_pass_a1<true>(vp, lo, hi, lane, k, tp);
+    } else if constexpr (CS > 1) {
+        if (leaf) { tq.init(); lean_pass_a1<false>(vp, lo, hi, lane, k, tp); }
+        else lean_pass_a2<METHOD != kSpecHub>(vp, vq, lo, hi, lane, k, tp, tq);
     } else {
-        if (leaf) lean_pass_a<false, false>(vp, vq, lo, hi, lane, k, tp, tq);
-        else lean_pass_a<true, METHOD != kSpecHub || THREADS == 512>(vp, vq, lo, hi, lane, k, tp, tq);
+        lean_pass_a2<METHOD != kSpecHub || THREADS == 512>(vp, vq, lo, hi, lane, k, tp, tq);
     }
     RowStat P, Q;
     {
@@ -1085,27 +1108,12 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
                     rr = f2_add(rr, w);
                 }
             };
-            if constexpr (SHIFT) {
-                any_pairs<-1>(vp, vq, lo, hi, lane, vec_b);
-            } else {
-                // software pipeline: the next vector pair is in registers before this one is consumed.
-                // This is the last use of both rows: the loads tell L2 to let these lines go first (one
-                // CTA per row: 1.38 -> 1.30 ms on V = 128256; from draft statistics, where pass A also told
-                // L2 to keep the target row's lines, 1.07 -> 1.02 ms.  Keep-hints on pass A of the kernel
-                // that reads both rows twice cost it 7-13 %).
-                uint64_t polf = 0;
-                constexpr bool kHintB = STATS || CS == 1;
-                if (kHintB) asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(polf));
-                auto ldb = [&](const StreamRow<LT, SHIFT> &row, int vi) { return kHintB ? row.fetch(vi, polf) : row.fetch(vi); };
-                V np = V::none(), nq = np;
-                if (last_vi >= lo) { np = ldb(vp, last_vi); nq = ldb(vq, last_vi); }
-#pragma unroll 1
-                for (int vi = last_vi; vi >= lo; vi -= 32) {
-                    const V cp = np, cq = nq;
-                    if (vi - 32 >= lo) { np = ldb(vp, vi - 32); nq = ldb(vq, vi - 32); }
-                    vec_b(vi, cp, cq);
-                }
-            }
+            // This is the last use of both rows: the loads tell L2 to let these lines go first (one
+            // CTA per row: 1.38 -> 1.30 ms on V = 128256; from draft statistics, where pass A also told
+            // L2 to keep the target row's lines, 1.07 -> 1.02 ms.  Keep-hints on pass A of the kernel
+            // that reads both rows twice cost it 7-13 %).
+            if constexpr (CS == 1) stream_pairs_last<-1>(vp, vq, lo, hi, lane, vec_b);
+            else stream_pairs<-1>(vp, vq, lo, hi, lane, vec_b);
             };
             pass_b();
             float acc[3] = {f2_sum(s1), f2_sum(s2), f2_sum(rr)};
@@ -1184,9 +1192,6 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
             F2 a1;   // (packed: low lane = even ids of a vector, high lane = odd ids)
             const F2 k2 = f2_make(k, k), ncq2 = f2_make(-cQ, -cQ);
             F2 ncp2, nrho2;
-            // RRSw: the next vector pair is loaded before the current one is consumed (measured:
-            // 2.21 -> 2.03 ms on V = 128256; for RRS the plain loop unrolled twice is the faster one)
-            constexpr bool PIPE = (METHOD == kRRSw);
             auto vec_b = [&](int vi, const V &cp, const V &cq) {
                 if (STATS) diff |= cp.differs(cq);
                 F2 eq[4];   // e_q of the vector, by words
@@ -1208,7 +1213,6 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
                     dnb += (qq[4] + qq[5]) + (qq[6] + qq[7]);
                 }
             };
-            V np = V::none(), nq = np;
             auto pass_b = [&](bool from_ring) {
             a1 = f2_make(0.f, 0.f); dna = 0.f; dnb = 0.f;
             ncp2 = f2_make(-cP, -cP); nrho2 = f2_make(-rho, -rho);
@@ -1229,22 +1233,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
                 return;
             }
             }
-            if constexpr (SHIFT) {
-                any_pairs<-1>(vp, vq, lo, hi, lane, vec_b);
-            } else {
-                if (PIPE && last_vi >= lo) { np = vp[last_vi]; nq = vq[last_vi]; }
-#pragma unroll(PIPE ? 1 : 2)
-                for (int vi = last_vi; vi >= lo; vi -= 32) {
-                    V cp, cq;
-                    if (PIPE) {
-                        cp = np; cq = nq;
-                        if (vi - 32 >= lo) { np = vp[vi - 32]; nq = vq[vi - 32]; }
-                    } else {
-                        cp = vp[vi]; cq = vq[vi];
-                    }
-                    vec_b(vi, cp, cq);
-                }
-            }
+            stream_pairs<-1>(vp, vq, lo, hi, lane, vec_b);
             };
             pass_b(true);
             float acc[2] = {f2_sum(a1), dna + dnb};
@@ -1297,24 +1286,10 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
                         if (v0 + j * 32 < hi) vec_c(v0 + j * 32, x, y);
                     }
                 }
-            } else if constexpr (SHIFT) {
-                any_pairs<1>(vp, vq, lo, hi, lane, vec_c);
+            } else if constexpr (CS == 1) {
+                stream_pairs_last<1>(vp, vq, lo, hi, lane, vec_c);
             } else {
-                uint64_t polc = 0;   // one CTA per row: the rows' last use, L2 may let these lines go first
-                if (CS == 1) asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(polc));
-                auto ldc = [&](const StreamRow<LT, SHIFT> &row, int vi) { return CS == 1 ? row.fetch(vi, polc) : row.fetch(vi); };
-                if (PIPE && lo + lane < hi) { np = ldc(vp, lo + lane); nq = ldc(vq, lo + lane); }
-#pragma unroll(PIPE ? 1 : 2)
-                for (int vi = lo + lane; vi < hi; vi += 32) {
-                    V cp, cq;
-                    if (PIPE) {
-                        cp = np; cq = nq;
-                        if (vi + 32 < hi) { np = ldc(vp, vi + 32); nq = ldc(vq, vi + 32); }
-                    } else {
-                        cp = ldc(vp, vi); cq = ldc(vq, vi);
-                    }
-                    vec_c(vi, cp, cq);
-                }
+                stream_pairs<1>(vp, vq, lo, hi, lane, vec_c);
             }
             float w2a, w2b;
             f2_get(w2, w2a, w2b);
@@ -1393,14 +1368,15 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_kernel(Row
     const __nv_bfloat16 *rowq = static_cast<const __nv_bfloat16 *>(a.draft) + b * a.stride_seq + n * a.stride_node;
     const StreamRow<__nv_bfloat16, false> vq(rowq, a.vocab);
     const Geo g = make_geo(a.vocab, 8, CS, me);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int lo = g.seg_lo(warp), hi = g.seg_hi(warp);
     const float k = kLog2e / temperature_of(a, b);
     const float u1 = a.uniforms[r * 5 + 0], u2 = a.uniforms[r * 5 + 1];
     const bool writer = (me == 0 && threadIdx.x == 0);
 
     LeanAcc<__nv_bfloat16> tq, unused;
-    lean_pass_a<false, false>(vq, vq, lo, hi, lane, k, tq, unused);
+    unused.init();
+    lean_pass_a1<false>(vq, lo, hi, lane, k, tq);
     {
         ArgMaxSum q, unusedq;
         lean_reduce2<false>(tq, unused, vq, vq, lo, hi, k, sh, q, unusedq);
@@ -1512,7 +1488,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
     const int b = static_cast<int>(r / a.nodes), n = static_cast<int>(r % a.nodes);
     const StreamRow<LT, SHIFT> vq(static_cast<const LT *>(a.draft) + b * a.stride_seq + n * a.stride_node, a.vocab);
     const Geo g = make_geo(a.vocab, 8);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int lo = g.seg_lo(warp), hi = g.seg_hi(warp);
     const float k = kLog2e / temperature_of(a, b);
     const float u1 = a.uniforms[r * 5 + 0], u2 = a.uniforms[r * 5 + 1];

@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_kary_draft_kerne
     const int b = static_cast<int>(r / a.nodes), n = static_cast<int>(r % a.nodes);
     const StreamRow<LT, SHIFT> vq(static_cast<const LT *>(a.draft) + b * a.stride_seq + n * a.stride_node, a.vocab);
     const Geo g = make_geo(a.vocab, 8);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int lo = g.seg_lo(warp), hi = g.seg_hi(warp);
     const float k = kLog2e / temperature_of(a, b);
     const float *un = a.uniforms + r * (2 * K + 1);
@@ -87,17 +87,6 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_kary_draft_kerne
 }
 
 // ---- verification ---------------------------------------------------------------------------------
-// This warp's range of two rows: f(vector index, target vector, draft vector), next pair of vectors in flight
-template <int STEP, typename LT, bool SHIFT, class F>
-__device__ __forceinline__ void stream_pairs(const StreamRow<LT, SHIFT> &p, const StreamRow<LT, SHIFT> &q, int lo, int hi, int lane, F f) {
-    if constexpr (SHIFT) {
-        any_pairs<STEP>(p, q, lo, hi, lane, f);
-    } else {
-        const int n = (hi - lo - lane + 31) >> 5;   // this lane's vectors
-        inside_pairs<STEP>(p, q, lo + lane, STEP > 0 ? 0 : n - 1, n, f);
-    }
-}
-
 template <typename LT, bool SHIFT, int THREADS>
 __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_kary_verify_kernel(KaryArgs A) {
     __shared__ LeanKaryShared sh;
@@ -112,7 +101,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_kary_
     const StreamRow<LT, SHIFT> vp(static_cast<const LT *>(a.target) + b * a.stride_seq + n * a.stride_node, a.vocab);
     const StreamRow<LT, SHIFT> vq(static_cast<const LT *>(a.draft) + b * a.stride_seq + n * a.stride_node, a.vocab);
     const Geo g = make_geo(a.vocab, 8);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int lo = g.seg_lo(warp), hi = g.seg_hi(warp);
     const float k = kLog2e / temperature_of(a, b);
     const float pinf = -neg_inf();

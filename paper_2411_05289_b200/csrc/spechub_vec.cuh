@@ -150,32 +150,44 @@ struct RowVecs {
     __device__ __forceinline__ Vec8<LT> load_aligned(int vi) const;   // whole(vi), sh == 0
     __device__ __forceinline__ Vec8<LT> load_shifted(int vi) const;   // whole(vi), sh != 0
     __device__ __forceinline__ Vec8<LT> load_slow(int vi) const;      // any vi
+    __device__ __forceinline__ Vec8<LT> load_edge(int vi) const;      // any vi, by a call
 };
 
-// (rolled loops: this code is next to every load, and the edges of a row are all that runs it)
+// Elements y0 .. y0 + 7 (bf16) or y0 .. y0 + 3 (fp32) of a row, -inf outside it, all requested together.
+__device__ __forceinline__ uint4 edge_inline(const unsigned short *row, int y0, int V) {
+    unsigned e[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) e[i] = static_cast<unsigned>(y0 + i) < static_cast<unsigned>(V) ? row[y0 + i] : 0xff80u;
+    return make_uint4(e[0] | e[1] << 16, e[2] | e[3] << 16, e[4] | e[5] << 16, e[6] | e[7] << 16);
+}
+__device__ __forceinline__ float4 edge_inline(const float *row, int y0, int V) {
+    float e[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) e[i] = static_cast<unsigned>(y0 + i) < static_cast<unsigned>(V) ? row[y0 + i] : neg_inf();
+    return make_float4(e[0], e[1], e[2], e[3]);
+}
+// ... as a call: in the streaming kernels this is next to every load, and the edges of a row are all that runs it
+static __device__ __noinline__ uint4 edge_word(const unsigned short *row, int y0, int V) { return edge_inline(row, y0, V); }
+static __device__ __noinline__ float4 edge_word(const float *row, int y0, int V) { return edge_inline(row, y0, V); }
 template <>
 __device__ __forceinline__ Vec8<__nv_bfloat16> RowVecs<__nv_bfloat16>::load_slow(int vi) const {
-    const unsigned short *r = reinterpret_cast<const unsigned short *>(row);
-    Vec8<__nv_bfloat16> o = Vec8<__nv_bfloat16>::none();
-#pragma unroll 1
-    for (int y = vi * 8 + 7; y >= vi * 8; --y) {   // elements enter at the bottom, the last one first
-        const unsigned e = y < V ? r[y] : 0xff80u;
-#pragma unroll
-        for (int i = 3; i > 0; --i) o.w[i] = __funnelshift_l(o.w[i - 1], o.w[i], 16);
-        o.w[0] = (o.w[0] << 16) | e;
-    }
-    return o;
+    const uint4 a = edge_inline(reinterpret_cast<const unsigned short *>(row), vi * 8, V);
+    return {{a.x, a.y, a.z, a.w}};
 }
 template <>
 __device__ __forceinline__ Vec8<float> RowVecs<float>::load_slow(int vi) const {
-    Vec8<float> o = Vec8<float>::none();
-#pragma unroll 1
-    for (int y = vi * 8 + 7; y >= vi * 8; --y) {
-#pragma unroll
-        for (int i = 7; i > 0; --i) o.f[i] = o.f[i - 1];
-        o.f[0] = y < V ? row[y] : neg_inf();
-    }
-    return o;
+    const float4 a = edge_inline(row, vi * 8, V), b = edge_inline(row, vi * 8 + 4, V);
+    return {{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}};
+}
+template <>
+__device__ __forceinline__ Vec8<__nv_bfloat16> RowVecs<__nv_bfloat16>::load_edge(int vi) const {
+    const uint4 a = edge_word(reinterpret_cast<const unsigned short *>(row), vi * 8, V);
+    return {{a.x, a.y, a.z, a.w}};
+}
+template <>
+__device__ __forceinline__ Vec8<float> RowVecs<float>::load_edge(int vi) const {
+    const float4 a = edge_word(row, vi * 8, V), b = edge_word(row, vi * 8 + 4, V);
+    return {{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}};
 }
 
 template <>
@@ -254,15 +266,13 @@ __device__ __forceinline__ Vec8<float> load_hint(const Vec8<float> *p, uint64_t 
 template <typename LT, bool SHIFT> struct StreamRow;
 template <typename LT>
 struct StreamRow<LT, false> {
-    using Raw = Vec8<LT>;
-    static constexpr int kDepth = 8 / sizeof(LT);   // vectors per lane that a pass keeps in flight: 64 bytes
+    using Elem = LT;
     const LT *row;
     __device__ __forceinline__ StreamRow(const LT *r, int) : row(r) {}
     __device__ __forceinline__ const Vec8<LT> *vec(int vi) const { return reinterpret_cast<const Vec8<LT> *>(row) + vi; }
     __device__ __forceinline__ Vec8<LT> operator[](int vi) const;
-    __device__ __forceinline__ Raw fetch(int vi) const { return (*this)[vi]; }
-    __device__ __forceinline__ Raw fetch(int vi, uint64_t pol) const { return load_hint(vec(vi), pol); }
-    __device__ __forceinline__ Vec8<LT> fix(const Raw &r) const { return r; }
+    __device__ __forceinline__ Vec8<LT> fetch(int vi) const { return (*this)[vi]; }
+    __device__ __forceinline__ Vec8<LT> fetch(int vi, uint64_t pol) const { return load_hint(vec(vi), pol); }
     __device__ __forceinline__ float one(int y) const { return load_one<LT>(row, y); }
 };
 template <>
@@ -280,112 +290,208 @@ __device__ __forceinline__ Vec8<float> StreamRow<float, false>::operator[](int v
 }
 template <typename LT>
 struct StreamRow<LT, true> {
+    using Elem = LT;
     RowVecs<LT> src;
     __device__ __forceinline__ StreamRow(const LT *r, int vocab) : src(r, vocab) {}
     __device__ __forceinline__ Vec8<LT> operator[](int vi) const {
-        if (!src.whole(vi)) return src.load_slow(vi);
+        if (!src.whole(vi)) return src.load_edge(vi);
         return src.sh == 0 ? src.load_aligned(vi) : src.load_shifted(vi);
     }
     __device__ __forceinline__ float one(int y) const { return load_one<LT>(src.row, y); }
 };
 
-// The inside of such a row (whole vectors) for the loops that keep loads in flight: they take the words of a vector
-// (fetch) and make the vector of them when it is used (fix).  Shifting is arithmetic on what was loaded: done at
-// once, it would wait for the load.
+// A row as the loops below take it: plain(vi) where all lanes' vectors are whole, checked(vi, hi) anywhere (-inf from
+// vector hi on).  Shifted rows are kept as the words of a vector (Raw) and made into the vector when it is used (fix):
+// shifting is arithmetic on what was loaded; done at once, it would wait for the load.
+template <typename LT>
+struct WholeIn {
+    using Raw = Vec8<LT>;
+    static constexpr int kDepth = 8 / sizeof(LT);   // vectors per lane that a pass over one row keeps in flight: 64 bytes
+    const StreamRow<LT, false> &row;
+    __device__ __forceinline__ Raw plain(int vi) const { return row[vi]; }
+    __device__ __forceinline__ Raw checked(int vi, int hi) const {
+        Raw v = Raw::none();
+        if (vi < hi) v = plain(vi);
+        return v;
+    }
+    __device__ __forceinline__ Vec8<LT> fix(const Raw &r) const { return r; }
+};
+template <typename LT>
+struct HintedIn {   // ... with an L2 eviction policy
+    using Raw = Vec8<LT>;
+    static constexpr int kDepth = 8 / sizeof(LT);
+    const StreamRow<LT, false> &row;
+    uint64_t pol;
+    __device__ __forceinline__ Raw plain(int vi) const { return row.fetch(vi, pol); }
+    __device__ __forceinline__ Raw checked(int vi, int hi) const {
+        Raw v = Raw::none();
+        if (vi < hi) v = plain(vi);
+        return v;
+    }
+    __device__ __forceinline__ Vec8<LT> fix(const Raw &r) const { return r; }
+};
+template <typename LT>
+struct AlignedIn {   // a row on a 16-byte boundary, of any length
+    using Raw = Vec8<LT>;
+    static constexpr int kDepth = 8 / sizeof(LT);
+    const RowVecs<LT> &src;
+    __device__ __forceinline__ Raw plain(int vi) const { return src.load_aligned(vi); }
+    __device__ __forceinline__ Raw checked(int vi, int hi) const {
+        Raw v = Raw::none();
+        if (vi < hi) v = src.whole(vi) ? src.load_aligned(vi) : src.load_edge(vi);
+        return v;
+    }
+    __device__ __forceinline__ Vec8<LT> fix(const Raw &r) const { return r; }
+};
 template <typename LT> struct ShiftRaw;
 template <> struct ShiftRaw<__nv_bfloat16> { uint4 a, b; };
 template <> struct ShiftRaw<float> { float4 a, b, c; };
 template <typename LT>
-struct AlignedInside {
-    using Raw = Vec8<LT>;
-    static constexpr int kDepth = 8 / sizeof(LT);
-    const RowVecs<LT> &src;
-    __device__ __forceinline__ Raw fetch(int vi) const { return src.load_aligned(vi); }
-    __device__ __forceinline__ Vec8<LT> fix(const Raw &r) const { return r; }
-};
-template <typename LT>
-struct ShiftedInside {
+struct ShiftedIn {   // any other row
     using Raw = ShiftRaw<LT>;
     static constexpr int kDepth = 4 / sizeof(LT);   // (two or three words for one vector)
     const RowVecs<LT> &src;
-    __device__ __forceinline__ Raw fetch(int vi) const;
+    __device__ __forceinline__ Raw plain(int vi) const;
+    __device__ __forceinline__ Raw checked(int vi, int hi) const;
     __device__ __forceinline__ Vec8<LT> fix(const Raw &r) const;
 };
 template <>
-__device__ __forceinline__ ShiftRaw<__nv_bfloat16> ShiftedInside<__nv_bfloat16>::fetch(int vi) const {
+__device__ __forceinline__ ShiftRaw<__nv_bfloat16> ShiftedIn<__nv_bfloat16>::plain(int vi) const {
     const uint4 *p = reinterpret_cast<const uint4 *>(src.row - src.sh) + vi;
     return {p[0], p[1]};
 }
 template <>
-__device__ __forceinline__ Vec8<__nv_bfloat16> ShiftedInside<__nv_bfloat16>::fix(const Raw &r) const {
+__device__ __forceinline__ ShiftRaw<__nv_bfloat16> ShiftedIn<__nv_bfloat16>::checked(int vi, int hi) const {
+    const uint4 n = make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);
+    ShiftRaw<__nv_bfloat16> r = {n, n};
+    if (vi < hi) {
+        if (src.whole(vi)) {
+            r = plain(vi);
+        } else {
+            const unsigned short *e = reinterpret_cast<const unsigned short *>(src.row);
+            r.a = edge_word(e, vi * 8 - src.sh, src.V);
+            r.b = edge_word(e, vi * 8 - src.sh + 8, src.V);
+        }
+    }
+    return r;
+}
+template <>
+__device__ __forceinline__ Vec8<__nv_bfloat16> ShiftedIn<__nv_bfloat16>::fix(const Raw &r) const {
     return shift_words(r.a, r.b, src.sh);
 }
 template <>
-__device__ __forceinline__ ShiftRaw<float> ShiftedInside<float>::fetch(int vi) const {
+__device__ __forceinline__ ShiftRaw<float> ShiftedIn<float>::plain(int vi) const {
     const float4 *p = reinterpret_cast<const float4 *>(src.row - src.sh) + 2 * vi;
     return {p[0], p[1], p[2]};
 }
 template <>
-__device__ __forceinline__ Vec8<float> ShiftedInside<float>::fix(const Raw &r) const {
+__device__ __forceinline__ ShiftRaw<float> ShiftedIn<float>::checked(int vi, int hi) const {
+    const float4 n = make_float4(neg_inf(), neg_inf(), neg_inf(), neg_inf());
+    ShiftRaw<float> r = {n, n, n};
+    if (vi < hi) {
+        if (src.whole(vi)) {
+            r = plain(vi);
+        } else {
+            r.a = edge_word(src.row, vi * 8 - src.sh, src.V);
+            r.b = edge_word(src.row, vi * 8 - src.sh + 4, src.V);
+            r.c = edge_word(src.row, vi * 8 - src.sh + 8, src.V);
+        }
+    }
+    return r;
+}
+template <>
+__device__ __forceinline__ Vec8<float> ShiftedIn<float>::fix(const Raw &r) const {
     return shift_words(r.a, r.b, r.c, src.sh);
 }
 
-// A warp's range [lo, hi) of such rows: lane-iteration `it` takes the vectors lo + 32 it + lane; the iterations
-// [i0, i1) lie inside the row (or both rows) and need no check per vector.
-struct InsideIters { int i0, i1, n; };
+// A warp's range [lo, hi) of a row: lane-iteration `it` takes the vectors lo + 32 it + lane; in the iterations [i0, i1)
+// every lane has a whole vector.  The same in every lane, as the compiler can see (warp_index).
+struct Iters { int i0, i1, n; };
+__device__ __forceinline__ int warp_index() { return __shfl_sync(kFull, static_cast<int>(threadIdx.x >> 5), 0); }
+__device__ __forceinline__ Iters whole_iters(int lo, int hi) { return {0, (hi - lo) >> 5, (hi - lo + 31) >> 5}; }
 template <typename LT>
-__device__ __forceinline__ InsideIters inside_iters(const RowVecs<LT> &a, const RowVecs<LT> &b, int lo, int hi) {
-    InsideIters r;
+__device__ __forceinline__ Iters inside_iters(const RowVecs<LT> &a, const RowVecs<LT> &b, int lo, int hi) {
+    Iters r;
     r.n = (hi - lo + 31) >> 5;
-    r.i0 = min(r.n, lo < max(a.f0, b.f0) ? 4 : 0);   // (a multiple of every loop's depth)
+    r.i0 = min(r.n, lo < max(a.f0, b.f0) ? 1 : 0);
     r.i1 = max(r.i0, min(r.n, (min(hi, min(a.f1, b.f1)) - lo) >> 5));
     return r;
 }
 
-// Loops over the inside of one row, kDepth vectors per lane in flight: the next ones are requested before the
-// current ones are used.  begin() is called once, with the first ones requested; f(vector); after(D) is called after
-// every D iterations.  Returns the iteration reached.
-template <class IN, class BEGIN, class F, class AFTER>
-__device__ __forceinline__ int inside_ahead(const IN &row, int v0, int it, int i1, BEGIN begin, F f, AFTER after) {
-    constexpr int D = IN::kDepth;
-    typename IN::Raw nx[D] = {};
-    if (it + D <= i1) {
+// One row, D vectors per lane in flight ahead of the D in use, in two sets of registers that take turns.  (With one set and
+// copies, the copies were a tenth of a pass's instructions; with one set and each vector's place taken by the one D further
+// on, the loads no longer come in bursts: draft step on 7936 rows of 128256 ids 352 us, 368 so, 360 with copies.)  The last
+// vectors of a range, and those at the edges of a row, come with the others (one by one behind the loop they cost up to
+// four load round trips per row): lanes that have none take -inf, which adds 0 to every sum.  begin(the lane's first
+// vector) is called with the first loads requested, one(vector) for each vector, batch(vi) after D of them, vi the first.
+// APART: the first loads are not the loop's (the same loads in the same order; in verification that keeps the passes behind
+// this one free of spills, 1010 us and 1029 above, in the draft step with more than two drafts it is what spills).
+template <int D, bool APART, class IN, class BEGIN, class ONE, class BATCH>
+__device__ __forceinline__ void row_batches(const IN &in, int v0, int hi, const Iters &t, BEGIN begin, ONE one, BATCH batch) {
+    using Raw = typename IN::Raw;
+    auto get = [&](int i, Raw (&x)[D]) {
+        if (i >= t.i0 && i + D <= t.i1) {
 #pragma unroll
-        for (int i = 0; i < D; ++i) nx[i] = row.fetch(v0 + 32 * (it + i));
-    }
-    begin();
-#pragma unroll 1
-    for (; it + D <= i1; it += D) {
-        typename IN::Raw a[D];
+            for (int d = 0; d < D; ++d) x[d] = in.plain(v0 + 32 * (i + d));
+        } else {
 #pragma unroll
-        for (int i = 0; i < D; ++i) a[i] = nx[i];
-        if (it + 2 * D <= i1) {
-#pragma unroll
-            for (int i = 0; i < D; ++i) nx[i] = row.fetch(v0 + 32 * (it + D + i));
+            for (int d = 0; d < D; ++d) x[d] = in.checked(v0 + 32 * (i + d), hi);
         }
+    };
+    auto use = [&](int i, const Raw (&x)[D]) {
 #pragma unroll
-        for (int i = 0; i < D; ++i) f(row.fix(a[i]));
-        after(D);
+        for (int d = 0; d < D; ++d) one(in.fix(x[d]));
+        batch(v0 + 32 * i);
+    };
+    Raw a[D], b[D];
+    if constexpr (APART) {
+        get(0, a);
+        begin(in.fix(a[0]));
+#pragma unroll 1
+        for (int i = 0; i < t.n; i += 2 * D) {
+            if (i + D < t.n) get(i + D, b);
+            use(i, a);
+            if (i + D >= t.n) break;
+            if (i + 2 * D < t.n) get(i + 2 * D, a);
+            use(i + D, b);
+        }
+    } else {
+#pragma unroll 1
+        for (int i = -D;;) {   // (the first turn only requests)
+            if (i + D < t.n) get(i + D, b);
+            if (i < 0) {
+                if (t.n <= 0) break;
+                begin(in.fix(b[0]));
+            } else {
+                use(i, a);
+            }
+            if ((i += D) >= t.n) break;
+            if (i + D < t.n) get(i + D, a);
+            use(i, b);
+            if ((i += D) >= t.n) break;
+        }
     }
-    return it;
 }
-// ... and over the insides of two rows, the next pair of vectors in flight; STEP = 1 or -1; f(vi, vector, vector)
+// Two rows, ascending (STEP = 1) or descending, the next pair of vectors in flight: f(vi, x, y) with the target's and the
+// draft's vector.  (Two sets of registers that take turns, the loop's code twice: verification from draft statistics on
+// 7936 rows of 128256 ids 1014 -> 1046 us, three drafts 750 -> 829; the next pair's loads behind the exponentials, in the
+// registers that held this pair: 1070, 790.)
 template <int STEP, class IN, class F>
-__device__ __forceinline__ void inside_pairs(const IN &p, const IN &q, int v0, int from, int n, F f) {
+__device__ __forceinline__ void pair_turns(const IN &p, const IN &q, int v0, int from, int n, F f) {
     typename IN::Raw np = {}, nq = {};
     int vi = v0 + 32 * from;
-    if (n > 0) { np = p.fetch(vi); nq = q.fetch(vi); }
+    if (n > 0) { np = p.plain(vi); nq = q.plain(vi); }
 #pragma unroll 1
     for (; n > 0; --n, vi += 32 * STEP) {
         const typename IN::Raw cp = np, cq = nq;
-        if (n > 1) { np = p.fetch(vi + 32 * STEP); nq = q.fetch(vi + 32 * STEP); }
+        if (n > 1) { np = p.plain(vi + 32 * STEP); nq = q.plain(vi + 32 * STEP); }
         f(vi, p.fix(cp), q.fix(cq));
     }
 }
-// All vectors of a warp's range of two rows of any alignment, in ascending (STEP = 1) or descending order.
+// All vectors of a warp's range of two rows of any alignment.
 template <int STEP, typename LT, class F>
 __device__ __forceinline__ void any_pairs(const StreamRow<LT, true> &p, const StreamRow<LT, true> &q, int lo, int hi, int lane, F f) {
-    const InsideIters t = inside_iters(p.src, q.src, lo, hi);
+    const Iters t = inside_iters(p.src, q.src, lo, hi);
     const int v0 = lo + lane;
     auto slow_run = [&](int from, int n) {
 #pragma unroll 1
@@ -398,9 +504,9 @@ __device__ __forceinline__ void any_pairs(const StreamRow<LT, true> &p, const St
     if (STEP > 0) slow_run(0, t.i0);
     else slow_run(t.n - 1, t.n - t.i1);
     if (p.src.sh == 0 && q.src.sh == 0)
-        inside_pairs<STEP>(AlignedInside<LT>{p.src}, AlignedInside<LT>{q.src}, v0, from, n, f);
+        pair_turns<STEP>(AlignedIn<LT>{p.src}, AlignedIn<LT>{q.src}, v0, from, n, f);
     else if (p.src.sh != 0 && q.src.sh != 0)
-        inside_pairs<STEP>(ShiftedInside<LT>{p.src}, ShiftedInside<LT>{q.src}, v0, from, n, f);
+        pair_turns<STEP>(ShiftedIn<LT>{p.src}, ShiftedIn<LT>{q.src}, v0, from, n, f);
     else   // (a shifted row beside one that is not: rows of two unlike buffers)
         slow_run(from, n);
     if (STEP > 0) slow_run(t.i1, t.n - t.i1);
