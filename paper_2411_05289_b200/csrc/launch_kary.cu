@@ -9,10 +9,10 @@ namespace spechub {
 template <typename LT, bool SHIFT>
 static int kary_draft(const KaryArgs &a, unsigned rows, cudaStream_t s) {
     const int th = draft_threads(a.r.vocab, rows);
-    if (th == 512) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 512>, rows, 512, 0, 1, s, a);
-    if (th == 256) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 256>, rows, 256, 0, 1, s, a);
-    if (th == 128) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 128>, rows, 128, 0, 1, s, a);
-    return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 64>, rows, 64, 0, 1, s, a);
+    if (th == 512) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 512>, rows, 512, kRowRingBytes<LT, SHIFT, 512>, 1, s, a);
+    if (th == 256) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 256>, rows, 256, kRowRingBytes<LT, SHIFT, 256>, 1, s, a);
+    if (th == 128) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 128>, rows, 128, kRowRingBytes<LT, SHIFT, 128>, 1, s, a);
+    return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 64>, rows, 64, kRowRingBytes<LT, SHIFT, 64>, 1, s, a);
 }
 template <typename LT, bool SHIFT>
 static int kary_verify(const KaryArgs &a, unsigned rows, cudaStream_t s) {

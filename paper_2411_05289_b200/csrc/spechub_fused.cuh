@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
 
     LeanAcc<__nv_bfloat16> tq, unused;
     unused.init();
-    lean_pass_a_ck<false>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * CS, sh.ckc + warp * CS, CS);
+    lean_pass_a_ck<false, THREADS>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * CS, sh.ckc + warp * CS, CS, sh.any[warp]);
     RowStat Q;
     {
         ArgMaxSum q, unusedq;
@@ -366,6 +366,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
         Q.set(q, k);
     }
     if (warp != 0) return;
+    const uint32_t missing = lean_late(sh, g) ? SPECHUB_ST_INTERNAL : 0;
     const float Zq = Q.sx + Q.own;
     if (t0 && a.draft_stats_out) {   // the record lean_draft_ck_kernel leaves, bit for bit
         DraftStat ds;
@@ -376,7 +377,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
         if (t0) {
             for (int m = 0; m < 3; ++m) {
                 A.tok_out[m][2 * r] = -1; A.tok_out[m][2 * r + 1] = -1;
-                if (A.dstatus[m]) A.dstatus[m][r] = SPECHUB_ST_NONFINITE;
+                if (A.dstatus[m]) A.dstatus[m][r] = SPECHUB_ST_NONFINITE | missing;
             }
             if (hub_out) hub_out[r] = -1;
             if (draft_prob) { draft_prob[2 * r] = 0.f; draft_prob[2 * r + 1] = 0.f; }
@@ -417,7 +418,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
         for (int m = 0; m < 3; ++m) {
             A.tok_out[m][2 * r] = x1;
             A.tok_out[m][2 * r + 1] = x2[m];
-            if (A.dstatus[m]) A.dstatus[m][r] = st[m];
+            if (A.dstatus[m]) A.dstatus[m][r] = st[m] | missing;
         }
         if (hub_out) hub_out[r] = hubtok;
         if (draft_prob) { draft_prob[2 * r] = prob0; draft_prob[2 * r + 1] = prob1; }

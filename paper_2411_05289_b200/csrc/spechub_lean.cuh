@@ -658,9 +658,19 @@ __device__ __forceinline__ int lean_ck_slots(const Geo &g, int CK) {   // sub-bl
     return (((g.seg + 31) >> 5) + CK - 1) / CK;
 }
 
-template <bool SHIFT, typename LT, class ROW>
+// The draft step's and the leaf rows' passes take bf16 rows in whole words from rings of bulk copies (spechub_ring.cuh) in
+// CTAs of 64 and 128 threads, the shapes for many long rows.  Not in one-warp CTAs (4000 rows of 10000 ids: 35 us, 39 from
+// rings), in those of 256 threads and more (448 rows of 32000: no difference) and for fp32 rows (480 rows of 128256: a step
+// 170 us, 173 from rings: a vector is 32 bytes, its reads from shared memory meet in the banks).
+template <typename LT, bool SHIFT, int THREADS>
+constexpr bool kRowRinged = sizeof(LT) == 2 && !SHIFT && (THREADS == 64 || THREADS == 128);
+template <typename LT, bool SHIFT, int THREADS>
+constexpr int kRowRingBytes = kRowRinged<LT, SHIFT, THREADS> ? THREADS / 32 * kRowWarpBytes : 0;
+
+// late: set if a bulk copy did not arrive within its bounded wait.
+template <bool SHIFT, int THREADS, typename LT, class ROW>
 __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, int lane, float k, int CK,
-                                               LeanAcc<LT> &Q, float *cks, float *ckc, int slots) {
+                                               LeanAcc<LT> &Q, float *cks, float *ckc, int slots, int &late) {
     LeanAcc<LT> st;
     st.init();
     float cref = 0.f;               // the reference every lane is expected to hold
@@ -695,28 +705,47 @@ __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, in
         st.s = 0.f;
     };
     int since = 0;
+    bool missing = false;
     LeanBatch<LT> B(st);
-    auto run = [&](const auto &in, const Iters &t) {   // (the loads of the next vectors also overlap the checkpoint's shuffle chain)
+    auto begin = [&](const Vec8<LT> &first) { reference(first); B.begin(k); };
+    auto one = [&](const Vec8<LT> &v) { B.push(v); };
+    auto batch = [&](const auto &in, int vi) {
         constexpr int D = std::decay_t<decltype(in)>::kDepth;
-        row_batches<D, false>(in, lo + lane, hi, t, [&](const Vec8<LT> &first) { reference(first); B.begin(k); },
-                       [&](const Vec8<LT> &v) { B.push(v); },
-                       [&](int vi) {
-                           B.template commit<D>(in, k, vi, hi);
-                           since += D;
-                           if (since >= CK) { checkpoint(); since = 0; B.again(); }
-                       });
+        B.template commit<D>(in, k, vi, hi);
+        since += D;
+        if (since >= CK) { checkpoint(); since = 0; B.again(); }
+    };
+    auto run = [&](const auto &in, const Iters &t) {   // (the loads of the next vectors also overlap the checkpoint's shuffle chain)
+        row_batches<std::decay_t<decltype(in)>::kDepth, false>(in, lo + lane, hi, t, begin, one, [&](int vi) { batch(in, vi); });
     };
     if constexpr (SHIFT) {
         const Iters t = inside_iters(rq.src, rq.src, lo, hi);
         if (rq.src.sh == 0) run(AlignedIn<LT>{rq.src}, t);
         else run(ShiftedIn<LT>{rq.src}, t);
+    } else if constexpr (kRowRinged<LT, SHIFT, THREADS>) {
+        extern __shared__ __align__(128) unsigned char row_ring_mem[];
+        __shared__ __align__(8) uint64_t row_ring_bars[THREADS / 32][kRowStages];
+        const int warp = warp_index();
+        const WholeIn<LT> in = {rq};
+        RowRing R;
+        row_ring_begin(R, row_ring_mem + warp * kRowWarpBytes, row_ring_bars[warp], rq.vec(lo),
+                       (hi - lo) * static_cast<int>(sizeof(Vec8<LT>)), lane);
+        ring_batches<LT>(R, lo, hi, lane, begin, one, [&](int vi) { batch(in, vi); });
+        missing = R.timed_out;
     } else {
         run(WholeIn<LT>{rq}, whole_iters(lo, hi));
     }
+    if (lane == 0) late = missing;
     if (since > 0) checkpoint();
     if (lane == 0)
         for (; j < slots; ++j) { cks[j] = 0.f; ckc[j] = 0.f; }
     Q.m2 = st.m2; Q.c = st.c; Q.s = tot;
+}
+
+// Did a copy of some warp's not arrive?  (Behind lean_reduce2; the whole warp.)
+__device__ __forceinline__ bool lean_late(const LeanCkShared &sh, const Geo &g) {
+    const int lane = threadIdx.x & 31;
+    return __any_sync(kFull, lane < g.nwarps && sh.any[lane] != 0);
 }
 
 // The draws are made by one warp, the others are done: a sub-block is a few vectors per lane, and a CTA-wide draw costs
@@ -869,7 +898,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_leaf_
     const int CK = lean_ck_interval(g), CS = lean_ck_slots(g, CK);
     LeanAcc<LT> tp, unused;
     unused.init();
-    lean_pass_a_ck<SHIFT>(vp, lo, hi, lane, k, CK, tp, sh.cks + warp * CS, sh.ckc + warp * CS, CS);
+    lean_pass_a_ck<SHIFT, THREADS>(vp, lo, hi, lane, k, CK, tp, sh.cks + warp * CS, sh.ckc + warp * CS, CS, sh.any[warp]);
     ArgMaxSum Ps, unusedq;
     lean_reduce2<false>(tp, unused, vp, vp, lo, hi, k, sh, Ps, unusedq);
     const float Zp = Ps.sx + Ps.own(k);
@@ -878,6 +907,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_leaf_
     int tok = -1;
     if (!(Ps.ml > neg_inf()) || !(Ps.ml < -neg_inf()) || !finite_pos(Zp)) status = SPECHUB_ST_NONFINITE;
     else if ((tok = lean_ck_draw(g, vp, k, Ps.c, CK, NoneOut{}, ures, sh)) < 0) tok = Ps.idx;   // (as in the draft step)
+    if (lean_late(sh, g)) status |= SPECHUB_ST_INTERNAL;
     if (threadIdx.x == 0) {
         for (int m = 0; m < A.n_out; ++m) {
             const NodeOutPtrs &o = A.out[m];
@@ -1496,7 +1526,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
 
     LeanAcc<LT> tq, unused;
     unused.init();
-    lean_pass_a_ck<SHIFT>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * CS, sh.ckc + warp * CS, CS);
+    lean_pass_a_ck<SHIFT, THREADS>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * CS, sh.ckc + warp * CS, CS, sh.any[warp]);
     RowStat Q;
     {
         ArgMaxSum q, unusedq;
@@ -1506,6 +1536,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
     if (warp != 0) return;
     const float Zq = Q.sx + Q.own;
     uint32_t st = 0;
+    const uint32_t missing = lean_late(sh, g) ? SPECHUB_ST_INTERNAL : 0;
     int x1 = -1, x2 = -1, hubtok = -1;
     float prob0 = 0.f, prob1 = 0.f;
     if (!(Q.ml > neg_inf()) || !finite_pos(Zq) || !(Q.ml < -neg_inf())) {
@@ -1548,7 +1579,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
         a.draft_tokens_out[2 * r + 1] = x2;
         if (a.hub) a.hub[r] = (method == kSpecHub) ? hubtok : -1;
         if (a.draft_prob) { a.draft_prob[2 * r] = prob0; a.draft_prob[2 * r + 1] = prob1; }
-        if (a.status) a.status[r] = st;
+        if (a.status) a.status[r] = st | missing;
     }
 }
 

@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_kary_draft_kerne
 
     LeanAcc<LT> tq, unused;
     unused.init();
-    lean_pass_a_ck<SHIFT>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * CS, sh.ckc + warp * CS, CS);
+    lean_pass_a_ck<SHIFT, THREADS>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * CS, sh.ckc + warp * CS, CS, sh.any[warp]);
     ArgMaxSum Q, unusedq;
     lean_reduce2<false>(tq, unused, vq, vq, lo, hi, k, sh, Q, unusedq);
     const float Zq = Q.sx + Q.own(k);
@@ -60,6 +60,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_kary_draft_kerne
     if (warp != 0) return;
     const bool bad = !(Q.ml > neg_inf()) || !finite_pos(Zq) || !(Q.ml < -neg_inf());
     if (bad) st = SPECHUB_ST_NONFINITE;
+    if (lean_late(sh, g)) st |= SPECHUB_ST_INTERNAL;
     for (int i = 0; i < K; ++i) {
         int t = -1;
         if (!bad) {

@@ -139,4 +139,92 @@ __device__ __forceinline__ void ring_drain(WarpRing &R) {
     R.ng = R.issued;
 }
 
+template <typename LT> __device__ __forceinline__ Vec8<LT> shared_vec(uint32_t at);
+template <>
+__device__ __forceinline__ Vec8<__nv_bfloat16> shared_vec(uint32_t at) {
+    Vec8<__nv_bfloat16> v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.w[0]), "=r"(v.w[1]), "=r"(v.w[2]), "=r"(v.w[3]) : "r"(at) : "memory");
+    return v;
+}
+template <>
+__device__ __forceinline__ Vec8<float> shared_vec(uint32_t at) {
+    Vec8<float> v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.f[0]), "=f"(v.f[1]), "=f"(v.f[2]), "=f"(v.f[3]) : "r"(at) : "memory");
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.f[4]), "=f"(v.f[5]), "=f"(v.f[6]), "=f"(v.f[7]) : "r"(at + 16) : "memory");
+    return v;
+}
+// ---- one row, once, forwards: the draft step and leaf rows ------------------------------------------------------------
+// Chunks of 2 KB (64 bytes per lane), two in flight per warp, in no registers and none of it in L1 (the draft step on 7936
+// rows of 128256 ids 351 us from registers, 339 so, 344 with three stages; 10000 rows of 65536: 238, 228, 235; of 32000:
+// 148, 141).
+constexpr int kRowStages = 2;
+constexpr int kRowChunkBytes = 2048;
+constexpr int kRowWarpBytes = kRowStages * kRowChunkBytes;
+
+struct RowRing {
+    uint32_t data, bars;   // shared-window addresses of this warp's stages and their mbarriers
+    const char *src;       // the warp's range
+    int bytes;             // of it
+    bool timed_out;
+};
+__device__ __forceinline__ void row_ring_issue(const RowRing &R, int c) {   // (one lane)
+    const uint32_t n = static_cast<uint32_t>(min(kRowChunkBytes, R.bytes - c * kRowChunkBytes));
+    const uint32_t bar = R.bars + 8u * (c % kRowStages), dst = R.data + (c % kRowStages) * kRowChunkBytes;
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(n) : "memory");
+    asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "l"(R.src + static_cast<long long>(c) * kRowChunkBytes), "r"(n), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void row_ring_begin(RowRing &R, void *data, uint64_t *bars, const void *src, int bytes, int lane) {
+    R.data = ring_saddr(data); R.bars = ring_saddr(bars);
+    R.src = static_cast<const char *>(src); R.bytes = bytes; R.timed_out = false;
+    if (lane == 0) {
+#pragma unroll
+        for (int i = 0; i < kRowStages; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(R.bars + 8u * i) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        for (int c = 0; c < kRowStages && c * kRowChunkBytes < bytes; ++c) row_ring_issue(R, c);
+    }
+    __syncwarp();
+}
+__device__ __forceinline__ void row_ring_wait(RowRing &R, int c) {
+    const uint32_t bar = R.bars + 8u * (c % kRowStages), phase = (c / kRowStages) & 1;
+    uint32_t done = 0;
+    for (unsigned i = 0; i < kRingSpinLimit && !done; ++i)
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(done) : "r"(bar), "r"(phase) : "memory");
+    if (!done) R.timed_out = true;
+}
+// As row_batches: begin(first vector), one(vector), batch(vi).
+template <typename LT, class BEGIN, class ONE, class BATCH>
+__device__ __forceinline__ void ring_batches(RowRing &R, int lo, int hi, int lane, BEGIN begin, ONE one, BATCH batch) {
+    constexpr int D = kRowChunkBytes / (32 * static_cast<int>(sizeof(Vec8<LT>)));
+    const int chunks = (hi - lo + 32 * D - 1) / (32 * D);
+#pragma unroll 1
+    for (int c = 0; c < chunks; ++c) {
+        const int v0 = lo + lane + 32 * D * c;
+        row_ring_wait(R, c);
+        Vec8<LT> x[D];
+        const uint32_t at = R.data + (c % kRowStages) * kRowChunkBytes + lane * static_cast<int>(sizeof(Vec8<LT>));
+        if (v0 - lane + 32 * D <= hi) {
+#pragma unroll
+            for (int d = 0; d < D; ++d) x[d] = shared_vec<LT>(at + 32 * d * sizeof(Vec8<LT>));
+        } else {
+#pragma unroll
+            for (int d = 0; d < D; ++d) {
+                x[d] = Vec8<LT>::none();
+                if (v0 + 32 * d < hi) x[d] = shared_vec<LT>(at + 32 * d * sizeof(Vec8<LT>));
+            }
+        }
+        __syncwarp();
+        if (lane == 0 && (c + kRowStages) * kRowChunkBytes < R.bytes) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            row_ring_issue(R, c + kRowStages);
+        }
+        if (c == 0) begin(x[0]);
+#pragma unroll
+        for (int d = 0; d < D; ++d) one(x[d]);
+        batch(v0);
+    }
+}
+
 }  // namespace spechub
