@@ -8,7 +8,10 @@ namespace spechub {
 
 template <typename LT, bool SHIFT>
 static int kary_draft(const KaryArgs &a, unsigned rows, cudaStream_t s) {
-    const int th = draft_threads(a.r.vocab, rows);
+    constexpr bool kWords = sizeof(LT) == 2 && !SHIFT;
+    const int th = draft_threads(a.r.vocab, rows, kWords);
+    if constexpr (kWords)
+        if (th == 32) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 32>, rows, 32, 0, 1, s, a);
     if (th == 512) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 512>, rows, 512, kRowRingBytes<LT, SHIFT, 512>, 1, s, a);
     if (th == 256) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 256>, rows, 256, kRowRingBytes<LT, SHIFT, 256>, 1, s, a);
     if (th == 128) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 128>, rows, 128, kRowRingBytes<LT, SHIFT, 128>, 1, s, a);

@@ -12,7 +12,10 @@ static int draft_group(const RowArgs &a, int method, unsigned rows, cudaStream_t
 
 template <typename LT, bool SHIFT>
 static int draft_rows(const RowArgs &a, int method, bool keep_stats, unsigned rows, cudaStream_t s) {
-    const int th = draft_threads(a.vocab, rows);
+    constexpr bool kWords = sizeof(LT) == 2 && !SHIFT;
+    const int th = draft_threads(a.vocab, rows, kWords);
+    if constexpr (kWords)
+        if (th == 32) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 32>, rows, 32, 0, 1, s, a, method, keep_stats);
     if (th == 512) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 512>, rows, 512, kRowRingBytes<LT, SHIFT, 512>, 1, s, a, method, keep_stats);
     if (th == 256) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 256>, rows, 256, kRowRingBytes<LT, SHIFT, 256>, 1, s, a, method, keep_stats);
     if (th == 128) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 128>, rows, 128, kRowRingBytes<LT, SHIFT, 128>, 1, s, a, method, keep_stats);
@@ -30,7 +33,7 @@ int launch_lean_draft(int format, int method, int cs, const RowArgs &a, bool kee
 
 template <typename LT, bool SHIFT>
 static int leaf_rows(const LeafArgs &la, unsigned rows, cudaStream_t s) {
-    const int th = draft_threads(la.r.vocab, rows);
+    const int th = draft_threads(la.r.vocab, rows, false);
     if (th == 512) return launch_grid(lean_leaf_kernel<LT, SHIFT, 512>, rows, 512, kRowRingBytes<LT, SHIFT, 512>, 1, s, la);
     if (th == 256) return launch_grid(lean_leaf_kernel<LT, SHIFT, 256>, rows, 256, kRowRingBytes<LT, SHIFT, 256>, 1, s, la);
     if (th == 128) return launch_grid(lean_leaf_kernel<LT, SHIFT, 128>, rows, 128, kRowRingBytes<LT, SHIFT, 128>, 1, s, la);

@@ -18,7 +18,13 @@ constexpr int threads_for_few(unsigned rows, int many) {
 // 64 threads: one warp draws while the others' registers idle, which weighs more the shorter the row and the more draws
 // it makes (3584 rows: RRSw V = 16384 44.0 -> 37.9 us, V = 32000 67.7 -> 61.8, SpecHub 58.6 -> 59.1; three drafts, 10240
 // rows of 32000 216 -> 199; but V = 65472 106 -> 109, SpecHub 95 -> 105, and 1400 rows of 32000 27.8 -> 31.8).
-constexpr int draft_threads(int vocab, unsigned rows) {
+// words: bf16 rows in whole words, of a draft step.  Short ones in more than a quarter of a wave of one-warp CTAs take
+// those: no warp idles while one draws, nothing waits at a barrier (64 / 32 threads, 2500 rows: V = 4096 22.5 / 19.2 us,
+// 8192 26.6 / 23.5; 20000 rows: V = 2500 88 / 64, 4096 100 / 76, 8192 121 / 102; but 800 rows of 8192 16.4 / 18.4, 5000 of
+// 12000 49 / 51, of 24000 74 / 84: more rows in flight than L2 holds until their draws.  Not fp32 or shifted rows, whose
+// passes are longer, and not leaf rows, which are half of a call's: a step on 1300 fp32 rows of 9999 ids 82 / 116).
+constexpr int draft_threads(int vocab, unsigned rows, bool words) {
+    if (words && vocab < 10240 && rows > 8 * kSms) return 32;
     return vocab < 8192 || (vocab < 40960 && rows > 16 * kSms) ? 64 : threads_for_few(rows, 128);
 }
 // Verification: 4 CTAs of 256 threads per SM (256/512/1024: 1.54/1.65/1.87 ms on V = 128256); 128 threads on rows too
