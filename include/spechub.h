@@ -243,10 +243,13 @@ int spechub_verify_tree(const spechub_desc *desc, const void *target_logits,
  * the recorded maximum -- flags the row SPECHUB_ST_STATS with outputs -1; other
  * inconsistencies are the caller's responsibility.  Only the default path of
  * the large-vocabulary shapes (no SPECHUB_FLAG_*, k = 2, rows on 16-byte (bf16)
- * or 32-byte (fp32) boundaries, vocab % 8 == 0, vocab >= 8192) writes and reads
+ * or 32-byte (fp32) boundaries, vocab % 8 == 0, vocab >= 8192; other rows from
+ * vocab >= 16384) writes and reads
  * records; on every
  * other path the draft call clears draft_stats and the verification call
- * ignores it, so the four calls may be used unconditionally.
+ * ignores it, so the four calls may be used unconditionally.  Of the other
+ * rows (off those boundaries, or vocab % 8 != 0) a record that cannot be the
+ * row's does not flag the row: verification goes on as the plain call does.
  */
 size_t spechub_draft_stats_bytes(const spechub_desc *desc);
 int spechub_draft_sample_stats(const spechub_desc *desc, const void *draft_logits, const float *uniforms,

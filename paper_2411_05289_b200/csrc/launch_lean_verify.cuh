@@ -44,8 +44,10 @@ int launch_lean_verify_method(int format, int cs, const RowArgs &a, unsigned row
         if (lrc != SPECHUB_OK) return lrc;
     }
     const bool stats = cs == 0 && a.draft_stats_in;
-    if (format == kBf16Shift) return verify_rows<__nv_bfloat16, true, METHOD, false>(a, rows, s);
-    if (format == kF32Shift) return verify_rows<float, true, METHOD, false>(a, rows, s);
+    if (format == kBf16Shift)
+        return stats ? verify_rows<__nv_bfloat16, true, METHOD, true>(a, rows, s) : verify_rows<__nv_bfloat16, true, METHOD, false>(a, rows, s);
+    if (format == kF32Shift)
+        return stats ? verify_rows<float, true, METHOD, true>(a, rows, s) : verify_rows<float, true, METHOD, false>(a, rows, s);
     if (format == kF32)
         return stats ? verify_rows<float, false, METHOD, true>(a, rows, s) : verify_rows<float, false, METHOD, false>(a, rows, s);
     if (stats) return verify_rows<__nv_bfloat16, false, METHOD, true>(a, rows, s);

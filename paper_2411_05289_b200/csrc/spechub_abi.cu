@@ -99,9 +99,11 @@ bool resident_shape(const spechub_desc *d, bool aligned, ResShape *out) {
     return (d->flags & SPECHUB_FLAG_RESIDENT) && resident_fits(d, aligned, out);
 }
 
-// Shapes whose draft step leaves records that verification reads (see spechub_draft_sample_stats).
+// Shapes whose draft step leaves records that verification reads (see spechub_draft_sample_stats): rows in whole words from
+// 8192 ids, rows of any alignment from 16384.  (The format is the draft rows' in a draft step and both rows' in verification:
+// a shape that verification takes records of is one that every draft step leaves them for.)
 bool keeps_stats(const spechub_desc *d, int format) {
-    return d->k == 2 && d->flags == 0 && (format == kBf16 || format == kF32) && d->vocab >= 8192;
+    return d->k == 2 && d->flags == 0 && d->vocab >= (format == kBf16 || format == kF32 ? 8192 : 16384);
 }
 
 // Rows held in registers: no flag asks for another kernel.
@@ -202,6 +204,8 @@ int verify_common(const spechub_desc *d, const void *target_logits, const void *
     ka.r = a; ka.k = d->k; ka.without_replacement = (method == kRRSw);
     const int cs = lean_ok(d, al) ? lean_split(d) : 0;
     if (use_reg(true, d, al, rows, &pl)) {
+        // (these kernels only check the records; beside rows of any alignment they are not refused, see lean_verify_kernel)
+        if (fmt != kBf16 && fmt != kF32) ka.r.draft_stats_in = nullptr;
         lrc = launch_reg_verify(pl, d->dtype, ka, method, rows, s);
     } else if (d->k > 2) {
         if (resident_shape(d, al, &rs)) lrc = launch_resident_kary(rs, ka, rows, s);

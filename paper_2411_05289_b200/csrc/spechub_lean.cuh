@@ -256,6 +256,22 @@ __device__ __forceinline__ void lean_pass_a1(const StreamRow<LT, false> &rp, int
     }
 }
 
+// ... of a row of any alignment
+template <bool KEEP, typename LT>
+__device__ __forceinline__ void lean_pass_a1(const StreamRow<LT, true> &rp, int lo, int hi, int lane, float k, LeanAcc<LT> &P) {
+    P.init();
+    LeanBatch<LT> B(P);
+    const Iters t = inside_iters(rp.src, rp.src, lo, hi);
+    auto run = [&](const auto &in) {
+        constexpr int D = std::decay_t<decltype(in)>::kDepth;
+        row_batches<D, false>(in, lo + lane, hi, t,
+                              [&](const Vec8<LT> &first) { P.c = lean_reference(first, rp, lo + lane, hi, k); B.begin(k); },
+                              [&](const Vec8<LT> &v) { B.push(v); }, [&](int vi) { B.template commit<D>(in, k, vi, hi); });
+    };
+    if (rp.src.sh == 0) run(AlignedIn<LT>{rp.src});
+    else run(ShiftedIn<LT>{rp.src});
+}
+
 // Pass A over both rows with the vectors coming from the warp's ring (the first pass of its stream, forwards).
 template <class ROW>
 __device__ __forceinline__ void lean_pass_a_ring(WarpRing &R, const ROW &vp, const ROW &vq, int lane, float k,
@@ -954,7 +970,7 @@ __device__ __forceinline__ float sum_without(const RowStat &st, const ROW &row, 
 // STATS (one CTA per row): the maximum, argmax and sum of the draft row come from the record the draft
 // step left (RowArgs::draft_stats_in), so pass A reads the target row only; a record that does not belong
 // to the row (tag, argmax out of range, or another logit there than the recorded maximum) flags the row
-// SPECHUB_ST_STATS.  The passes are register-fed, with L2 eviction hints on the loads (keep the target row
+// SPECHUB_ST_STATS (shifted rows: is not looked at).  The passes are register-fed, with L2 eviction hints on the loads (keep the target row
 // after pass A, let the rows go at their last use): with a single row to keep in L2 between passes that
 // beats the rings (RRS 1.53 -> 1.46 ms, RRSw 1.62 -> 1.60 ms on V = 128256, 7936 rows).
 template <typename LT, bool SHIFT, int METHOD, int THREADS, int CS, bool RING = false, bool STATS = false>
@@ -1042,8 +1058,18 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
             sh.x_ml[0] = Ps.ml; sh.x_sx[0] = Ps.sx; sh.x_idx[0] = Ps.idx;
             if (!STATS) { sh.x_ml[1] = Qs.ml; sh.x_sx[1] = Qs.sx; sh.x_idx[1] = Qs.idx; }
         }
+        bool from_record = STATS;
+        if constexpr (STATS && SHIFT) {
+            // A record that is not the row's: as if there were none (rows that were once read without looking at records
+            // still come with whatever their caller has).  Same vectors, same order, so the plain call's bits.
+            if (!sh.stat_ok) {
+                lean_pass_a1<false>(vq, lo, hi, lane, k, tq);
+                lean_reduce2<true>(tp, tq, vp, vq, lo, hi, k, sh, Ps, Qs);
+                from_record = false;
+            }
+        }
         if (CS == 1) {   // (the published values are read by a draw from p only, after further barriers)
-            if (STATS) { Qs.ml = sh.x_ml[1]; Qs.c = shift_of(Qs.ml, k); Qs.sx = sh.x_sx[1]; Qs.idx = sh.x_idx[1]; }
+            if (from_record) { Qs.ml = sh.x_ml[1]; Qs.c = shift_of(Qs.ml, k); Qs.sx = sh.x_sx[1]; Qs.idx = sh.x_idx[1]; }
             P.set(Ps, k);
             Q.set(Qs, k);
         }
@@ -1077,7 +1103,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
     };
 
     do {
-        if (STATS && !sh.stat_ok) { o.status = SPECHUB_ST_STATS; break; }
+        if (STATS && !SHIFT && !sh.stat_ok) { o.status = SPECHUB_ST_STATS; break; }
         if (!(P.ml > neg_inf()) || !(P.ml < pinf) || !finite_pos(Zp)) { o.status = SPECHUB_ST_NONFINITE; break; }
         if (leaf) {
             // bonus token after the last accepted draft (Figure 2): a draw from p
