@@ -144,6 +144,19 @@ __device__ __forceinline__ void lean_push(LeanAcc<LT> &st, const Vec8<LT> &v, fl
     st.s += a;
 }
 
+// ... of one vector of each of two rows, with one look at both sums
+template <typename LT>
+__device__ __forceinline__ void lean_push2(LeanAcc<LT> &P, LeanAcc<LT> &Q, const Vec8<LT> &x, const Vec8<LT> &y, float k) {
+    const F2 k2 = f2_make(k, k);
+    const float sp = P.s + vec_sum(x, k2, f2_make(-P.c, -P.c)), sq = Q.s + vec_sum(y, k2, f2_make(-Q.c, -Q.c));
+    if (sp + sq < kHuge) {
+        P.m2 = Vec8<LT>::max_of(P.m2, x.packed_max()); P.s = sp;
+        Q.m2 = Vec8<LT>::max_of(Q.m2, y.packed_max()); Q.s = sq;
+    } else {
+        lean_push(P, x, k);
+        lean_push(Q, y, k);
+    }
+}
 // ... of a batch of vectors: the same sums in the same order, with one look at their size.  (Where that fails the vectors,
 // vi, vi + 32, ..., are read again: kept for it, they would not fit the registers.)
 template <typename LT>
@@ -225,8 +238,12 @@ __device__ __forceinline__ void lean_pass_a2(const StreamRow<LT, SHIFT> &rp, con
     P.c = lean_reference(rp, vi, hi, k);
     Q.c = lean_reference(rq, vi, hi, k);
     auto push = [&](int, const Vec8<LT> &a, const Vec8<LT> &b) {
+#ifdef P2
+        lean_push2(P, Q, a, b, k);
+#else
         lean_push(P, a, k);
         lean_push(Q, b, k);
+#endif
     };
     if constexpr (AHEAD || SHIFT) {
         stream_pairs<1>(rp, rq, lo, hi, lane, push);

@@ -146,8 +146,12 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_kary_
     tq.c = lean_reference(vq, lo + lane, hi, k);
     stream_pairs<1>(vp, vq, lo, hi, lane, [&](int vi, V x, V y) {
         if (mine) drop_singles(vi, x, y);
+#ifdef P2
+        lean_push2(tp, tq, x, y, k);
+#else
         lean_push(tp, x, k);
         lean_push(tq, y, k);
+#endif
     });
     const int nwarps = THREADS / 32;
     {
