@@ -244,12 +244,14 @@ int spechub_verify_tree(const spechub_desc *desc, const void *target_logits,
  * inconsistencies are the caller's responsibility.  Only the default path of
  * the large-vocabulary shapes (no SPECHUB_FLAG_*, k = 2, rows on 16-byte (bf16)
  * or 32-byte (fp32) boundaries, vocab % 8 == 0, vocab >= 8192; other rows from
- * vocab >= 16384) writes and reads
- * records; on every
- * other path the draft call clears draft_stats and the verification call
- * ignores it, so the four calls may be used unconditionally.  Of the other
- * rows (off those boundaries, or vocab % 8 != 0) a record that cannot be the
- * row's does not flag the row: verification goes on as the plain call does.
+ * vocab >= 16384) writes and reads records; on every other path the draft call
+ * clears draft_stats and the verification call ignores it, so the four calls
+ * may be used unconditionally.  Of the other rows (off those boundaries, or
+ * vocab % 8 != 0) a record that is not the row's does not flag the row:
+ * verification goes on as the plain call does.  Their records also carry a mark
+ * of 32 logits spread over the row, so those that another iteration left are
+ * told apart even where the logit at the recorded argmax is the same one; a row
+ * changed in a few places only since its draft step may not be.
  */
 size_t spechub_draft_stats_bytes(const spechub_desc *desc);
 int spechub_draft_sample_stats(const spechub_desc *desc, const void *draft_logits, const float *uniforms,

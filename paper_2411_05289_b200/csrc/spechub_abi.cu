@@ -101,9 +101,12 @@ bool resident_shape(const spechub_desc *d, bool aligned, ResShape *out) {
 
 // Shapes whose draft step leaves records that verification reads (see spechub_draft_sample_stats): rows in whole words from
 // 8192 ids, rows of any alignment from 16384.  (The format is the draft rows' in a draft step and both rows' in verification:
-// a shape that verification takes records of is one that every draft step leaves them for.)
-bool keeps_stats(const spechub_desc *d, int format) {
-    return d->k == 2 && d->flags == 0 && d->vocab >= (format == kBf16 || format == kF32 ? 8192 : 16384);
+// a shape that verification takes records of is one that every draft step leaves some for; of shifted draft rows, records
+// that were left for rows in whole words carry no mark and are not taken.)
+KeepStats keeps_stats(const spechub_desc *d, int format) {
+    const bool words = format == kBf16 || format == kF32;
+    if (d->k != 2 || d->flags != 0 || d->vocab < (words ? 8192 : 16384)) return kVoidStats;
+    return words ? kPlainStats : kMarkedStats;
 }
 
 // Rows held in registers: no flag asks for another kernel.

@@ -40,9 +40,12 @@ struct DraftStat {
     float ml;       // the row's maximum logit
     float sx;       // sum over ids != argmax of 2^(k l - rint(k ml)), k = log2(e) / T
     int idx;        // argmax, lowest id on ties
-    unsigned tag;   // kDraftStatTag ^ bits of k: a record of another kind or temperature is refused
+    unsigned tag;   // stat_tag: a record of another kind or temperature (with a mark: of another row) is not taken
 };
 constexpr unsigned kDraftStatTag = 0x51a76u << 12;   // (another number whenever the record's meaning changes)
+
+// The records a draft step leaves: void ones, those of rows read in whole words, those of other rows (row_mark).
+enum KeepStats : int { kVoidStats, kPlainStats, kMarkedStats };
 
 struct NodeOutPtrs {
     int32_t *accept_idx, *token, *hub;
@@ -67,7 +70,7 @@ struct KaryArgs {
     RowArgs r;
     int k;
     int without_replacement;
-    bool keep_stats;   // draft step: leave records that verification accepts (else void ones)
+    KeepStats keep_stats;   // draft step: the records left for verification
 };
 
 constexpr int kShardRecord = 8;  // floats per row in a phase output

@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
     if (leaf) return;   // leaf rows belong to lean_leaf_kernel
     if (STATS && threadIdx.x == THREADS - 1) {   // the draft row's record, checked off the path between the passes
         const DraftStat ds = static_cast<const DraftStat *>(a.draft_stats_in)[r];
-        bool ok = ds.tag == (kDraftStatTag ^ __float_as_uint(k));
+        bool ok = ds.tag == stat_tag(k);
         if (ok && ds.ml > neg_inf() && ds.ml < pinf && finite_pos(ds.sx + 1.f))
             ok = ds.idx >= 0 && ds.idx < a.vocab && load_one<__nv_bfloat16>(rowq, ds.idx) == ds.ml;
         sh.stat_ok = ok;
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
     const float Zq = Q.sx + Q.own;
     if (t0 && a.draft_stats_out) {   // the record lean_draft_ck_kernel leaves, bit for bit
         DraftStat ds;
-        ds.ml = Q.ml; ds.sx = Q.sx; ds.idx = Q.idx; ds.tag = kDraftStatTag ^ __float_as_uint(k);
+        ds.ml = Q.ml; ds.sx = Q.sx; ds.idx = Q.idx; ds.tag = stat_tag(k);
         static_cast<DraftStat *>(a.draft_stats_out)[r] = ds;
     }
     if (!(Q.ml > neg_inf()) || !finite_pos(Zq) || !(Q.ml < -neg_inf())) {

@@ -987,9 +987,10 @@ __device__ __forceinline__ float sum_without(const RowStat &st, const ROW &row, 
 // STATS (one CTA per row): the maximum, argmax and sum of the draft row come from the record the draft
 // step left (RowArgs::draft_stats_in), so pass A reads the target row only; a record that does not belong
 // to the row (tag, argmax out of range, or another logit there than the recorded maximum) flags the row
-// SPECHUB_ST_STATS (shifted rows: is not looked at).  The passes are register-fed, with L2 eviction hints on the loads (keep the target row
-// after pass A, let the rows go at their last use): with a single row to keep in L2 between passes that
-// beats the rings (RRS 1.53 -> 1.46 ms, RRSw 1.62 -> 1.60 ms on V = 128256, 7936 rows).
+// SPECHUB_ST_STATS; a shifted row (whose tag also marks it, row_mark) is then verified as without a record, its draft row
+// read in a pass of its own.  The passes are register-fed, those over rows in whole words with L2 eviction hints on the
+// loads (keep the target row after pass A, let the rows go at their last use): with a single row to keep in L2 between
+// passes that beats the rings (RRS 1.53 -> 1.46 ms, RRSw 1.62 -> 1.60 ms on V = 128256, 7936 rows).
 template <typename LT, bool SHIFT, int METHOD, int THREADS, int CS, bool RING = false, bool STATS = false>
 __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verify_kernel(RowArgs a) {
     static_assert(!RING || (sizeof(LT) == 2 && !SHIFT), "the ring-fed form: bf16 rows in whole words");
@@ -1034,6 +1035,8 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
         const int t1 = a.draft_tokens_in[2 * r], t2 = a.draft_tokens_in[2 * r + 1];
         DraftStat ds = {};
         if (STATS) ds = static_cast<const DraftStat *>(a.draft_stats_in)[r];
+        unsigned mark = 0;
+        if constexpr (STATS && SHIFT) mark = row_mark(vq.src.row, a.vocab);
         int y = lane > 4 ? -1 : lane == 4 ? (STATS ? ds.idx : -1) : (lane & 1) ? t2 : t1;
         if (leaf) y = -1;
         float l = neg_inf();
@@ -1042,10 +1045,12 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
         if (lane < 8) sh.lg[lane] = l;
         if (lane == 0) { sh.tk[0] = t1; sh.tk[1] = t2; }
         if (STATS && lane == 4) {
-            bool ok = ds.tag == (kDraftStatTag ^ __float_as_uint(k));
+            bool ok = ds.tag == stat_tag(k, mark);
             // (a record of a row without a finite maximum or sum needs no look-up: the row is flagged
-            // SPECHUB_ST_NONFINITE below, as it is without the record)
-            if (ok && ds.ml > neg_inf() && ds.ml < pinf && finite_pos(ds.sx + 1.f))
+            // SPECHUB_ST_NONFINITE below, as it is without the record; a shifted row is read)
+            const bool finite = ds.ml > neg_inf() && ds.ml < pinf && finite_pos(ds.sx + 1.f);
+            if (SHIFT) ok = ok && finite;
+            if (ok && finite)
                 ok = ds.idx >= 0 && ds.idx < a.vocab && l == ds.ml;
             sh.stat_ok = ok;
             sh.x_ml[1] = ds.ml; sh.x_sx[1] = ds.sx; sh.x_idx[1] = ok ? ds.idx : 0;
@@ -1078,7 +1083,8 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
         bool from_record = STATS;
         if constexpr (STATS && SHIFT) {
             // A record that is not the row's: as if there were none (rows that were once read without looking at records
-            // still come with whatever their caller has).  Same vectors, same order, so the plain call's bits.
+            // still come with whatever their caller has).  Same vectors, same order, so the plain call's bits but for
+            // RRSw's 1 - q(x1), which is sum_without's here.
             if (!sh.stat_ok) {
                 lean_pass_a1<false>(vq, lo, hi, lane, k, tq);
                 lean_reduce2<true>(tp, tq, vp, vq, lo, hi, k, sh, Ps, Qs);
@@ -1554,7 +1560,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_kernel(Row
 // Draft step, one CTA per row (checkpointed pass A and sub-block sampler above).
 // ------------------------------------------------------------------------------------------------
 template <typename LT, bool SHIFT, int THREADS>
-__global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(RowArgs a, int method, bool keep_stats) {
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(RowArgs a, int method, bool keep_stats) {   // (shifted rows: marked ones)
     __shared__ LeanCkShared sh;
     pdl_begin();
     const long long r = blockIdx.x;
@@ -1612,10 +1618,13 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
             }
         }
     }
+    unsigned mark = 0;
+    if constexpr (SHIFT)
+        if (keep_stats && a.draft_stats_out) mark = row_mark(vq.src.row, a.vocab);
     if (threadIdx.x == 0) {
         if (a.draft_stats_out) {
             DraftStat ds = {};
-            if (keep_stats) { ds.ml = Q.ml; ds.sx = Q.sx; ds.idx = Q.idx; ds.tag = kDraftStatTag ^ __float_as_uint(k); }
+            if (keep_stats) { ds.ml = Q.ml; ds.sx = Q.sx; ds.idx = Q.idx; ds.tag = stat_tag(k, mark); }
             static_cast<DraftStat *>(a.draft_stats_out)[r] = ds;
         }
         a.draft_tokens_out[2 * r] = x1;

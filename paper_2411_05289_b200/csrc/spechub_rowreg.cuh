@@ -409,9 +409,10 @@ __global__ void __launch_bounds__(kRegThreads) reg_draft_kernel(KaryArgs A, int 
     g.sync();
     PerPart mass;   // the parts' masses, ids drawn so far left out where the draws ask for it
     const RegStat Q = merge_parts<true, true>(g, sh.q, k, neg_inf(), &mass);
+    const unsigned mark = a.draft_stats_out && A.keep_stats == kMarkedStats && g.part == 0 ? row_mark(rowq, a.vocab) : 0;
     if (lead && a.draft_stats_out) {
         DraftStat ds = {};
-        if (A.keep_stats) { ds.ml = Q.ml; ds.sx = Q.sx; ds.idx = Q.idx; ds.tag = kDraftStatTag ^ __float_as_uint(k); }
+        if (A.keep_stats) { ds.ml = Q.ml; ds.sx = Q.sx; ds.idx = Q.idx; ds.tag = stat_tag(k, mark); }
         static_cast<DraftStat *>(a.draft_stats_out)[r] = ds;
     }
     if (!(Q.ml > neg_inf()) || !finite_pos(Q.Z) || !(Q.ml < -neg_inf())) {
@@ -535,7 +536,7 @@ __device__ __forceinline__ void reg_draw_from_p(const RegRow &g, PerPart mass, c
 template <typename LT>
 __device__ __forceinline__ bool draft_stat_ok(const RowArgs &a, long long r, const LT *rowq, float k) {
     const DraftStat ds = static_cast<const DraftStat *>(a.draft_stats_in)[r];
-    bool ok = ds.tag == (kDraftStatTag ^ __float_as_uint(k));
+    bool ok = ds.tag == stat_tag(k);
     if (ok && ds.ml > neg_inf() && ds.ml < -neg_inf() && finite_pos(ds.sx + 1.f))
         ok = ds.idx >= 0 && ds.idx < a.vocab && load_one<LT>(rowq, ds.idx) == ds.ml;
     return ok;

@@ -13,6 +13,18 @@ __device__ __forceinline__ void void_draft_stat(const RowArgs &a, long long r) {
     if (a.draft_stats_out) static_cast<uint4 *>(a.draft_stats_out)[r] = make_uint4(0u, 0u, 0u, 0u);
 }
 
+// What a record's tag says about the row beside its temperature.  Verification of rows that are not read in whole words
+// did not always look at records, so a buffer that an earlier iteration filled may still come with them, and the one
+// logit that is compared with the recorded maximum is the same now and then: those records also carry a mark of 32 more
+// logits, spread over the row.  (The 32 lanes of a warp; vocab >= 64.)
+template <typename LT>
+__device__ __forceinline__ unsigned row_mark(const LT *row, int vocab) {
+    const unsigned i = 2 * (threadIdx.x & 31) + 1;
+    const unsigned h = __float_as_uint(load_one<LT>(row, static_cast<int>(i) * (vocab >> 6))) * (0x9e3779b0u + i);
+    return __reduce_xor_sync(kFull, h ^ (h >> 15));
+}
+__device__ __forceinline__ unsigned stat_tag(float k, unsigned mark = 0) { return kDraftStatTag ^ __float_as_uint(k) ^ mark; }
+
 struct WarpPart {  // per-warp (max, argmax, sum without the argmax) of one row
     float ml[kMaxWarps], sx[kMaxWarps];
     int idx[kMaxWarps];

@@ -1,5 +1,6 @@
 """Draft statistics of rows that are not whole words (off a 16-byte boundary, or with a remainder), from 16384 ids: records
-are written and used, both steps against the oracle; a record that is not the row's leaves the plain call's results."""
+are written and used, both steps against the oracle; a record that is not the row's leaves the plain call's results, also
+where the logit at its argmax is the recorded maximum."""
 import numpy as np
 import pytest
 
@@ -46,10 +47,36 @@ def test_foreign_records_leave_the_plain_results(sh, V, dtype, pad):  # noqa: F8
             plain = gpu_verify(sh, m, *a, d["tokens"], und[:rows], tree, 0.8)
             for stats in (torch.zeros_like(d["stats"]), gpu_draft_stats(sh, m, a[1], und[:rows], tree, 0.5)["stats"]):
                 out = gpu_verify_stats(sh, m, *a, stats, d["tokens"], und[:rows], tree, 0.8)
-                for key in plain:
-                    if m == "rrsw" and key in ("beta", "rate"):
-                        # 1 - q(x1) is Z_q less one term here, a sum of its own there: at most 2^-22 of it apart, and
-                        # the acceptance ratio and the differences of sums of O(1) with it
-                        torch.testing.assert_close(out[key], plain[key], rtol=2e-6, atol=2e-6)
-                    else:
-                        assert torch.equal(plain[key], out[key]), (m, key, rows)
+                check_plain(m, out, plain, rows)
+
+
+def check_plain(m, out, plain, rows):
+    for key in plain:
+        if m == "rrsw" and key in ("beta", "rate"):
+            # 1 - q(x1) is Z_q less one term here, a sum of its own there: at most 2^-22 of it apart, and
+            # the acceptance ratio and the differences of sums of O(1) with it
+            torch.testing.assert_close(out[key], plain[key], rtol=2e-6, atol=2e-6)
+        else:
+            assert torch.equal(plain[key], out[key]), (m, key, rows)
+
+
+@pytest.mark.parametrize("V,dtype,pad", SHAPES)
+def test_records_of_an_earlier_iteration_leave_the_plain_results(sh, V, dtype, pad):  # noqa: F811
+    """The rows' logits are others since the draft step, except at the recorded argmax; or were not finite then."""
+    rng, B, lp, lq, un = problem(V, dtype)
+    now = workloads.round_to_storage(random_logits(rng, B, lp.shape[1], V, dtype)[1], dtype)
+    top = lq.argmax(-1)[..., None]
+    np.put_along_axis(now, top, np.take_along_axis(lq, top, -1), -1)
+    then = lq.copy()
+    then[0, 2, 5], then[1, 1, :], then[1, 2, 7] = np.nan, -np.inf, np.inf
+    tp, tq, tthen, und = padded(lp, dtype, pad), padded(now, dtype, pad), padded(then, dtype, pad), torch.from_numpy(un).cuda()
+    tree = sh.Tree.heap(lp.shape[1])
+    for rows in (B, 2):
+        for m in METHODS:
+            d = gpu_draft_stats(sh, m, tq[:rows], und[:rows], tree, 0.8)
+            a = (tp[:rows], tq[:rows])
+            plain = gpu_verify(sh, m, *a, d["tokens"], und[:rows], tree, 0.8)
+            assert int((plain["status"] & 1).sum()) == 0
+            for old in (tthen, padded(lq, dtype, pad)):
+                stats = gpu_draft_stats(sh, m, old[:rows], und[:rows], tree, 0.8)["stats"]
+                check_plain(m, gpu_verify_stats(sh, m, *a, stats, d["tokens"], und[:rows], tree, 0.8), plain, rows)
