@@ -366,18 +366,18 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
         Q.set(q, k);
     }
     if (warp != 0) return;
-    const uint32_t missing = lean_late(sh, g) ? SPECHUB_ST_INTERNAL : 0;
+    const bool late = lean_late(sh, g);   // (as in lean_draft_ck_kernel)
     const float Zq = Q.sx + Q.own;
     if (t0 && a.draft_stats_out) {   // the record lean_draft_ck_kernel leaves, bit for bit
-        DraftStat ds;
-        ds.ml = Q.ml; ds.sx = Q.sx; ds.idx = Q.idx; ds.tag = stat_tag(k);
+        DraftStat ds = {};
+        if (!late) { ds.ml = Q.ml; ds.sx = Q.sx; ds.idx = Q.idx; ds.tag = stat_tag(k); }
         static_cast<DraftStat *>(a.draft_stats_out)[r] = ds;
     }
-    if (!(Q.ml > neg_inf()) || !finite_pos(Zq) || !(Q.ml < -neg_inf())) {
+    if (late || !(Q.ml > neg_inf()) || !finite_pos(Zq) || !(Q.ml < -neg_inf())) {
         if (t0) {
             for (int m = 0; m < 3; ++m) {
                 A.tok_out[m][2 * r] = -1; A.tok_out[m][2 * r + 1] = -1;
-                if (A.dstatus[m]) A.dstatus[m][r] = SPECHUB_ST_NONFINITE | missing;
+                if (A.dstatus[m]) A.dstatus[m][r] = late ? SPECHUB_ST_INTERNAL : SPECHUB_ST_NONFINITE;
             }
             if (hub_out) hub_out[r] = -1;
             if (draft_prob) { draft_prob[2 * r] = 0.f; draft_prob[2 * r + 1] = 0.f; }
@@ -418,7 +418,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
         for (int m = 0; m < 3; ++m) {
             A.tok_out[m][2 * r] = x1;
             A.tok_out[m][2 * r + 1] = x2[m];
-            if (A.dstatus[m]) A.dstatus[m][r] = st[m] | missing;
+            if (A.dstatus[m]) A.dstatus[m][r] = st[m];
         }
         if (hub_out) hub_out[r] = hubtok;
         if (draft_prob) { draft_prob[2 * r] = prob0; draft_prob[2 * r + 1] = prob1; }

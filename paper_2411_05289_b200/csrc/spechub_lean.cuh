@@ -700,7 +700,7 @@ constexpr bool kRowRinged = sizeof(LT) == 2 && !SHIFT && (THREADS == 64 || THREA
 template <typename LT, bool SHIFT, int THREADS>
 constexpr int kRowRingBytes = kRowRinged<LT, SHIFT, THREADS> ? THREADS / 32 * kRowWarpBytes : 0;
 
-// late: set if a bulk copy did not arrive within its bounded wait.
+// late: set if a bulk copy did not arrive within its bounded wait (the results are then of the part in front of it).
 template <bool SHIFT, int THREADS, typename LT, class ROW>
 __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, int lane, float k, int CK,
                                                LeanAcc<LT> &Q, float *cks, float *ckc, int slots, int &late) {
@@ -763,8 +763,7 @@ __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, in
         RowRing R;
         row_ring_begin(R, row_ring_mem + warp * kRowWarpBytes, row_ring_bars[warp], rq.vec(lo),
                        (hi - lo) * static_cast<int>(sizeof(Vec8<LT>)), lane);
-        ring_batches<LT>(R, lo, hi, lane, begin, one, [&](int vi) { batch(in, vi); });
-        missing = R.timed_out;
+        missing = !ring_batches<LT>(R, lo, hi, lane, begin, one, [&](int vi) { batch(in, vi); });
     } else {
         run(WholeIn<LT>{rq}, whole_iters(lo, hi));
     }
@@ -938,9 +937,9 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_leaf_
     if (warp != 0) return;
     uint32_t status = 0;
     int tok = -1;
-    if (!(Ps.ml > neg_inf()) || !(Ps.ml < -neg_inf()) || !finite_pos(Zp)) status = SPECHUB_ST_NONFINITE;
+    if (lean_late(sh, g)) status = SPECHUB_ST_INTERNAL;   // (nothing is drawn from a part of the row)
+    else if (!(Ps.ml > neg_inf()) || !(Ps.ml < -neg_inf()) || !finite_pos(Zp)) status = SPECHUB_ST_NONFINITE;
     else if ((tok = lean_ck_draw(g, vp, k, Ps.c, CK, NoneOut{}, ures, sh)) < 0) tok = Ps.idx;   // (as in the draft step)
-    if (lean_late(sh, g)) status |= SPECHUB_ST_INTERNAL;
     if (threadIdx.x == 0) {
         for (int m = 0; m < A.n_out; ++m) {
             const NodeOutPtrs &o = A.out[m];
@@ -1585,10 +1584,12 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
     if (warp != 0) return;
     const float Zq = Q.sx + Q.own;
     uint32_t st = 0;
-    const uint32_t missing = lean_late(sh, g) ? SPECHUB_ST_INTERNAL : 0;
+    const bool late = lean_late(sh, g);   // (nothing is drawn from, or recorded of, a part of the row)
     int x1 = -1, x2 = -1, hubtok = -1;
     float prob0 = 0.f, prob1 = 0.f;
-    if (!(Q.ml > neg_inf()) || !finite_pos(Zq) || !(Q.ml < -neg_inf())) {
+    if (late) {
+        st = SPECHUB_ST_INTERNAL;
+    } else if (!(Q.ml > neg_inf()) || !finite_pos(Zq) || !(Q.ml < -neg_inf())) {
         st = SPECHUB_ST_NONFINITE;
     } else {
         hubtok = Q.idx;
@@ -1624,14 +1625,14 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
     if (threadIdx.x == 0) {
         if (a.draft_stats_out) {
             DraftStat ds = {};
-            if (keep_stats) { ds.ml = Q.ml; ds.sx = Q.sx; ds.idx = Q.idx; ds.tag = stat_tag(k, mark); }
+            if (keep_stats && !late) { ds.ml = Q.ml; ds.sx = Q.sx; ds.idx = Q.idx; ds.tag = stat_tag(k, mark); }
             static_cast<DraftStat *>(a.draft_stats_out)[r] = ds;
         }
         a.draft_tokens_out[2 * r] = x1;
         a.draft_tokens_out[2 * r + 1] = x2;
         if (a.hub) a.hub[r] = (method == kSpecHub) ? hubtok : -1;
         if (a.draft_prob) { a.draft_prob[2 * r] = prob0; a.draft_prob[2 * r + 1] = prob1; }
-        if (a.status) a.status[r] = st | missing;
+        if (a.status) a.status[r] = st;
     }
 }
 

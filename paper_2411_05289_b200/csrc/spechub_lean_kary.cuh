@@ -58,9 +58,8 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_kary_draft_kerne
     const float Zq = Q.sx + Q.own(k);
     uint32_t st = 0;
     if (warp != 0) return;
-    const bool bad = !(Q.ml > neg_inf()) || !finite_pos(Zq) || !(Q.ml < -neg_inf());
-    if (bad) st = SPECHUB_ST_NONFINITE;
-    if (lean_late(sh, g)) st |= SPECHUB_ST_INTERNAL;
+    const bool late = lean_late(sh, g), bad = late || !(Q.ml > neg_inf()) || !finite_pos(Zq) || !(Q.ml < -neg_inf());
+    if (bad) st = late ? SPECHUB_ST_INTERNAL : SPECHUB_ST_NONFINITE;
     for (int i = 0; i < K; ++i) {
         int t = -1;
         if (!bad) {

@@ -17,6 +17,7 @@
 
 #include <cstdint>
 
+#include "spechub_ring_run.h"
 #include "spechub_vec.cuh"
 
 namespace spechub {
@@ -165,7 +166,6 @@ struct RowRing {
     uint32_t data, bars;   // shared-window addresses of this warp's stages and their mbarriers
     const char *src;       // the warp's range
     int bytes;             // of it
-    bool timed_out;
 };
 __device__ __forceinline__ void row_ring_issue(const RowRing &R, int c) {   // (one lane)
     const uint32_t n = static_cast<uint32_t>(min(kRowChunkBytes, R.bytes - c * kRowChunkBytes));
@@ -176,7 +176,7 @@ __device__ __forceinline__ void row_ring_issue(const RowRing &R, int c) {   // (
 }
 __device__ __forceinline__ void row_ring_begin(RowRing &R, void *data, uint64_t *bars, const void *src, int bytes, int lane) {
     R.data = ring_saddr(data); R.bars = ring_saddr(bars);
-    R.src = static_cast<const char *>(src); R.bytes = bytes; R.timed_out = false;
+    R.src = static_cast<const char *>(src); R.bytes = bytes;
     if (lane == 0) {
 #pragma unroll
         for (int i = 0; i < kRowStages; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(R.bars + 8u * i) : "memory");
@@ -186,45 +186,49 @@ __device__ __forceinline__ void row_ring_begin(RowRing &R, void *data, uint64_t 
     }
     __syncwarp();
 }
-__device__ __forceinline__ void row_ring_wait(RowRing &R, int c) {
+// Did chunk c arrive, within a bounded wait?  The same in every lane.
+__device__ __forceinline__ bool row_ring_wait(const RowRing &R, int c) {
     const uint32_t bar = R.bars + 8u * (c % kRowStages), phase = (c / kRowStages) & 1;
     uint32_t done = 0;
     for (unsigned i = 0; i < kRingSpinLimit && !done; ++i)
         asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
                      : "=r"(done) : "r"(bar), "r"(phase) : "memory");
-    if (!done) R.timed_out = true;
+    return __all_sync(kFull, done);
 }
-// As row_batches: begin(first vector), one(vector), batch(vi).
+// As row_batches: begin(first vector), one(vector), batch(vi).  False: a chunk did not arrive (within its bounded wait), and
+// it and those behind it are in no sum.
 template <typename LT, class BEGIN, class ONE, class BATCH>
-__device__ __forceinline__ void ring_batches(RowRing &R, int lo, int hi, int lane, BEGIN begin, ONE one, BATCH batch) {
+__device__ __forceinline__ bool ring_batches(const RowRing &R, int lo, int hi, int lane, BEGIN begin, ONE one, BATCH batch) {
     constexpr int D = kRowChunkBytes / (32 * static_cast<int>(sizeof(Vec8<LT>)));
-    const int chunks = (hi - lo + 32 * D - 1) / (32 * D);
-#pragma unroll 1
-    for (int c = 0; c < chunks; ++c) {
-        const int v0 = lo + lane + 32 * D * c;
-        row_ring_wait(R, c);
-        Vec8<LT> x[D];
-        const uint32_t at = R.data + (c % kRowStages) * kRowChunkBytes + lane * static_cast<int>(sizeof(Vec8<LT>));
-        if (v0 - lane + 32 * D <= hi) {
+    Vec8<LT> x[D];
+    return ring_run<kRowStages>(
+        (hi - lo + 32 * D - 1) / (32 * D), [&](int c) { return row_ring_wait(R, c); },
+        [&](int c) {
+            const int v0 = lo + lane + 32 * D * c;
+            const uint32_t at = R.data + (c % kRowStages) * kRowChunkBytes + lane * static_cast<int>(sizeof(Vec8<LT>));
+            if (v0 - lane + 32 * D <= hi) {
 #pragma unroll
-            for (int d = 0; d < D; ++d) x[d] = shared_vec<LT>(at + 32 * d * sizeof(Vec8<LT>));
-        } else {
+                for (int d = 0; d < D; ++d) x[d] = shared_vec<LT>(at + 32 * d * sizeof(Vec8<LT>));
+            } else {
 #pragma unroll
-            for (int d = 0; d < D; ++d) {
-                x[d] = Vec8<LT>::none();
-                if (v0 + 32 * d < hi) x[d] = shared_vec<LT>(at + 32 * d * sizeof(Vec8<LT>));
+                for (int d = 0; d < D; ++d) {
+                    x[d] = Vec8<LT>::none();
+                    if (v0 + 32 * d < hi) x[d] = shared_vec<LT>(at + 32 * d * sizeof(Vec8<LT>));
+                }
             }
-        }
-        __syncwarp();
-        if (lane == 0 && (c + kRowStages) * kRowChunkBytes < R.bytes) {
+            __syncwarp();
+        },
+        [&](int c) {
+            if (lane != 0) return;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            row_ring_issue(R, c + kRowStages);
-        }
-        if (c == 0) begin(x[0]);
+            row_ring_issue(R, c);
+        },
+        [&](int c) {
+            if (c == 0) begin(x[0]);
 #pragma unroll
-        for (int d = 0; d < D; ++d) one(x[d]);
-        batch(v0);
-    }
+            for (int d = 0; d < D; ++d) one(x[d]);
+            batch(lo + lane + 32 * D * c);
+        });
 }
 
 }  // namespace spechub
