@@ -1264,6 +1264,11 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
                 }
                 o.status = 0;
             }
+            // RRS on bf16 rows in whole words takes plain loops unrolled twice, two pairs of loads at once, through passes B
+            // and C.  With one pair ahead instead: from draft statistics 7936 rows of 128256 ids 1412 -> 1543 us, of 32000
+            // 397 -> 399, without them 1920 rows of 50048 195 -> 199; but fp32 rows, 840 of 128256, 444 -> 432, 1920 of 32000
+            // 199 -> 184, and RRSw, whose pass B also keeps x1's place, 2.21 -> 2.03 ms on 7936 rows of 128256.
+            constexpr bool kTwoAtOnce = METHOD == kRRS && !SHIFT && sizeof(LT) == 2;
             // pass B: A1 = sum max(p - q, 0); RRSw also sums q outside x1 directly
             const int x1vec = x1 >> 3, x1el = x1 & 7;
             float dna = 0.f, dnb = 0.f;
@@ -1311,7 +1316,13 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
                 return;
             }
             }
-            stream_pairs<-1>(vp, vq, lo, hi, lane, vec_b);
+            if constexpr (kTwoAtOnce) {
+                const int n = (hi - lo - lane + 31) >> 5;   // this lane's vectors
+#pragma unroll 2
+                for (int vi = lo + lane + 32 * (n - 1); vi >= lo; vi -= 32) vec_b(vi, vp[vi], vq[vi]);
+            } else {
+                stream_pairs<-1>(vp, vq, lo, hi, lane, vec_b);
+            }
             };
             pass_b(true);
             float acc[2] = {f2_sum(a1), dna + dnb};
@@ -1363,6 +1374,14 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
                         if (j == kRingCh - 1) ring_release(R, lane);
                         if (v0 + j * 32 < hi) vec_c(v0 + j * 32, x, y);
                     }
+                }
+            } else if constexpr (kTwoAtOnce) {
+                uint64_t pol = 0;   // one CTA per row: the rows' last use, as in stream_pairs_last
+                if (CS == 1) asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+#pragma unroll 2
+                for (int vi = lo + lane; vi < hi; vi += 32) {
+                    if (CS == 1) vec_c(vi, vp.fetch(vi, pol), vq.fetch(vi, pol));
+                    else vec_c(vi, vp[vi], vq[vi]);
                 }
             } else if constexpr (CS == 1) {
                 stream_pairs_last<1>(vp, vq, lo, hi, lane, vec_c);
