@@ -15,11 +15,13 @@ static int draft_rows(const RowArgs &a, int method, bool keep_stats, unsigned ro
     constexpr bool kWords = sizeof(LT) == 2 && !SHIFT;
     const int th = draft_threads(a.vocab, rows, kWords);
     if constexpr (kWords)
-        if (th == 32) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 32>, rows, 32, 0, 1, s, a, method, keep_stats);
-    if (th == 512) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 512>, rows, 512, kRowRingBytes<LT, SHIFT, 512>, 1, s, a, method, keep_stats);
-    if (th == 256) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 256>, rows, 256, kRowRingBytes<LT, SHIFT, 256>, 1, s, a, method, keep_stats);
-    if (th == 128) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 128>, rows, 128, kRowRingBytes<LT, SHIFT, 128>, 1, s, a, method, keep_stats);
-    return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 64>, rows, 64, kRowRingBytes<LT, SHIFT, 64>, 1, s, a, method, keep_stats);
+        if (th == 32) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 32, false>, rows, 32, 0, 1, s, a, method, keep_stats);
+    if (th == 512) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 512, false>, rows, 512, 0, 1, s, a, method, keep_stats);
+    if (th == 256) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 256, false>, rows, 256, 0, 1, s, a, method, keep_stats);
+    if (th == 128 && many_rows(th, rows)) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 128, true>, rows, 128, kRowRingBytes<LT, SHIFT, 128, true>, 1, s, a, method, keep_stats);
+    if (th == 128) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 128, false>, rows, 128, 0, 1, s, a, method, keep_stats);
+    if (many_rows(th, rows)) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 64, true>, rows, 64, kRowRingBytes<LT, SHIFT, 64, true>, 1, s, a, method, keep_stats);
+    return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 64, false>, rows, 64, 0, 1, s, a, method, keep_stats);
 }
 
 int launch_lean_draft(int format, int method, int cs, const RowArgs &a, bool keep_stats, unsigned rows, cudaStream_t s) {
@@ -34,10 +36,12 @@ int launch_lean_draft(int format, int method, int cs, const RowArgs &a, bool kee
 template <typename LT, bool SHIFT>
 static int leaf_rows(const LeafArgs &la, unsigned rows, cudaStream_t s) {
     const int th = draft_threads(la.r.vocab, rows, false);
-    if (th == 512) return launch_grid(lean_leaf_kernel<LT, SHIFT, 512>, rows, 512, kRowRingBytes<LT, SHIFT, 512>, 1, s, la);
-    if (th == 256) return launch_grid(lean_leaf_kernel<LT, SHIFT, 256>, rows, 256, kRowRingBytes<LT, SHIFT, 256>, 1, s, la);
-    if (th == 128) return launch_grid(lean_leaf_kernel<LT, SHIFT, 128>, rows, 128, kRowRingBytes<LT, SHIFT, 128>, 1, s, la);
-    return launch_grid(lean_leaf_kernel<LT, SHIFT, 64>, rows, 64, kRowRingBytes<LT, SHIFT, 64>, 1, s, la);
+    if (th == 512) return launch_grid(lean_leaf_kernel<LT, SHIFT, 512, false>, rows, 512, 0, 1, s, la);
+    if (th == 256) return launch_grid(lean_leaf_kernel<LT, SHIFT, 256, false>, rows, 256, 0, 1, s, la);
+    if (th == 128 && many_rows(th, rows)) return launch_grid(lean_leaf_kernel<LT, SHIFT, 128, true>, rows, 128, kRowRingBytes<LT, SHIFT, 128, true>, 1, s, la);
+    if (th == 128) return launch_grid(lean_leaf_kernel<LT, SHIFT, 128, false>, rows, 128, 0, 1, s, la);
+    if (many_rows(th, rows)) return launch_grid(lean_leaf_kernel<LT, SHIFT, 64, true>, rows, 64, kRowRingBytes<LT, SHIFT, 64, true>, 1, s, la);
+    return launch_grid(lean_leaf_kernel<LT, SHIFT, 64, false>, rows, 64, 0, 1, s, la);
 }
 
 // The leaf rows of an unsplit call (same CTA shape as the draft step).

@@ -691,17 +691,24 @@ __device__ __forceinline__ int lean_ck_slots(const Geo &g, int CK) {   // sub-bl
     return (((g.seg + 31) >> 5) + CK - 1) / CK;
 }
 
-// The draft step's and the leaf rows' passes take bf16 rows in whole words from rings of bulk copies (spechub_ring.cuh) in
-// CTAs of 64 and 128 threads, the shapes for many long rows.  Not in one-warp CTAs (4000 rows of 10000 ids: 35 us, 39 from
-// rings), in those of 256 threads and more (448 rows of 32000: no difference) and for fp32 rows (480 rows of 128256: a step
-// 170 us, 173 from rings: a vector is 32 bytes, its reads from shared memory meet in the banks).
-template <typename LT, bool SHIFT, int THREADS>
-constexpr bool kRowRinged = sizeof(LT) == 2 && !SHIFT && (THREADS == 64 || THREADS == 128);
-template <typename LT, bool SHIFT, int THREADS>
-constexpr int kRowRingBytes = kRowRinged<LT, SHIFT, THREADS> ? THREADS / 32 * kRowWarpBytes : 0;
+// How the draft step's and the leaf rows' passes take their rows.  MANY: more rows than one wave of these CTAs (many_rows),
+// of 64 or 128 threads.  bf16 rows in whole words come from rings of bulk copies then (spechub_ring.cuh; draft step on 7936
+// rows of 128256 ids 321 us, from registers 333; 3840 of 64000 100, 110; 1792 of 32000 34.5, 35.5).  In less than a wave
+// an SM's rings hold too few bytes in flight, and a row is not behind others that hide its end (651 rows of 12800 ids 12.4
+// us, from rings 13.8; 651 of 101056 45.6, 57.7; 896 of 64000 33.3, 37.1).  Not in one-warp CTAs (4000 rows of 10000 ids: 35
+// us, 39 from rings), in those of 256 threads and more (448 rows of 32000: no difference) and for fp32 rows (480 rows of
+// 128256: a step 170 us, 173 from rings: a vector is 32 bytes, its reads from shared memory meet in the banks).
+// From registers: row_turns, whose last batch goes as far as the range does (exponentials of padding made a draft step of
+// three methods on 1170 rows of 12800 ids 16.1 us, 14.75 so); shifted rows, longer to make into vectors, row_batches while
+// they are less than a wave (448 rows of 16393 ids 14.0 us, with row_turns 14.3, 224 of 64001 17.7, 18.5; but 3840 of 64001
+// 159, 147).
+template <typename LT, bool SHIFT, int THREADS, bool MANY>
+constexpr bool kRowRinged = sizeof(LT) == 2 && !SHIFT && MANY && (THREADS == 64 || THREADS == 128);
+template <typename LT, bool SHIFT, int THREADS, bool MANY>
+constexpr int kRowRingBytes = kRowRinged<LT, SHIFT, THREADS, MANY> ? THREADS / 32 * kRowWarpBytes : 0;
 
 // late: set if a bulk copy did not arrive within its bounded wait (the results are then of the part in front of it).
-template <bool SHIFT, int THREADS, typename LT, class ROW>
+template <bool SHIFT, int THREADS, bool MANY, typename LT, class ROW>
 __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, int lane, float k, int CK,
                                                LeanAcc<LT> &Q, float *cks, float *ckc, int slots, int &late) {
     LeanAcc<LT> st;
@@ -749,13 +756,15 @@ __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, in
         if (since >= CK) { checkpoint(); since = 0; B.again(); }
     };
     auto run = [&](const auto &in, const Iters &t) {   // (the loads of the next vectors also overlap the checkpoint's shuffle chain)
-        row_batches<std::decay_t<decltype(in)>::kDepth, false>(in, lo + lane, hi, t, begin, one, [&](int vi) { batch(in, vi); });
+        constexpr int D = std::decay_t<decltype(in)>::kDepth;
+        if constexpr (SHIFT && !MANY) row_batches<D, false>(in, lo + lane, hi, t, begin, one, [&](int vi) { batch(in, vi); });
+        else row_turns<D>(in, lo + lane, hi, t, begin, one, [&](int vi) { batch(in, vi); });
     };
     if constexpr (SHIFT) {
         const Iters t = inside_iters(rq.src, rq.src, lo, hi);
         if (rq.src.sh == 0) run(AlignedIn<LT>{rq.src}, t);
         else run(ShiftedIn<LT>{rq.src}, t);
-    } else if constexpr (kRowRinged<LT, SHIFT, THREADS>) {
+    } else if constexpr (kRowRinged<LT, SHIFT, THREADS, MANY>) {
         extern __shared__ __align__(128) unsigned char row_ring_mem[];
         __shared__ __align__(8) uint64_t row_ring_bars[THREADS / 32][kRowStages];
         const int warp = warp_index();
@@ -912,7 +921,7 @@ __device__ __forceinline__ int lean_ck_draw(const Geo &g, const ROW &row, float 
 // pass A over p with checkpoints, then the sub-block sampler.  CTAs of verifying rows leave at
 // once; the verification kernels skip the leaf rows.  Up to three output sets receive the result
 // (the three-method call: the methods share u_res, hence the bonus token).
-template <typename LT, bool SHIFT, int THREADS>
+template <typename LT, bool SHIFT, int THREADS, bool MANY>
 __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_leaf_kernel(LeafArgs A) {
     __shared__ LeanCkShared sh;
     pdl_begin();
@@ -930,7 +939,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_leaf_
     const int CK = lean_ck_interval(g), CS = lean_ck_slots(g, CK);
     LeanAcc<LT> tp, unused;
     unused.init();
-    lean_pass_a_ck<SHIFT, THREADS>(vp, lo, hi, lane, k, CK, tp, sh.cks + warp * CS, sh.ckc + warp * CS, CS, sh.any[warp]);
+    lean_pass_a_ck<SHIFT, THREADS, MANY>(vp, lo, hi, lane, k, CK, tp, sh.cks + warp * CS, sh.ckc + warp * CS, CS, sh.any[warp]);
     ArgMaxSum Ps, unusedq;
     lean_reduce2<false>(tp, unused, vp, vp, lo, hi, k, sh, Ps, unusedq);
     const float Zp = Ps.sx + Ps.own(k);
@@ -1266,7 +1275,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
             }
             // RRS on bf16 rows in whole words takes plain loops unrolled twice, two pairs of loads at once, through passes B
             // and C.  With one pair ahead instead: from draft statistics 7936 rows of 128256 ids 1412 -> 1543 us, of 32000
-            // 397 -> 399, without them 1920 rows of 50048 195 -> 199; but fp32 rows, 840 of 128256, 444 -> 432, 1920 of 32000
+            // 397 -> 399, without them 1920 rows of 50048 195 -> 199; but fp32 rows, 992 of 128256, 444 -> 432, 1920 of 32000
             // 199 -> 184, and RRSw, whose pass B also keeps x1's place, 2.21 -> 2.03 ms on 7936 rows of 128256.
             constexpr bool kTwoAtOnce = METHOD == kRRS && !SHIFT && sizeof(LT) == 2;
             // pass B: A1 = sum max(p - q, 0); RRSw also sums q outside x1 directly
@@ -1577,7 +1586,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_kernel(Row
 // ------------------------------------------------------------------------------------------------
 // Draft step, one CTA per row (checkpointed pass A and sub-block sampler above).
 // ------------------------------------------------------------------------------------------------
-template <typename LT, bool SHIFT, int THREADS>
+template <typename LT, bool SHIFT, int THREADS, bool MANY>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(RowArgs a, int method, bool keep_stats) {   // (shifted rows: marked ones)
     __shared__ LeanCkShared sh;
     pdl_begin();
@@ -1593,7 +1602,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
 
     LeanAcc<LT> tq, unused;
     unused.init();
-    lean_pass_a_ck<SHIFT, THREADS>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * CS, sh.ckc + warp * CS, CS, sh.any[warp]);
+    lean_pass_a_ck<SHIFT, THREADS, MANY>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * CS, sh.ckc + warp * CS, CS, sh.any[warp]);
     RowStat Q;
     {
         ArgMaxSum q, unusedq;

@@ -425,7 +425,7 @@ __device__ __forceinline__ Iters inside_iters(const RowVecs<LT> &a, const RowVec
 // four load round trips per row): lanes that have none take -inf, which adds 0 to every sum.  begin(the lane's first
 // vector) is called with the first loads requested, one(vector) for each vector, batch(vi) after D of them, vi the first.
 // APART: the first loads are not the loop's (the same loads in the same order; in verification that keeps the passes behind
-// this one free of spills, 1010 us and 1029 above, in the draft step with more than two drafts it is what spills).
+// this one free of spills, 1010 us and 1029 above, in shifted rows' draft steps it is what spills).
 template <int D, bool APART, class IN, class BEGIN, class ONE, class BATCH>
 __device__ __forceinline__ void row_batches(const IN &in, int v0, int hi, const Iters &t, BEGIN begin, ONE one, BATCH batch) {
     using Raw = typename IN::Raw;
@@ -470,6 +470,41 @@ __device__ __forceinline__ void row_batches(const IN &in, int v0, int hi, const 
             use(i, b);
             if ((i += D) >= t.n) break;
         }
+    }
+}
+// ... with one set of registers, copied behind the request of the next: longer by the copies, shorter in code and in
+// registers, and the last batch goes as far as the range does.  (The order of the sums is the same one.)
+template <int D, class IN, class BEGIN, class ONE, class BATCH>
+__device__ __forceinline__ void row_turns(const IN &in, int v0, int hi, const Iters &t, BEGIN begin, ONE one, BATCH batch) {
+    using Raw = typename IN::Raw;
+    auto get = [&](int i, Raw (&x)[D]) {
+        if (i >= t.i0 && i + D <= t.i1) {
+#pragma unroll
+            for (int d = 0; d < D; ++d) x[d] = in.plain(v0 + 32 * (i + d));
+        } else {
+#pragma unroll
+            for (int d = 0; d < D; ++d) x[d] = in.checked(v0 + 32 * (i + d), hi);
+        }
+    };
+    if (t.n <= 0) return;
+    Raw nx[D];
+    get(0, nx);
+    begin(in.fix(nx[0]));
+#pragma unroll 1
+    for (int i = 0; i < t.n; i += D) {
+        Raw a[D];
+#pragma unroll
+        for (int d = 0; d < D; ++d) a[d] = nx[d];
+        if (i + D < t.n) get(i + D, nx);
+        if (i + D <= t.n) {
+#pragma unroll
+            for (int d = 0; d < D; ++d) one(in.fix(a[d]));
+        } else {
+#pragma unroll
+            for (int d = 0; d < D - 1; ++d)
+                if (i + d < t.n) one(in.fix(a[d]));
+        }
+        batch(v0 + 32 * i);
     }
 }
 // Two rows, ascending (STEP = 1) or descending, the next pair of vectors in flight: f(vi, x, y) with the target's and the
