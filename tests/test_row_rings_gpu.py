@@ -1,5 +1,7 @@
-"""Draft step and leaf rows of one warp each, and those whose passes take their rows from rings of bulk copies (bf16 rows in whole words, CTAs of 64
-and 128 threads): rows at which a warp's last chunk is full, one vector long or missing, against the oracle on a sample."""
+"""Draft step and leaf rows by the shape of their CTAs: one warp per row; passes that take their rows from rings of bulk
+copies (bf16 rows in whole words, more rows than one wave of CTAs of 64 or 128 threads); rows that come with the next
+vectors in registers.  Rows at which a warp's last chunk or batch is full, one vector long or missing, and rows that are hard
+on sums and references, against the oracle on a sample; the three-method draft step bit for bit."""
 import numpy as np
 import pytest
 
@@ -8,11 +10,14 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 import workloads  # noqa: E402
+from test_compare_gpu import METHODS, bits, separate_draft  # noqa: E402
 from test_parity_gpu import random_logits, random_uniforms, sh  # noqa: E402,F401
-from test_streaming_gpu import check_more_drafts, check_two_drafts, sample  # noqa: E402
+from test_streaming_gpu import check_more_drafts, check_two_drafts, hard_rows, sample  # noqa: E402
 
-# ids a warp's chunk holds: 1024.  64 threads: below 8192 ids and, in many rows, below 40960; 128: more than 592 rows
-SIZES = [(4104, 340), (6144, 340), (8192, 90), (8200, 90), (12296, 90), (16384 + 8, 90), (40960, 90), (16384, 340)]
+# A chunk is 1024 ids of a warp's range.  Seven rows per sequence: 340 sequences fill more than a wave of 64 threads (below
+# 40960 ids; below 10240 ids only leaf rows take those, draft steps one warp), 170 more than one of 128, 90 less than that.
+SIZES = [(4104, 340), (6144, 340), (10248, 340), (12288, 340), (12296, 340), (16384, 170), (16392, 170), (16416, 170), (40968, 170),
+         (8192, 90), (8200, 90), (16392, 90), (40960, 90)]
 
 
 @pytest.mark.parametrize("V,B", SIZES)
@@ -52,7 +57,7 @@ def test_rows_of_one_warp(sh, V, dtype, pad):  # noqa: F811
     check_more_drafts(sh, 3, True, lp, lq, dtype, pad, 1.0, un, True, sample(rng, B, 4, 6), "one warp")
 
 
-@pytest.mark.parametrize("V,B", [(8200, 160), (32000, 160), (16384, 620)])
+@pytest.mark.parametrize("V,B", [(8200, 160), (32000, 160), (16384, 620), (12296, 620), (16392, 310)])
 def test_three_drafts(sh, V, B):  # noqa: F811
     rng = np.random.default_rng(V + 1)
     N, k = 4, 3
@@ -60,3 +65,44 @@ def test_three_drafts(sh, V, B):  # noqa: F811
     un = rng.integers(0, 1 << 24, (B, N, 2 * k + 1)).astype(np.float32) * np.float32(2.0 ** -24)
     for wo in (False, True):
         check_more_drafts(sh, k, wo, lp, lq, "bf16", 0, 1.0, un, True, sample(rng, B, 4, 6), "rings")
+
+
+# shifted rows: more than a wave of 128 and of 64 threads, and less
+@pytest.mark.parametrize("V,B,dtype", [(16393, 170, "bf16"), (12291, 340, "bf16"), (16393, 90, "bf16"), (16387, 170, "fp32")])
+def test_shifted_rows(sh, V, B, dtype):  # noqa: F811
+    rng = np.random.default_rng(V + B)
+    lp, lq = random_logits(rng, B, 7, V, dtype)
+    lq[0, 0, : V // 2] = -np.inf
+    lq[1, 0, V - 64:] += 64.0
+    lp, lq = workloads.round_to_storage(lp, dtype), workloads.round_to_storage(lq, dtype)
+    for leaves in (False, True):
+        check_two_drafts(sh, lp, lq, dtype, 0, 0.8, random_uniforms(rng, B, 7), leaves, sample(rng, B, 4, 6), "shifted")
+
+
+# (rows: three per sequence) one warp; 64 threads, leaf rows only and all; 128 threads, more than a wave and less
+MANY = [(4104, 410), (9000, 410), (4104, 810), (12296, 810), (16392, 410), (16392, 230)]
+
+
+@pytest.mark.parametrize("V,B", MANY)
+def test_hard_rows(sh, V, B):  # noqa: F811
+    rng = np.random.default_rng(V + B)
+    lp, lq = random_logits(rng, B, 3, V, "bf16")
+    hard_rows(lp, lq)
+    lp, lq = workloads.round_to_storage(lp, "bf16"), workloads.round_to_storage(lq, "bf16")
+    un, pick = random_uniforms(rng, B, 3), sample(rng, B, n=6)
+    for leaves in (False, True):
+        check_two_drafts(sh, lp, lq, "bf16", 0, 1.0, un, leaves, pick, "hard", stats=True)
+
+
+@pytest.mark.parametrize("V,B", MANY[1:] + [(40960, 800), (40968, 410), (32000, 130), (32000, 90)])
+def test_three_methods(sh, V, B):  # noqa: F811
+    rng = np.random.default_rng(V + B + 1)
+    _, lq = random_logits(rng, B, 3, V, "bf16")
+    hard_rows(lq.copy(), lq)
+    tq, und = workloads.to_device(workloads.round_to_storage(lq, "bf16"), "bf16", "cuda"), torch.from_numpy(random_uniforms(rng, B, 3)).cuda()
+    tree = sh.Tree.heap(3)
+    out = sh.mdsd_compare_draft_sample(tq, und, tree, 0.8)
+    for m in METHODS:
+        one = separate_draft(sh, m, tq, und, tree, 0.8)
+        for key in one:
+            np.testing.assert_array_equal(bits(out[m][key]), bits(one[key]), err_msg="%s %s" % (m, key))

@@ -34,6 +34,14 @@ def test_records_are_used(sh, V, dtype, pad):  # noqa: F811
     assert bool((d["stats"].view(-1, 4)[:, 3] != 0).all())
     for leaves in (False, True):
         check_two_drafts(sh, lp, lq, dtype, pad, 0.8, un, leaves, sample(rng, B, 3, 5), "records", stats=True)
+    # a record whose sum is another one is believed: the reported rates are others
+    wrong = d["stats"].clone()
+    words = wrong.view(-1, 4)
+    words[:, 1] = (words[:, 1].contiguous().view(torch.float32) * 1.5).view(wrong.dtype)
+    a, und = (padded(lp, dtype, pad), tq), torch.from_numpy(un).cuda()
+    plain = gpu_verify(sh, "spechub", *a, d["tokens"], und, tree, 0.8)
+    out = gpu_verify_stats(sh, "spechub", *a, wrong, d["tokens"], und, tree, 0.8)
+    assert bool(((out["rate"] - plain["rate"]).abs().amax(-1)[2:] > 1e-3).all())
 
 
 @pytest.mark.parametrize("V,dtype,pad", SHAPES)
