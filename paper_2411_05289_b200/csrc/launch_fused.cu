@@ -6,14 +6,16 @@
 namespace spechub {
 
 int launch_fused_draft(const FusedArgs &f, int32_t *hub, float *draft_prob, unsigned rows, cudaStream_t s) {
+    constexpr RowPass kFew = kFewRows<__nv_bfloat16, false>, kMany = kManyDrafts<__nv_bfloat16, false>;
     const int th = draft_threads(f.r.vocab, rows, true);
-    if (th == 512) return launch_grid(fused_draft_kernel<512, false>, rows, 512, 0, 1, s, f, hub, draft_prob);
-    if (th == 256) return launch_grid(fused_draft_kernel<256, false>, rows, 256, 0, 1, s, f, hub, draft_prob);
-    if (th == 128 && many_rows(th, rows)) return launch_grid(fused_draft_kernel<128, true>, rows, 128, kRowRingBytes<__nv_bfloat16, false, 128, true>, 1, s, f, hub, draft_prob);
-    if (th == 128) return launch_grid(fused_draft_kernel<128, false>, rows, 128, 0, 1, s, f, hub, draft_prob);
-    if (th == 64 && many_rows(th, rows)) return launch_grid(fused_draft_kernel<64, true>, rows, 64, kRowRingBytes<__nv_bfloat16, false, 64, true>, 1, s, f, hub, draft_prob);
-    if (th == 64) return launch_grid(fused_draft_kernel<64, false>, rows, 64, 0, 1, s, f, hub, draft_prob);
-    return launch_grid(fused_draft_kernel<32, false>, rows, 32, 0, 1, s, f, hub, draft_prob);
+    const bool many = many_rows(th, rows) && f.r.vocab >= kRowRingVocab;
+    if (th == 512) return launch_grid(fused_draft_kernel<512, kFew>, rows, 512, 0, 1, s, f, hub, draft_prob);
+    if (th == 256) return launch_grid(fused_draft_kernel<256, kFew>, rows, 256, 0, 1, s, f, hub, draft_prob);
+    if (th == 128 && many) return launch_grid(fused_draft_kernel<128, kMany>, rows, 128, kRowRingBytes<128, kMany>, 1, s, f, hub, draft_prob);
+    if (th == 128) return launch_grid(fused_draft_kernel<128, kFew>, rows, 128, 0, 1, s, f, hub, draft_prob);
+    if (th == 64 && many) return launch_grid(fused_draft_kernel<64, kMany>, rows, 64, kRowRingBytes<64, kMany>, 1, s, f, hub, draft_prob);
+    if (th == 64) return launch_grid(fused_draft_kernel<64, kFew>, rows, 64, 0, 1, s, f, hub, draft_prob);
+    return launch_grid(fused_draft_kernel<32, kFew>, rows, 32, 0, 1, s, f, hub, draft_prob);
 }
 
 int launch_fused_verify(const FusedArgs &f, unsigned rows, cudaStream_t s) {

@@ -9,15 +9,16 @@ namespace spechub {
 template <typename LT, bool SHIFT>
 static int kary_draft(const KaryArgs &a, unsigned rows, cudaStream_t s) {
     constexpr bool kWords = sizeof(LT) == 2 && !SHIFT;
+    constexpr RowPass kFew = kFewRows<LT, SHIFT>, kMany = kManyRows<LT, SHIFT>;
     const int th = draft_threads(a.r.vocab, rows, kWords);
     if constexpr (kWords)
-        if (th == 32) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 32, false>, rows, 32, 0, 1, s, a);
-    if (th == 512) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 512, false>, rows, 512, 0, 1, s, a);
-    if (th == 256) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 256, false>, rows, 256, 0, 1, s, a);
-    if (th == 128 && many_rows(th, rows)) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 128, true>, rows, 128, kRowRingBytes<LT, SHIFT, 128, true>, 1, s, a);
-    if (th == 128) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 128, false>, rows, 128, 0, 1, s, a);
-    if (many_rows(th, rows)) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 64, true>, rows, 64, kRowRingBytes<LT, SHIFT, 64, true>, 1, s, a);
-    return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 64, false>, rows, 64, 0, 1, s, a);
+        if (th == 32) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 32, kFew>, rows, 32, 0, 1, s, a);
+    if (th == 512) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 512, kFew>, rows, 512, 0, 1, s, a);
+    if (th == 256) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 256, kFew>, rows, 256, 0, 1, s, a);
+    if (th == 128 && many_rows(th, rows)) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 128, kMany>, rows, 128, 0, 1, s, a);
+    if (th == 128) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 128, kFew>, rows, 128, 0, 1, s, a);
+    if (many_rows(th, rows)) return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 64, kMany>, rows, 64, 0, 1, s, a);
+    return launch_grid(lean_kary_draft_kernel<LT, SHIFT, 64, kFew>, rows, 64, 0, 1, s, a);
 }
 template <typename LT, bool SHIFT>
 static int kary_verify(const KaryArgs &a, unsigned rows, cudaStream_t s) {

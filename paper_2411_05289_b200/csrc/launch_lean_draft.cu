@@ -13,15 +13,17 @@ static int draft_group(const RowArgs &a, int method, unsigned rows, cudaStream_t
 template <typename LT, bool SHIFT>
 static int draft_rows(const RowArgs &a, int method, bool keep_stats, unsigned rows, cudaStream_t s) {
     constexpr bool kWords = sizeof(LT) == 2 && !SHIFT;
+    constexpr RowPass kFew = kFewRows<LT, SHIFT>, kMany = kManyDrafts<LT, SHIFT>;
     const int th = draft_threads(a.vocab, rows, kWords);
+    const bool many = many_rows(th, rows) && (kMany != kRing || a.vocab >= kRowRingVocab);
     if constexpr (kWords)
-        if (th == 32) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 32, false>, rows, 32, 0, 1, s, a, method, keep_stats);
-    if (th == 512) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 512, false>, rows, 512, 0, 1, s, a, method, keep_stats);
-    if (th == 256) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 256, false>, rows, 256, 0, 1, s, a, method, keep_stats);
-    if (th == 128 && many_rows(th, rows)) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 128, true>, rows, 128, kRowRingBytes<LT, SHIFT, 128, true>, 1, s, a, method, keep_stats);
-    if (th == 128) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 128, false>, rows, 128, 0, 1, s, a, method, keep_stats);
-    if (many_rows(th, rows)) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 64, true>, rows, 64, kRowRingBytes<LT, SHIFT, 64, true>, 1, s, a, method, keep_stats);
-    return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 64, false>, rows, 64, 0, 1, s, a, method, keep_stats);
+        if (th == 32) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 32, kFew>, rows, 32, 0, 1, s, a, method, keep_stats);
+    if (th == 512) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 512, kFew>, rows, 512, 0, 1, s, a, method, keep_stats);
+    if (th == 256) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 256, kFew>, rows, 256, 0, 1, s, a, method, keep_stats);
+    if (th == 128 && many) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 128, kMany>, rows, 128, kRowRingBytes<128, kMany>, 1, s, a, method, keep_stats);
+    if (th == 128) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 128, kFew>, rows, 128, 0, 1, s, a, method, keep_stats);
+    if (many) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 64, kMany>, rows, 64, kRowRingBytes<64, kMany>, 1, s, a, method, keep_stats);
+    return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 64, kFew>, rows, 64, 0, 1, s, a, method, keep_stats);
 }
 
 int launch_lean_draft(int format, int method, int cs, const RowArgs &a, bool keep_stats, unsigned rows, cudaStream_t s) {
@@ -35,13 +37,14 @@ int launch_lean_draft(int format, int method, int cs, const RowArgs &a, bool kee
 
 template <typename LT, bool SHIFT>
 static int leaf_rows(const LeafArgs &la, unsigned rows, cudaStream_t s) {
+    constexpr RowPass kFew = kFewRows<LT, SHIFT>, kMany = kManyRows<LT, SHIFT>;
     const int th = draft_threads(la.r.vocab, rows, false);
-    if (th == 512) return launch_grid(lean_leaf_kernel<LT, SHIFT, 512, false>, rows, 512, 0, 1, s, la);
-    if (th == 256) return launch_grid(lean_leaf_kernel<LT, SHIFT, 256, false>, rows, 256, 0, 1, s, la);
-    if (th == 128 && many_rows(th, rows)) return launch_grid(lean_leaf_kernel<LT, SHIFT, 128, true>, rows, 128, kRowRingBytes<LT, SHIFT, 128, true>, 1, s, la);
-    if (th == 128) return launch_grid(lean_leaf_kernel<LT, SHIFT, 128, false>, rows, 128, 0, 1, s, la);
-    if (many_rows(th, rows)) return launch_grid(lean_leaf_kernel<LT, SHIFT, 64, true>, rows, 64, kRowRingBytes<LT, SHIFT, 64, true>, 1, s, la);
-    return launch_grid(lean_leaf_kernel<LT, SHIFT, 64, false>, rows, 64, 0, 1, s, la);
+    if (th == 512) return launch_grid(lean_leaf_kernel<LT, SHIFT, 512, kFew>, rows, 512, 0, 1, s, la);
+    if (th == 256) return launch_grid(lean_leaf_kernel<LT, SHIFT, 256, kFew>, rows, 256, 0, 1, s, la);
+    if (th == 128 && many_rows(th, rows)) return launch_grid(lean_leaf_kernel<LT, SHIFT, 128, kMany>, rows, 128, 0, 1, s, la);
+    if (th == 128) return launch_grid(lean_leaf_kernel<LT, SHIFT, 128, kFew>, rows, 128, 0, 1, s, la);
+    if (many_rows(th, rows)) return launch_grid(lean_leaf_kernel<LT, SHIFT, 64, kMany>, rows, 64, 0, 1, s, la);
+    return launch_grid(lean_leaf_kernel<LT, SHIFT, 64, kFew>, rows, 64, 0, 1, s, la);
 }
 
 // The leaf rows of an unsplit call (same CTA shape as the draft step).

@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
 
 // Draft step of the three methods from one read of q (the checkpointed pass A and sampler of
 // lean_draft_ck_kernel).  x1 ~ q is the same draw for all three: they share u_d1.
-template <int THREADS, bool MANY>
+template <int THREADS, RowPass PASS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(FusedArgs A, int32_t *hub_out,
                                                                             float *draft_prob) {
     __shared__ LeanCkShared sh;
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
 
     LeanAcc<__nv_bfloat16> tq, unused;
     unused.init();
-    lean_pass_a_ck<false, THREADS, MANY>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * CS, sh.ckc + warp * CS, CS, sh.any[warp]);
+    lean_pass_a_ck<false, THREADS, PASS>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * CS, sh.ckc + warp * CS, CS, sh.any[warp]);
     RowStat Q;
     {
         ArgMaxSum q, unusedq;

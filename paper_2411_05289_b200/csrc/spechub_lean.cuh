@@ -691,24 +691,28 @@ __device__ __forceinline__ int lean_ck_slots(const Geo &g, int CK) {   // sub-bl
     return (((g.seg + 31) >> 5) + CK - 1) / CK;
 }
 
-// How the draft step's and the leaf rows' passes take their rows.  MANY: more rows than one wave of these CTAs (many_rows),
-// of 64 or 128 threads.  bf16 rows in whole words come from rings of bulk copies then (spechub_ring.cuh; draft step on 7936
-// rows of 128256 ids 321 us, from registers 333; 3840 of 64000 100, 110; 1792 of 32000 34.5, 35.5).  In less than a wave
-// an SM's rings hold too few bytes in flight, and a row is not behind others that hide its end (651 rows of 12800 ids 12.4
-// us, from rings 13.8; 651 of 101056 45.6, 57.7; 896 of 64000 33.3, 37.1).  Not in one-warp CTAs (4000 rows of 10000 ids: 35
-// us, 39 from rings), in those of 256 threads and more (448 rows of 32000: no difference) and for fp32 rows (480 rows of
-// 128256: a step 170 us, 173 from rings: a vector is 32 bytes, its reads from shared memory meet in the banks).
-// From registers: row_turns, whose last batch goes as far as the range does (exponentials of padding made a draft step of
-// three methods on 1170 rows of 12800 ids 16.1 us, 14.75 so); shifted rows, longer to make into vectors, row_batches while
-// they are less than a wave (448 rows of 16393 ids 14.0 us, with row_turns 14.3, 224 of 64001 17.7, 18.5; but 3840 of 64001
-// 159, 147).
-template <typename LT, bool SHIFT, int THREADS, bool MANY>
-constexpr bool kRowRinged = sizeof(LT) == 2 && !SHIFT && MANY && (THREADS == 64 || THREADS == 128);
-template <typename LT, bool SHIFT, int THREADS, bool MANY>
-constexpr int kRowRingBytes = kRowRinged<LT, SHIFT, THREADS, MANY> ? THREADS / 32 * kRowWarpBytes : 0;
+// How the draft step's and the leaf rows' passes take their rows (us of the draft step unless it says otherwise).
+//   kTurns    from registers, one set (row_turns): rows in whole words, and bf16 shifted rows of more than one wave of these
+//             CTAs (many_rows; 3840 of 64001 ids 147, by two sets 159; 4900 of 8201 52.2, 56.8)
+//   kBatches  from registers, two sets that take turns (row_batches): other shifted rows, longer to make into vectors (448
+//             bf16 rows of 16393 ids 14.0, by one set 14.3, 224 of 64001 17.7, 18.5; 1400 fp32 rows of 64001 91.5, 104)
+//   kRing     from rings of bulk copies (spechub_ring.cuh), CTAs of 64 or 128 threads: the draft step of two drafts on bf16 rows
+//             in whole words, from 24576 ids, in more than one wave (7936 of 128256 ids 322, by one set 333; 7680 of 40000
+//             122, 125; 10500 of 32000 128, 129; but 4900 of 24000 57.3, 57.2, of 16392 47.3, 45.9).  In less than a wave an
+//             SM's rings hold too few bytes in flight, and no row is behind others that hide its end (651 of 101056 57.7,
+//             45.6; 896 of 64000 37.1, 33.3).  More drafts wait for their draws longer than for the bytes (three drafts, 3250
+//             rows of 32000: 75.2, 70.1), as do leaf rows behind a draft step (verification, 7680 rows of 32000, half of them
+//             leaves: 212, 206).  Not one-warp CTAs (4000 of 10000: 39, 35) or fp32 rows (480 of 128256, a step 173, 170:
+//             a vector is 32 bytes, its reads from shared memory meet in the banks).
+enum RowPass { kTurns, kBatches, kRing };
+template <typename LT, bool SHIFT> constexpr RowPass kFewRows = SHIFT ? kBatches : kTurns;
+template <typename LT, bool SHIFT> constexpr RowPass kManyRows = SHIFT && sizeof(LT) == 2 ? kTurns : kFewRows<LT, SHIFT>;
+template <typename LT, bool SHIFT> constexpr RowPass kManyDrafts = !SHIFT && sizeof(LT) == 2 ? kRing : kManyRows<LT, SHIFT>;
+constexpr int kRowRingVocab = 24576;
+template <int THREADS, RowPass PASS> constexpr int kRowRingBytes = PASS == kRing ? THREADS / 32 * kRowWarpBytes : 0;
 
 // late: set if a bulk copy did not arrive within its bounded wait (the results are then of the part in front of it).
-template <bool SHIFT, int THREADS, bool MANY, typename LT, class ROW>
+template <bool SHIFT, int THREADS, RowPass PASS, typename LT, class ROW>
 __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, int lane, float k, int CK,
                                                LeanAcc<LT> &Q, float *cks, float *ckc, int slots, int &late) {
     LeanAcc<LT> st;
@@ -757,14 +761,14 @@ __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, in
     };
     auto run = [&](const auto &in, const Iters &t) {   // (the loads of the next vectors also overlap the checkpoint's shuffle chain)
         constexpr int D = std::decay_t<decltype(in)>::kDepth;
-        if constexpr (SHIFT && !MANY) row_batches<D, false>(in, lo + lane, hi, t, begin, one, [&](int vi) { batch(in, vi); });
+        if constexpr (PASS == kBatches) row_batches<D, false>(in, lo + lane, hi, t, begin, one, [&](int vi) { batch(in, vi); });
         else row_turns<D>(in, lo + lane, hi, t, begin, one, [&](int vi) { batch(in, vi); });
     };
     if constexpr (SHIFT) {
         const Iters t = inside_iters(rq.src, rq.src, lo, hi);
         if (rq.src.sh == 0) run(AlignedIn<LT>{rq.src}, t);
         else run(ShiftedIn<LT>{rq.src}, t);
-    } else if constexpr (kRowRinged<LT, SHIFT, THREADS, MANY>) {
+    } else if constexpr (PASS == kRing) {
         extern __shared__ __align__(128) unsigned char row_ring_mem[];
         __shared__ __align__(8) uint64_t row_ring_bars[THREADS / 32][kRowStages];
         const int warp = warp_index();
@@ -921,7 +925,7 @@ __device__ __forceinline__ int lean_ck_draw(const Geo &g, const ROW &row, float 
 // pass A over p with checkpoints, then the sub-block sampler.  CTAs of verifying rows leave at
 // once; the verification kernels skip the leaf rows.  Up to three output sets receive the result
 // (the three-method call: the methods share u_res, hence the bonus token).
-template <typename LT, bool SHIFT, int THREADS, bool MANY>
+template <typename LT, bool SHIFT, int THREADS, RowPass PASS>
 __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_leaf_kernel(LeafArgs A) {
     __shared__ LeanCkShared sh;
     pdl_begin();
@@ -939,7 +943,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_leaf_
     const int CK = lean_ck_interval(g), CS = lean_ck_slots(g, CK);
     LeanAcc<LT> tp, unused;
     unused.init();
-    lean_pass_a_ck<SHIFT, THREADS, MANY>(vp, lo, hi, lane, k, CK, tp, sh.cks + warp * CS, sh.ckc + warp * CS, CS, sh.any[warp]);
+    lean_pass_a_ck<SHIFT, THREADS, PASS>(vp, lo, hi, lane, k, CK, tp, sh.cks + warp * CS, sh.ckc + warp * CS, CS, sh.any[warp]);
     ArgMaxSum Ps, unusedq;
     lean_reduce2<false>(tp, unused, vp, vp, lo, hi, k, sh, Ps, unusedq);
     const float Zp = Ps.sx + Ps.own(k);
@@ -1586,7 +1590,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_kernel(Row
 // ------------------------------------------------------------------------------------------------
 // Draft step, one CTA per row (checkpointed pass A and sub-block sampler above).
 // ------------------------------------------------------------------------------------------------
-template <typename LT, bool SHIFT, int THREADS, bool MANY>
+template <typename LT, bool SHIFT, int THREADS, RowPass PASS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(RowArgs a, int method, bool keep_stats) {   // (shifted rows: marked ones)
     __shared__ LeanCkShared sh;
     pdl_begin();
@@ -1602,7 +1606,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
 
     LeanAcc<LT> tq, unused;
     unused.init();
-    lean_pass_a_ck<SHIFT, THREADS, MANY>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * CS, sh.ckc + warp * CS, CS, sh.any[warp]);
+    lean_pass_a_ck<SHIFT, THREADS, PASS>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * CS, sh.ckc + warp * CS, CS, sh.any[warp]);
     RowStat Q;
     {
         ArgMaxSum q, unusedq;

@@ -34,7 +34,7 @@ __device__ __forceinline__ bool one_of(const int *x, int n, int y) {
 }
 
 // ---- draft step -----------------------------------------------------------------------------------
-template <typename LT, bool SHIFT, int THREADS, bool MANY>
+template <typename LT, bool SHIFT, int THREADS, RowPass PASS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_kary_draft_kernel(KaryArgs A) {
     __shared__ LeanKaryShared sh;
     pdl_begin();
@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_kary_draft_kerne
 
     LeanAcc<LT> tq, unused;
     unused.init();
-    lean_pass_a_ck<SHIFT, THREADS, MANY>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * CS, sh.ckc + warp * CS, CS, sh.any[warp]);
+    lean_pass_a_ck<SHIFT, THREADS, PASS>(vq, lo, hi, lane, k, CK, tq, sh.cks + warp * CS, sh.ckc + warp * CS, CS, sh.any[warp]);
     ArgMaxSum Q, unusedq;
     lean_reduce2<false>(tq, unused, vq, vq, lo, hi, k, sh, Q, unusedq);
     const float Zq = Q.sx + Q.own(k);

@@ -33,7 +33,7 @@ constexpr int draft_threads(int vocab, unsigned rows, bool words) {
 constexpr int verify_threads(int vocab, unsigned rows, int per_sm) {
     return rows <= unsigned(per_sm / 512 * kSms) ? 512 : rows <= unsigned(per_sm / 256 * kSms) || vocab >= 16384 ? 256 : 128;
 }
-// More rows than one wave of the draft step's CTAs of these many threads?  (What that decides: kRowRinged.)
+// More rows than one wave of the draft step's CTAs of these many threads?  (What that decides: RowPass.)
 constexpr bool many_rows(int threads, unsigned rows) { return rows > unsigned(1024 / threads * kSms); }
 constexpr int kLeanThreads = 256;   // split rows, and the rings of bulk copies
 
