@@ -92,8 +92,8 @@ extern "C" {
 /* descriptor flags: how many CTAs of a thread-block cluster share one row in the large-vocabulary
  * bf16 kernels (a tuning hint; results do not depend on it beyond fp32 summation order).  At most
  * one of the three may be set; none = the library chooses by rows, length and type: rows held in
- * registers, one CTA per row of 64 to 512 threads, or (RRS / RRSw on many long rows) rings of bulk
- * copies into shared memory.  SPECHUB_FLAG_SPLIT_1 asks for one CTA of 256 threads per row whose loads
+ * registers, one CTA per row of 32 to 512 threads, or (the draft step and RRS / RRSw on many long
+ * rows) rings of bulk copies into shared memory.  SPECHUB_FLAG_SPLIT_1 asks for one CTA of 256 threads per row whose loads
  * go to registers. */
 #define SPECHUB_FLAG_SPLIT_1 1u
 #define SPECHUB_FLAG_SPLIT_2 2u

@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_draft_kernel(Fu
         Q.set(q, k);
     }
     if (warp != 0) return;
-    const bool late = lean_late(sh, g);   // (as in lean_draft_ck_kernel)
+    const bool late = PASS == kRing && lean_late(sh, g);   // (as in lean_draft_ck_kernel)
     const float Zq = Q.sx + Q.own;
     if (t0 && a.draft_stats_out) {   // the record lean_draft_ck_kernel leaves, bit for bit
         DraftStat ds = {};

@@ -144,19 +144,6 @@ __device__ __forceinline__ void lean_push(LeanAcc<LT> &st, const Vec8<LT> &v, fl
     st.s += a;
 }
 
-// ... of one vector of each of two rows, with one look at both sums
-template <typename LT>
-__device__ __forceinline__ void lean_push2(LeanAcc<LT> &P, LeanAcc<LT> &Q, const Vec8<LT> &x, const Vec8<LT> &y, float k) {
-    const F2 k2 = f2_make(k, k);
-    const float sp = P.s + vec_sum(x, k2, f2_make(-P.c, -P.c)), sq = Q.s + vec_sum(y, k2, f2_make(-Q.c, -Q.c));
-    if (sp + sq < kHuge) {
-        P.m2 = Vec8<LT>::max_of(P.m2, x.packed_max()); P.s = sp;
-        Q.m2 = Vec8<LT>::max_of(Q.m2, y.packed_max()); Q.s = sq;
-    } else {
-        lean_push(P, x, k);
-        lean_push(Q, y, k);
-    }
-}
 // ... of a batch of vectors: the same sums in the same order, with one look at their size.  (Where that fails the vectors,
 // vi, vi + 32, ..., are read again: kept for it, they would not fit the registers.)
 template <typename LT>
@@ -238,12 +225,8 @@ __device__ __forceinline__ void lean_pass_a2(const StreamRow<LT, SHIFT> &rp, con
     P.c = lean_reference(rp, vi, hi, k);
     Q.c = lean_reference(rq, vi, hi, k);
     auto push = [&](int, const Vec8<LT> &a, const Vec8<LT> &b) {
-#ifdef P2
-        lean_push2(P, Q, a, b, k);
-#else
         lean_push(P, a, k);
         lean_push(Q, b, k);
-#endif
     };
     if constexpr (AHEAD || SHIFT) {
         stream_pairs<1>(rp, rq, lo, hi, lane, push);
@@ -711,7 +694,7 @@ template <typename LT, bool SHIFT> constexpr RowPass kManyDrafts = !SHIFT && siz
 constexpr int kRowRingVocab = 24576;
 template <int THREADS, RowPass PASS> constexpr int kRowRingBytes = PASS == kRing ? THREADS / 32 * kRowWarpBytes : 0;
 
-// late: set if a bulk copy did not arrive within its bounded wait (the results are then of the part in front of it).
+// late (kRing): whether a bulk copy did not arrive within its bounded wait (the results are of the part in front of it).
 template <bool SHIFT, int THREADS, RowPass PASS, typename LT, class ROW>
 __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, int lane, float k, int CK,
                                                LeanAcc<LT> &Q, float *cks, float *ckc, int slots, int &late) {
@@ -776,11 +759,11 @@ __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, in
         RowRing R;
         row_ring_begin(R, row_ring_mem + warp * kRowWarpBytes, row_ring_bars[warp], rq.vec(lo),
                        (hi - lo) * static_cast<int>(sizeof(Vec8<LT>)), lane);
-        missing = !ring_batches<LT>(R, lo, hi, lane, begin, one, [&](int vi) { batch(in, vi); });
+        missing = !ring_batches(R, lo, hi, lane, begin, one, [&](int vi) { batch(in, vi); });
     } else {
         run(WholeIn<LT>{rq}, whole_iters(lo, hi));
     }
-    if (lane == 0) late = missing;
+    if (PASS == kRing && lane == 0) late = missing;
     if (since > 0) checkpoint();
     if (lane == 0)
         for (; j < slots; ++j) { cks[j] = 0.f; ckc[j] = 0.f; }
@@ -950,8 +933,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_leaf_
     if (warp != 0) return;
     uint32_t status = 0;
     int tok = -1;
-    if (lean_late(sh, g)) status = SPECHUB_ST_INTERNAL;   // (nothing is drawn from a part of the row)
-    else if (!(Ps.ml > neg_inf()) || !(Ps.ml < -neg_inf()) || !finite_pos(Zp)) status = SPECHUB_ST_NONFINITE;
+    if (!(Ps.ml > neg_inf()) || !(Ps.ml < -neg_inf()) || !finite_pos(Zp)) status = SPECHUB_ST_NONFINITE;
     else if ((tok = lean_ck_draw(g, vp, k, Ps.c, CK, NoneOut{}, ures, sh)) < 0) tok = Ps.idx;   // (as in the draft step)
     if (threadIdx.x == 0) {
         for (int m = 0; m < A.n_out; ++m) {
@@ -1616,7 +1598,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_ck_kernel(
     if (warp != 0) return;
     const float Zq = Q.sx + Q.own;
     uint32_t st = 0;
-    const bool late = lean_late(sh, g);   // (nothing is drawn from, or recorded of, a part of the row)
+    const bool late = PASS == kRing && lean_late(sh, g);   // (nothing is drawn from, or recorded of, a part of the row)
     int x1 = -1, x2 = -1, hubtok = -1;
     float prob0 = 0.f, prob1 = 0.f;
     if (late) {

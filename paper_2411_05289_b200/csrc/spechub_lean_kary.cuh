@@ -58,8 +58,8 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_kary_draft_kerne
     const float Zq = Q.sx + Q.own(k);
     uint32_t st = 0;
     if (warp != 0) return;
-    const bool late = lean_late(sh, g), bad = late || !(Q.ml > neg_inf()) || !finite_pos(Zq) || !(Q.ml < -neg_inf());
-    if (bad) st = late ? SPECHUB_ST_INTERNAL : SPECHUB_ST_NONFINITE;
+    const bool bad = !(Q.ml > neg_inf()) || !finite_pos(Zq) || !(Q.ml < -neg_inf());
+    if (bad) st = SPECHUB_ST_NONFINITE;
     for (int i = 0; i < K; ++i) {
         int t = -1;
         if (!bad) {
@@ -145,12 +145,8 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_kary_
     tq.c = lean_reference(vq, lo + lane, hi, k);
     stream_pairs<1>(vp, vq, lo, hi, lane, [&](int vi, V x, V y) {
         if (mine) drop_singles(vi, x, y);
-#ifdef P2
-        lean_push2(tp, tq, x, y, k);
-#else
         lean_push(tp, x, k);
         lean_push(tq, y, k);
-#endif
     });
     const int nwarps = THREADS / 32;
     {

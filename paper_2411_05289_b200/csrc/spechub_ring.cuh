@@ -1,7 +1,7 @@
-// Per-warp rings of bulk copies (cp.async.bulk, global -> shared, completion on an mbarrier) that feed
-// the passes of the streaming verification kernels.
+// Per-warp rings of bulk copies (cp.async.bulk, global -> shared, completion on an mbarrier): of two bf16 rows, over several
+// passes, for streaming verification (WarpRing), and of one, once, for the draft step (RowRing, below).
 //
-// A warp owns a contiguous range [lo, hi) of 16-byte vectors of the target row and of the draft row and
+// Two rows: a warp owns a contiguous range [lo, hi) of 16-byte vectors of the target row and of the draft row and
 // goes over it once per pass, forwards or backwards.  The passes of a row form one stream of chunks
 // (kRingCh vectors per lane of each row): lane 0 keeps kRingStages chunks of that stream in flight, also
 // across the boundary between two passes, so that the loads of a pass are under way while the warp still
@@ -140,21 +140,12 @@ __device__ __forceinline__ void ring_drain(WarpRing &R) {
     R.ng = R.issued;
 }
 
-template <typename LT> __device__ __forceinline__ Vec8<LT> shared_vec(uint32_t at);
-template <>
 __device__ __forceinline__ Vec8<__nv_bfloat16> shared_vec(uint32_t at) {
     Vec8<__nv_bfloat16> v;
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.w[0]), "=r"(v.w[1]), "=r"(v.w[2]), "=r"(v.w[3]) : "r"(at) : "memory");
     return v;
 }
-template <>
-__device__ __forceinline__ Vec8<float> shared_vec(uint32_t at) {
-    Vec8<float> v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.f[0]), "=f"(v.f[1]), "=f"(v.f[2]), "=f"(v.f[3]) : "r"(at) : "memory");
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.f[4]), "=f"(v.f[5]), "=f"(v.f[6]), "=f"(v.f[7]) : "r"(at + 16) : "memory");
-    return v;
-}
-// ---- one row, once, forwards: the draft step and leaf rows ------------------------------------------------------------
+// ---- one row, once, forwards: the draft step ------------------------------------------------------------
 // Chunks of 2 KB (64 bytes per lane), two in flight per warp, in no registers and none of it in L1 (the draft step on 7936
 // rows of 128256 ids 351 us from registers, 339 so, 344 with three stages; 10000 rows of 65536: 238, 228, 235; of 32000:
 // 148, 141).
@@ -197,23 +188,24 @@ __device__ __forceinline__ bool row_ring_wait(const RowRing &R, int c) {
 }
 // As row_batches: begin(first vector), one(vector), batch(vi).  False: a chunk did not arrive (within its bounded wait), and
 // it and those behind it are in no sum.
-template <typename LT, class BEGIN, class ONE, class BATCH>
+template <class BEGIN, class ONE, class BATCH>
 __device__ __forceinline__ bool ring_batches(const RowRing &R, int lo, int hi, int lane, BEGIN begin, ONE one, BATCH batch) {
-    constexpr int D = kRowChunkBytes / (32 * static_cast<int>(sizeof(Vec8<LT>)));
-    Vec8<LT> x[D];
+    using V = Vec8<__nv_bfloat16>;
+    constexpr int D = kRowChunkBytes / (32 * static_cast<int>(sizeof(V)));
+    V x[D];
     return ring_run<kRowStages>(
         (hi - lo + 32 * D - 1) / (32 * D), [&](int c) { return row_ring_wait(R, c); },
         [&](int c) {
             const int v0 = lo + lane + 32 * D * c;
-            const uint32_t at = R.data + (c % kRowStages) * kRowChunkBytes + lane * static_cast<int>(sizeof(Vec8<LT>));
+            const uint32_t at = R.data + (c % kRowStages) * kRowChunkBytes + lane * static_cast<int>(sizeof(V));
             if (v0 - lane + 32 * D <= hi) {
 #pragma unroll
-                for (int d = 0; d < D; ++d) x[d] = shared_vec<LT>(at + 32 * d * sizeof(Vec8<LT>));
+                for (int d = 0; d < D; ++d) x[d] = shared_vec(at + 32 * d * sizeof(V));
             } else {
 #pragma unroll
                 for (int d = 0; d < D; ++d) {
-                    x[d] = Vec8<LT>::none();
-                    if (v0 + 32 * d < hi) x[d] = shared_vec<LT>(at + 32 * d * sizeof(Vec8<LT>));
+                    x[d] = V::none();
+                    if (v0 + 32 * d < hi) x[d] = shared_vec(at + 32 * d * sizeof(V));
                 }
             }
             __syncwarp();
