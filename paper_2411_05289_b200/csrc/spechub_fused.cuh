@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
         sh.x_ml[1] = ds.ml; sh.x_sx[1] = ds.sx; sh.x_idx[1] = ok ? ds.idx : 0;
     }
     LeanAcc<__nv_bfloat16> tp, tq;
-    if constexpr (STATS) lean_pass_a1<true>(vp, lo, hi, lane, k, tp);
+    if constexpr (STATS) lean_pass_a1<true, true>(vp, lo, hi, lane, k, tp);
     else lean_pass_a2<false>(vp, vq, lo, hi, lane, k, tp, tq);
     RowStat P, Q;
     {

@@ -236,16 +236,20 @@ __device__ __forceinline__ void lean_pass_a2(const StreamRow<LT, SHIFT> &rp, con
     }
 }
 
-// Pass A over one row.  KEEP: the row is read again by pass B, and L2 is asked to keep it.
-template <bool KEEP, typename LT>
+// Pass A over one row.  KEEP: the row is read again by pass B, and L2 is asked to keep it.  TURNS: through one set of
+// registers (row_turns): in the three-method kernel two sets cost the later passes spills (7936 rows of 32000 ids 518 -> 511
+// us, 3968 of 128256 907 -> 896), in RRSw's the copies cost more than those (7936 of 32000 402 -> 424).
+template <bool KEEP, bool TURNS, typename LT>
 __device__ __forceinline__ void lean_pass_a1(const StreamRow<LT, false> &rp, int lo, int hi, int lane, float k, LeanAcc<LT> &P) {
     P.init();
     LeanBatch<LT> B(P);
     auto run = [&](const auto &in) {
         constexpr int D = std::decay_t<decltype(in)>::kDepth;
-        row_batches<D, true>(in, lo + lane, hi, whole_iters(lo, hi),
-                             [&](const Vec8<LT> &first) { P.c = lean_reference(first, rp, lo + lane, hi, k); B.begin(k); },
-                             [&](const Vec8<LT> &v) { B.push(v); }, [&](int vi) { B.template commit<D>(in, k, vi, hi); });
+        auto begin = [&](const Vec8<LT> &first) { P.c = lean_reference(first, rp, lo + lane, hi, k); B.begin(k); };
+        auto one = [&](const Vec8<LT> &v) { B.push(v); };
+        auto batch = [&](int vi) { B.template commit<D>(in, k, vi, hi); };
+        if constexpr (TURNS) row_turns<D>(in, lo + lane, hi, whole_iters(lo, hi), begin, one, batch);
+        else row_batches<D, true>(in, lo + lane, hi, whole_iters(lo, hi), begin, one, batch);
     };
     if constexpr (KEEP) {
         uint64_t pol;
@@ -256,8 +260,8 @@ __device__ __forceinline__ void lean_pass_a1(const StreamRow<LT, false> &rp, int
     }
 }
 
-// ... of a row of any alignment
-template <bool KEEP, typename LT>
+// ... of a row of any alignment (neither applies)
+template <bool KEEP, bool TURNS, typename LT>
 __device__ __forceinline__ void lean_pass_a1(const StreamRow<LT, true> &rp, int lo, int hi, int lane, float k, LeanAcc<LT> &P) {
     P.init();
     LeanBatch<LT> B(P);
@@ -1058,9 +1062,9 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
                    reinterpret_cast<const uint4 *>(vq.row), lo, hi, 3, 2u, lane);
         lean_pass_a_ring(R, vp, vq, lane, k, tp, tq);
     } else if constexpr (STATS) {
-        lean_pass_a1<true>(vp, lo, hi, lane, k, tp);
+        lean_pass_a1<true, false>(vp, lo, hi, lane, k, tp);
     } else if constexpr (CS > 1) {
-        if (leaf) { tq.init(); lean_pass_a1<false>(vp, lo, hi, lane, k, tp); }
+        if (leaf) { tq.init(); lean_pass_a1<false, false>(vp, lo, hi, lane, k, tp); }
         else lean_pass_a2<METHOD != kSpecHub>(vp, vq, lo, hi, lane, k, tp, tq);
     } else {
         lean_pass_a2<METHOD != kSpecHub || THREADS == 512>(vp, vq, lo, hi, lane, k, tp, tq);
@@ -1080,7 +1084,7 @@ __global__ void __launch_bounds__(THREADS, lean_ctas<SHIFT>(THREADS)) lean_verif
             // still come with whatever their caller has).  Same vectors, same order, so the plain call's bits but for
             // RRSw's 1 - q(x1), which is sum_without's here.
             if (!sh.stat_ok) {
-                lean_pass_a1<false>(vq, lo, hi, lane, k, tq);
+                lean_pass_a1<false, false>(vq, lo, hi, lane, k, tq);
                 lean_reduce2<true>(tp, tq, vp, vq, lo, hi, k, sh, Ps, Qs);
                 from_record = false;
             }
@@ -1468,7 +1472,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) lean_draft_kernel(Row
 
     LeanAcc<__nv_bfloat16> tq, unused;
     unused.init();
-    lean_pass_a1<false>(vq, lo, hi, lane, k, tq);
+    lean_pass_a1<false, false>(vq, lo, hi, lane, k, tq);
     {
         ArgMaxSum q, unusedq;
         lean_reduce2<false>(tq, unused, vq, vq, lo, hi, k, sh, q, unusedq);
