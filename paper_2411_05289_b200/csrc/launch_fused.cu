@@ -13,7 +13,6 @@ int launch_fused_draft(const FusedArgs &f, int32_t *hub, float *draft_prob, unsi
     if (th == 256) return launch_grid(fused_draft_kernel<256, kFew>, rows, 256, 0, 1, s, f, hub, draft_prob);
     if (th == 128 && many) return launch_grid(fused_draft_kernel<128, kMany>, rows, 128, kRowRingBytes<128, kMany>, 1, s, f, hub, draft_prob);
     if (th == 128) return launch_grid(fused_draft_kernel<128, kFew>, rows, 128, 0, 1, s, f, hub, draft_prob);
-    if (th == 64 && many) return launch_grid(fused_draft_kernel<64, kMany>, rows, 64, kRowRingBytes<64, kMany>, 1, s, f, hub, draft_prob);
     if (th == 64) return launch_grid(fused_draft_kernel<64, kFew>, rows, 64, 0, 1, s, f, hub, draft_prob);
     return launch_grid(fused_draft_kernel<32, kFew>, rows, 32, 0, 1, s, f, hub, draft_prob);
 }

@@ -16,13 +16,14 @@ static int draft_rows(const RowArgs &a, int method, bool keep_stats, unsigned ro
     constexpr RowPass kFew = kFewRows<LT, SHIFT>, kMany = kManyDrafts<LT, SHIFT>;
     const int th = draft_threads(a.vocab, rows, kWords);
     const bool many = many_rows(th, rows) && (kMany != kRing || a.vocab >= kRowRingVocab);
+    constexpr RowPass kMany64 = kManyRows<LT, SHIFT>;   // (rings: rows of 128 threads)
     if constexpr (kWords)
         if (th == 32) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 32, kFew>, rows, 32, 0, 1, s, a, method, keep_stats);
     if (th == 512) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 512, kFew>, rows, 512, 0, 1, s, a, method, keep_stats);
     if (th == 256) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 256, kFew>, rows, 256, 0, 1, s, a, method, keep_stats);
     if (th == 128 && many) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 128, kMany>, rows, 128, kRowRingBytes<128, kMany>, 1, s, a, method, keep_stats);
     if (th == 128) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 128, kFew>, rows, 128, 0, 1, s, a, method, keep_stats);
-    if (many) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 64, kMany>, rows, 64, kRowRingBytes<64, kMany>, 1, s, a, method, keep_stats);
+    if (many) return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 64, kMany64>, rows, 64, 0, 1, s, a, method, keep_stats);
     return launch_grid(lean_draft_ck_kernel<LT, SHIFT, 64, kFew>, rows, 64, 0, 1, s, a, method, keep_stats);
 }
 

@@ -680,22 +680,25 @@ __device__ __forceinline__ int lean_ck_slots(const Geo &g, int CK) {   // sub-bl
 
 // How the draft step's and the leaf rows' passes take their rows (us of the draft step unless it says otherwise).
 //   kTurns    from registers, one set (row_turns): rows in whole words, and bf16 shifted rows of more than one wave of these
-//             CTAs (many_rows; 3840 of 64001 ids 147, by two sets 159; 4900 of 8201 52.2, 56.8)
+//             CTAs (many_rows; 3840 of 64001 ids 147, by two sets 159; 4900 of 8201 52.2, 56.8), whose sums are looked at
+//             after every vector then: a batch's own sum and maximum are registers that these kernels would spill (7680 of
+//             50257 ids 203, by batches 214; 3968 of 128257 236, 251)
 //   kBatches  from registers, two sets that take turns (row_batches): other shifted rows, longer to make into vectors (448
 //             bf16 rows of 16393 ids 14.0, by one set 14.3, 224 of 64001 17.7, 18.5; 1400 fp32 rows of 64001 91.5, 104)
-//   kRing     from rings of bulk copies (spechub_ring.cuh), CTAs of 64 or 128 threads: the draft step of two drafts on bf16 rows
-//             in whole words, from 24576 ids, in more than one wave (7936 of 128256 ids 322, by one set 333; 7680 of 40000
-//             122, 125; 10500 of 32000 128, 129; but 4900 of 24000 57.3, 57.2, of 16392 47.3, 45.9).  In less than a wave an
-//             SM's rings hold too few bytes in flight, and no row is behind others that hide its end (651 of 101056 57.7,
-//             45.6; 896 of 64000 37.1, 33.3).  More drafts wait for their draws longer than for the bytes (three drafts, 3250
-//             rows of 32000: 75.2, 70.1), as do leaf rows behind a draft step (verification, 7680 rows of 32000, half of them
-//             leaves: 212, 206).  Not one-warp CTAs (4000 of 10000: 39, 35) or fp32 rows (480 of 128256, a step 173, 170:
-//             a vector is 32 bytes, its reads from shared memory meet in the banks).
+//   kRing     from rings of bulk copies (spechub_ring.cuh): the draft step of two drafts on bf16 rows in whole words of 40960 ids
+//             and more, in more than one wave of CTAs of 128 threads (7936 of 128256 ids 322, by one set 333; 3584 of 48000
+//             70.4, 72.7).  In less than a wave an SM's rings hold too few bytes in flight, and no row is behind others that
+//             hide its end (651 of 101056 57.7, 45.6; 896 of 64000 37.1, 33.3).  Shorter rows gain 1 to 3 % by themselves, but
+//             verification behind them starts later (RRSw step on 3840 rows of 32000 with leaves 165, without rings 158:
+//             kernels of other needs of shared memory do not meet on an SM).  More drafts wait for their draws longer than
+//             for the bytes (three drafts, 3250 rows of 32000: 75.2, 70.1), as do leaf rows behind a draft step
+//             (verification, 7680 rows of 32000, half of them leaves: 212, 206).  Not fp32 rows (480 of 128256, a step
+//             173, 170: a vector is 32 bytes, its reads from shared memory meet in the banks).
 enum RowPass { kTurns, kBatches, kRing };
 template <typename LT, bool SHIFT> constexpr RowPass kFewRows = SHIFT ? kBatches : kTurns;
 template <typename LT, bool SHIFT> constexpr RowPass kManyRows = SHIFT && sizeof(LT) == 2 ? kTurns : kFewRows<LT, SHIFT>;
 template <typename LT, bool SHIFT> constexpr RowPass kManyDrafts = !SHIFT && sizeof(LT) == 2 ? kRing : kManyRows<LT, SHIFT>;
-constexpr int kRowRingVocab = 24576;
+constexpr int kRowRingVocab = 40960;   // (draft_threads: 128 threads in more than a wave of rows)
 template <int THREADS, RowPass PASS> constexpr int kRowRingBytes = PASS == kRing ? THREADS / 32 * kRowWarpBytes : 0;
 
 // late (kRing): whether a bulk copy did not arrive within its bounded wait (the results are of the part in front of it).
@@ -739,10 +742,14 @@ __device__ __forceinline__ void lean_pass_a_ck(const ROW &rq, int lo, int hi, in
     bool missing = false;
     LeanBatch<LT> B(st);
     auto begin = [&](const Vec8<LT> &first) { reference(first); B.begin(k); };
-    auto one = [&](const Vec8<LT> &v) { B.push(v); };
+    constexpr bool kByVector = SHIFT && PASS == kTurns;   // (the same sums)
+    auto one = [&](const Vec8<LT> &v) {
+        if constexpr (kByVector) lean_push(st, v, k);
+        else B.push(v);
+    };
     auto batch = [&](const auto &in, int vi) {
         constexpr int D = std::decay_t<decltype(in)>::kDepth;
-        B.template commit<D>(in, k, vi, hi);
+        if constexpr (!kByVector) B.template commit<D>(in, k, vi, hi);
         since += D;
         if (since >= CK) { checkpoint(); since = 0; B.again(); }
     };
