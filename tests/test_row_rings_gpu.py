@@ -1,6 +1,6 @@
 """Draft step and leaf rows by the shape of their CTAs: one warp per row; passes that take their rows from rings of bulk
-copies (bf16 rows in whole words, more rows than one wave of CTAs of 64 or 128 threads); rows that come with the next
-vectors in registers.  Rows at which a warp's last chunk or batch is full, one vector long or missing, and rows that are hard
+copies (draft step, bf16 rows in whole words of 40960 ids and more, more rows than one wave of CTAs of 128 threads); rows that
+come with the next vectors in registers.  Rows at which a warp's last chunk or batch is full, one vector long or missing, and rows that are hard
 on sums and references, against the oracle on a sample; the three-method draft step bit for bit."""
 import numpy as np
 import pytest
@@ -14,9 +14,10 @@ from test_compare_gpu import METHODS, bits, separate_draft  # noqa: E402
 from test_parity_gpu import random_logits, random_uniforms, sh  # noqa: E402,F401
 from test_streaming_gpu import check_more_drafts, check_two_drafts, hard_rows, sample  # noqa: E402
 
-# A chunk is 1024 ids of a warp's range.  Seven rows per sequence: 340 sequences fill more than a wave of 64 threads (below
+# A chunk of a ring, as a batch of vectors, is 1024 ids of a warp's range.  Seven rows per sequence: 340 sequences fill more than a wave of 64 threads (below
 # 40960 ids; below 10240 ids only leaf rows take those, draft steps one warp), 170 more than one of 128, 90 less than that.
-SIZES = [(4104, 340), (6144, 340), (10248, 340), (12288, 340), (12296, 340), (16384, 170), (16392, 170), (16416, 170), (40968, 170),
+SIZES = [(4104, 340), (6144, 340), (10248, 340), (12288, 340), (12296, 340), (16384, 170), (16392, 170), (16416, 170), (40960, 170),
+         (40968, 170), (40992, 170),
          (8192, 90), (8200, 90), (16392, 90), (40960, 90)]
 
 
@@ -33,7 +34,7 @@ def test_two_drafts(sh, V, B):  # noqa: F811
     un = random_uniforms(rng, B, N)
     pick = sample(rng, B, 4, 6)
     for leaves in (False, True):
-        check_two_drafts(sh, lp, lq, "bf16", 0, 0.8, un, leaves, pick, "rings")
+        check_two_drafts(sh, lp, lq, "bf16", 0, 0.8, un, leaves, pick, "passes")
 
 
 # one warp per row: bf16 in whole words, below 10240 ids in more than 1184 rows; beside it rows that do not take it
@@ -80,7 +81,7 @@ def test_shifted_rows(sh, V, B, dtype):  # noqa: F811
 
 
 # (rows: three per sequence) one warp; 64 threads, leaf rows only and all; 128 threads, more than a wave and less
-MANY = [(4104, 410), (9000, 410), (4104, 810), (12296, 810), (16392, 410), (16392, 230)]
+MANY = [(4104, 410), (9000, 410), (4104, 810), (12296, 810), (16392, 410), (16392, 230), (40968, 410)]
 
 
 @pytest.mark.parametrize("V,B", MANY)
@@ -94,7 +95,7 @@ def test_hard_rows(sh, V, B):  # noqa: F811
         check_two_drafts(sh, lp, lq, "bf16", 0, 1.0, un, leaves, pick, "hard", stats=True)
 
 
-@pytest.mark.parametrize("V,B", MANY[1:] + [(40960, 800), (40968, 410), (32000, 130), (32000, 90)])
+@pytest.mark.parametrize("V,B", MANY[1:] + [(40960, 800), (40992, 410), (32000, 130), (32000, 90)])
 def test_three_methods(sh, V, B):  # noqa: F811
     rng = np.random.default_rng(V + B + 1)
     _, lq = random_logits(rng, B, 3, V, "bf16")
