@@ -44,7 +44,9 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) fused_verify_kernel(F
     using V = Vec8<__nv_bfloat16>;
     const StreamRow<__nv_bfloat16, false> vp(rowp, a.vocab), vq(rowq, a.vocab);
     const Geo g = make_geo(a.vocab, 8);
-    const int warp = warp_index(), lane = threadIdx.x & 31;
+    // (Known to be the same in every lane only where pass A reads one row, whose loop asks whole warps: 3968 rows of 128256 ids
+    // 902 -> 894 us; from the draft row, too, 1984 rows of 128256 579 -> 609, 7936 of 32000 603 -> 623.)
+    const int warp = STATS ? warp_index() : static_cast<int>(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int lo = g.seg_lo(warp), hi = g.seg_hi(warp);
     const int last_vi = (lo + lane < hi) ? lo + lane + ((hi - 1 - lo - lane) / 32) * 32 : lo - 1;
     const float k = kLog2e / temperature_of(a, b);
